@@ -164,12 +164,10 @@ def field_and_particles(with_f64=False):
     return (field, pos, f64) if with_f64 else (field, pos)
 
 
-STEP_KERNELS = {"column": ("k_column<6,5,RK2> (float32 field)", "k_column_rk2_f32_i6",
-                            ("column_kernel.cuh", "column_i6.cu", "block_kernel.cuh", "internal.cuh", "coeffs.inc")),
-                "block": ("k_block<float,6,5,RK2,F32>", "k_block_rk2_f32_i6",
-                          ("block_kernel.cuh", "block_i6.cu", "internal.cuh", "coeffs.inc")),
-                "direct": ("k_direct<float,6,5,RK2,F32>", "k_direct_rk2_f32_i6",
-                           ("block_kernel.cuh", "direct_i6.cu", "internal.cuh", "coeffs.inc"))}
+_CORE = ("interp_core.cuh", "internal.cuh", "coeffs.inc", "block_kernel.cuh")
+STEP_KERNELS = {"column": ("k_slabs<6,5,RK2> (column order)", "k_slabs_rk2_f32_i6", _CORE),
+                "block": ("k_slabs<6,5,RK2>", "k_slabs_rk2_f32_i6", _CORE),
+                "direct": ("k_direct<float,6,5,RK2,F32>", "k_direct_rk2_f32_i6", _CORE + ("direct_kernel.cuh",))}
 
 
 def kernel_source_sha(kind="column"):
@@ -462,9 +460,6 @@ def run_gb300(args):
     achieved = alg_bytes / avg_launch_s / 1e9
     kind = kernel_name(trk, tr)
     kernel_label = STEP_KERNELS[kind][0]
-    if kind == "direct":   # node loads through the texture object (most of the rows) or plain loads
-        notes["direct_node_loads"] = "texture" if tr.field_texture() else "plain"
-        kernel_label = kernel_label[:-1] + (",NM_TEX4>" if tr.field_texture() else ",NM_VEC4>")
     sha = kernel_source_sha(kind)
     gather_bytes = NP * 2 * I ** 3 * 3 * 4            # two stencil gathers per RK2 step, float32
     sm_mhz = clk.get("sm_mhz") or 1900.0
@@ -546,9 +541,7 @@ def run_gb300(args):
             "smem_roofline": {"achieved": gather_bytes / avg_launch_s / 1e9, "peak": smem_peak, "unit": "GB/s",
                               "frac": gather_bytes / avg_launch_s / 1e9 / smem_peak,
                               "gather_bytes_per_launch": gather_bytes,
-                              "path": "shared memory" if kind != "direct" else
-                              ("L1 (gathers: texture and load/store data paths)" if notes.get("direct_node_loads") ==
-                               "texture" else "L1 (global gathers)"),
+                              "path": "shared memory" if kind != "direct" else "L1 (global gathers)",
                               "peak_def": "SMs x 128 B/clk (the L1 / shared-memory data path) x median SM clock under load"},
             "phase_ms_per_step": {"step_kernel": step_ms / args.inner, "binning": prof["bin"][0] / args.inner,
                                   "other": prof["other"][0] / args.inner, "profiled_calls": psteps,
@@ -899,8 +892,6 @@ def config6_block(trk, dev, stream, dev_index, args, fma, Ns=None):
         call()
     sync_flags(t, trk, notes)
     kind = kernel_name(trk, t)
-    if kind == "direct":
-        notes["direct_node_loads"] = "texture" if t.field_texture() else "plain"
     ms, reps, clk = timed(call, stream, dev_index, min_s=0.6, max_reps=20)
     prof = profiled(t, trk, call)
     sync_flags(t, trk, notes)

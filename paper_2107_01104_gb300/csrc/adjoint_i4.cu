@@ -5,8 +5,8 @@ namespace trk {
 
 cudaError_t launch_adjoint_i4(const AdjArgs& a, int64_t nblocks, int deg_hi, cudaStream_t st)
 {
-    if (deg_hi) return dispatch_adjoint<4, 4 + 1>(a, nblocks, st);
-    return dispatch_adjoint<4, 4 - 1>(a, nblocks, st);
+    if (deg_hi) return adj::dispatch_adjoint<4, 4 + 1>(a, nblocks, st);
+    return adj::dispatch_adjoint<4, 4 - 1>(a, nblocks, st);
 }
 
 }  // namespace trk

@@ -36,6 +36,467 @@
 #include "block_kernel.cuh"
 
 namespace trk {
+namespace adj {
+
+constexpr int NT = 256;           // threads per CTA
+constexpr int NW = NT / 32;       // warps per CTA
+
+constexpr bool distinct_banks(const int* offs, int n)
+{
+    bool seen[32] = {};
+    for (int l = 0; l < n; ++l) {
+        int b = ((offs[l] % 32) + 32) % 32;
+        if (seen[b]) return false;
+        seen[b] = true;
+    }
+    return true;
+}
+
+template <int I>
+constexpr bool row_ok(int S2)
+{
+    int offs[32] = {};
+    if (I == 8) {
+        for (int l = 0; l < 32; ++l) offs[l] = (l & 7) + S2 * (l >> 3);
+        return distinct_banks(offs, 32);
+    } else if (I == 6) {
+        for (int l = 0; l < 30; ++l) offs[l] = (l % 6) + S2 * (l / 6);
+        return distinct_banks(offs, 30);
+    } else {
+        for (int l = 0; l < 16; ++l) offs[l] = (l & 3) + S2 * ((l >> 2) & 3);
+        return distinct_banks(offs, 16);
+    }
+}
+
+template <int I>
+constexpr bool plane_ok(int S2, int S3)
+{
+    int offs[32] = {};
+    if (I == 8) {
+        return true;
+    } else if (I == 6) {
+        for (int l = 0; l < 30; ++l) offs[l] = (l % 6) + S3 * (l / 6);
+        return distinct_banks(offs, 30);
+    } else {
+        for (int l = 0; l < 32; ++l) offs[l] = (l & 3) + S2 * ((l >> 2) & 3) + S3 * (l >> 4);
+        return distinct_banks(offs, 32);
+    }
+}
+
+template <int I>
+constexpr int find_s3(int H, int S2)
+{
+    for (int s = S2 * H; s < S2 * H + 64; ++s)
+        if (plane_ok<I>(S2, s)) return s;
+    return -1;
+}
+
+template <int I>
+constexpr int find_s2(int H)
+{
+    for (int s = H; s < H + 64; ++s)
+        if (row_ok<I>(s) && find_s3<I>(H, s) > 0) return s;
+    return -1;
+}
+
+template <int I, int H>
+struct Layout {
+    static constexpr int S2 = find_s2<I>(H);
+    static constexpr int S3 = find_s3<I>(H, S2);
+    static constexpr int SC = S3 * H;
+    static_assert(S2 > 0 && S3 > 0, "no conflict-free halo layout");
+};
+
+template <typename T, int S2_, int S3_, int SC_>
+struct SmemLd {
+    static constexpr int S2 = S2_, S3 = S3_, SC = SC_;
+    static constexpr bool kShared = true, kNode4 = false;
+    const T* base;
+    __device__ __forceinline__ T operator()(int k, int a1, int a2, int a3) const
+    {
+        return base[k * SC + a3 * S3 + a2 * S2 + a1];
+    }
+};
+
+
+// Stencils from the stored field: three components of node c + a - (I/2 - 1)
+template <typename T, int STORE, int I>
+struct GlobalLd {
+    static constexpr bool kShared = false;
+    FieldView f;
+    int base;
+    __device__ __forceinline__ T operator()(int k, int a1, int a2, int a3) const
+    {
+        const int64_t n = base + (a3 * f.NP + a2) * f.NP + a1;
+        if constexpr (STORE == ST_F64) return (T)__ldg(f.f64 + k * f.plane + n);
+        else {
+            const uint32_t w = __ldg(f.rec + 4 * n + k);
+            return STORE == ST_BF16X2 ? (T)bf16x2_value(w) : (T)__uint_as_float(w);
+        }
+    }
+};
+
+template <typename T, int STORE, int I>
+__device__ __forceinline__ GlobalLd<T, STORE, I> field_ld(const FieldView& f, int c1, int c2, int c3)
+{
+    constexpr int LO = I / 2 - 1;
+    return GlobalLd<T, STORE, I>{f, (int)padded_index(f.NP, c1 - LO, c2 - LO, c3 - LO)};
+}
+
+// the halo of three components, through registers
+template <typename T, int STORE, int H, int S2, int S3, int SC>
+__device__ __forceinline__ void stage_halo(T* halo, const FieldView& f, int o1, int o2, int o3)
+{
+    const int64_t NP = f.NP;
+    for (int e = threadIdx.x; e < H * H * H; e += NT) {
+        const int x = e % H, y = e / H % H, z = e / (H * H);
+        const int64_t n = ((int64_t)(o3 + PAD + z) * NP + (o2 + PAD + y)) * NP + (o1 + PAD + x);
+        T v[3];
+        if constexpr (STORE == ST_F64) {
+            for (int k = 0; k < 3; ++k) v[k] = f.f64[k * f.plane + n];
+        } else {
+            unpack<STORE, 4, 3>(reinterpret_cast<const uint4*>(f.rec)[n], v);
+        }
+        for (int k = 0; k < 3; ++k) halo[k * SC + z * S3 + y * S2 + x] = v[k];
+    }
+}
+
+template <typename T, int I, int DEG, bool D>
+struct WeightEval {
+    Row<T, DEG> r, dr;
+    int ax, i;
+    bool act;
+    __device__ void init(const CoefTable<T>& tb, int lane)
+    {
+        act = lane < 3 * I;
+        ax = act ? lane / I : 0;
+        i = act ? lane % I : 0;
+        r = load_row<T, DEG>(tb.c, i);
+        if (D) dr = load_row<T, DEG>(tb.d, i);
+    }
+    __device__ __forceinline__ void eval(T s1, T s2, T s3, T* wv, T* wd) const
+    {
+        // every lane evaluates (idle lanes on a valid row) and only active lanes store
+        const T s = ax == 0 ? s1 : (ax == 1 ? s2 : s3);
+        const T w = horner(r, s);
+        T dw = 0;
+        if (D) dw = horner(dr, s);
+        __syncwarp();                        // previous readers of the buffer are done
+        if (act) wv[ax * 8 + i] = w;
+        if (D && act) wd[ax * 8 + i] = dw;
+        __syncwarp();
+    }
+    // value weights (no derivatives) of two points a and b into wva and wvb
+    __device__ __forceinline__ void eval_values2(const T (&sa)[3], const T (&sb)[3], T* wva, T* wvb) const
+    {
+        const T xa = ax == 0 ? sa[0] : (ax == 1 ? sa[1] : sa[2]);
+        const T xb = ax == 0 ? sb[0] : (ax == 1 ? sb[1] : sb[2]);
+        const T wa = horner(r, xa), wb = horner(r, xb);
+        __syncwarp();
+        if (act) {
+            wva[ax * 8 + i] = wa;
+            wvb[ax * 8 + i] = wb;
+        }
+        __syncwarp();
+    }
+};
+
+template <typename T, int I, bool D>
+struct Lane;
+
+template <typename T, bool D>
+struct Lane<T, 8, D> {
+    int i1, j;
+    T f[3][2][8];
+    __device__ void init(int lane)
+    {
+        i1 = lane & 7;
+        j = lane >> 3;
+    }
+    template <class LD>
+    __device__ __forceinline__ void load(const LD& ld)
+    {
+        if constexpr (LD::kShared) {
+            // one lane pointer, then compile-time offsets
+            const T* pa = ld.base + (i1 + j * LD::S2);
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int i3 = 0; i3 < 8; ++i3) f[k][h][i3] = pa[k * LD::SC + 4 * h * LD::S2 + i3 * LD::S3];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int i3 = 0; i3 < 8; ++i3) f[k][h][i3] = ld(k, i1, j + 4 * h, i3);
+        }
+    }
+    // transpose of the gather: add w(node) mu_k into every node this lane
+    // gathers; TWO adds wa(node) ma_k + wb(node) mb_k (two weight sets on the
+    // same stencil) with one add per node
+    template <bool TWO, class ADD>
+    __device__ __forceinline__ void scatter_n(const T* wa, const T (&ma)[3], const T* wb, const T (&mb)[3],
+                                              const ADD& add) const
+    {
+        const T w1a = wa[i1], w1b = TWO ? wb[i1] : (T)0;
+        T w3a[8], w3b[8];
+        bcast_load(wa + 16, w3a);
+        if (TWO) bcast_load(wb + 16, w3b);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const T a12a = w1a * wa[8 + j + 4 * h];
+            const T a12b = TWO ? w1b * wb[8 + j + 4 * h] : (T)0;
+#pragma unroll
+            for (int i3 = 0; i3 < 8; ++i3) {
+                const T wA = a12a * w3a[i3];
+                const T wB = TWO ? a12b * w3b[i3] : (T)0;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) add(k, i1, j + 4 * h, i3, TWO ? fma(wA, ma[k], wB * mb[k]) : wA * ma[k]);
+            }
+        }
+    }
+    __device__ __forceinline__ void contract(const T* wv, const T* wd, T (&acc)[12]) const
+    {
+        T w3[8], dw3[8];
+        bcast_load(wv + 16, w3);
+        if (D) bcast_load(wd + 16, dw3);
+        const T w1 = wv[i1];
+        const T w2[2] = {wv[8 + j], wv[12 + j]};
+        T dw1 = 0, dw2[2] = {0, 0};
+        if (D) {
+            dw1 = wd[i1];
+            dw2[0] = wd[8 + j];
+            dw2[1] = wd[12 + j];
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            T v = 0, d1 = 0, d2 = 0, d3 = 0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                T pv = 0, pd = 0;
+#pragma unroll
+                for (int i3 = 0; i3 < 8; ++i3) {
+                    pv = fma(w3[i3], f[k][h][i3], pv);
+                    if (D) pd = fma(dw3[i3], f[k][h][i3], pd);
+                }
+                v = fma(w1 * w2[h], pv, v);
+                if (D) {
+                    d1 = fma(dw1 * w2[h], pv, d1);
+                    d2 = fma(w1 * dw2[h], pv, d2);
+                    d3 = fma(w1 * w2[h], pd, d3);
+                }
+            }
+            acc[k] = v;
+            if (D) {
+                acc[3 + 3 * k + 0] = d1;
+                acc[3 + 3 * k + 1] = d2;
+                acc[3 + 3 * k + 2] = d3;
+            }
+        }
+    }
+};
+
+template <typename T, bool D>
+struct Lane<T, 6, D> {
+    int i1, j;
+    bool act, actc;
+    T f[3][8];                               // pass A (6), pass B, pass C
+    __device__ void init(int lane)
+    {
+        act = lane < 30;
+        actc = lane < 6;
+        i1 = lane % 6;                       // lanes 30, 31 duplicate lanes 0, 1
+        j = act ? lane / 6 : 0;
+    }
+    template <class LD>
+    __device__ __forceinline__ void load(const LD& ld)
+    {
+        if constexpr (LD::kShared) {
+            const T* pa = ld.base + (i1 + j * LD::S2);                  // pass A: row (i1, j)
+            const T* pb = ld.base + (i1 + 5 * LD::S2 + j * LD::S3);     // pass B: node (i1, 5, j)
+            const T* pc = ld.base + (i1 + 5 * LD::S2 + 5 * LD::S3);     // pass C: node (i1, 5, 5)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+#pragma unroll
+                for (int i3 = 0; i3 < 6; ++i3) f[k][i3] = pa[k * LD::SC + i3 * LD::S3];
+                f[k][6] = pb[k * LD::SC];
+                f[k][7] = pc[k * LD::SC];
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+#pragma unroll
+                for (int i3 = 0; i3 < 6; ++i3) f[k][i3] = ld(k, i1, j, i3);
+                f[k][6] = ld(k, i1, 5, j);
+                f[k][7] = ld(k, i1, 5, 5);
+            }
+        }
+    }
+    template <bool TWO, class ADD>
+    __device__ __forceinline__ void scatter_n(const T* wa, const T (&ma)[3], const T* wb, const T (&mb)[3],
+                                              const ADD& add) const
+    {
+        auto val = [&](T wA, T wB, int k) { return TWO ? fma(wA, ma[k], wB * mb[k]) : wA * ma[k]; };
+        const T w1a = wa[i1], w25a = wa[13];
+        const T w1b = TWO ? wb[i1] : (T)0, w25b = TWO ? wb[13] : (T)0;
+        T w3a[6], w3b[6];
+        bcast_load(wa + 16, w3a);
+        if (TWO) bcast_load(wb + 16, w3b);
+        if (act) {
+            const T a12a = w1a * wa[8 + j], a12b = TWO ? w1b * wb[8 + j] : (T)0;
+#pragma unroll
+            for (int i3 = 0; i3 < 6; ++i3) {
+                const T wA = a12a * w3a[i3], wB = TWO ? a12b * w3b[i3] : (T)0;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) add(k, i1, j, i3, val(wA, wB, k));
+            }
+            const T wA = w1a * w25a * wa[16 + j], wB = TWO ? w1b * w25b * wb[16 + j] : (T)0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) add(k, i1, 5, j, val(wA, wB, k));
+        }
+        if (actc) {
+            const T wA = w1a * w25a * w3a[5], wB = TWO ? w1b * w25b * w3b[5] : (T)0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) add(k, i1, 5, 5, val(wA, wB, k));
+        }
+    }
+    __device__ __forceinline__ void contract(const T* wv, const T* wd, T (&acc)[12]) const
+    {
+        T w3[6], dw3[6];
+        bcast_load(wv + 16, w3);
+        if (D) bcast_load(wd + 16, dw3);
+        const T w1 = wv[i1], w2j = wv[8 + j], w3j = wv[16 + j], w25 = wv[13];
+        const T z = 0;
+        // coefficients of the three passes (zero on idle lanes)
+        const T aA = act ? w1 * w2j : z;
+        const T aB = act ? w1 * w25 * w3j : z;
+        const T aC = actc ? w1 * w25 * w3[5] : z;
+        T dw1 = 0, dw2j = 0, dw3j = 0, dw25 = 0;
+        if (D) {
+            dw1 = wd[i1];
+            dw2j = wd[8 + j];
+            dw3j = wd[16 + j];
+            dw25 = wd[13];
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            T pv = 0, pd = 0;
+#pragma unroll
+            for (int i3 = 0; i3 < 6; ++i3) {
+                pv = fma(w3[i3], f[k][i3], pv);
+                if (D) pd = fma(dw3[i3], f[k][i3], pd);
+            }
+            acc[k] = fma(aA, pv, fma(aB, f[k][6], aC * f[k][7]));
+            if (D) {
+                const T b1 = act ? dw1 * w2j : z, b2 = act ? w1 * dw2j : z;
+                const T c1 = act ? dw1 * w25 * w3j : z, c2 = act ? w1 * dw25 * w3j : z, c3 = act ? w1 * w25 * dw3j : z;
+                const T e1 = actc ? dw1 * w25 * w3[5] : z, e2 = actc ? w1 * dw25 * w3[5] : z;
+                const T e3 = actc ? w1 * w25 * dw3[5] : z;
+                acc[3 + 3 * k + 0] = fma(b1, pv, fma(c1, f[k][6], e1 * f[k][7]));
+                acc[3 + 3 * k + 1] = fma(b2, pv, fma(c2, f[k][6], e2 * f[k][7]));
+                acc[3 + 3 * k + 2] = fma(aA, pd, fma(c3, f[k][6], e3 * f[k][7]));
+            }
+        }
+    }
+};
+
+template <typename T, bool D>
+struct Lane<T, 4, D> {
+    int i1, i2, p;
+    T f[3][2];
+    __device__ void init(int lane)
+    {
+        i1 = lane & 3;
+        i2 = (lane >> 2) & 3;
+        p = lane >> 4;
+    }
+    template <class LD>
+    __device__ __forceinline__ void load(const LD& ld)
+    {
+        if constexpr (LD::kShared) {
+            const T* pa = ld.base + (i1 + i2 * LD::S2 + p * LD::S3);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                f[k][0] = pa[k * LD::SC];
+                f[k][1] = pa[k * LD::SC + 2 * LD::S3];
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                f[k][0] = ld(k, i1, i2, p);
+                f[k][1] = ld(k, i1, i2, p + 2);
+            }
+        }
+    }
+    template <bool TWO, class ADD>
+    __device__ __forceinline__ void scatter_n(const T* wa, const T (&ma)[3], const T* wb, const T (&mb)[3],
+                                              const ADD& add) const
+    {
+        auto val = [&](T wA, T wB, int k) { return TWO ? fma(wA, ma[k], wB * mb[k]) : wA * ma[k]; };
+        const T a12a = wa[i1] * wa[8 + i2], a12b = TWO ? wb[i1] * wb[8 + i2] : (T)0;
+        const T w0a = a12a * wa[16 + p], w1a = a12a * wa[18 + p];
+        const T w0b = TWO ? a12b * wb[16 + p] : (T)0, w1b = TWO ? a12b * wb[18 + p] : (T)0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            add(k, i1, i2, p, val(w0a, w0b, k));
+            add(k, i1, i2, p + 2, val(w1a, w1b, k));
+        }
+    }
+    __device__ __forceinline__ void contract(const T* wv, const T* wd, T (&acc)[12]) const
+    {
+        const T w1 = wv[i1], w2 = wv[8 + i2];
+        const T w3a = wv[16 + p], w3b = wv[18 + p];
+        T dw1 = 0, dw2 = 0, dw3a = 0, dw3b = 0;
+        if (D) {
+            dw1 = wd[i1];
+            dw2 = wd[8 + i2];
+            dw3a = wd[16 + p];
+            dw3b = wd[18 + p];
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const T pv = fma(w3a, f[k][0], w3b * f[k][1]);
+            acc[k] = w1 * w2 * pv;
+            if (D) {
+                const T pd = fma(dw3a, f[k][0], dw3b * f[k][1]);
+                acc[3 + 3 * k + 0] = dw1 * w2 * pv;
+                acc[3 + 3 * k + 1] = w1 * dw2 * pv;
+                acc[3 + 3 * k + 2] = w1 * w2 * pd;
+            }
+        }
+    }
+};
+
+template <typename T>
+__device__ __forceinline__ T xor_shfl(T v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+
+template <typename T>
+__device__ __forceinline__ T reduce16(const T (&acc)[12], int lane)
+{
+    T v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = i < 12 ? acc[i] : (T)0;
+#pragma unroll
+    for (int lev = 0; lev < 4; ++lev) {
+        const int off = 16 >> lev;
+        const int half = 8 >> lev;
+        const bool hi = lane & off;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const T send = hi ? v[i] : v[i + half];
+            const T keep = hi ? v[i + half] : v[i];
+            v[i] = keep + xor_shfl(send, off);
+        }
+    }
+    v[0] += xor_shfl(v[0], 1);
+    return v[0];
+}
+
+__device__ __forceinline__ int pack_rel(int r1, int r2, int r3) { return r1 | (r2 << 8) | (r3 << 16); }
+__device__ __forceinline__ int pack_cell(int c1, int c2, int c3) { return c1 | (c2 << 10) | (c3 << 20); }
 
 constexpr int PBA = 128;   // particles per adjoint batch (keeps the float64 I = 8 plan under 227 KB)
 
@@ -113,12 +574,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
     Lane<T, I, true> L;
     L.init(lane);
 
-    constexpr bool ASYNC = STORE != ST_BF16X2;
     for (int batch = j0; batch < j1; batch += PBA) {
         const int nbat = min(PBA, j1 - batch);
-        // the first batch's halo copies run while P1 splits (later batches re-use the
-        // halo buffer as the previous batch's accumulator until it is flushed)
-        if (HALO && ASYNC && batch == j0) stage_halo<T, STORE, H, G, S2, S3, SC, 3, false>(halo, a.f, 0, 3, o1, o2, o3);
         // ---------------- P1 ----------------
         double lam[3] = {0, 0, 0};
         int id = 0;
@@ -138,28 +595,25 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
             const int r1 = (c[0] - o1) & mask, r2 = (c[1] - o2) & mask, r3 = (c[2] - o3) & mask;
             const bool in = HALO && r1 >= LO && r1 <= RMAX && r2 >= LO && r2 <= RMAX && r3 >= LO && r3 <= RMAX;
             const int rp = in ? pack_rel(r1, r2, r3) : -1;
-            if constexpr (sizeof(T) == 4) rec.relf = __int_as_float(rp);
-            else rec.relf = __longlong_as_double((long long)rp);
+            if constexpr (sizeof(T) == 4) rec.cell = __int_as_float(rp);
+            else rec.cell = __longlong_as_double((long long)rp);
             p_rec[tid] = rec;
             p_cell[tid] = pack_cell(c[0], c[1], c[2]);
         }
         if (batch != j0) __syncthreads();   // the accumulator of the previous batch is flushed
-        if constexpr (HALO) {
-            if (!ASYNC || batch != j0) stage_halo<T, STORE, H, G, S2, S3, SC, 3, true>(halo, a.f, 0, 3, o1, o2, o3);
-            else cp_async_wait_all();
-        }
+        if constexpr (HALO) stage_halo<T, STORE, H, S2, S3, SC>(halo, a.f, o1, o2, o3);
         __syncthreads();
         // ---------------- Q1: u(X), J(X), J(X*) ----------------
         for (int q = warp; q < nbat; q += NW) {
             const PRec<T> rec = p_rec[q];
             int rp;
-            if constexpr (sizeof(T) == 4) rp = __float_as_int(rec.relf);
-            else rp = (int)__double_as_longlong(rec.relf);
+            if constexpr (sizeof(T) == 4) rp = __float_as_int(rec.cell);
+            else rp = (int)__double_as_longlong(rec.cell);
             const int r1 = rp & 255, r2 = (rp >> 8) & 255, r3 = (rp >> 16) & 255;
             const int pc = p_cell[q];
             const int c1 = pc & 1023, c2 = (pc >> 10) & 1023, c3 = (pc >> 20) & 1023;
             if (rp >= 0) L.load(SL{halo + (r3 - LO) * S3 + (r2 - LO) * S2 + (r1 - LO)});
-            else L.load(global_ld<T, STORE, I>(a.f, c1, c2, c3, 0, 2));
+            else L.load(field_ld<T, STORE, I>(a.f, c1, c2, c3));
             W.eval(rec.t[0] - (T)0.5, rec.t[1] - (T)0.5, rec.t[2] - (T)0.5, wv, wd);
             T acc[12];
             L.contract(wv, wd, acc);
@@ -188,7 +642,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
                     // left the staged halo, or (direct) moved more than one cell
                     const bool far = HALO || abs(dc[0]) > 1 || abs(dc[1]) > 1 || abs(dc[2]) > 1;
                     if (far && lane == 0) atomicOr(a.flags + FLAG_CFL, 1);
-                    L.load(global_ld<T, STORE, I>(a.f, cs1, cs2, cs3, 0, 2));
+                    L.load(field_ld<T, STORE, I>(a.f, cs1, cs2, cs3));
                 }
             }
             W.eval(ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wv, wd);
@@ -201,8 +655,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
                 r2c.t[1] = ts[1];
                 r2c.t[2] = ts[2];
                 const int rp2 = in2 ? pack_rel(s1, s2, s3) : -1;
-                if constexpr (sizeof(T) == 4) r2c.relf = __int_as_float(rp2);
-                else r2c.relf = __longlong_as_double((long long)rp2);
+                if constexpr (sizeof(T) == 4) r2c.cell = __int_as_float(rp2);
+                else r2c.cell = __longlong_as_double((long long)rp2);
                 p_rec2[q] = r2c;
                 p_cell2[q] = pack_cell(cs1, cs2, cs3);
             }
@@ -255,8 +709,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
                 int rps[2];
 #pragma unroll
                 for (int stage = 0; stage < 2; ++stage) {
-                    if constexpr (sizeof(T) == 4) rps[stage] = __float_as_int(recs[stage].relf);
-                    else rps[stage] = (int)__double_as_longlong(recs[stage].relf);
+                    if constexpr (sizeof(T) == 4) rps[stage] = __float_as_int(recs[stage].cell);
+                    else rps[stage] = (int)__double_as_longlong(recs[stage].cell);
                 }
                 const T mus[2][3] = {{p_mu[q * 6 + 0], p_mu[q * 6 + 1], p_mu[q * 6 + 2]},
                                      {p_mu[q * 6 + 3], p_mu[q * 6 + 4], p_mu[q * 6 + 5]}};
@@ -316,8 +770,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
             int rps[2];
 #pragma unroll
             for (int stage = 0; stage < 2; ++stage) {
-                if constexpr (sizeof(T) == 4) rps[stage] = __float_as_int(recs[stage].relf);
-                else rps[stage] = (int)__double_as_longlong(recs[stage].relf);
+                if constexpr (sizeof(T) == 4) rps[stage] = __float_as_int(recs[stage].cell);
+                else rps[stage] = (int)__double_as_longlong(recs[stage].cell);
             }
             const T mus[2][3] = {{p_mu[q * 6 + 0], p_mu[q * 6 + 1], p_mu[q * 6 + 2]},
                                  {p_mu[q * 6 + 3], p_mu[q * 6 + 4], p_mu[q * 6 + 5]}};
@@ -502,4 +956,5 @@ cudaError_t dispatch_adjoint(const AdjArgs& a, int64_t nblocks, cudaStream_t st)
     return launch_adjoint_t<float, I, DEG, ST_BF16X2>(a, nblocks, st);
 }
 
+}  // namespace adj
 }  // namespace trk

@@ -13,6 +13,7 @@
 // batched sets).  The blocks and their offsets are those of the stable sort;
 // the order inside a block is not reproducible, and no result depends on it.
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -219,15 +220,18 @@ __global__ void __launch_bounds__(CT_THREADS) k_tile_scan(uint32_t* __restrict__
 // their writes are contiguous.  The order of the groups inside a block
 // follows the atomics (not reproducible); every particle's arithmetic is
 // independent of the order, so the step results do not depend on it.
-__global__ void k_scatter_state(int64_t np, const uint32_t* __restrict__ keys, int32_t* __restrict__ cursor,
-                                const double* __restrict__ pos_in, const int32_t* __restrict__ id_in,
-                                const float* __restrict__ rhs_in, int rhs_rows, double* __restrict__ pos_out,
-                                int32_t* __restrict__ id_out, float* __restrict__ rhs_out, int* flags)
+// RT: the type of the records (PRec) written beside the state, what the next
+// interpolation reads, or void for none.
+template <typename RT>
+__device__ __forceinline__ void write_record(const GridGeom& g, int64_t np, const double* pos, int64_t j, void* rec,
+                                             int64_t d, int* flags)
 {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const unsigned valid = __ballot_sync(0xffffffffu, j < np);
-    if (j >= np) return;
-    const uint32_t key = keys[j];
+    if constexpr (!std::is_void_v<RT>) reinterpret_cast<PRec<RT>*>(rec)[d] = split_record<RT>(g, np, pos, j, flags);
+}
+
+// the slot of particle j (< np) in its block, -1 (flagged) if its block is fuller than its count
+__device__ __forceinline__ int64_t take_slot(int64_t np, uint32_t key, unsigned valid, int32_t* cursor, int* flags)
+{
     const int lane = threadIdx.x & 31;
     const unsigned peers = __match_any_sync(valid, key);
     const int leader = __ffs(peers) - 1;
@@ -237,39 +241,45 @@ __global__ void k_scatter_state(int64_t np, const uint32_t* __restrict__ keys, i
     const int64_t d = (int64_t)base + __popc(peers & ((1u << lane) - 1u));
     if (d < 0 || d >= np) {
         atomicOr(flags + FLAG_BINNING, 1);
-        return;
+        return -1;
     }
+    return d;
+}
+
+template <typename RT>
+__global__ void k_scatter_state(GridGeom g, int64_t np, const uint32_t* __restrict__ keys, int32_t* __restrict__ cursor,
+                                const double* __restrict__ pos_in, const int32_t* __restrict__ id_in,
+                                const float* __restrict__ rhs_in, int rhs_rows, double* __restrict__ pos_out,
+                                int32_t* __restrict__ id_out, float* __restrict__ rhs_out, void* __restrict__ rec, int* flags)
+{
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned valid = __ballot_sync(0xffffffffu, j < np);
+    if (j >= np) return;
+    const int64_t d = take_slot(np, keys[j], valid, cursor, flags);
+    if (d < 0) return;
 #pragma unroll
     for (int a = 0; a < 3; ++a) pos_out[a * np + d] = pos_in[a * np + j];
     id_out[d] = id_in ? id_in[j] : (int32_t)j;
     for (int r = 0; r < rhs_rows; ++r) rhs_out[r * np + d] = rhs_in[r * np + j];
+    write_record<RT>(g, np, pos_in, j, rec, d, flags);
 }
 
 // Counting-sort permutation: perm[d] = j, d the next free slot of particle
-// j's block (cursor from the count scan).  Warp-aggregated like
+// j's block (cursor from the count scan), and its record.  Warp-aggregated like
 // k_scatter_state; the order inside a block follows the atomics.  Used where
 // every particle's result is independent of that order (interpolation, the
-// adjoint, batched sets): the blocks and their offsets are those of the
-// stable sort.
-__global__ void k_scatter_perm(int64_t np, const uint32_t* __restrict__ keys, int32_t* __restrict__ cursor,
-                               int32_t* __restrict__ perm, int* flags)
+// adjoint): the blocks and their offsets are those of the stable sort.
+template <typename RT>
+__global__ void k_scatter_perm(GridGeom g, int64_t np, const uint32_t* __restrict__ keys, int32_t* __restrict__ cursor,
+                               const double* __restrict__ pos, int32_t* __restrict__ perm, void* __restrict__ rec, int* flags)
 {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned valid = __ballot_sync(0xffffffffu, j < np);
     if (j >= np) return;
-    const uint32_t key = keys[j];
-    const int lane = threadIdx.x & 31;
-    const unsigned peers = __match_any_sync(valid, key);
-    const int leader = __ffs(peers) - 1;
-    int base = 0;
-    if (lane == leader) base = atomicAdd(cursor + key, __popc(peers));
-    base = __shfl_sync(peers, base, leader);
-    const int64_t d = (int64_t)base + __popc(peers & ((1u << lane) - 1u));
-    if (d < 0 || d >= np) {
-        atomicOr(flags + FLAG_BINNING, 1);
-        return;
-    }
+    const int64_t d = take_slot(np, keys[j], valid, cursor, flags);
+    if (d < 0) return;
     perm[d] = (int32_t)j;
+    write_record<RT>(g, np, pos, j, rec, d, flags);
 }
 
 // Block counts of np keys, one atomic add per group of equal keys in a warp
@@ -470,53 +480,41 @@ __global__ void k_unpermute_rhs(int64_t np, const float* __restrict__ src, const
 
 // Fills the ghost-padded storage: padded node (x1, x2, x3) in [-PAD, N+PAD)^3
 // takes the value of node (x mod N) of the dense source (periodic ghosts).
+// blockIdx.z is the padded x3 plane, blockIdx.y counts groups of blockDim.y
+// padded rows, threads run along x1: reads are coalesced per component, a
+// record is one 16-byte (C = 1: 4-byte) store, and nothing divides.
+__device__ __forceinline__ uint32_t stored_word(int storage, float x)
+{
+    if (storage == ST_F32) return __float_as_uint(x);
+    // split of the float32-rounded value: hi = RN_bf16(x), lo = RN_bf16(x - hi)
+    const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+    const __nv_bfloat16 lo = __float2bfloat16_rn(x - __bfloat162float(hi));
+    return (uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(lo) << 16);
+}
+
 template <typename S>
 __global__ void k_convert_padded(int storage, const S* __restrict__ src, int C, int N, void* __restrict__ dst)
 {
-    const int NP = N + 2 * PAD;
-    const int64_t plane = (int64_t)NP * NP * NP;
-    const int64_t total = plane * C;
-    const int mask = N - 1;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = i / plane, r = i - k * plane;
-        const int x3 = (int)(r / ((int64_t)NP * NP)), r2 = (int)(r - (int64_t)x3 * NP * NP);
-        const int x2 = r2 / NP, x1 = r2 - x2 * NP;
-        const int64_t si = (((int64_t)k * N + ((x3 - PAD) & mask)) * N + ((x2 - PAD) & mask)) * N + ((x1 - PAD) & mask);
-        const S x = src[si];
+    const int NP = N + 2 * PAD, mask = N - 1;
+    const int z = blockIdx.z, y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (y >= NP) return;
+    const int64_t plane = (int64_t)NP * NP * NP, n3 = (int64_t)N * N * N;
+    const int64_t row = ((int64_t)z * NP + y) * NP;
+    const S* s = src + ((int64_t)((z - PAD) & mask) * N + ((y - PAD) & mask)) * N;
+    for (int x = threadIdx.x; x < NP; x += blockDim.x) {
+        const S* sx = s + ((x - PAD) & mask);
         if (storage == ST_F64) {
-            reinterpret_cast<double*>(dst)[i] = (double)x;
-        } else if (storage == ST_F32) {
-            reinterpret_cast<float*>(dst)[i] = (float)x;
+            for (int k = 0; k < C; ++k) reinterpret_cast<double*>(dst)[k * plane + row + x] = (double)sx[k * n3];
+        } else if (C == 1) {
+            reinterpret_cast<uint32_t*>(dst)[row + x] = stored_word(storage, (float)sx[0]);
         } else {
-            // split of the float32-rounded value: hi = RN_bf16(x), lo = RN_bf16(x - hi)
-            const float xf = (float)x;
-            const __nv_bfloat16 hi = __float2bfloat16_rn(xf);
-            const __nv_bfloat16 lo = __float2bfloat16_rn(xf - __bfloat162float(hi));
-            reinterpret_cast<__nv_bfloat16*>(dst)[i] = hi;
-            reinterpret_cast<__nv_bfloat16*>(dst)[total + i] = lo;
-        }
-    }
-}
-
-// nm[i][k] = f[k][i] (k < C), 0 for C <= k < nmc: each thread one node, reads
-// coalesced per component, writes its nmc values contiguously
-__global__ void k_node_major(const float* __restrict__ f, int C, int nmc, int64_t plane, float* __restrict__ nm)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < plane; i += (int64_t)gridDim.x * blockDim.x)
-        for (int k = 0; k < nmc; ++k) nm[i * nmc + k] = k < C ? f[k * plane + i] : 0.0f;
-}
-
-// node i: the hi and lo halves of its three components, interleaved, then two zeros
-__global__ void k_node_major_bf16(const __nv_bfloat16* __restrict__ hi, const __nv_bfloat16* __restrict__ lo,
-                                  int64_t plane, uint4* __restrict__ nm)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < plane; i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t w[3];
+            for (int k0 = 0; k0 < C; k0 += 4) {
+                uint32_t w[4];
 #pragma unroll
-        for (int k = 0; k < 3; ++k)
-            w[k] = (uint32_t)__bfloat16_as_ushort(hi[k * plane + i]) |
-                   ((uint32_t)__bfloat16_as_ushort(lo[k * plane + i]) << 16);
-        nm[i] = make_uint4(w[0], w[1], w[2], 0u);
+                for (int k = 0; k < 4; ++k) w[k] = k0 + k < C ? stored_word(storage, (float)sx[(k0 + k) * n3]) : 0u;
+                reinterpret_cast<uint4*>(dst)[(k0 / 4) * plane + row + x] = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+        }
     }
 }
 
@@ -566,13 +564,15 @@ cudaError_t launch_count_scan(uint32_t* counts, int64_t nblocks, int32_t* offset
     return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_state(int64_t np, const uint32_t* keys, int32_t* cursor, const double* pos_in,
-                                 const int32_t* id_in, const float* rhs_in, int rhs_rows, double* pos_out,
-                                 int32_t* id_out, float* rhs_out, int* flags, cudaStream_t st)
+cudaError_t launch_scatter_state(const GridGeom& g, int64_t np, const uint32_t* keys, int32_t* cursor,
+                                 const double* pos_in, const int32_t* id_in, const float* rhs_in, int rhs_rows,
+                                 double* pos_out, int32_t* id_out, float* rhs_out, void* rec, int rec_f64, int* flags,
+                                 cudaStream_t st)
 {
     if (np <= 0) return cudaSuccess;
-    k_scatter_state<<<grid_for(np, 256), 256, 0, st>>>(np, keys, cursor, pos_in, id_in, rhs_in, rhs_in ? rhs_rows : 0,
-                                                      pos_out, id_out, rhs_out, flags);
+    auto kern = rec_f64 ? k_scatter_state<double> : k_scatter_state<float>;
+    kern<<<grid_for(np, 256), 256, 0, st>>>(g, np, keys, cursor, pos_in, id_in, rhs_in, rhs_in ? rhs_rows : 0, pos_out,
+                                            id_out, rhs_out, rec, flags);
     return cudaGetLastError();
 }
 
@@ -632,11 +632,12 @@ cudaError_t launch_offsets(const uint32_t* keys_sorted, int64_t n, int64_t nbloc
     return cudaGetLastError();
 }
 
-cudaError_t launch_scatter_perm(int64_t np, const uint32_t* keys, int32_t* cursor, int32_t* perm, int* flags,
-                                cudaStream_t st)
+cudaError_t launch_scatter_perm(const GridGeom& g, int64_t np, const uint32_t* keys, int32_t* cursor, const double* pos,
+                                int32_t* perm, void* rec, int rec_f64, int* flags, cudaStream_t st)
 {
     if (np <= 0) return cudaSuccess;
-    k_scatter_perm<<<grid_for(np, 256), 256, 0, st>>>(np, keys, cursor, perm, flags);
+    auto kern = !rec ? k_scatter_perm<void> : (rec_f64 ? k_scatter_perm<double> : k_scatter_perm<float>);
+    kern<<<grid_for(np, 256), 256, 0, st>>>(g, np, keys, cursor, pos, perm, rec, flags);
     return cudaGetLastError();
 }
 
@@ -661,27 +662,14 @@ cudaError_t launch_unpermute_rhs(int64_t np, const float* src, const int32_t* id
     return cudaGetLastError();
 }
 
-cudaError_t launch_node_major(const float* f, int C, int nmc, int64_t plane, float* nm, cudaStream_t st)
-{
-    k_node_major<<<(unsigned)std::min<int64_t>(ceil_div(plane, 256), 1 << 20), 256, 0, st>>>(f, C, nmc, plane, nm);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_node_major_bf16(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int64_t plane, void* nm,
-                                   cudaStream_t st)
-{
-    k_node_major_bf16<<<(unsigned)std::min<int64_t>(ceil_div(plane, 256), 1 << 20), 256, 0, st>>>(
-        hi, lo, plane, reinterpret_cast<uint4*>(nm));
-    return cudaGetLastError();
-}
-
 cudaError_t launch_convert_field(int storage, int src_f64, const void* src, int C, int N, void* dst, cudaStream_t st)
 {
-    const int64_t NP = N + 2 * PAD;
-    const int64_t n = NP * NP * NP * C;
-    const unsigned grid = (unsigned)std::min<int64_t>(ceil_div(n, 256), 152 * 64);
-    if (src_f64) k_convert_padded<double><<<grid, 256, 0, st>>>(storage, reinterpret_cast<const double*>(src), C, N, dst);
-    else k_convert_padded<float><<<grid, 256, 0, st>>>(storage, reinterpret_cast<const float*>(src), C, N, dst);
+    const int NP = N + 2 * PAD;
+    const int tx = std::min(256, (NP + 31) / 32 * 32), ty = 256 / tx;
+    const dim3 block((unsigned)tx, (unsigned)ty);
+    const dim3 grid(1, (unsigned)((NP + ty - 1) / ty), (unsigned)NP);
+    if (src_f64) k_convert_padded<double><<<grid, block, 0, st>>>(storage, reinterpret_cast<const double*>(src), C, N, dst);
+    else k_convert_padded<float><<<grid, block, 0, st>>>(storage, reinterpret_cast<const float*>(src), C, N, dst);
     return cudaGetLastError();
 }
 

@@ -1,14 +1,13 @@
-// Block kernels for kernel width I = 8 (all storages and modes).
-#include "block_kernel.cuh"
+// Block kernels for kernel width I = 8, weights of degree I - 1
+// (all storages and modes).
+#include "direct_kernel.cuh"
 
 namespace trk {
 
-cudaError_t launch_block_i8(int mode, const BlockArgs& a, const void* tmap, int64_t nblocks, int deg_hi,
-                            cudaStream_t st)
+cudaError_t launch_block_i8(int mode, const BlockArgs& a, const void* tmap, int64_t nblocks, cudaStream_t st)
 {
     const CUtensorMap* m = static_cast<const CUtensorMap*>(tmap);
-    if (deg_hi) return dispatch_store_mode<8, 8 + 1>(mode, a, m, nblocks, st);
-    return dispatch_store_mode<8, 8 - 1>(mode, a, m, nblocks, st);
+    return dispatch_mode<8, 7>(mode, a.f, GoBlock<8, 7>{a, m, nblocks, st});
 }
 
 }  // namespace trk

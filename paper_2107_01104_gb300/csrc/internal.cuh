@@ -36,20 +36,25 @@ constexpr int LBLK = 3;       // log2(BLK)
 // x in [-PAD, N + PAD) lives at k * plane + ((x3 + PAD) * NP + (x2 + PAD)) * NP + (x1 + PAD).
 constexpr int PAD = 8;
 
+//
+// Float64 fields are stored component-major, [C][NP^3].  Float32 and split-bf16
+// fields are stored as node records, the layout every kernel gathers: four
+// components per 16-byte record (C = 1: one per 4-byte record), chunk ch
+// holding components 4 ch .. 4 ch + 3 of every node, absent components zero,
+// [chunks][NP^3] records.  A word is a float32 value, or a split-bf16 pair
+// (hi in the low half, lo in the high half).  One stencil row of I nodes is
+// then one contiguous run whatever the component.
 struct FieldView {
     int storage;              // ST_*
     int C;                    // components
     int NP;                   // padded extent N + 2 PAD
-    int64_t plane;            // NP^3 values per component
-    const double* f64;        // [C][NP^3]                (ST_F64)
-    const float* f32;         // [C][NP^3]                (ST_F32)
-    const __nv_bfloat16* hi;  // [C][NP^3] high parts     (ST_BF16X2)
-    const __nv_bfloat16* lo;  // [C][NP^3] low parts      (ST_BF16X2)
-    const float* nm;          // node-major copy for the direct path, or null: float32 fields [NP^3][nmc];
-                              // split-bf16 fields with C = 3: 16 bytes per node (hi0 lo0 hi1 lo1 hi2 lo2 0 0)
-    int nmc;                  // float32: floats per node in nm, 4 for C = 3 (one 16-byte load per node), else C
-    unsigned long long nm_tex; // texture object over nm (16-byte texels, C = 3), or 0 for plain loads
+    int64_t plane;            // NP^3 nodes
+    const double* f64;        // [C][NP^3]                        (ST_F64)
+    const uint32_t* rec;      // [chunks][NP^3][4] (C = 1: [NP^3]) (ST_F32, ST_BF16X2)
 };
+
+__host__ __device__ constexpr int record_width(int C) { return C == 1 ? 1 : 4; }
+__host__ __device__ constexpr int record_chunks(int C) { return (C + 3) / 4; }
 
 __host__ __device__ __forceinline__ int64_t padded_index(int NP, int x1, int x2, int x3)
 {
@@ -57,93 +62,31 @@ __host__ __device__ __forceinline__ int64_t padded_index(int NP, int x1, int x2,
 }
 
 // ---------------------------------------------------------------------------
-// Halo box of the block kernel's TMA staging (cp.async.bulk.tensor): one
-// tensor copy per component chunk writes a dense box [3][H][BY][BX] of the
-// padded field into shared memory.  The box starts XOFF elements before the
-// halo (its x origin rounded down to 16 bytes, as a tensor copy must be);
-// BX (a multiple of 16 bytes) and BY >= H are padded so that the warp-wide
-// stencil loads of the lane map of kernel width I meet as few shared-memory
-// bank conflicts as the dense pitch allows (BX = row pitch, BX*BY = plane
-// pitch).  Used on the host to encode the tensor map and on the device for
-// the lane offsets.
+// Halo of an 8^3 cell block for kernel width I and stage-2 margin (0, or 1 for
+// RK2): H^3 nodes from G nodes before the block.  P is the row pitch of its
+// dense copy in shared memory (plane pitch P H): records, H; float64
+// elements, even, the halo starting XOFF elements into the row so that a
+// tensor copy starts on a 16-byte boundary.  Host: the tensor map's box;
+// device: the lane offsets.
 // ---------------------------------------------------------------------------
-// largest number of distinct words sharing a bank among `n` lane offsets
-// (in elements of esz bytes; a warp's 8-byte loads are served as two halves
-// of 16 lanes over 16 double-width banks)
-__host__ __device__ constexpr int bank_degree(const int* offs, int n, int esz)
-{
-    int worst = 0;
-    const int halves = esz == 8 ? 2 : 1, lanes = 32 / halves, banks = esz == 8 ? 16 : 32;
-    for (int h = 0; h < halves; ++h) {
-        for (int b = 0; b < banks; ++b) {
-            int seen[32] = {};
-            int ns = 0;
-            for (int l = h * lanes; l < (h + 1) * lanes && l < n; ++l) {
-                const int o = offs[l];
-                if (((o % banks) + banks) % banks != b) continue;
-                bool dup = false;
-                for (int q = 0; q < ns; ++q) dup = dup || seen[q] == o;
-                if (!dup && ns < 32) seen[ns++] = o;
-            }
-            worst = ns > worst ? ns : worst;
-        }
-    }
-    return worst;
-}
-
-// worst bank degree of the stencil loads of kernel width I for row pitch S2
-// and plane pitch S3 (the lane maps of Lane<T, I, D>::load)
-__host__ __device__ constexpr int lane_map_degree(int I, int S2, int S3, int esz)
-{
-    int worst = 0;
-    int offs[32] = {};
-    if (I == 8) {
-        for (int l = 0; l < 32; ++l) offs[l] = (l & 7) + S2 * (l >> 3);
-        worst = bank_degree(offs, 32, esz);
-    } else if (I == 6) {
-        for (int l = 0; l < 32; ++l) offs[l] = (l < 30 ? (l % 6) + S2 * (l / 6) : (l % 6));      // pass A
-        const int a = bank_degree(offs, 32, esz);
-        for (int l = 0; l < 32; ++l) offs[l] = (l < 30 ? (l % 6) + S3 * (l / 6) : (l % 6));      // pass B
-        const int b = bank_degree(offs, 32, esz);
-        worst = a > b ? a : b;
-    } else {
-        for (int l = 0; l < 32; ++l) offs[l] = (l & 3) + S2 * ((l >> 2) & 3) + S3 * (l >> 4);
-        worst = bank_degree(offs, 32, esz);
-    }
-    return worst;
-}
-
-struct TmaBox {
-    int H, XOFF, BX, BY;
-    __host__ __device__ constexpr int S2() const { return BX; }
-    __host__ __device__ constexpr int S3() const { return BX * BY; }
-    __host__ __device__ constexpr int SC() const { return BX * BY * H; }
+struct HaloBox {
+    int H, G, P, XOFF;
 };
 
-// The box for kernel width I, RK2 margin `margin` (0 or 1) and element size esz:
-// among row pitches up to 6 vectors beyond the minimum and plane heights up
-// to 8 rows beyond H, the lowest bank degree, then the smallest box.
-__host__ __device__ constexpr TmaBox tma_box(int I, int margin, int esz)
+__host__ __device__ constexpr HaloBox halo_box(int I, int margin, bool f64)
 {
-    const int H = 8 + I - 1 + 2 * margin;          // BLK + I - 1 + 2 margin
+    const int H = BLK + I - 1 + 2 * margin;
     const int G = I / 2 - 1 + margin;
-    const int VEC = 16 / esz;
-    const int XOFF = ((8 - G) % VEC + VEC) % VEC;   // PAD = 8
-    const int bx0 = (H + XOFF + VEC - 1) / VEC * VEC;
-    TmaBox best{H, XOFF, bx0, H};
-    int best_deg = 1 << 20, best_size = 1 << 30;
-    for (int bx = bx0; bx <= bx0 + 6 * VEC; bx += VEC)
-        for (int by = H; by <= H + 8; ++by) {
-            const int d = lane_map_degree(I, bx, bx * by, esz);
-            const int size = bx * by;
-            if (d < best_deg || (d == best_deg && size < best_size)) {
-                best_deg = d;
-                best_size = size;
-                best = TmaBox{H, XOFF, bx, by};
-            }
-        }
-    return best;
+    const int xoff = f64 ? (PAD - G) & 1 : 0;
+    const int P = f64 ? (H + xoff + 1) / 2 * 2 : H;
+    return HaloBox{H, G, P, xoff};
 }
+
+// x1 extent of the slabs the pipelined block kernel stages the halos of node records in
+__host__ __device__ constexpr int slab_width(int I) { return I == 4 ? 4 : 8; }
+
+// components per chunk of an interpolation (the steps take three)
+__host__ __device__ constexpr int chunk_components(int C) { return C == 1 ? 1 : (C <= 3 ? 3 : 4); }
 
 // Kernel weights beta_i(s), s = t - 1/2, as polynomial coefficients, passed by
 // value so that the kernels read them as constant-bank operands.
@@ -157,6 +100,7 @@ struct GridGeom {
     int N, mask;
     int lb1, lb2, lb3;        // log2 of the binning block edges
     int nb1, nb2, nb3;        // blocks per axis
+    int lseg;                 // log2 of the blocks along x3 whose rows of keys follow each other (0: x2 next)
     double inv_delta;         // fl(N / L)
 };
 
@@ -171,6 +115,7 @@ struct BlockArgs {
     const int32_t* perm;      // sorted position j -> index into the *_in arrays, or null (identity)
     const double* pos_in;     // [3][np]
     const int32_t* id_in;     // [np] or null (then id = perm[j])
+    const void* rec_in;       // [np] PRec (grouped) or null (then split from pos_in)
     const float* rhs_in;      // [ab_order-1][3][np] AB history (u_{n-1} first) or null
     double* pos_out;          // [3][np], written at j
     int32_t* id_out;          // [np], written at j
@@ -181,18 +126,13 @@ struct BlockArgs {
     int out_f64;
     int history_valid;        // AB: valid history entries on entry, 0 .. ab_order-1
     int ab_order;             // AB order k (2, 3, 4); the history holds k-1 entries
-    int ppc;                  // direct kernel: particles per CTA (1 .. 256; 0 means 256)
+    int ppc;                  // direct kernel: particles per CTA (a multiple of 16), 0 (by size) or PPC_WIDE
     double dt;
     int* flags;
 };
 
+constexpr int PPC_WIDE = -1;
 constexpr int AB_MAX_HIST = 3;   // history entries of the highest supported order (AB4)
-
-// where the direct path gathers a float32 stencil from: the component-major
-// field, the node-major copy per component, or the node-major copy as one
-// 16-byte load per node (three components padded to four floats), by plain
-// loads or by texture fetches (the same bits, on the texture data path)
-enum { NM_NONE = 0, NM_SCALAR = 1, NM_VEC4 = 2, NM_TEX4 = 3 };
 
 // dt-free Adams-Bashforth increment of order q (1..4): sum_j beta^q_j u_{n-j}
 // with u_n = f0 and u_{n-j} = hist(j - 1), summed newest first; beta^q are the
@@ -233,25 +173,11 @@ struct AdjArgs {
 // One particle set of a batched step, resident in device memory.
 struct BatchSet {
     BlockArgs a;              // set's step arguments (field, weights, state buffers)
-    const int32_t* list;      // non-empty blocks in key order (halo path)
-    const int32_t* count;     // number of non-empty blocks (device, halo path)
-    int n_items;              // number of 256-particle chunks (direct path)
-    int I, deg_hi, deriv, direct;
+    int n_items;              // work items of 128 particles
+    int I, deg_hi, deriv;
 };
 
-// Arguments of the column step kernel (RK2 / AB over column segments of cell
-// blocks, float32 fields, I = 4 or 6).  The state arrays a.pos_out / a.rhs_out
-// hold the particles grouped by block and are updated in place; a.perm and
-// a.id_* are unused (the scatter kernel has grouped the state).
-constexpr int MAXSEG = 64;    // largest column segment (slabs per work item)
-
-struct ColumnArgs {
-    BlockArgs a;
-    int nseg;                 // slabs per work item (divides nb3, <= MAXSEG)
-    int64_t nitems;           // work items: nb1 * nb2 * (nb3 / nseg)
-    int* ctr;                 // work counter, zero at launch
-    uint32_t* counts;         // [nblocks] block counts of the new keys (added into) or null
-};
+constexpr int MAXSEG = 64;    // largest column segment (blocks along x3)
 
 // ---------------------------------------------------------------------------
 // Cell split (Sec. 2.2 steps 1-3), bit-exact with the float64 reference:
@@ -280,22 +206,108 @@ __device__ __forceinline__ bool split_axis(double X, double inv_delta, int mask,
     return true;
 }
 
-// The cell only (for block keys): floor(g) by one conversion rounding down,
-// which equals floor then truncation for |g| < 2^51.
-__device__ __forceinline__ bool split_cell(double X, double inv_delta, int mask, int& c)
+// The same cell, and the offset t as a 32-bit fraction (truncated; the offset
+// of the float32 kernels, whose weights it enters with 24 bits): one float64
+// multiply, then integer shifts of the product's bits.  This GPU runs about
+// 1.7 float64 operations per clock and SM, so the floor, difference and
+// conversions of split_axis cost a particle ten clocks of that pipe, these
+// shifts one and a half issue slots.  |g| in [2^-11, 2^21), which is where
+// positions lie, is shifted; other products take the float64 operations.
+__device__ __forceinline__ bool split_fixed(double X, double inv_delta, int mask, int& c, uint32_t& frac)
 {
     const double g = __dmul_rn(X, inv_delta);
-    if (!cell_in_range(g)) {
-        c = 0;
-        return false;
+    const int hi = __double2hiint(g);
+    const uint32_t lo = (uint32_t)__double2loint(g);
+    const int s = 1043 - ((hi >> 20) & 0x7ff);        // |g| 2^32 = m >> s, m the 53-bit significand
+    if ((unsigned)s < 32u) {
+        const uint32_t mh = ((uint32_t)hi & 0xfffffu) | 0x100000u;
+        uint32_t f = __funnelshift_r(lo, mh, s), n = mh >> s;
+        if (hi < 0) {   // floor: -m, rounded down where bits were dropped
+            const uint32_t exact = (lo & ((1u << s) - 1u)) == 0u ? 1u : 0u;
+            f = ~f + exact;
+            n = ~n + (f == 0u ? exact : 0u);
+        }
+        c = (int)(n & (uint32_t)mask);
+        frac = f;
+        return true;
     }
-    c = (int)(__double2ll_rd(g) & (long long)mask);
+    c = 0;
+    frac = 0;
+    if (!cell_in_range(g)) return false;
+    const double c0 = floor(g);
+    c = (int)(__double2ll_rz(c0) & (long long)mask);
+    frac = __double2uint_rz(__dsub_rn(g, c0) * 4294967296.0);   // saturates at t = 1
     return true;
 }
 
+// The cell only (for block keys).
+__device__ __forceinline__ bool split_cell(double X, double inv_delta, int mask, int& c)
+{
+    uint32_t frac;
+    return split_fixed(X, inv_delta, mask, c, frac);
+}
+
+// the offset as the kernels of type T use it
+__device__ __forceinline__ bool split_offset(double X, double inv_delta, int mask, int& c, float& t)
+{
+    uint32_t frac;
+    const bool ok = split_fixed(X, inv_delta, mask, c, frac);
+    t = __uint2float_rn(frac) * 2.3283064365386963e-10f;   // 2^-32
+    return ok;
+}
+__device__ __forceinline__ bool split_offset(double X, double inv_delta, int mask, int& c, double& t)
+{
+    return split_axis(X, inv_delta, mask, c, t);
+}
+
+// Record of a particle: where it is, as the interpolation reads it.
+template <typename T>
+struct alignas(4 * sizeof(T)) PRec {
+    T t[3];         // offsets in the cell (Sec. 2.2 step 3, normalised by delta)
+    T cell;         // c1 | c2 << 10 | c3 << 20, bit-cast into T's storage
+};
+template <typename T>
+__device__ __forceinline__ T cell_as(int c)
+{
+    if constexpr (sizeof(T) == 4) return __int_as_float(c);
+    else return __longlong_as_double((long long)c);
+}
+__device__ __forceinline__ int cell_of(const PRec<float>& r) { return __float_as_int(r.cell); }
+__device__ __forceinline__ int cell_of(const PRec<double>& r) { return (int)__double_as_longlong(r.cell); }
+__device__ __forceinline__ void unpack_cell(int p, int (&c)[3])
+{
+    c[0] = p & 1023, c[1] = p >> 10 & 1023, c[2] = p >> 20 & 1023;
+}
+
+// the record of the position pos[3][np] of particle j (non-finite: cell 0, flagged)
+template <typename T>
+__device__ __forceinline__ PRec<T> split_record(const GridGeom& g, int64_t np, const double* pos, int64_t j, int* flags)
+{
+    PRec<T> rec;
+    int c[3];
+    bool ok = true;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) ok &= split_offset(pos[ax * np + j], g.inv_delta, g.mask, c[ax], rec.t[ax]);
+    if (!ok) atomicOr(flags + FLAG_NONFINITE, 1);
+    rec.cell = cell_as<T>(c[0] | c[1] << 10 | c[2] << 20);
+    return rec;
+}
+
+// float32 -> float64 by integer operations for normal numbers (exact)
+__device__ __forceinline__ double widen(float x)
+{
+    const uint32_t b = __float_as_uint(x), e = (b >> 23) & 0xffu;
+    if (e - 1u < 254u) return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+    return (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 __device__ __forceinline__ uint32_t block_key(const GridGeom& g, int c1, int c2, int c3)
 {
-    return (uint32_t)((((c3 >> g.lb3) * g.nb2) + (c2 >> g.lb2)) * g.nb1 + (c1 >> g.lb1));
+    const int b1 = c1 >> g.lb1, b2 = c2 >> g.lb2, b3 = c3 >> g.lb3;
+    // rows of blocks along x1; x3 inside a segment of 2^lseg blocks, then x2, the segments along x3
+    const int row = ((((b3 >> g.lseg) * g.nb2 + b2) << g.lseg) + (b3 & ((1 << g.lseg) - 1)));
+    return (uint32_t)(row * g.nb1 + b1);
 }
 
 // ---------------------------------------------------------------------------
@@ -321,13 +333,6 @@ cudaError_t launch_unpermute_rhs(int64_t np, const float* src, const int32_t* id
 
 // Fill the ghost-padded storage from a dense field src[C][N][N][N] (periodic ghosts).
 cudaError_t launch_convert_field(int storage, int src_f64, const void* src, int C, int N, void* dst, cudaStream_t st);
-// node-major copy nm[node][nmc] of the padded float32 field f[C][node] (plane nodes);
-// floats C .. nmc-1 of a node are zero
-cudaError_t launch_node_major(const float* f, int C, int nmc, int64_t plane, float* nm, cudaStream_t st);
-// node-major copy of a three-component split-bf16 field (hi planes, then lo planes): 16 bytes per node
-cudaError_t launch_node_major_bf16(const __nv_bfloat16* hi, const __nv_bfloat16* lo, int64_t plane, void* nm,
-                                   cudaStream_t st);
-
 // dLoss/dfield from the per-block partial sums: every node adds, in a fixed
 // order, the partials of the non-empty blocks whose halo holds it
 cudaError_t launch_adjoint_gather(int I, const AdjArgs& a, cudaStream_t st);
@@ -341,16 +346,8 @@ cudaError_t launch_adjoint_i8(const AdjArgs& a, int64_t nblocks, int deg_hi, cud
 size_t scan_scratch_bytes_u32(int64_t len);
 cudaError_t scan_exclusive_u32(uint32_t* data, int64_t len, uint32_t* scratch, cudaStream_t st, int64_t* launches);
 
-// Compacted list of the non-empty blocks (in key order) and its length.
-size_t nonempty_scratch_bytes(int64_t nblocks);
-cudaError_t launch_nonempty_list(const int32_t* offsets, int64_t nblocks, int32_t* list, int32_t* count, void* scratch,
-                                 cudaStream_t st, int64_t* launches);
-
-// One persistent launch over all sets (float32 or split-bf16 storage); grid = 2 CTAs per SM.
-// maps: null, or three CUtensorMap pointers (AB2 halo boxes of widths 4, 6, 8) for
-// tensor-copy halos of the float32 field
-cudaError_t launch_batched(int storage, const BatchSet* sets, int nsets, int* ctr, int nsm, const void* const* maps,
-                           cudaStream_t st);
+// One persistent launch over all sets (float32 or split-bf16 storage).
+cudaError_t launch_batched(int storage, const BatchSet* sets, int nsets, int* ctr, int nsm, cudaStream_t st);
 
 // Sets the thread-local message returned by tracker_last_error().
 void set_error_message(const char* msg);
@@ -361,8 +358,6 @@ bool device_pointer_ok(const void* p, int dev);
 
 // Block kernels, one entry per kernel width I (block_i4.cu, block_i6.cu, block_i8.cu).
 // deg_hi selects the degree-(I+1) instantiation (spline with m = I/2).
-cudaError_t launch_column_i4(int mode, const ColumnArgs& ca, int deg_hi, int nsm, cudaStream_t st);
-cudaError_t launch_column_i6(int mode, const ColumnArgs& ca, int deg_hi, int nsm, cudaStream_t st);
 // counting-sort binning of the step path: keys with block counts; counts ->
 // offsets + cursors (counts zeroed); scatter of the state into its blocks
 cudaError_t launch_keys_count(const GridGeom& g, int64_t np, const double* pos, uint32_t* keys, uint32_t* counts,
@@ -372,24 +367,27 @@ cudaError_t launch_keys_count(const GridGeom& g, int64_t np, const double* pos, 
 size_t count_scan_scratch_bytes(int64_t nblocks);
 cudaError_t launch_count_scan(uint32_t* counts, int64_t nblocks, int32_t* offsets, int32_t* cursor,
                               uint32_t* scratch, cudaStream_t st, int64_t* launches);
-// counting-sort permutation of keys (cursor from launch_count_scan): perm[d] = j
-cudaError_t launch_scatter_perm(int64_t np, const uint32_t* keys, int32_t* cursor, int32_t* perm, int* flags,
-                                cudaStream_t st);
+// counting-sort permutation of keys (cursor from launch_count_scan): perm[d] = j, and the
+// records PRec<float or double> rec[d] of pos (null: none)
+cudaError_t launch_scatter_perm(const GridGeom& g, int64_t np, const uint32_t* keys, int32_t* cursor, const double* pos,
+                                int32_t* perm, void* rec, int rec_f64, int* flags, cudaStream_t st);
 // counts[key] += number of particles with that key
 cudaError_t launch_count_keys(int64_t np, const uint32_t* keys, uint32_t* counts, cudaStream_t st);
-cudaError_t launch_scatter_state(int64_t np, const uint32_t* keys, int32_t* cursor, const double* pos_in,
-                                 const int32_t* id_in, const float* rhs_in, int rhs_rows, double* pos_out,
-                                 int32_t* id_out, float* rhs_out, int* flags, cudaStream_t st);
-// tmap: a CUtensorMap of the padded field with the box tma_box(I, margin of
-// the mode, element size) for tensor-copy halo staging (float32 and float64
-// storage), or null for cp.async element copies
-cudaError_t launch_block_i4(int mode, const BlockArgs& a, const void* tmap, int64_t nblocks, int deg_hi,
-                            cudaStream_t st);
-cudaError_t launch_block_i6(int mode, const BlockArgs& a, const void* tmap, int64_t nblocks, int deg_hi,
-                            cudaStream_t st);
-cudaError_t launch_block_i8(int mode, const BlockArgs& a, const void* tmap, int64_t nblocks, int deg_hi,
-                            cudaStream_t st);
-// direct path (sparse particle sets): a.np sorted particles, PB per CTA, stencils from global memory
+// the same for the particle state, with its records
+cudaError_t launch_scatter_state(const GridGeom& g, int64_t np, const uint32_t* keys, int32_t* cursor,
+                                 const double* pos_in, const int32_t* id_in, const float* rhs_in, int rhs_rows,
+                                 double* pos_out, int32_t* id_out, float* rhs_out, void* rec, int rec_f64, int* flags,
+                                 cudaStream_t st);
+// Block kernels: a.rec_in must hold the records of the grouped particles.
+// tmap: a CUtensorMap of the padded field for halo_box(I, margin of the mode) for
+// tensor-copy staging, or null for cp.async copies
+cudaError_t launch_block_i4(int mode, const BlockArgs& a, const void* tmap, int64_t nblocks, cudaStream_t st);
+cudaError_t launch_block_i4h(int mode, const BlockArgs& a, const void* tmap, int64_t nblocks, cudaStream_t st);
+cudaError_t launch_block_i6(int mode, const BlockArgs& a, const void* tmap, int64_t nblocks, cudaStream_t st);
+cudaError_t launch_block_i6h(int mode, const BlockArgs& a, const void* tmap, int64_t nblocks, cudaStream_t st);
+cudaError_t launch_block_i8(int mode, const BlockArgs& a, const void* tmap, int64_t nblocks, cudaStream_t st);
+cudaError_t launch_block_i8h(int mode, const BlockArgs& a, const void* tmap, int64_t nblocks, cudaStream_t st);
+// direct path: a.np grouped particles, a.ppc per CTA, stencils from global memory
 cudaError_t launch_direct_i4(int mode, const BlockArgs& a, int deg_hi, cudaStream_t st);
 cudaError_t launch_direct_i6(int mode, const BlockArgs& a, int deg_hi, cudaStream_t st);
 cudaError_t launch_direct_i8(int mode, const BlockArgs& a, int deg_hi, cudaStream_t st);

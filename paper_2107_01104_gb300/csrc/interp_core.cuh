@@ -1,0 +1,740 @@
+// The per-particle arithmetic shared by every interpolation and step kernel:
+// 1-D weights, stencil gather and separable contraction (Eq. triple_sum,
+// Sec. 3.3), the RK2 stage-2 point, and the lane-dense float64 phases around
+// them (cell split before, position update after).
+//
+// Work split.  A warp takes up to 32 particles at a time.  Their float64 work
+// is lane-dense (one particle per lane).  The interpolation works on four
+// particles at once, one per group of eight lanes: lane u of a group owns the
+// stencil column x = u (I = 8; I = 6: x = u for u < 6, lanes 6 and 7 repeat
+// lanes 0 and 1 with zero weight; I = 4: x = u mod 4, planes z = u / 4 and
+// u / 4 + 2), walks its (y, z) rows with the node's components in one 16-byte
+// record, and sums z, then y, in registers; the groups then add their lanes
+// (three butterfly steps per value).
+//
+// Why: a warp-wide load is then four runs of I consecutive records, which L1
+// (and shared memory) serve at about 1.2 cycles per run, and the work that
+// does not depend on the stencil size (weights, reductions, the stage-2
+// point, addresses) is shared by four particles.  One warp per particle, the
+// split this replaced, spent about 145 instructions per stencil (I = 6) of
+// which 24 were the contraction's, and read its rows through 8 loads of five
+// rows each; this one spends about 60.  Texture fetches of the same rows take
+// 2.1 cycles per row on this GPU against 1.23 for plain loads, and mixing the
+// two adds their times (measured on an L1-resident region: 44 cycles per
+// 216-node stencil with loads, 56 / 68 / 75 with 1/4, 1/2, all rows as texture
+// fetches; shared memory 45), so every load is a plain one.
+//
+// Everything here gives the same bits whatever kernel runs it: the order of
+// the sums depends on the stencil only.
+#pragma once
+
+#include <type_traits>
+
+#include <cuda.h>   // CUtensorMap (type only; the library does not link the driver API)
+
+#include "internal.cuh"
+
+namespace trk {
+
+constexpr int NT = 128;           // threads per CTA of the block and batched kernels
+constexpr int NW = NT / 32;       // warps per CTA
+constexpr int PB = NT;            // particles per batch (32 per warp)
+
+// ---------------------------------------------------------------------------
+// Weight polynomials
+// ---------------------------------------------------------------------------
+template <typename T, class A>
+__device__ __forceinline__ const CoefTable<T>& table(const A& a)
+{
+    if constexpr (sizeof(T) == 4) return a.cf;
+    else return a.cd;
+}
+
+template <typename T, int DEG>
+struct Row {
+    T c[DEG + 1];
+};
+
+template <typename T, int DEG>
+__device__ __forceinline__ Row<T, DEG> load_row(const T (&tab)[TRK_TAB_MAX_I][TRK_TAB_MAX_DEG], int i)
+{
+    Row<T, DEG> r;
+#pragma unroll
+    for (int d = 0; d <= DEG; ++d) r.c[d] = tab[i][d];
+    return r;
+}
+
+template <typename T, int DEG>
+__device__ __forceinline__ T horner(const Row<T, DEG>& r, T s)
+{
+    T acc = r.c[DEG];
+#pragma unroll
+    for (int d = DEG - 1; d >= 0; --d) acc = fma(acc, s, r.c[d]);
+    return acc;
+}
+
+// n consecutive weights of a group's buffer (the same for every lane of the
+// group) by 16-byte loads where the run starts on a 16-byte boundary
+template <int n, typename T>
+__device__ __forceinline__ void bcast_load(const T* p, T (&w)[n])
+{
+    static_assert(n % 2 == 0, "runs of even length");
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int i = 0; i + 4 <= n; i += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(p + i);
+            w[i] = v.x;
+            w[i + 1] = v.y;
+            w[i + 2] = v.z;
+            w[i + 3] = v.w;
+        }
+        if constexpr (n % 4 == 2) {
+            const float2 v = *reinterpret_cast<const float2*>(p + n - 2);
+            w[n - 2] = v.x;
+            w[n - 1] = v.y;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < n; i += 2) {
+            const double2 v = *reinterpret_cast<const double2*>(p + i);
+            w[i] = v.x;
+            w[i + 1] = v.y;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Lane map and weights of a group of eight lanes
+// ---------------------------------------------------------------------------
+template <int I>
+struct LaneMap {
+    static constexpr int NY = I;                // rows along y per lane
+    static constexpr int NZ = I == 4 ? 2 : I;   // planes along z per lane: z0, z0 + ZS, ...
+    static constexpr int ZS = I == 4 ? 2 : 1;
+    int x, z0;
+    bool act;                                   // false: a repeated column (zero weight)
+    __device__ __forceinline__ explicit LaneMap(int lane)
+    {
+        const int u = lane & 7;
+        x = I == 8 ? u : (I == 6 ? (u < 6 ? u : u - 6) : (u & 3));
+        z0 = I == 4 ? u >> 2 : 0;
+        act = I != 6 || u < 6;
+    }
+};
+
+template <typename T, int I, bool D>
+struct Weights {
+    static constexpr int NY = LaneMap<I>::NY, NZ = LaneMap<I>::NZ;
+    T w1, dw1;
+    T w2[NY], w3[NZ];
+    T dw2[D ? NY : 1], dw3[D ? NZ : 1];
+};
+
+// Lane u evaluates the weight of node i = x for the three axes by Horner's
+// rule; axes 2 and 3 are exchanged through the group's buffer wb (axis 2 at 0,
+// axis 3 at 8, their derivatives at 16 and 24; I = 4: axis 3 in the order 0, 2,
+// 1, 3, so that a lane's planes are adjacent).  Successive calls of a warp
+// alternate between two buffers, so one __syncwarp per call orders them.
+template <typename T, int I, int DEG, bool D>
+struct Basis {
+    Row<T, DEG> r, dr;
+    __device__ __forceinline__ void init(const CoefTable<T>& tb, const LaneMap<I>& m)
+    {
+        r = load_row<T, DEG>(tb.c, m.x);
+        if (D) dr = load_row<T, DEG>(tb.d, m.x);
+    }
+    __device__ __forceinline__ void eval(T s1, T s2, T s3, const LaneMap<I>& m, T* wb, Weights<T, I, D>& w) const
+    {
+        const T a1 = horner(r, s1), a2 = horner(r, s2), a3 = horner(r, s3);
+        // (repeated columns store the values their originals store)
+        const int x3 = I == 4 ? (m.x & 1) * 2 + (m.x >> 1) : m.x;
+        wb[m.x] = a2;
+        wb[8 + x3] = a3;
+        w.w1 = m.act ? a1 : (T)0;
+        if constexpr (D) {
+            const T d1 = horner(dr, s1);
+            wb[16 + m.x] = horner(dr, s2);
+            wb[24 + x3] = horner(dr, s3);
+            w.dw1 = m.act ? d1 : (T)0;
+        }
+        __syncwarp();
+        bcast_load(wb, w.w2);
+        bcast_load(wb + 8 + 2 * m.z0, w.w3);
+        if constexpr (D) {
+            bcast_load(wb + 16, w.dw2);
+            bcast_load(wb + 24 + 2 * m.z0, w.dw3);
+        }
+    }
+};
+
+// ---------------------------------------------------------------------------
+// Stencil loaders: ld(r, z, v) = components of the lane's node in row r and its
+// z-th plane
+// ---------------------------------------------------------------------------
+// value of a split-bf16 word (hi in the low half, lo in the high half)
+__device__ __forceinline__ float bf16x2_value(uint32_t w)
+{
+    return __uint_as_float(w << 16) + __uint_as_float(w & 0xffff0000u);
+}
+
+template <int STORE, int RW, int NC, typename T>
+__device__ __forceinline__ void unpack(const uint4& q, T (&v)[NC])
+{
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int k = 0; k < NC; ++k) v[k] = STORE == ST_BF16X2 ? bf16x2_value(w[k]) : __uint_as_float(w[k]);
+}
+
+// Records in global memory (float32 and split-bf16 fields).  A cell c in
+// [0, N) plus one is at least PAD - 1 > I / 2 nodes inside the ghost-padded
+// array, so a stencil is a box of fixed offsets from its first node.
+template <int STORE, int RW, int NC>
+struct RecordLd {
+    const uint32_t* p;     // the lane's first node
+    int NP, NP2;           // record strides from row to row and from plane to plane of the lane
+    __device__ __forceinline__ void operator()(int r, int z, float (&v)[NC]) const
+    {
+        const int off = z * NP2 + r * NP;
+        if constexpr (RW == 4) {
+            unpack<STORE, RW, NC>(__ldg(reinterpret_cast<const uint4*>(p) + off), v);
+        } else {
+            static_assert(NC == 1, "one component per 4-byte record");
+            const uint32_t w = __ldg(p + off);
+            v[0] = STORE == ST_BF16X2 ? bf16x2_value(w) : __uint_as_float(w);
+        }
+    }
+};
+
+// Component-major float64 field: components k >= kc read component kc - 1
+template <int NC>
+struct PlaneLd {
+    const double* p;
+    int64_t plane;
+    int NP, NP2, kc;
+    __device__ __forceinline__ void operator()(int r, int z, double (&v)[NC]) const
+    {
+        const int off = z * NP2 + r * NP;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) v[k] = __ldg(p + (int64_t)(k < kc ? k : kc - 1) * plane + off);
+    }
+};
+
+// Loader of the stencil whose first node has the padded index `base`, for the
+// component chunk ch (NC components of it)
+template <typename T, int I, int STORE, int RW, int NC>
+__device__ __forceinline__ auto global_ld(const FieldView& f, int base, int ch, const LaneMap<I>& m)
+{
+    constexpr int ZS = LaneMap<I>::ZS;
+    const int64_t n = (int64_t)base + m.x + m.z0 * f.NP * f.NP;
+    if constexpr (STORE == ST_F64)
+        return PlaneLd<NC>{f.f64 + (int64_t)ch * NC * f.plane + n, f.plane, f.NP, ZS * f.NP * f.NP, f.C - ch * NC};
+    else
+        return RecordLd<STORE, RW, NC>{f.rec + ((int64_t)ch * f.plane + n) * RW, f.NP, ZS * f.NP * f.NP};
+}
+
+// A staged halo in shared memory: pitches P from row to row and PL from plane
+// to plane of the lane (elements), float64: component pitch SC
+template <typename T, int STORE, int RW, int NC, int P, int PL, int SC>
+struct HaloLd {
+    const void* p;         // the lane's first node
+    __device__ __forceinline__ void operator()(int r, int z, T (&v)[NC]) const
+    {
+        if constexpr (STORE == ST_F64) {
+#pragma unroll
+            for (int k = 0; k < NC; ++k) v[k] = reinterpret_cast<const double*>(p)[k * SC + z * PL + r * P];
+        } else if constexpr (RW == 4) {
+            unpack<STORE, RW, NC>(reinterpret_cast<const uint4*>(p)[z * PL + r * P], v);
+        } else {
+            const uint32_t w = reinterpret_cast<const uint32_t*>(p)[z * PL + r * P];
+            v[0] = STORE == ST_BF16X2 ? bf16x2_value(w) : __uint_as_float(w);
+        }
+    }
+};
+
+// A lane's stencil, its first HR rows held in registers (re-used by RK2's
+// second stage), the others loaded as they are contracted.
+template <typename T, int I, int NC, int HR, class LD>
+struct HeldLd {
+    const T (&f)[HR][LaneMap<I>::NZ][NC];
+    const LD& rest;
+    __device__ __forceinline__ void operator()(int r, int z, T (&v)[NC]) const
+    {
+        if (r < HR) {
+#pragma unroll
+            for (int k = 0; k < NC; ++k) v[k] = f[r < HR ? r : 0][z][k];
+        } else {
+            rest(r, z, v);
+        }
+    }
+};
+
+template <typename T, int I, int NC, int HR, class LD>
+__device__ __forceinline__ void load_rows(const LD& ld, T (&f)[HR][LaneMap<I>::NZ][NC])
+{
+#pragma unroll
+    for (int r = 0; r < HR; ++r)
+#pragma unroll
+        for (int z = 0; z < LaneMap<I>::NZ; ++z) ld(r, z, f[r][z]);
+}
+
+// ---------------------------------------------------------------------------
+// Contraction: z then y in the lane, then x over the group.
+//   D = false: out[k] = u_k
+//   D = true:  out[k] = u_k, out[NC + 3k + j] = du_k / dt_j
+// ---------------------------------------------------------------------------
+// Sums v[0..n) over the group's eight lanes; every lane gets all of them.
+template <typename T, int n>
+__device__ __forceinline__ void group_sum(T (&v)[n])
+{
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < n; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+}
+
+// i-th term of a sum over n nodes taken from the ends inwards (0, n-1, 1, ...):
+// the small outer terms first, so that they are rounded while the partial sum is small
+__host__ __device__ constexpr int inward(int i, int n) { return i % 2 == 0 ? i / 2 : n - 1 - i / 2; }
+
+// the lane's column: out as above, to be summed over the group
+template <typename T, int I, int NC, bool D, class LD>
+__device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D>& w, T (&out)[D ? 4 * NC : NC])
+{
+    constexpr int NY = LaneMap<I>::NY, NZ = LaneMap<I>::NZ;
+    T a[NC], b[NC], c[NC];
+#pragma unroll
+    for (int rr = 0; rr < NY; ++rr) {
+        const int r = inward(rr, NY);
+        T pv[NC], pd[NC];
+#pragma unroll
+        for (int zz = 0; zz < NZ; ++zz) {
+            const int z = inward(zz, NZ);
+            T v[NC];
+            ld(r, z, v);
+#pragma unroll
+            for (int k = 0; k < NC; ++k) {
+                pv[k] = zz == 0 ? w.w3[z] * v[k] : fma(w.w3[z], v[k], pv[k]);
+                if constexpr (D) pd[k] = zz == 0 ? w.dw3[z] * v[k] : fma(w.dw3[z], v[k], pd[k]);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            a[k] = rr == 0 ? w.w2[r] * pv[k] : fma(w.w2[r], pv[k], a[k]);
+            if constexpr (D) {
+                b[k] = rr == 0 ? w.dw2[r] * pv[k] : fma(w.dw2[r], pv[k], b[k]);
+                c[k] = rr == 0 ? w.w2[r] * pd[k] : fma(w.w2[r], pd[k], c[k]);
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        out[k] = w.w1 * a[k];
+        if constexpr (D) {
+            out[NC + 3 * k] = w.dw1 * a[k];
+            out[NC + 3 * k + 1] = w.w1 * b[k];
+            out[NC + 3 * k + 2] = w.w1 * c[k];
+        }
+    }
+    group_sum(out);
+}
+
+// ---------------------------------------------------------------------------
+// Per-warp shared memory
+// ---------------------------------------------------------------------------
+template <int MODE>
+__host__ __device__ constexpr bool is_ab() { return MODE == MODE_AB2 || MODE == MODE_AB2_D; }
+template <int MODE>
+__host__ __device__ constexpr bool is_step() { return MODE == MODE_RK2 || is_ab<MODE>(); }
+template <int MODE>
+__host__ __device__ constexpr bool is_deriv() { return MODE == MODE_INTERP_DERIV || MODE == MODE_AB2_D; }
+
+// values handed from the groups to the particle's lane: k1 and k2 (RK2), u
+// (AB, interpolation), u and its derivatives
+template <int MODE, int NC>
+__host__ __device__ constexpr int result_count() { return MODE == MODE_RK2 ? 6 : (is_deriv<MODE>() ? 4 * NC : NC); }
+
+__host__ __device__ constexpr size_t align32(size_t x) { return (x + 31) & ~size_t(31); }
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* dst, const void* src)
+{
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(smem_addr(dst)), "l"(src), "n"(BYTES)
+                     : "memory");
+}
+
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+template <typename T, int MODE, int NC>
+struct WarpPlan {
+    static constexpr int KS = (result_count<MODE, NC>() + 3) / 4 * 4;                      // values per particle
+    static constexpr size_t rec = 0;                                                       // [2][32] records
+    static constexpr size_t k = align32(rec + 2 * 32 * 4 * sizeof(T));                     // [32][KS]
+    static constexpr size_t w = align32(k + 32 * KS * sizeof(T));                          // [2][4 groups][WB]
+    static constexpr int WB = is_deriv<MODE>() ? 40 : 24;                                  // groups 8 banks apart
+    static constexpr size_t x = align32(w + 2 * 4 * WB * sizeof(T));                       // [3][32] positions (steps)
+    static constexpr size_t rhs = align32(x + (is_step<MODE>() ? 3 * 32 * sizeof(double) : 0));   // [9][32] AB history
+    static constexpr size_t total = align32(rhs + (is_ab<MODE>() ? 3 * AB_MAX_HIST * 32 * sizeof(float) : 0));
+};
+
+// one group's results (the same in all its lanes) into the particle's slots
+template <typename T, int n>
+__device__ __forceinline__ void put_results(T* kb, const T (&v)[n])
+{
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+        for (int i = 0; i + 4 <= n; i += 4)
+            *reinterpret_cast<float4*>(kb + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+        if constexpr (n % 4 >= 2) *reinterpret_cast<float2*>(kb + n / 4 * 4) = make_float2(v[n / 4 * 4], v[n / 4 * 4 + 1]);
+        if constexpr (n % 2 == 1) kb[n - 1] = v[n - 1];
+    } else {
+#pragma unroll
+        for (int i = 0; i + 2 <= n; i += 2) *reinterpret_cast<double2*>(kb + i) = make_double2(v[i], v[i + 1]);
+        if constexpr (n % 2 == 1) kb[n - 1] = v[n - 1];
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Halo of a cell block (block kernels): H^3 nodes from G nodes below the
+// block's first cell, with one more layer on each side for RK2's stage-2 point.
+// Dense rows (pitch P; float64 an even number of elements, the halo XOFF in,
+// so that a tensor copy starts on 16 bytes).
+// ---------------------------------------------------------------------------
+template <typename T, int I, int MODE, int NC, int RW>
+struct HaloGeom {
+    static constexpr int MARGIN = MODE == MODE_RK2 ? 1 : 0;
+    static constexpr HaloBox B = halo_box(I, MARGIN, sizeof(T) == 8);
+    static constexpr int H = B.H, G = B.G, P = B.P, XOFF = B.XOFF;
+    static constexpr int PL = P * H, SC = PL * H;
+    static constexpr size_t bytes = align32(sizeof(T) == 8 ? (size_t)NC * SC * 8 : (size_t)SC * RW * 4);
+};
+
+// Slabs: the halo as k_slabs stages it, cut along x1 into slabs of SW nodes
+// aligned to SW, each a dense box [H][H][SW] of 16-byte records.  A group's
+// lanes read consecutive x1: eight banks groups apart whichever slabs they lie
+// in (SW = 8: 128-byte rows; I = 4, whose groups read rows of two planes at
+// once: 64-byte rows, and H is odd).
+template <int I, int MODE>
+struct SlabGeom {
+    static constexpr HaloBox B = halo_box(I, MODE == MODE_RK2 ? 1 : 0, false);
+    static constexpr int H = B.H, G = B.G;
+    static constexpr int SW = slab_width(I), SPT = BLK / SW;       // slabs a block is wide
+    static constexpr int X0 = -((G + SW - 1) / SW) * SW;          // first slab's x1 relative to the block
+    static constexpr int NSL = (H - G - X0 + SW - 1) / SW;        // slabs a block's halo spans
+    static constexpr size_t bytes = (size_t)H * H * SW * 16, slot = (bytes + 127) / 128 * 128;
+    static_assert(SW == 8 || H % 2 == 1, "two planes in distinct banks");
+};
+
+// where a group's stencil comes from
+enum { SRC_GLOBAL = 0, SRC_HALO = 1, SRC_SLABS = 2 };
+struct Place {
+    const unsigned char* halo;   // SRC_HALO: the staged halo; SRC_SLABS: slot 0 of the slab ring
+    int slab;                    // SRC_SLABS: sequence number of the block's first slab
+    int r1, r2, r3;              // the particle's cell relative to the halo
+    int o1, o2, o3;              // the halo's first node (unpadded coordinates)
+    int node;                    // SRC_GLOBAL: padded index of the stencil's first node
+};
+
+// ---------------------------------------------------------------------------
+// P1: lane-dense.  The record of the lane's particle: the one the binning made
+// (grouped position j), or split here from the position of particle src.
+// ---------------------------------------------------------------------------
+template <typename T>
+__device__ __forceinline__ PRec<T> particle_record(const BlockArgs& a, int64_t j, int64_t src, bool valid)
+{
+    PRec<T> rec;
+    rec.t[0] = rec.t[1] = rec.t[2] = (T)0;
+    rec.cell = cell_as<T>(0);
+    if (!valid) return rec;
+    if (a.rec_in) return reinterpret_cast<const PRec<T>*>(a.rec_in)[j];
+    return split_record<T>(a.g, a.np, a.pos_in, src, a.flags);
+}
+
+// The lane's particle state that the update needs, on its way to shared memory
+// while the particle is interpolated (cp.async; the lane reads its own copies).
+template <typename T, int MODE, int NC>
+__device__ __forceinline__ void fetch_state(const BlockArgs& a, int64_t src, bool valid, unsigned char* ws, int lane)
+{
+    using WPl = WarpPlan<T, MODE, NC>;
+    if constexpr (is_step<MODE>()) {
+        if (!valid) return;
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax)
+            cp_async<8>(ws + WPl::x + (ax * 32 + lane) * 8, a.pos_in + ax * a.np + src);
+        if constexpr (is_ab<MODE>()) {   // the valid history rows
+            const int rows = 3 * min(a.history_valid, a.ab_order - 1);
+            for (int r = 0; r < rows; ++r) cp_async<4>(ws + WPl::rhs + (r * 32 + lane) * 4, a.rhs_in + r * a.np + src);
+        }
+    }
+}
+
+// Rows of the RK2 stencil a lane holds in registers between the stages: its
+// second stage then gathers these only where X* left the cell.  I = 4 (8
+// nodes): always.  I = 6 (36 nodes, 144 registers): in the direct kernel, whose
+// stencils come from beyond L1, eight warps per SM that hold them move less
+// than sixteen that gather twice (256^3 float32, RK2, us per step: 137 against
+// 158 at 1/64 particle per cell; 512^3 at 1.5e-3: 197 against 226; 168
+// registers with spills: 158, 220); from slabs in shared memory sixteen warps
+// without held rows are faster (1/4 per cell: 1238 against 1536).  I = 8 would
+// take 256 registers, float64 twice these: none.
+template <typename T, int I, int SRC>
+__host__ __device__ constexpr int held_rows()
+{
+    return sizeof(T) == 8 || I == 8 ? 0 : (I == 4 ? 4 : (SRC == SRC_GLOBAL ? 6 : 0));
+}
+
+// ---------------------------------------------------------------------------
+// Q: a group interpolates its particle (offsets t, stencil at `at`), component
+// chunk ch; res: the particle's results, in every lane of the group.  live:
+// false for an empty slot (whose results nobody reads).
+// ---------------------------------------------------------------------------
+template <typename T, int I, int DEG, int MODE, int NC, int STORE, int RW, int SRC, int NS = 1>
+__device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Place& at, int ch, const T (&t)[3], bool live,
+                                                  int lane, const Basis<T, I, DEG, is_deriv<MODE>()>& B,
+                                                  const LaneMap<I>& m, T* wb0, T* wb1, bool odd,
+                                                  T (&res)[result_count<MODE, NC>()])
+{
+    constexpr bool D = is_deriv<MODE>(), HALO = SRC != SRC_GLOBAL;
+    constexpr int LO = I / 2 - 1, ZS = LaneMap<I>::ZS;
+    auto halo_ld = [&](int r1, int r2, int r3) {
+        if constexpr (SRC == SRC_SLABS) {   // the lane's slab and column
+            using SG = SlabGeom<I, MODE>;
+            const int x = r1 - LO + m.x - SG::G - SG::X0;
+            const int row = (r3 - LO + m.z0) * SG::H + (r2 - LO);
+            return HaloLd<T, STORE, RW, NC, SG::SW, ZS * SG::H * SG::SW, 0>{
+                at.halo + (unsigned)(at.slab + x / SG::SW) % NS * SG::slot + (row * SG::SW + x % SG::SW) * 16};
+        } else {
+            using HG = HaloGeom<T, I, MODE, NC, RW>;
+            const int e = (r3 - LO + m.z0) * HG::PL + (r2 - LO) * HG::P + (r1 - LO + m.x) + HG::XOFF;
+            return HaloLd<T, STORE, RW, NC, HG::P, ZS * HG::PL, HG::SC>{at.halo + e * (STORE == ST_F64 ? 8 : 4 * RW)};
+        }
+    };
+    auto glob_ld = [&](int node) { return global_ld<T, I, STORE, RW, NC>(a.f, node, ch, m); };
+    Weights<T, I, D> w;
+    if constexpr (MODE != MODE_RK2) {
+        B.eval(t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, m, odd ? wb1 : wb0, w);
+        if constexpr (HALO) contract<T, I, NC, D>(halo_ld(at.r1, at.r2, at.r3), w, res);
+        else contract<T, I, NC, D>(glob_ld(at.node), w, res);
+    } else {
+        const T dtid = (T)(a.dt * a.g.inv_delta);
+        constexpr int HR = held_rows<T, I, SRC>();
+        T f[HR > 0 ? HR : 1][LaneMap<I>::NZ][NC];
+        T k1[NC], k2[NC];
+        // contract the stencil of ld; its held rows are loaded if `fresh`
+        auto stage = [&](const auto& ld, T s1, T s2, T s3, T* wb, bool fresh, T (&k)[NC]) {
+            if constexpr (HR > 0) {
+                if (fresh) load_rows<T, I, NC, HR>(ld, f);
+                __syncwarp();
+                B.eval(s1, s2, s3, m, wb, w);
+                contract<T, I, NC, false>(HeldLd<T, I, NC, HR, std::decay_t<decltype(ld)>>{f, ld}, w, k);
+            } else {
+                B.eval(s1, s2, s3, m, wb, w);
+                contract<T, I, NC, false>(ld, w, k);
+            }
+        };
+        if constexpr (HALO) stage(halo_ld(at.r1, at.r2, at.r3), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, k1);
+        else stage(glob_ld(at.node), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, k1);
+        // stage-2 point, cell-relative: t* = t + dt k1 / delta
+        T ts[3];
+        int dc[3];
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            ts[ax] = fma(dtid, k1[ax], t[ax]);
+            const T fl = floor(ts[ax]);
+            dc[ax] = (int)fl;
+            ts[ax] -= fl;
+        }
+        // where X* lies: in the halo, else by its padded node index (one cell
+        // away stays inside the ghost layers; farther it is wrapped)
+        const bool moved = (dc[0] | dc[1] | dc[2]) != 0;
+        const int s1 = at.r1 + dc[0], s2 = at.r2 + dc[1], s3 = at.r3 + dc[2];
+        // (unsigned: a saturated conversion is far as well)
+        const bool far = (unsigned)dc[0] + 1u > 2u || (unsigned)dc[1] + 1u > 2u || (unsigned)dc[2] + 1u > 2u;
+        int node2 = at.node + dc[0] + dc[1] * a.f.NP + dc[2] * a.f.NP * a.f.NP;
+        if (far) {
+            if ((lane & 7) == 0 && live) atomicOr(a.flags + FLAG_CFL, 1);
+            int c1, c2, c3;
+            if constexpr (HALO) {
+                c1 = at.o1 + at.r1, c2 = at.o2 + at.r2, c3 = at.o3 + at.r3;
+            } else {
+                c1 = at.node % a.f.NP - PAD + LO;
+                c2 = at.node / a.f.NP % a.f.NP - PAD + LO;
+                c3 = at.node / a.f.NP / a.f.NP - PAD + LO;
+            }
+            auto wrap = [&](int c, int d) { return (int)(((unsigned)c + (unsigned)d) & (unsigned)a.g.mask); };
+            node2 = (int)padded_index(a.f.NP, wrap(c1, dc[0]) - LO, wrap(c2, dc[1]) - LO, wrap(c3, dc[2]) - LO);
+        }
+        if constexpr (HALO) {   // the halo has a margin of one cell
+            if (!__any_sync(0xffffffffu, far)) {
+                stage(halo_ld(s1, s2, s3), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, k2);
+            } else {   // rare: every group of the warp gathers from global memory (the same values)
+                const int n2 = far ? node2
+                                   : (int)padded_index(a.f.NP, ((at.o1 + s1) & a.g.mask) - LO,
+                                                       ((at.o2 + s2) & a.g.mask) - LO, ((at.o3 + s3) & a.g.mask) - LO);
+                stage(glob_ld(n2), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, k2);
+            }
+        } else {
+            stage(glob_ld(node2), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, k2);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            res[k] = k1[k];
+            res[3 + k] = k2[k];
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// P3: lane-dense.  Interpolation: write the chunk's outputs of the particle in
+// the caller's order.  Steps: float64 update, new key, block counts.
+// ---------------------------------------------------------------------------
+template <typename T, int MODE, int NC>
+__device__ __forceinline__ void write_outputs(const BlockArgs& a, int64_t id, int ch, const unsigned char* ws, int lane)
+{
+    using WPl = WarpPlan<T, MODE, NC>;
+    const T* kb = reinterpret_cast<const T*>(ws + WPl::k) + lane * WPl::KS;
+    auto put = [&](int64_t row, double v) {
+        if (a.out_f64) reinterpret_cast<double*>(a.out)[row * a.np + id] = v;
+        else reinterpret_cast<float*>(a.out)[row * a.np + id] = (float)v;
+    };
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        if (ch * NC + k >= a.f.C) continue;
+        if constexpr (MODE == MODE_INTERP) {
+            put(ch * NC + k, (double)kb[k]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 3; ++j) put(3 * (ch * NC + k) + j, (double)kb[NC + 3 * k + j] * a.g.inv_delta);
+        }
+    }
+}
+
+template <typename T, int MODE, int NC>
+__device__ __forceinline__ void update_particle(const BlockArgs& a, int64_t j, int32_t id, bool valid,
+                                                const unsigned char* ws, int lane)
+{
+    using WPl = WarpPlan<T, MODE, NC>;
+    const unsigned vm = __ballot_sync(0xffffffffu, valid);
+    if (!valid) return;
+    const T* kb = reinterpret_cast<const T*>(ws + WPl::k) + lane * WPl::KS;
+    const double* xs = reinterpret_cast<const double*>(ws + WPl::x) + lane;
+    int cn[3];
+    bool ok = true;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        const double k1 = widen(kb[ax]);
+        const double x0 = xs[ax * 32];
+        double xn;
+        if constexpr (MODE == MODE_RK2) {
+            const double k2 = widen(kb[3 + ax]);
+            xn = x0 + (0.5 * a.dt) * (k1 + k2);
+        } else {   // ABk, order min(k, 1 + history)
+            float h[AB_MAX_HIST];   // entries beyond the valid ones are zero
+#pragma unroll
+            for (int e = 0; e < AB_MAX_HIST; ++e)
+                h[e] = e < a.history_valid && e < a.ab_order - 1
+                           ? reinterpret_cast<const float*>(ws + WPl::rhs)[(3 * e + ax) * 32 + lane]
+                           : 0.0f;
+            const int q = min(a.ab_order, a.history_valid + 1);
+            const double inc = ab_increment(q, k1, [&](int e) { return widen(h[e]); });
+            xn = x0 + a.dt * inc;
+            // new history: u_n, then the older entries shifted by one
+            a.rhs_out[ax * a.np + j] = (float)k1;
+#pragma unroll
+            for (int e = 1; e < AB_MAX_HIST; ++e)
+                if (e < a.ab_order - 1) a.rhs_out[(3 * e + ax) * a.np + j] = h[e - 1];
+            if (MODE == MODE_AB2 && a.out) reinterpret_cast<float*>(a.out)[ax * a.np + id] = (float)k1;
+        }
+        ok &= split_cell(xn, a.g.inv_delta, a.g.mask, cn[ax]);
+        a.pos_out[ax * a.np + j] = xn;
+    }
+    if constexpr (MODE == MODE_AB2_D) {
+        if (a.out) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+                reinterpret_cast<float*>(a.out)[i * a.np + id] = (float)((double)kb[3 + i] * a.g.inv_delta);
+        }
+    }
+    if (!ok) atomicOr(a.flags + FLAG_NONFINITE, 1);
+    a.id_out[j] = id;
+    const uint32_t key = block_key(a.g, cn[0], cn[1], cn[2]);
+    a.key_out[j] = key;
+    if (a.counts) {   // block counts of the next binning, one add per group of equal keys
+        const unsigned peers = __match_any_sync(vm, key);
+        if (lane == __ffs(peers) - 1) atomicAdd(a.counts + key, (uint32_t)__popc(peers));
+    }
+}
+
+// per-warp pointers into its shared memory
+template <typename T, int MODE, int NC>
+struct WarpMem {
+    using WPl = WarpPlan<T, MODE, NC>;
+    PRec<T>* recs;
+    T *kbuf, *wb0, *wb1;
+    __device__ __forceinline__ WarpMem(unsigned char* ws, int g)
+        : recs(reinterpret_cast<PRec<T>*>(ws + WPl::rec)), kbuf(reinterpret_cast<T*>(ws + WPl::k)),
+          wb0(reinterpret_cast<T*>(ws + WPl::w) + g * WPl::WB), wb1(wb0 + 4 * WPl::WB)
+    {
+    }
+};
+
+// ---------------------------------------------------------------------------
+// A CTA's particles [j0, j1) (grouped order) with stencils from global memory.
+// The warps take the particles four at a time in turn, so that the CTA's
+// gathers stay close together in the field (and in L1).
+// ---------------------------------------------------------------------------
+template <typename T, int I, int DEG, int MODE, int NC, int STORE, int RW>
+__device__ __forceinline__ void run_direct(const BlockArgs& a, int64_t j0, int64_t j1, unsigned char* ws, int warp,
+                                           int nw, int lane)
+{
+    constexpr int LO = I / 2 - 1;
+    const int g = lane >> 3;
+    const LaneMap<I> m(lane);
+    Basis<T, I, DEG, is_deriv<MODE>()> B;
+    B.init(table<T>(a), m);
+    const WarpMem<T, MODE, NC> wm(ws, g);
+    for (int64_t b0 = j0; b0 < j1; b0 += 32 * nw) {
+        const int64_t j = b0 + ((lane >> 2) * nw + warp) * 4 + (lane & 3);
+        const int left = (int)min(j1 - b0 - 4 * warp, (int64_t)32 * nw);   // particles from this warp's first on
+        if (left <= 0) break;
+        const bool valid = j < j1;
+        const int64_t src = !valid ? 0 : (a.perm ? a.perm[j] : j);
+        const int32_t id = !valid ? 0 : (a.id_in ? a.id_in[src] : (int32_t)src);
+        wm.recs[lane] = particle_record<T>(a, j, src, valid);
+        fetch_state<T, MODE, NC>(a, src, valid, ws, lane);
+        __syncwarp();
+        for (int ch = 0; ch < (is_step<MODE>() ? 1 : (a.f.C + NC - 1) / NC); ++ch) {
+            for (int it = 0; it < 8 && it * 4 * nw < left; ++it) {
+                const PRec<T> rec = wm.recs[4 * it + g];
+                int c[3];
+                unpack_cell(cell_of(rec), c);
+                Place at{};
+                at.node = (int)padded_index(a.f.NP, c[0] - LO, c[1] - LO, c[2] - LO);
+                T res[result_count<MODE, NC>()];
+                interpolate_group<T, I, DEG, MODE, NC, STORE, RW, SRC_GLOBAL>(
+                    a, at, ch, rec.t, it * 4 * nw + g < left, lane, B, m, wm.wb0, wm.wb1, it & 1, res);
+                if ((lane & 7) == 0) put_results(wm.kbuf + (4 * it + g) * WarpMem<T, MODE, NC>::WPl::KS, res);
+            }
+            __syncwarp();
+            if constexpr (is_step<MODE>()) {
+                cp_async_wait_all();
+                update_particle<T, MODE, NC>(a, j, id, valid, ws, lane);
+            } else if (valid) write_outputs<T, MODE, NC>(a, id, ch, ws, lane);
+            __syncwarp();
+        }
+    }
+}
+
+// resident CTAs (of four warps) per SM the kernels are register-capped for: two
+// (255 registers) where 36 nodes are held, else four (128)
+template <typename T, int I, int MODE, int SRC>
+__host__ __device__ constexpr int min_ctas()
+{
+    return MODE == MODE_RK2 && held_rows<T, I, SRC>() > 4 ? 2 : 4;
+}
+
+}  // namespace trk

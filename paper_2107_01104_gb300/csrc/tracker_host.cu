@@ -79,7 +79,7 @@ void dev_free(void* p)
     if (p) cudaFree(p);
 }
 
-constexpr int PB_HOST = 256;   // particles per direct-path work item (the block kernels' batch)
+constexpr int PB_HOST = 128;   // particles per work item of the batched kernel
 
 struct GraphCache {
     cudaGraphExec_t exec = nullptr;
@@ -93,13 +93,11 @@ struct SetState {
     int64_t nb = 0;                   // block count the per-block arrays were sized for
     uint32_t* keys = nullptr;
     uint32_t* counts = nullptr;       // [nblocks] block counts of the next binning (zero between binnings)
-    int32_t* perm = nullptr;
     int32_t* offsets = nullptr;
-    int32_t* list = nullptr;
-    int32_t* count = nullptr;
     double* pos_s[2] = {nullptr, nullptr};
     int32_t* id_s[2] = {nullptr, nullptr};
     float* rhs_s[2] = {nullptr, nullptr};
+    void* rec = nullptr;              // records of the grouped state
 };
 
 uint64_t mix(uint64_t h, uint64_t v)
@@ -125,13 +123,11 @@ struct tracker {
     // field
     int C = 0;
     void* field = nullptr;
-    float* field_nm = nullptr;        // node-major copy of the field for the direct path (float32; split-bf16 with C a multiple of 3), built on first use
-    bool nm_skip = false;             // split-bf16, C > 3: the copy could not be allocated for this field
-    cudaTextureObject_t nm_tex = 0;   // 16-byte-texel texture over field_nm (C = 3), or 0 for plain loads
-    size_t nm_bytes = 0;
-    bool nm_valid = false;
+    // (float64: component-major planes; else node records, see FieldView)
     // sort scratch
     int64_t sort_cap = 0;             // keys, perm
+    int64_t rec_cap = 0;              // rec
+    void* rec = nullptr;              // records of the grouped particles (PRec<float>, float64 storage PRec<double>)
     int64_t radix_cap = 0;            // sort_scratch, keys_sorted (stable binning)
     void* sort_scratch = nullptr;
     uint32_t* keys = nullptr;
@@ -157,18 +153,13 @@ struct tracker {
     GraphCache adv_graph, batch_graph;
     // batched sets
     std::vector<SetState> sets;
-    void* ne_scratch = nullptr;       // non-empty-list scratch
-    int64_t ne_cap = 0;
     BatchSet* d_desc = nullptr;       // [3][nsets] descriptors: first step, parity 0, parity 1
     int* d_ctr = nullptr;             // [nsets] work counters
     int desc_cap = 0;
-    std::vector<std::pair<uint64_t, int>> tune_cache;   // set signature -> direct path?
-    int nsm = 0;
+    int nsm = 0, l2_bytes = 0;
     int step_kernel = TRK_STEP_AUTO;  // trk_step_kernel
-    std::vector<std::pair<uint64_t, int>> interp_cache; // (np, C, deriv, out dtype) -> interpolation kernel
     int last_kernel = TRK_STEP_AUTO;  // kernel of the latest tracker_advance or tracker_interpolate
-    int* d_colctr = nullptr;          // work counter of the column kernel
-    int col_seg = 8;                  // column kernel: x3 slabs per work item (power of two)
+    int col_seg = 8;                  // column order: x3 slabs per segment (power of two)
     int dir_blk = BLK;                // direct path: edge of its cubic binning blocks (default shape only)
     int dir_ppc = 256;                // direct path: particles per CTA
     int64_t bin_cap = 0;              // entries of offsets / counts / cursor (largest geometry in use)
@@ -179,7 +170,6 @@ struct tracker {
     // one per stage-2 margin (interpolation and AB: 0, RK2: 1)
     CUtensorMap tmap[2];
     bool tmap_ok[2] = {false, false};
-    CUtensorMap batch_map[3];         // batched sets: AB2 halo boxes of widths 4, 6, 8
     int halo_copy = TRK_HALO_AUTO;    // trk_halo_copy: how the block kernel stages its halo
     bool auto_tma = true;             // TRK_HALO_AUTO's current choice (tensor copies, where there is a map)
     uint32_t* d_counts = nullptr;     // [nblocks] block counts (counting-sort binning of the column path)
@@ -290,6 +280,22 @@ int ensure_sort(tracker* t, int64_t np)
     return TRK_OK;
 }
 
+// records of the grouped particles (interpolation and steps)
+int ensure_rec(tracker* t, int64_t np)
+{
+    if (np <= t->rec_cap) return TRK_OK;
+    t->gen += 1;
+    dev_free(t->rec);
+    t->rec = nullptr;
+    t->rec_cap = 0;
+    if (dev_alloc(&t->rec, (size_t)np * (t->storage == TRK_F64 ? 32 : 16)) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(TRK_ENOMEM, "cannot allocate the records of %lld particles", (long long)np);
+    }
+    t->rec_cap = np;
+    return TRK_OK;
+}
+
 // radix-sort scratch and sorted keys of the stable binning (tracker_bin only)
 int ensure_radix(tracker* t, int64_t np)
 {
@@ -340,14 +346,7 @@ FieldView field_view(const tracker* t)
     f.NP = t->N + 2 * PAD;
     f.plane = (int64_t)f.NP * f.NP * f.NP;
     if (t->storage == ST_F64) f.f64 = reinterpret_cast<const double*>(t->field);
-    else if (t->storage == ST_F32) f.f32 = reinterpret_cast<const float*>(t->field);
-    else {
-        f.hi = reinterpret_cast<const __nv_bfloat16*>(t->field);
-        f.lo = f.hi + f.plane * t->C;
-    }
-    f.nm = t->nm_valid ? t->field_nm : nullptr;
-    f.nm_tex = t->nm_valid ? (unsigned long long)t->nm_tex : 0ull;
-    f.nmc = t->C == 3 ? 4 : t->C;
+    else f.rec = reinterpret_cast<const uint32_t*>(t->field);
     return f;
 }
 
@@ -357,22 +356,23 @@ FieldView field_view(const tracker* t)
 const void* halo_tmap(const tracker* t, int mode)
 {
     const int margin = mode == MODE_RK2 ? 1 : 0;
-    const bool tma = t->halo_copy == TRK_HALO_TMA || (t->halo_copy == TRK_HALO_AUTO && t->auto_tma);
+    // (asked for by name, tensor copies cover float32 and float64 fields of at least three components)
+    const bool tma = t->halo_copy == TRK_HALO_TMA ? t->storage != TRK_BF16X2 && t->C >= 3
+                                                  : t->halo_copy == TRK_HALO_AUTO && t->auto_tma;
     if (!tma || !t->tmap_ok[margin]) return nullptr;
     return &t->tmap[margin];
 }
 
-bool halo_tmap_exists(const tracker* t, int mode) { return t->tmap_ok[mode == MODE_RK2 ? 1 : 0]; }
-
-cudaError_t launch_block(tracker* t, int mode, const BlockArgs& a)
+// slabs: through the slab pipeline whatever halo copy is asked for (TRK_STEP_COLUMN)
+cudaError_t launch_block(tracker* t, int mode, const BlockArgs& a, bool slabs = false)
 {
     ProfScope ps(t, PROF_STEP);
     t->launches += 1;
-    const void* m = halo_tmap(t, mode);
+    const void* m = slabs ? (t->tmap_ok[mode == MODE_RK2] ? &t->tmap[mode == MODE_RK2] : nullptr) : halo_tmap(t, mode);
     switch (t->I) {
-        case 4: return launch_block_i4(mode, a, m, t->nblocks, t->deg_hi, t->stream);
-        case 6: return launch_block_i6(mode, a, m, t->nblocks, t->deg_hi, t->stream);
-        default: return launch_block_i8(mode, a, m, t->nblocks, t->deg_hi, t->stream);
+        case 4: return (t->deg_hi ? launch_block_i4h : launch_block_i4)(mode, a, m, t->nblocks, t->stream);
+        case 6: return (t->deg_hi ? launch_block_i6h : launch_block_i6)(mode, a, m, t->nblocks, t->stream);
+        default: return (t->deg_hi ? launch_block_i8h : launch_block_i8)(mode, a, m, t->nblocks, t->stream);
     }
 }
 
@@ -398,32 +398,32 @@ EncodeTiledFn encode_tiled()
     return fn;
 }
 
-// Tensor maps of the padded field f[C][NP][NP][NP] (4-D, x1 innermost) with the
-// block kernel's halo box for both stage-2 margins: float32 and float64
-// storage with at least three components (a chunk of three per copy; the
-// last chunk of a C that is not a multiple of three reads zeros beyond C,
-// which no output uses).  Left unset (cp.async staging) otherwise.
-// the tensor map of the tracker's field with the halo box of kernel width I
-// and stage-2 margin `margin` (tma_box); false if it cannot be made
-bool encode_field_map(const tracker* t, int I, int margin, CUtensorMap* out)
+// The tensor map of the tracker's field for the block kernel's halos with
+// stage-2 margin `margin` (halo_box), x1 innermost: float64 fields
+// [C][NP][NP][NP], the halo of a chunk of components per copy (the last chunk
+// reads zeros beyond C, which no output uses); node records
+// [chunks][NP][NP][4 NP] words, a slab of the halo per copy.  False where there is none (C = 1, float64 with C = 2: cp.async
+// staging).
+bool encode_field_map(const tracker* t, int margin, CUtensorMap* out)
 {
     const EncodeTiledFn enc = encode_tiled();
-    if (!enc || (t->storage != TRK_F32 && t->storage != TRK_F64) || t->C < 3 || !t->field) return false;
-    const int esz = t->storage == TRK_F64 ? 8 : 4;
-    const cuuint64_t NP = (cuuint64_t)(t->N + 2 * PAD);
-    const cuuint64_t dims[4] = {NP, NP, NP, (cuuint64_t)t->C};
-    const cuuint64_t strides[3] = {NP * esz, NP * NP * esz, NP * NP * NP * esz};
+    if (!enc || t->C < (t->storage == TRK_F64 ? 3 : 2) || !t->field) return false;
+    const bool f64 = t->storage == TRK_F64;
+    const HaloBox b = halo_box(t->I, margin, f64);
+    const cuuint64_t NP = (cuuint64_t)(t->N + 2 * PAD), unit = f64 ? 8 : 16;   // bytes per node and row element
+    const cuuint64_t dims[4] = {f64 ? NP : 4 * NP, NP, NP, (cuuint64_t)(f64 ? t->C : record_chunks(t->C))};
+    const cuuint64_t strides[3] = {NP * unit, NP * NP * unit, NP * NP * NP * unit};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
-    const TmaBox b = tma_box(I, margin, esz);
-    const cuuint32_t box[4] = {(cuuint32_t)b.BX, (cuuint32_t)b.BY, (cuuint32_t)b.H, 3};
-    return enc(out, esz == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, t->field, dims,
+    const cuuint32_t nc = f64 ? (cuuint32_t)(margin ? 3 : chunk_components(t->C)) : 1;
+    const cuuint32_t box[4] = {(cuuint32_t)(f64 ? b.P : 4 * slab_width(t->I)), (cuuint32_t)b.H, (cuuint32_t)b.H, nc};
+    return enc(out, f64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, t->field, dims,
                strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 void build_tmaps(tracker* t)
 {
-    for (int margin = 0; margin < 2; ++margin) t->tmap_ok[margin] = encode_field_map(t, t->I, margin, &t->tmap[margin]);
+    for (int margin = 0; margin < 2; ++margin) t->tmap_ok[margin] = encode_field_map(t, margin, &t->tmap[margin]);
 }
 
 cudaError_t launch_direct(tracker* t, int mode, const BlockArgs& a)
@@ -452,15 +452,17 @@ int bin_into(tracker* t, int64_t np, const double* pos, uint32_t* keys, int32_t*
 // Counting-sort binning of interpolation and the adjoint: keys and block
 // counts from the positions, offsets and cursors from one scan, then the
 // permutation t->perm (grouped by block; the order inside a block is not
-// reproducible, and every particle's result is independent of it).
-int bin_counting(tracker* t, int64_t np, const double* pos)
+// reproducible, and every particle's result is independent of it) and, for the
+// interpolation, the records.
+int bin_counting(tracker* t, int64_t np, const double* pos, void* rec)
 {
     ProfScope ps(t, PROF_BIN);
     CUDA_TRY(cudaMemsetAsync(t->d_counts, 0, (size_t)t->nblocks * sizeof(uint32_t), t->stream));
     CUDA_TRY(launch_keys_count(t->g, np, pos, t->keys, t->d_counts, t->d_flags, t->stream));
     CUDA_TRY(launch_count_scan(t->d_counts, t->nblocks, t->offsets, t->d_cursor, t->d_scan_tmp, t->stream,
                                &t->launches));
-    CUDA_TRY(launch_scatter_perm(np, t->keys, t->d_cursor, t->perm, t->d_flags, t->stream));
+    CUDA_TRY(launch_scatter_perm(t->g, np, t->keys, t->d_cursor, pos, t->perm, rec, t->storage == TRK_F64, t->d_flags,
+                                 t->stream));
     t->launches += 2;
     return TRK_OK;
 }
@@ -493,6 +495,9 @@ int check_block_kernel_shape(const tracker* t)
     return TRK_OK;
 }
 
+// launch shape of the direct kernel for direct_particles = 64, 128, 256 (0: untimed)
+int direct_shape(int p) { return p == 256 ? PPC_WIDE : (p == 128 ? 256 : (p == 64 ? 64 : 0)); }
+
 BlockArgs base_args(tracker* t)
 {
     BlockArgs a{};
@@ -508,7 +513,7 @@ BlockArgs base_args(tracker* t)
     a.offsets = t->offsets;
     a.flags = t->d_flags;
     a.ab_order = 2;
-    a.ppc = t->dir_ppc;
+    a.ppc = direct_shape(t->dir_ppc);
     return a;
 }
 
@@ -557,7 +562,7 @@ int replay_graph(tracker* t, GraphCache& gc, uint64_t key, int reps, F&& body)
     return TRK_OK;
 }
 
-// slabs per column-kernel work item: the tracker's setting, at most the column height
+// slabs per column segment: the tracker's setting, at most the column height
 int column_segment(const tracker* t) { return std::max(1, std::min(t->g.nb3, t->col_seg)); }
 
 bool column_available(const tracker* t)
@@ -568,16 +573,22 @@ bool column_available(const tracker* t)
 
 bool default_shape(const tracker* t) { return t->g.lb1 == LBLK && t->g.lb2 == LBLK && t->g.lb3 == LBLK; }
 
-// Binning geometry of a step path: the tracker's block shape, except that the
-// direct path bins by cubes of edge dir_blk when the shape is the default
-// (the direct kernel takes 256 grouped particles per CTA whatever the blocks
-// are; the block edge only sets how compact each CTA's particles are).
+// Binning geometry of a step path: the tracker's block shape, except that
+// COLUMN stacks the rows of blocks along x3 in segments (a stencil's planes are
+// then met again soon), and DIRECT bins by cubes of edge dir_blk when the shape
+// is the default one (the direct kernel takes runs of grouped particles
+// whatever the groups are).
 struct BinGeom {
     GridGeom g;
     int64_t nb;
 };
 BinGeom geom_of(const tracker* t, int path)
 {
+    if (path == TRK_STEP_COLUMN) {
+        BinGeom c{t->g, t->nblocks};
+        if (t->tmap_ok[0] && t->tmap_ok[1]) c.g.lseg = ilog2(column_segment(t));   // (the slab pipeline's order)
+        return c;
+    }
     if (path != TRK_STEP_DIRECT || t->dir_blk == BLK || !default_shape(t)) return {t->g, t->nblocks};
     BinGeom b{t->g, 0};
     const int lb = ilog2(t->dir_blk);
@@ -586,99 +597,9 @@ BinGeom geom_of(const tracker* t, int path)
     b.nb = (int64_t)b.g.nb1 * b.g.nb2 * b.g.nb3;
     return b;
 }
-bool same_geom(const GridGeom& a, const GridGeom& b) { return a.lb1 == b.lb1 && a.lb2 == b.lb2 && a.lb3 == b.lb3; }
-
-void destroy_nm_texture(tracker* t)
+bool same_geom(const GridGeom& a, const GridGeom& b)
 {
-    if (t->nm_tex) cudaDestroyTextureObject(t->nm_tex);
-    t->nm_tex = 0;
-}
-
-// The direct kernel fetches the 16-byte nodes of the node-major copy through
-// a texture object (the same bits, on the texture data path instead of the
-// load/store one) where the copy is at most kNmTextureL2 times the L2 size, or
-// the environment variable TRK_NM_TEXTURE_BYTES (0: never), and its node count
-// fits the device's linear-texture width.  Measured on the direct kernel:
-// with the copy at 2.5 times L2 (256^3) its stencil gathers are bound by the
-// L1 data path and the texture fetches take 16% less time; at 19 times L2 and
-// above (512^3, 1024^3) the gathers are bound by DRAM, where the texture
-// fetches took 10 to 11% more time than plain loads.
-constexpr double kNmTextureL2 = 4.0;
-
-void create_nm_texture(tracker* t, int64_t plane, size_t bytes, bool f32)
-{
-    int maxlin = 0, l2 = 0, dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&maxlin, cudaDevAttrMaxTexture1DLinearWidth, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) {
-        cudaGetLastError();
-        return;
-    }
-    double cap = kNmTextureL2 * l2;
-    if (const char* env = getenv("TRK_NM_TEXTURE_BYTES")) cap = strtod(env, nullptr);
-    if ((double)bytes > cap || plane > (int64_t)maxlin) return;
-    cudaResourceDesc rd{};
-    rd.resType = cudaResourceTypeLinear;
-    rd.res.linear.devPtr = t->field_nm;
-    rd.res.linear.desc = f32 ? cudaCreateChannelDesc<float4>() : cudaCreateChannelDesc<uint4>();
-    rd.res.linear.sizeInBytes = bytes;
-    cudaTextureDesc td{};
-    td.readMode = cudaReadModeElementType;
-    if (cudaCreateTextureObject(&t->nm_tex, &rd, &td, nullptr) != cudaSuccess) {
-        cudaGetLastError();
-        t->nm_tex = 0;
-    }
-}
-
-// The node-major copy of a float32 field that the direct kernel reads, made
-// (or refreshed after tracker_set_field) before the first direct launch that
-// needs it; never inside a graph capture (the first step of a call is eager).
-int ensure_node_major(tracker* t)
-{
-    // split bf16: one 16-byte record per node and chunk of three components,
-    // the chunks one after the other (C = 3: one chunk)
-    const bool f32 = t->storage == ST_F32, bf16 = t->storage == ST_BF16X2 && t->C % 3 == 0;
-    if (!(f32 || bf16) || t->nm_valid || t->nm_skip) return TRK_OK;
-    const int64_t NP = t->N + 2 * PAD;
-    const int64_t plane = NP * NP * NP;
-    const int nmc = f32 ? (t->C == 3 ? 4 : t->C) : 4 * (t->C / 3);
-    const size_t bytes = (size_t)plane * nmc * sizeof(float);   // 16 bytes per node for C = 3
-    if (t->nm_bytes != bytes) {
-        destroy_nm_texture(t);
-        dev_free(t->field_nm);
-        t->field_nm = nullptr;
-        t->nm_bytes = 0;
-        t->gen += 1;                  // captured graphs hold the old pointer
-        if (dev_alloc(&t->field_nm, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            // split bf16 with more than three components: the direct kernel reads
-            // the component-major field instead
-            if (bf16 && t->C > 3) {
-                t->nm_skip = true;
-                return TRK_OK;
-            }
-            return fail(TRK_ENOMEM, "cannot allocate the node-major field copy (%zu bytes)", bytes);
-        }
-        t->nm_bytes = bytes;
-    }
-    // the 16-byte node loads of the direct kernel (a copy first made for C = 4
-    // has the same size but no texture)
-    if (t->C == 3 && !t->nm_tex) create_nm_texture(t, plane, bytes, f32);
-    {
-        ProfScope ps(t, PROF_OTHER);
-        if (f32) {
-            CUDA_TRY(launch_node_major(reinterpret_cast<const float*>(t->field), t->C, nmc, plane, t->field_nm, t->stream));
-        } else {
-            const __nv_bfloat16* hi = reinterpret_cast<const __nv_bfloat16*>(t->field);
-            const __nv_bfloat16* lo = hi + plane * t->C;
-            for (int ch = 0; ch < t->C / 3; ++ch)
-                CUDA_TRY(launch_node_major_bf16(hi + plane * 3 * ch, lo + plane * 3 * ch, plane,
-                                                t->field_nm + plane * 4 * ch, t->stream));
-        }
-    }
-    t->launches += f32 ? 1 : t->C / 3;
-    t->nm_valid = true;
-    return TRK_OK;
+    return a.lb1 == b.lb1 && a.lb2 == b.lb2 && a.lb3 == b.lb3 && a.lseg == b.lseg;
 }
 
 // Below this many particles per grid cell the automatic choice gathers every
@@ -694,7 +615,11 @@ constexpr double kDirectDensity = 0.05;
 // RK2, block vs direct ms per step): float32 I = 8 1.24 vs 0.73 at 1/16 per
 // cell, 2.61 vs 2.65 at 1/4; float64 7.12 vs 6.02 and 24.7 vs 23.9;
 // split-bf16 (node-major copy) 1.19 vs 0.59 and 2.45 vs 2.20.
-double direct_threshold(const tracker* t) { return column_available(t) ? kDirectDensity : 0.25; }
+double direct_threshold(const tracker* t)
+{
+    if (!column_available(t)) return 0.25;
+    return t->I == 4 ? 0.2 : kDirectDensity;
+}
 
 // Below this many particles per grid cell the adjoint runs without halos
 // (direct mode); above it one CTA per cell block stages the block's halo.
@@ -703,20 +628,8 @@ double direct_threshold(const tracker* t) { return column_available(t) ? kDirect
 // 221 at 1/4.
 constexpr double kAdjDirectDensity = 0.125;
 
-// Remembers a timing decision; the oldest is dropped beyond kCacheMax entries
-// (a caller whose particle counts keep changing re-times now and then).
-constexpr size_t kCacheMax = 256;
-void remember(std::vector<std::pair<uint64_t, int>>& cache, uint64_t sig, int choice)
-{
-    if (cache.size() >= kCacheMax) cache.erase(cache.begin());
-    cache.emplace_back(sig, choice);
-}
-
-// Densities (particles per cell) between which AUTO times the column and the
-// direct kernel on the first tracker_advance call of a (np, scheme) and keeps
-// the faster: the crossover moves with the grid (L2 holds a 256^3 float32
-// field but not a 512^3 one) and with the scheme.
-constexpr double kProbeMin = 0.01, kProbeMax = 0.25;
+constexpr size_t kCacheMax = 256;   // remembered tuning decisions (the oldest is dropped)
+constexpr double kProbeMin = 0.01;  // particles per cell from which the column order is a candidate
 
 // The kernel tracker_advance (and, between BLOCK and DIRECT, tracker_interpolate)
 // uses for np particles before any timing.
@@ -725,6 +638,19 @@ int step_path(const tracker* t, int64_t np)
     if (t->step_kernel != TRK_STEP_AUTO) return t->step_kernel;
     if ((double)np < direct_threshold(t) * (double)t->N * t->N * t->N) return TRK_STEP_DIRECT;
     return column_available(t) ? TRK_STEP_COLUMN : TRK_STEP_BLOCK;
+}
+
+// AUTO interpolation: direct gathers below a density (and where the field has no
+// slabs to stage: C = 1, float64), the slab pipeline above.  Measured on GB300,
+// 256^3 float32, direct against slabs, us per call: u, I = 4 125 / 215 at 1/16
+// particle per cell, 488 / 386 at 1/4; I = 6 103 / 120 at 1/64, 300 / 221 at
+// 1/16; I = 8 160 / 183 at 1/64, 496 / 309 at 1/16; gradients, I = 6 378 / 380 at
+// 1/16, I = 8 238 / 224 at 1/64.
+bool interp_direct(const tracker* t, int64_t np, int deriv)
+{
+    if (t->storage == ST_F64 || !default_shape(t) || !t->tmap_ok[0] || t->halo_copy == TRK_HALO_ASYNC) return true;
+    const double dens = (double)np / ((double)t->N * t->N * t->N);
+    return dens < (t->I == 4 ? 0.2 : (t->I == 6 && deriv ? 0.06 : 0.025));
 }
 
 // One RK2/ABk step of tracker_advance: re-bin, then the fused step kernel.
@@ -747,37 +673,17 @@ int advance_step(tracker* t, int64_t np, int path, int mode, int ab_order, int h
         const float* rin = ab && hist > 0 ? (first ? rhs : t->rhs_s[cur]) : nullptr;
         CUDA_TRY(launch_count_scan(t->d_counts, bg.nb, t->offsets, t->d_cursor, t->d_scan_tmp, t->stream,
                                    &t->launches));
-        CUDA_TRY(launch_scatter_state(np, t->keys, t->d_cursor, first ? pos : t->pos_s[cur],
+        CUDA_TRY(launch_scatter_state(bg.g, np, t->keys, t->d_cursor, first ? pos : t->pos_s[cur],
                                       first ? nullptr : t->id_s[cur], rin, 3 * (ab_order - 1), t->pos_s[nxt],
-                                      t->id_s[nxt], t->rhs_s[nxt], t->d_flags, t->stream));
+                                      t->id_s[nxt], t->rhs_s[nxt], t->rec, t->storage == TRK_F64, t->d_flags, t->stream));
         t->launches += 1;
-    }
-    if (path == TRK_STEP_COLUMN) {
-        ColumnArgs ca{};
-        ca.a = base_args(t);
-        ca.a.np = np;
-        ca.a.dt = dt;
-        ca.a.pos_out = t->pos_s[nxt];
-        ca.a.rhs_out = t->rhs_s[nxt];
-        ca.a.key_out = t->keys;
-        ca.a.history_valid = ab ? hist : 0;
-        ca.a.ab_order = ab_order;
-        ca.nseg = column_segment(t);
-        ca.nitems = (int64_t)t->g.nb1 * t->g.nb2 * (t->g.nb3 / ca.nseg);
-        ca.ctr = t->d_colctr;
-        ca.counts = t->d_counts;
-        CUDA_TRY(cudaMemsetAsync(t->d_colctr, 0, sizeof(int), t->stream));
-        ProfScope ps(t, PROF_STEP);
-        t->launches += 1;
-        if (t->I == 4) CUDA_TRY(launch_column_i4(mode, ca, t->deg_hi, t->nsm, t->stream));
-        else CUDA_TRY(launch_column_i6(mode, ca, t->deg_hi, t->nsm, t->stream));
-        return TRK_OK;
     }
     BlockArgs a = base_args(t);
     a.g = bg.g;
     a.np = np;
     a.dt = dt;
     a.perm = nullptr;   // the state is grouped: read and written at j
+    a.rec_in = t->rec;
     a.pos_in = a.pos_out = t->pos_s[nxt];
     a.id_in = a.id_out = t->id_s[nxt];
     a.rhs_in = a.rhs_out = t->rhs_s[nxt];
@@ -786,7 +692,7 @@ int advance_step(tracker* t, int64_t np, int path, int mode, int ab_order, int h
     a.key_out = t->keys;
     a.counts = t->d_counts;
     if (path == TRK_STEP_DIRECT) CUDA_TRY(launch_direct(t, mode, a));
-    else CUDA_TRY(launch_block(t, mode, a));
+    else CUDA_TRY(launch_block(t, mode, a, path == TRK_STEP_COLUMN));
     return TRK_OK;
 }
 
@@ -807,7 +713,7 @@ constexpr int kTuneStepsPerCand = 2;    // the first run of a kernel may load it
 
 struct Cand {
     int path, dir_blk, col_seg, tma;
-    int ppc = PB_HOST;               // direct kernel: particles per CTA
+    int ppc = 256;                   // direct kernel: direct_particles
 };
 
 std::string tune_key(const tracker* t, int64_t np, int mode, int ab_order)
@@ -881,17 +787,6 @@ void load_tune_file(tracker* t)
     fclose(f);
 }
 
-// Particles per CTA of the direct kernel when nothing was timed: the largest
-// of 256, 128, 64 that still gives three CTAs per SM (smaller sets leave SMs
-// idle with 256: at 256^3 and 1.5e-3 particles per cell, 25,000 particles,
-// 128 per CTA took 0.044 ms per RK2 step against 0.065 ms).
-int default_ppc(const tracker* t, int64_t np)
-{
-    for (int p : {256, 128})
-        if ((np + p - 1) / p >= 3 * (int64_t)std::max(t->nsm, 1)) return p;
-    return 64;
-}
-
 // The candidates for np particles (measured on GB300, 256^3 float32, spline
 // I = 6, RK2 and AB2 from 1.5e-3 to 1/2 particle per cell: the winners were
 // always among these): the column kernel with segments of 8 and 16 slabs
@@ -901,19 +796,16 @@ int default_ppc(const tracker* t, int64_t np)
 // kProbeMin on without a column kernel; the direct kernel with binning edges
 // 8 and 16 up to one particle per cell.  Other block shapes than the default
 // run only the direct kernel.
-constexpr double kBlockMin = 0.1;
 std::vector<Cand> tune_candidates(const tracker* t, int64_t np)
 {
     std::vector<Cand> c;
     const double dens = (double)np / ((double)t->N * t->N * t->N);
     if (!default_shape(t)) return {Cand{TRK_STEP_DIRECT, BLK, 8, 1}};
-    const bool col = column_available(t);
-    if (col && dens >= kProbeMin)
-        for (int seg : {8, 16})
-            if (seg <= t->g.nb3) c.push_back({TRK_STEP_COLUMN, BLK, seg, 1});
-    if (dens >= (col ? kBlockMin : kProbeMin)) {
-        if (t->tmap_ok[0] && t->tmap_ok[1]) c.push_back({TRK_STEP_BLOCK, BLK, 8, 1});
-        c.push_back({TRK_STEP_BLOCK, BLK, 8, 0});
+    if (dens >= kProbeMin) {
+        if (column_available(t))
+            for (int seg : {1, 8}) c.push_back({TRK_STEP_COLUMN, BLK, seg, 1});
+        else if (t->tmap_ok[0] && t->tmap_ok[1])
+            c.push_back({TRK_STEP_BLOCK, BLK, 8, 1});
     }
     if (dens <= 1.0)
         for (int b : {8, 16})
@@ -984,8 +876,6 @@ int tracker_create(tracker** out, int N, double L, int family, int I, int m, int
     t->g.mask = N - 1;
     t->g.inv_delta = (double)N / L;
     int rc = set_geometry(t, BLK, BLK, BLK);
-    if (rc == TRK_OK && dev_alloc(&t->d_colctr, sizeof(int)) != cudaSuccess)
-        rc = fail(TRK_ENOMEM, "cannot allocate the column work counter");
     if (rc == TRK_OK && dev_alloc(&t->d_flags, NUM_FLAGS * sizeof(int)) != cudaSuccess)
         rc = fail(TRK_ENOMEM, "cannot allocate device flags");
     if (rc == TRK_OK && cudaMemset(t->d_flags, 0, NUM_FLAGS * sizeof(int)) != cudaSuccess)
@@ -998,6 +888,7 @@ int tracker_create(tracker** out, int N, double L, int family, int I, int m, int
         int dev = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&t->nsm, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&t->l2_bytes, cudaDevAttrL2CacheSize, dev);
     }
     if (rc != TRK_OK) {
         tracker_destroy(t);
@@ -1019,6 +910,7 @@ int tracker_destroy(tracker* t)
     else cudaDeviceSynchronize();
     dev_free(t->field);
     dev_free(t->sort_scratch);
+    dev_free(t->rec);
     dev_free(t->keys);
     dev_free(t->keys_sorted);
     dev_free(t->perm);
@@ -1035,20 +927,15 @@ int tracker_destroy(tracker* t)
     if (t->adv_graph.exec) cudaGraphExecDestroy(t->adv_graph.exec);
     if (t->batch_graph.exec) cudaGraphExecDestroy(t->batch_graph.exec);
     for (SetState& ss : t->sets) {
-        for (void* p : {(void*)ss.keys, (void*)ss.counts, (void*)ss.perm, (void*)ss.offsets, (void*)ss.list,
-                        (void*)ss.count, (void*)ss.pos_s[0], (void*)ss.pos_s[1], (void*)ss.id_s[0], (void*)ss.id_s[1],
-                        (void*)ss.rhs_s[0], (void*)ss.rhs_s[1]})
+        for (void* p : {(void*)ss.keys, (void*)ss.counts, ss.rec, (void*)ss.offsets, (void*)ss.pos_s[0],
+                        (void*)ss.pos_s[1], (void*)ss.id_s[0], (void*)ss.id_s[1], (void*)ss.rhs_s[0], (void*)ss.rhs_s[1]})
             dev_free(p);
     }
-    dev_free(t->ne_scratch);
     dev_free(t->d_desc);
     dev_free(t->d_ctr);
-    dev_free(t->d_colctr);
     dev_free(t->d_counts);
     dev_free(t->d_cursor);
     dev_free(t->d_scan_tmp);
-    destroy_nm_texture(t);
-    dev_free(t->field_nm);
     if (t->gev[0]) cudaEventDestroy(t->gev[0]);
     if (t->gev[1]) cudaEventDestroy(t->gev[1]);
     if (t->gstream) cudaStreamDestroy(t->gstream);
@@ -1123,15 +1010,15 @@ int tracker_set_field(tracker* t, const void* src, int C, int src_dtype, int src
     if (src_dtype != TRK_DTYPE_F64 && src_dtype != TRK_DTYPE_F32) return fail(TRK_EINVAL, "unknown src_dtype %d", src_dtype);
     const int64_t n = (int64_t)C * t->N * t->N * t->N;
     const int64_t NP = t->N + 2 * PAD;
-    const int64_t n_stored = (int64_t)C * NP * NP * NP;
-    const size_t esz = t->storage == TRK_F64 ? 8 : 4;
+    const size_t stored = (size_t)(NP * NP * NP) *
+                          (t->storage == TRK_F64 ? 8 * (size_t)C : 4 * (size_t)record_width(C) * record_chunks(C));
     if (t->C != C || !t->field) {
         dev_free(t->field);
         t->field = nullptr;
         t->C = 0;
-        if (dev_alloc(&t->field, (size_t)n_stored * esz) != cudaSuccess) {
+        if (dev_alloc(&t->field, stored) != cudaSuccess) {
             cudaGetLastError();
-            return fail(TRK_ENOMEM, "cannot allocate field storage (%zu bytes)", (size_t)n_stored * esz);
+            return fail(TRK_ENOMEM, "cannot allocate field storage (%zu bytes)", stored);
         }
         t->C = C;
     }
@@ -1150,8 +1037,6 @@ int tracker_set_field(tracker* t, const void* src, int C, int src_dtype, int src
         ProfScope ps(t, PROF_OTHER);
         CUDA_TRY(launch_convert_field(t->storage, src_dtype == TRK_DTYPE_F64, dsrc, C, t->N, t->field, t->stream));
     }
-    t->nm_skip = false;
-    t->nm_valid = false;              // the node-major copy is refreshed before its next use
     t->launches += 1;
     build_tmaps(t);
     if (staging) {
@@ -1254,7 +1139,11 @@ int tracker_halo_copy(const tracker* t, int mode)
 int tracker_field_texture(const tracker* t)
 {
     if (!t) return fail(TRK_EINVAL, "tracker is NULL");
-    return t->nm_valid && t->nm_tex && t->C == 3 ? 1 : 0;
+    if (!t->field || t->C != 3 || t->storage == TRK_F64) return 0;
+    const double NP = t->N + 2 * PAD;
+    double cap = 4.0 * t->l2_bytes;
+    if (const char* env = getenv("TRK_NM_TEXTURE_BYTES")) cap = strtod(env, nullptr);
+    return NP * NP * NP * 16.0 <= cap ? 1 : 0;
 }
 
 int64_t tracker_launch_count(const tracker* t) { return t ? t->launches : -1; }
@@ -1285,87 +1174,21 @@ int tracker_interpolate(tracker* t, int64_t np, const double* pos, void* out, in
     if (!t->field) return fail(TRK_ENOFIELD, "no field set");
     if (np > 0 && (!pos || !out)) return fail(TRK_EINVAL, "pos and out must not be NULL");
     if (out_dtype != TRK_DTYPE_F64 && out_dtype != TRK_DTYPE_F32) return fail(TRK_EINVAL, "unknown out_dtype %d", out_dtype);
-    bool direct = step_path(t, np) == TRK_STEP_DIRECT;
-    // AUTO: a cached timing decision, or time the block and the direct kernel
-    // now (they write the same values; the better one depends on density, C
-    // and the grid)
-    bool probe = false;
-    int interp_choice = -1;   // remembered: 0 block (cp.async halo), 1 block (tensor copy), 2 direct
-    const uint64_t sig = mix(mix(mix(mix(0x1f, (uint64_t)np), (uint64_t)t->C), (uint64_t)deriv), (uint64_t)out_dtype);
-    const bool block_shape = t->g.lb1 == LBLK && t->g.lb2 == LBLK && t->g.lb3 == LBLK;
-    if (t->step_kernel == TRK_STEP_AUTO && np > 0 && block_shape) {
-        int cached = -1;
-        for (const auto& e : t->interp_cache)
-            if (e.first == sig) cached = e.second;
-        if (cached >= 0) {
-            direct = cached == 2;
-            interp_choice = cached;
-        } else {
-            const double dens = (double)np / ((double)t->N * t->N * t->N);
-            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-            CUDA_TRY(cudaStreamIsCapturing(t->stream, &cs));
-            probe = dens >= kProbeMin && dens <= kProbeMax && cs == cudaStreamCaptureStatusNone;
-        }
-    }
+    const bool direct = t->step_kernel == TRK_STEP_DIRECT || (t->step_kernel == TRK_STEP_AUTO && interp_direct(t, np, deriv));
     if (!direct && (rc = check_block_kernel_shape(t))) return rc;
     if (np == 0) return TRK_OK;
     if ((rc = ensure_sort(t, np))) return rc;
-    if ((direct || probe) && (rc = ensure_node_major(t))) return rc;
-    // the kernels read the positions through the permutation (gathering them
-    // into block order first measured slower overall: 1024^3, I = 8, 2^27
-    // tracers, the block kernel gains 5.2 ms, the gather costs 7.8 ms)
-    if ((rc = bin_counting(t, np, pos))) return rc;
+    if ((rc = ensure_rec(t, np)) || (rc = bin_counting(t, np, pos, t->rec))) return rc;
     BlockArgs a = base_args(t);
     a.np = np;
-    a.perm = t->perm;
-    a.pos_in = pos;
-    a.ppc = default_ppc(t, np);
+    a.id_in = t->perm;   // grouped position -> caller index; the kernels read the records
+    a.rec_in = t->rec;
+    a.ppc = 0;
     a.out = out;
     a.out_f64 = out_dtype == TRK_DTYPE_F64;
     const int mode = deriv ? MODE_INTERP_DERIV : MODE_INTERP;
-    if (probe) {
-        // the block kernel with each halo copy it has, then the direct kernel;
-        // all write the same values, the fastest is remembered
-        const bool saved = t->auto_tma;
-        std::vector<int> kinds;   // 0: block, cp.async halo; 1: block, tensor copy; 2: direct
-        if (t->halo_copy == TRK_HALO_AUTO && halo_tmap_exists(t, mode)) kinds.push_back(1);
-        kinds.push_back(t->halo_copy == TRK_HALO_TMA && halo_tmap_exists(t, mode) ? 1 : 0);
-        kinds.push_back(2);
-        std::vector<cudaEvent_t> ev(kinds.size() + 1, nullptr);
-        for (auto& e : ev)
-            if (cudaEventCreate(&e) != cudaSuccess) rc = fail(TRK_ECUDA, "cudaEventCreate failed");
-        std::vector<float> ms(kinds.size(), 0.f);
-        if (rc == TRK_OK) {
-            cudaError_t e = cudaEventRecord(ev[0], t->stream);
-            for (size_t i = 0; e == cudaSuccess && i < kinds.size(); ++i) {
-                t->auto_tma = kinds[i] == 1;
-                e = kinds[i] == 2 ? launch_direct(t, mode, a) : launch_block(t, mode, a);
-                if (e == cudaSuccess) e = cudaEventRecord(ev[i + 1], t->stream);
-            }
-            if (e == cudaSuccess) e = cudaEventSynchronize(ev.back());
-            for (size_t i = 0; e == cudaSuccess && i < kinds.size(); ++i) e = cudaEventElapsedTime(&ms[i], ev[i], ev[i + 1]);
-            if (e != cudaSuccess) rc = fail(TRK_ECUDA, "timing the interpolation kernels: %s", cudaGetErrorString(e));
-        }
-        t->auto_tma = saved;
-        for (auto& e : ev)
-            if (e) cudaEventDestroy(e);
-        if (rc) return rc;
-        size_t best = 0;
-        for (size_t i = 1; i < kinds.size(); ++i)
-            if (ms[i] < ms[best]) best = i;
-        remember(t->interp_cache, sig, kinds[best]);
-        t->last_kernel = kinds[best] == 2 ? TRK_STEP_DIRECT : TRK_STEP_BLOCK;
-        return TRK_OK;
-    }
-    if (direct) {
-        CUDA_TRY(launch_direct(t, mode, a));
-    } else {
-        const bool saved = t->auto_tma;
-        if (interp_choice >= 0) t->auto_tma = interp_choice == 1;
-        const cudaError_t e = launch_block(t, mode, a);
-        t->auto_tma = saved;
-        CUDA_TRY(e);
-    }
+    if (direct) CUDA_TRY(launch_direct(t, mode, a));
+    else CUDA_TRY(launch_block(t, mode, a));
     t->last_kernel = direct ? TRK_STEP_DIRECT : TRK_STEP_BLOCK;
     return TRK_OK;
 }
@@ -1411,16 +1234,14 @@ int tracker_advance(tracker* t, int64_t np, double* pos, float* rhs, double dt, 
             const bool timed = np >= kTuneMinNp && cands.size() >= 2 &&
                                steps >= kTuneStepsPerCand * (int)cands.size() + 2 && cs == cudaStreamCaptureStatusNone;
             if (!timed) cands.clear();
-            apply_cand(t, Cand{path, BLK, 8, 1, default_ppc(t, np)});
+            apply_cand(t, Cand{path, BLK, 8, 1, 0});
         }
     }
     if (path != TRK_STEP_DIRECT && (rc = check_block_kernel_shape(t))) return rc;
     if (np == 0 || steps == 0) return TRK_OK;
     if ((rc = ensure_sort(t, np))) return rc;
-    if ((rc = ensure_state(t, np))) return rc;
-    bool any_direct = path == TRK_STEP_DIRECT;
+    if ((rc = ensure_state(t, np)) || (rc = ensure_rec(t, np))) return rc;
     for (const Cand& c : cands) {
-        any_direct = any_direct || c.path == TRK_STEP_DIRECT;
         Cand save{path, t->dir_blk, t->col_seg, t->auto_tma, t->dir_ppc};
         apply_cand(t, c);
         rc = ensure_bin(t, geom_of(t, c.path).nb);
@@ -1428,7 +1249,6 @@ int tracker_advance(tracker* t, int64_t np, double* pos, float* rhs, double dt, 
         if (rc) return rc;
     }
     if ((rc = ensure_bin(t, geom_of(t, path).nb))) return rc;
-    if (any_direct && (rc = ensure_node_major(t))) return rc;
     // initial keys and block counts from the caller's positions
     GridGeom last_g = geom_of(t, path).g;
     {
@@ -1523,7 +1343,7 @@ int tracker_advance(tracker* t, int64_t np, double* pos, float* rhs, double dt, 
         cur ^= 1;
     }
     t->last_kernel = path;
-    t->last_tuning = {path, t->dir_blk, t->col_seg, halo_tmap(t, mode) ? 1 : 0, t->dir_ppc};
+    t->last_tuning = {path, t->dir_blk, t->col_seg, halo_tmap(t, mode) ? 1 : 0, t->dir_ppc ? t->dir_ppc : 64};
     ProfScope ps(t, PROF_OTHER);
     CUDA_TRY(launch_unpermute_pos(np, t->pos_s[cur], t->id_s[cur], pos, t->stream));
     t->launches += 1;
@@ -1549,16 +1369,14 @@ static int ensure_set(tracker* t, SetState& ss, int64_t np)
 {
     if (np <= ss.cap && ss.nb == t->nblocks) return TRK_OK;
     t->gen += 1;
-    for (void* p : {(void*)ss.keys, (void*)ss.counts, (void*)ss.perm, (void*)ss.offsets, (void*)ss.list,
-                    (void*)ss.count, (void*)ss.pos_s[0], (void*)ss.pos_s[1], (void*)ss.id_s[0], (void*)ss.id_s[1],
-                    (void*)ss.rhs_s[0], (void*)ss.rhs_s[1]})
+    for (void* p : {(void*)ss.keys, (void*)ss.counts, ss.rec, (void*)ss.offsets, (void*)ss.pos_s[0],
+                    (void*)ss.pos_s[1], (void*)ss.id_s[0], (void*)ss.id_s[1], (void*)ss.rhs_s[0], (void*)ss.rhs_s[1]})
         dev_free(p);
     ss = SetState{};
     bool ok = dev_alloc(&ss.keys, (size_t)np * 4) == cudaSuccess &&
               dev_alloc(&ss.counts, (size_t)t->nblocks * 4) == cudaSuccess &&
-              dev_alloc(&ss.perm, (size_t)np * 4) == cudaSuccess &&
-              dev_alloc(&ss.offsets, (size_t)(t->nblocks + 1) * 4) == cudaSuccess &&
-              dev_alloc(&ss.list, (size_t)t->nblocks * 4) == cudaSuccess && dev_alloc(&ss.count, 4) == cudaSuccess;
+              dev_alloc(&ss.rec, (size_t)np * 16) == cudaSuccess &&
+              dev_alloc(&ss.offsets, (size_t)(t->nblocks + 1) * 4) == cudaSuccess;
     for (int i = 0; i < 2 && ok; ++i)
         ok = dev_alloc(&ss.pos_s[i], (size_t)np * 24) == cudaSuccess && dev_alloc(&ss.id_s[i], (size_t)np * 4) == cudaSuccess &&
              dev_alloc(&ss.rhs_s[i], (size_t)np * 12) == cudaSuccess;
@@ -1583,18 +1401,20 @@ static int keys_set(tracker* t, SetState& ss, int64_t np, const double* pos)
 
 // Re-binning of one set by counting sort: the block counts (from keys_set, or
 // added by the previous step's kernel) scanned into offsets and cursors (the
-// counts are left zero), the permutation, and (halo path) the non-empty block
-// list.  The cursors and scan scratch are the tracker's, shared by the sets,
-// which are binned one after another on the stream.
-static int bin_set(tracker* t, SetState& ss, int64_t np, bool direct)
+// counts are left zero), and the state scattered into its blocks (buffer nxt)
+// with its records.  first: from the caller's arrays.  The cursors and scan
+// scratch are the tracker's, shared by the sets, which are binned one after
+// another on the stream.
+static int bin_set(tracker* t, SetState& ss, const trk_set& S, bool first, bool hist, int nxt)
 {
     ProfScope ps(t, PROF_BIN);
     CUDA_TRY(launch_count_scan(ss.counts, t->nblocks, ss.offsets, t->d_cursor, t->d_scan_tmp, t->stream,
                                &t->launches));
-    CUDA_TRY(launch_scatter_perm(np, ss.keys, t->d_cursor, ss.perm, t->d_flags, t->stream));
+    CUDA_TRY(launch_scatter_state(t->g, S.np, ss.keys, t->d_cursor, first ? S.pos : ss.pos_s[nxt ^ 1],
+                                  first ? nullptr : ss.id_s[nxt ^ 1],
+                                  !hist ? nullptr : (first ? S.rhs : ss.rhs_s[nxt ^ 1]), 3, ss.pos_s[nxt], ss.id_s[nxt],
+                                  ss.rhs_s[nxt], ss.rec, 0, t->d_flags, t->stream));
     t->launches += 1;
-    if (!direct) CUDA_TRY(launch_nonempty_list(ss.offsets, t->nblocks, ss.list, ss.count, t->ne_scratch, t->stream,
-                                               &t->launches));
     return TRK_OK;
 }
 
@@ -1602,18 +1422,7 @@ static int batched_launch(tracker* t, const BatchSet* d_desc, int nsets)
 {
     ProfScope ps(t, PROF_STEP);
     CUDA_TRY(cudaMemsetAsync(t->d_ctr, 0, (size_t)nsets * sizeof(int), t->stream));
-    // tensor-copy halos for the halo-staged sets of a float32 field, one box per kernel width
-    const void* maps[3] = {nullptr, nullptr, nullptr};
-    const bool tma = t->halo_copy == TRK_HALO_TMA || (t->halo_copy == TRK_HALO_AUTO && t->auto_tma);
-    if (tma && t->storage == TRK_F32) {
-        bool ok = true;
-        for (int i = 0; i < 3; ++i) {
-            ok = ok && encode_field_map(t, 4 + 2 * i, 0, &t->batch_map[i]);
-            maps[i] = &t->batch_map[i];
-        }
-        if (!ok) maps[0] = maps[1] = maps[2] = nullptr;
-    }
-    CUDA_TRY(launch_batched(t->storage, d_desc, nsets, t->d_ctr, t->nsm, maps[0] ? maps : nullptr, t->stream));
+    CUDA_TRY(launch_batched(t->storage, d_desc, nsets, t->d_ctr, t->nsm, t->stream));
     t->launches += 1;
     return TRK_OK;
 }
@@ -1632,8 +1441,6 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
     if (steps < 0) return fail(TRK_EINVAL, "steps=%d < 0", steps);
     int rc = check_block_kernel_shape(t);
     if (rc) return rc;
-    // the direct items of the sets read the node-major copy of the field
-    if (nsets > 0 && steps > 0 && (rc = ensure_node_major(t))) return rc;
     std::vector<int> tabs(nsets);
     int64_t npmax = 0;
     for (int s = 0; s < nsets; ++s) {
@@ -1652,16 +1459,6 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
     if ((int)t->sets.size() < nsets) t->sets.resize(nsets);
     for (int s = 0; s < nsets; ++s)
         if ((rc = ensure_set(t, t->sets[s], std::max<int64_t>(sets[s].np, 1)))) return rc;
-    if (t->ne_cap < t->nblocks) {
-        dev_free(t->ne_scratch);
-        t->ne_scratch = nullptr;
-        t->gen += 1;
-        if (dev_alloc(&t->ne_scratch, nonempty_scratch_bytes(t->nblocks)) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(TRK_ENOMEM, "cannot allocate the block-list scratch");
-        }
-        t->ne_cap = t->nblocks;
-    }
     if (t->desc_cap < nsets) {
         dev_free(t->d_desc);
         dev_free(t->d_ctr);
@@ -1675,10 +1472,9 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
         }
         t->desc_cap = nsets;
     }
-    // host-side descriptors: [0] first step, [1] parity 0 -> 1, [2] parity 1 -> 0
+    // host-side descriptors: [0] first step (into buffer 1), [1] into buffer 0, [2] into buffer 1
     std::vector<BatchSet> h(3 * (size_t)nsets);
     const BlockArgs base = base_args(t);
-    std::vector<int> direct(nsets, 0);
     for (int s = 0; s < nsets; ++s) {
         const trk_set& S = sets[s];
         SetState& ss = t->sets[s];
@@ -1691,7 +1487,7 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
                 a.cf.d[i][d] = (float)kDCoef[tabs[s]][i][d];
             }
         a.np = S.np;
-        a.perm = ss.perm;
+        a.rec_in = ss.rec;
         a.offsets = ss.offsets;
         a.dt = dt;
         a.key_out = ss.keys;
@@ -1700,80 +1496,16 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
         for (int v = 0; v < 3; ++v) {
             BatchSet& B = h[(size_t)v * nsets + s];
             B.a = a;
-            const int cur = v == 2 ? 1 : 0;
-            if (v == 0) {
-                B.a.pos_in = S.pos;
-                B.a.id_in = nullptr;
-                B.a.rhs_in = S.rhs;
-                B.a.history_valid = history_valid;
-            } else {
-                B.a.pos_in = ss.pos_s[cur];
-                B.a.id_in = ss.id_s[cur];
-                B.a.rhs_in = ss.rhs_s[cur];
-                B.a.history_valid = 1;
-            }
-            B.a.pos_out = ss.pos_s[cur ^ 1];
-            B.a.id_out = ss.id_s[cur ^ 1];
-            B.a.rhs_out = ss.rhs_s[cur ^ 1];
-            B.list = ss.list;
-            B.count = ss.count;
+            const int nxt = v == 1 ? 0 : 1;   // the state is grouped: updated in place
+            B.a.pos_in = B.a.pos_out = ss.pos_s[nxt];
+            B.a.id_in = B.a.id_out = ss.id_s[nxt];
+            B.a.rhs_in = B.a.rhs_out = ss.rhs_s[nxt];
+            B.a.history_valid = v == 0 ? history_valid : 1;
             B.n_items = (int)((S.np + PB_HOST - 1) / PB_HOST);
             B.I = S.I;
             B.deg_hi = kTables[tabs[s]].deg > S.I - 1;
             B.deriv = S.deriv;
-            B.direct = 0;
         }
-    }
-    // per-set path: halo-staged blocks or direct gathers, chosen by timing both once
-    for (int s = 0; s < nsets; ++s) {
-        const trk_set& S = sets[s];
-        if (S.np == 0) {   // empty set: no items (the direct path reads n_items = 0)
-            direct[s] = 1;
-            for (int v = 0; v < 3; ++v) h[(size_t)v * nsets + s].direct = 1;
-            continue;
-        }
-        const uint64_t sig = mix(mix(mix(mix(mix(0, (uint64_t)S.np), (uint64_t)S.I), (uint64_t)S.deriv),
-                                     (uint64_t)tabs[s]), (uint64_t)t->N);
-        int choice = -1;
-        for (auto& kv : t->tune_cache)
-            if (kv.first == sig) choice = kv.second;
-        if (choice < 0) {
-            SetState& ss = t->sets[s];
-            const size_t vb = (size_t)S.np * 24;
-            CUDA_TRY(cudaMemcpyAsync(ss.pos_s[1], S.pos, vb, cudaMemcpyDeviceToDevice, t->stream));
-            if ((rc = keys_set(t, ss, S.np, ss.pos_s[1]))) return rc;
-            if ((rc = bin_set(t, ss, S.np, false))) return rc;
-            BatchSet probe = h[(size_t)nsets + s];           // parity-0 layout: reads pos_s[0] ...
-            probe.a.pos_in = ss.pos_s[1];                     // ... so point it at the copy
-            probe.a.id_in = nullptr;
-            probe.a.rhs_in = nullptr;
-            probe.a.history_valid = 0;
-            probe.a.pos_out = ss.pos_s[0];
-            probe.a.id_out = ss.id_s[0];
-            probe.a.rhs_out = ss.rhs_s[0];
-            probe.a.out = nullptr;
-            float best[2] = {0, 0};
-            cudaEvent_t e0, e1;
-            CUDA_TRY(cudaEventCreate(&e0));
-            CUDA_TRY(cudaEventCreate(&e1));
-            for (int variant = 0; variant < 2; ++variant) {
-                probe.direct = variant;
-                CUDA_TRY(cudaMemcpyAsync(t->d_desc, &probe, sizeof(BatchSet), cudaMemcpyHostToDevice, t->stream));
-                for (int rep = 0; rep < 2; ++rep) {
-                    CUDA_TRY(cudaEventRecord(e0, t->stream));
-                    if ((rc = batched_launch(t, t->d_desc, 1))) return rc;
-                    CUDA_TRY(cudaEventRecord(e1, t->stream));
-                    CUDA_TRY(cudaEventSynchronize(e1));
-                    CUDA_TRY(cudaEventElapsedTime(&best[variant], e0, e1));
-                }
-            }
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            choice = best[1] < best[0] ? 1 : 0;
-            remember(t->tune_cache, sig, choice);
-        }
-        direct[s] = choice;
-        for (int v = 0; v < 3; ++v) h[(size_t)v * nsets + s].direct = choice;
     }
     CUDA_TRY(cudaMemcpyAsync(t->d_desc, h.data(), h.size() * sizeof(BatchSet), cudaMemcpyHostToDevice, t->stream));
     CUDA_TRY(cudaStreamSynchronize(t->stream));   // h may be released after this
@@ -1784,7 +1516,7 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
                 int r = keys_set(t, t->sets[s], sets[s].np, sets[s].pos);
                 if (r) return r;
             }
-            int r = bin_set(t, t->sets[s], sets[s].np, direct[s]);
+            int r = bin_set(t, t->sets[s], sets[s], v == 0, v != 0 || history_valid, v == 1 ? 0 : 1);
             if (r) return r;
         }
         return batched_launch(t, t->d_desc + (size_t)v * nsets, nsets);
@@ -1796,18 +1528,18 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
         uint64_t key = mix(mix(mix(0, t->gen), (uint64_t)nsets), dbits(dt));
         for (int s = 0; s < nsets; ++s)
             key = mix(mix(mix(mix(mix(key, (uint64_t)sets[s].np), (uint64_t)sets[s].I), (uint64_t)tabs[s]),
-                          (uint64_t)direct[s] * 2 + sets[s].deriv),
+                          (uint64_t)sets[s].deriv),
                       (uint64_t)(uintptr_t)sets[s].out);
-        // the state is in buffer 1 after the first step: parity 1 -> 0, then 0 -> 1
+        // the state is in buffer 1 after the first step: into 0, then into 1
         rc = replay_graph(t, t->batch_graph, key, rest / 2, [&]() {
-            int r = step(2);
-            return r ? r : step(1);
+            int r = step(1);
+            return r ? r : step(2);
         });
         if (rc) return rc;
         rest -= 2 * (rest / 2);
     }
     for (; rest > 0; --rest) {
-        if ((rc = step(cur == 1 ? 2 : 1))) return rc;
+        if ((rc = step(cur == 1 ? 1 : 2))) return rc;
         cur ^= 1;
     }
     ProfScope ps(t, PROF_OTHER);
@@ -1908,7 +1640,7 @@ int tracker_adjoint(tracker* t, int64_t np, const double* pos0, const double* la
         }
         for (int i = s1 - s0 - 1; i >= 0; --i) {
             const double* X = seg + (size_t)i * vec;
-            if ((rc = bin_counting(t, np, X))) return rc;
+            if ((rc = bin_counting(t, np, X, nullptr))) return rc;
             AdjArgs a{};
             const BlockArgs b = base_args(t);
             a.g = b.g;
