@@ -907,10 +907,11 @@ __global__ void k_adj_gather(const __grid_constant__ AdjArgs a)
     }
     // every slab value is read by exactly one node: leave the slabs zero for the
     // next step's atomic adds
+    // (the float32 scatter writes whole slabs and needs no zeros)
     T* gz = reinterpret_cast<T*>(a.gscratch);
 #pragma unroll
     for (int c = 0; c < NA * NA * NA; ++c)
-        if (use[c]) {
+        if (sizeof(T) == 8 && use[c]) {
             T* sb = gz + bidx[c] * 3 * H3 + hoff[c];
             sb[0] = (T)0;
             sb[H3] = (T)0;
@@ -951,9 +952,7 @@ cudaError_t launch_adjoint_t(const AdjArgs& a, int64_t nblocks, cudaStream_t st)
 template <int I, int DEG>
 cudaError_t dispatch_adjoint(const AdjArgs& a, int64_t nblocks, cudaStream_t st)
 {
-    if (a.f.storage == ST_F64) return launch_adjoint_t<double, I, DEG, ST_F64>(a, nblocks, st);
-    if (a.f.storage == ST_F32) return launch_adjoint_t<float, I, DEG, ST_F32>(a, nblocks, st);
-    return launch_adjoint_t<float, I, DEG, ST_BF16X2>(a, nblocks, st);
+    return launch_adjoint_t<double, I, DEG, ST_F64>(a, nblocks, st);
 }
 
 }  // namespace adj

@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(CS_THREADS) k_count_scan(uint32_t* __restrict_
 }
 
 // The same for large grids, over all SMs: tiles of CT_TILE counts (nblocks a
-// multiple of CT_TILE).  k_tile_sums sums each tile; k_tile_scan adds the sums
+// multiple of CT_TILE; counts, offsets and cursor on 16-byte boundaries).  k_tile_sums sums each tile; k_tile_scan adds the sums
 // of the preceding tiles and scans its own tile, CT_PER counts per thread
 // read and written as 16-byte vectors.
 constexpr int CT_THREADS = 256, CT_PER = 16, CT_TILE = CT_THREADS * CT_PER;

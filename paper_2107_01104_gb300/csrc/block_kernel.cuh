@@ -116,9 +116,8 @@ __global__ void __launch_bounds__(NT, 4)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 3;
     Place at{};
     at.halo = smem_raw;
-    at.o1 = b % a.g.nb1 * BLK - HG::G;
-    at.o2 = b / a.g.nb1 % a.g.nb2 * BLK - HG::G;
-    at.o3 = b / (a.g.nb1 * a.g.nb2) * BLK - HG::G;
+    const int o1 = b % a.g.nb1 * BLK - HG::G, o2 = b / a.g.nb1 % a.g.nb2 * BLK - HG::G,
+              o3 = b / (a.g.nb1 * a.g.nb2) * BLK - HG::G;
     uint64_t* mbar = reinterpret_cast<uint64_t*>(smem_raw + PL::mbar);
     unsigned char* ws = smem_raw + PL::warp + warp * WarpPlan<T, MODE, NC>::total;
     const WarpMem<T, MODE, NC> wm(ws, g);
@@ -136,10 +135,10 @@ __global__ void __launch_bounds__(NT, 4)
     auto issue_halo = [&](int ch) {
         if constexpr (HC == HC_TMA) {
             if (tid == 0)
-                tma_issue(smem_raw, &tmap, at.o1 + PAD - HG::XOFF, at.o2 + PAD, at.o3 + PAD, NC * ch, mbar,
+                tma_issue(smem_raw, &tmap, o1 + PAD - HG::XOFF, o2 + PAD, o3 + PAD, NC * ch, mbar,
                           (uint32_t)(NC * HG::SC * sizeof(double)));
         } else {
-            stage_halo_async<T, I, MODE, NC, STORE, RW>(smem_raw, a.f, ch, at.o1, at.o2, at.o3);
+            stage_halo_async<T, I, MODE, NC, STORE, RW>(smem_raw, a.f, ch, o1, o2, o3);
         }
     };
     for (int b0 = j0; b0 < j1; b0 += PB) {
@@ -176,9 +175,7 @@ __global__ void __launch_bounds__(NT, 4)
             }
             for (int it = 0; it < 8 && it * 4 * NW < left; ++it) {
                 const PRec<T> rec = wm.recs[4 * it + g];
-                int c[3];
-                unpack_cell(cell_of(rec), c);   // (a particle lies in its own block)
-                at.r1 = (c[0] & 7) + HG::G, at.r2 = (c[1] & 7) + HG::G, at.r3 = (c[2] & 7) + HG::G;
+                unpack_cell(cell_of(rec), at.c);   // (a particle lies in its own block)
                 T res[result_count<MODE, NC>()];
                 interpolate_group<T, I, DEG, MODE, NC, STORE, RW, SRC_HALO>(
                     a, at, ch, rec.t, it * 4 * NW + g < left, lane, B, m, wm.wb0, wm.wb1, it & 1, res);
@@ -229,7 +226,8 @@ __global__ void __launch_bounds__(NT, 4)
 template <int I, int MODE, int NC>
 struct SlabPlan {
     using SG = SlabGeom<I, MODE>;
-    static constexpr int warps = 4 * min_ctas<float, I, MODE, SRC_SLABS>();
+    // (the adjoint hands 22 values per particle over: fewer warps leave room for the slabs)
+    static constexpr int warps = MODE == MODE_ADJ ? (I == 8 ? 8 : 12) : 4 * min_ctas<float, I, MODE, SRC_SLABS>();
     static constexpr size_t slab = SG::slot;
     static constexpr size_t per_warp = WarpPlan<float, MODE, NC>::total;
     static constexpr size_t room = 232448 - 256 - warps * per_warp;
@@ -387,7 +385,8 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
         const int left = (int)min(j1 - b0 - 4 * warp, (int64_t)4 * nw * rounds);
         if (left <= 0) break;
         const bool valid = j < j1 && (lane >> 2) < rounds;
-        fetch_state<T, MODE, NC>(a, j, valid, ws, lane);
+        const int32_t id = !valid ? 0 : (a.id_in ? a.id_in[j] : (int32_t)j);
+        fetch_state<T, MODE, NC>(a, MODE == MODE_ADJ ? id : j, valid, ws, lane);
         fetch_records(bn, 8, buf ^ 1);
         cp_async_commit();
         cp_async_wait_group<1>();
@@ -406,14 +405,11 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
                 const int lo = (int)__reduce_min_sync(0xffffffffu, todo ? (unsigned)q : 0x7fffffffu);
                 const bool now = todo && q - lo <= SG::SPT;
                 Place at{};
+                at.c[0] = c[0], at.c[1] = c[1], at.c[2] = c[2];
                 at.slab = now ? q : lo;
                 slabs.release_to(lo, lane, nw);
                 slabs.need((int)__reduce_max_sync(0xffffffffu, (unsigned)at.slab) + SG::NSL - 1);
                 at.halo = smem_raw;
-                at.r1 = (c[0] & 7) + SG::G, at.r2 = (c[1] & 7) + SG::G, at.r3 = (c[2] & 7) + SG::G;
-                if constexpr (MODE == MODE_RK2) {
-                    at.o1 = (c[0] & ~7) - SG::G, at.o2 = (c[1] & ~7) - SG::G, at.o3 = (c[2] & ~7) - SG::G;
-                }
                 T res[result_count<MODE, NC>()];
                 interpolate_group<T, I, DEG, MODE, NC, STORE, 4, SRC_SLABS, SP::NS>(a, at, slabs.ch, rec.t, now, lane, B, m,
                                                                                     wm.wb0, wm.wb1, odd & 1, res);
@@ -422,11 +418,13 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
                 todo = todo && !now;
             } while (__any_sync(0xffffffffu, todo));
         }
-        const int32_t id = !valid ? 0 : (a.id_in ? a.id_in[j] : (int32_t)j);
         __syncwarp();
         if constexpr (is_step<MODE>()) {
             cp_async_wait_all();
             update_particle<T, MODE, NC>(a, j, id, valid, ws, lane);
+        } else if constexpr (MODE == MODE_ADJ) {
+            cp_async_wait_all();
+            adjoint_particle<T, MODE, NC>(a, j, id, valid, ws, lane);
         } else if (valid) {
             write_outputs<T, MODE, NC>(a, id, slabs.ch, ws, lane);
         }
@@ -470,7 +468,7 @@ cudaError_t launch_slabs(BlockArgs a, const CUtensorMap& tmap, cudaStream_t st)
     if (a.np <= 0) return cudaSuccess;
     // one contiguous run of particles per SM, whole fours
     a.ppc = (int)(((a.np + nsm - 1) / nsm + 3) / 4 * 4);
-    const dim3 grid((unsigned)((a.np + a.ppc - 1) / a.ppc), is_step<MODE>() ? 1 : (unsigned)((a.f.C + NC - 1) / NC));
+    const dim3 grid((unsigned)((a.np + a.ppc - 1) / a.ppc), WarpPlan<float, MODE, NC>::HAS_X ? 1 : (unsigned)((a.f.C + NC - 1) / NC));
     kern<<<grid, 32 * SP::warps, SP::total, st>>>(a, tmap);
     return cudaGetLastError();
 }

@@ -25,7 +25,8 @@ enum { ST_F64 = 0, ST_F32 = 1, ST_BF16X2 = 2 };
 
 // Block-kernel modes.
 // MODE_AB2_D: AB2 step that also writes du_k/dX_j at the step's start.
-enum { MODE_INTERP = 0, MODE_INTERP_DERIV = 1, MODE_RK2 = 2, MODE_AB2 = 3, MODE_AB2_D = 4 };
+// MODE_ADJ: the adjoint of an RK2 step (Jacobians at X and X*, lambda recurrence).
+enum { MODE_INTERP = 0, MODE_INTERP_DERIV = 1, MODE_RK2 = 2, MODE_AB2 = 3, MODE_AB2_D = 4, MODE_ADJ = 5 };
 
 constexpr int BLK = 8;        // cell-block edge used by the block kernels
 constexpr int LBLK = 3;       // log2(BLK)
@@ -129,6 +130,7 @@ struct BlockArgs {
     int ppc;                  // direct kernel: particles per CTA (a multiple of 16), 0 (by size) or PPC_WIDE
     double dt;
     int* flags;
+    float4* adj;              // MODE_ADJ: [3][np] X* (offsets, cell), mu, dt/2 lambda (grouped) or null
 };
 
 constexpr int PPC_WIDE = -1;
@@ -168,6 +170,18 @@ struct AdjArgs {
                               // float64 storage), or null: float64 atomics instead
     double dt;
     int* flags;
+};
+
+// Arguments of the field-gradient scatter (float32 / split-bf16 fields).
+struct AdjScatterArgs {
+    GridGeom g;
+    CoefTable<float> cf;
+    int64_t np;
+    const int32_t* offsets;   // [nblocks + 1] of the grouped particles
+    const float4* rec;        // [np] records of X
+    const float4* adj;        // [3][np] X*, mu, dt/2 lambda (BlockArgs::adj)
+    double* gfield;           // [3][N^3] dLoss/dfield (added into)
+    float* gscratch;          // [nblocks][3][H^3] per-block sums, or null: float64 atomics instead
 };
 
 // One particle set of a batched step, resident in device memory.
@@ -338,6 +352,13 @@ cudaError_t launch_convert_field(int storage, int src_f64, const void* src, int 
 cudaError_t launch_adjoint_gather(int I, const AdjArgs& a, cudaStream_t st);
 // halo edge of the adjoint kernel for kernel width I (stage-2 margin included)
 constexpr int adj_halo(int I) { return BLK + I - 1 + 2; }
+cudaError_t launch_adj_particles_i4(const BlockArgs& a, const void* tmap, int deg_hi, cudaStream_t st);
+cudaError_t launch_adj_particles_i6(const BlockArgs& a, const void* tmap, int deg_hi, cudaStream_t st);
+cudaError_t launch_adj_particles_i8(const BlockArgs& a, const void* tmap, int deg_hi, cudaStream_t st);
+cudaError_t launch_adj_scatter_i4(const AdjScatterArgs& a, int64_t nblocks, int deg_hi, cudaStream_t st);
+cudaError_t launch_adj_scatter_i6(const AdjScatterArgs& a, int64_t nblocks, int deg_hi, cudaStream_t st);
+cudaError_t launch_adj_scatter_i8(const AdjScatterArgs& a, int64_t nblocks, int deg_hi, cudaStream_t st);
+// float64 fields
 cudaError_t launch_adjoint_i4(const AdjArgs& a, int64_t nblocks, int deg_hi, cudaStream_t st);
 cudaError_t launch_adjoint_i6(const AdjArgs& a, int64_t nblocks, int deg_hi, cudaStream_t st);
 cudaError_t launch_adjoint_i8(const AdjArgs& a, int64_t nblocks, int deg_hi, cudaStream_t st);

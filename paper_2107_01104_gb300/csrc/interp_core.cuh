@@ -346,12 +346,22 @@ __host__ __device__ constexpr bool is_ab() { return MODE == MODE_AB2 || MODE == 
 template <int MODE>
 __host__ __device__ constexpr bool is_step() { return MODE == MODE_RK2 || is_ab<MODE>(); }
 template <int MODE>
-__host__ __device__ constexpr bool is_deriv() { return MODE == MODE_INTERP_DERIV || MODE == MODE_AB2_D; }
+__host__ __device__ constexpr bool is_deriv()
+{
+    return MODE == MODE_INTERP_DERIV || MODE == MODE_AB2_D || MODE == MODE_ADJ;
+}
+// a second stage one step along (its halo has a margin of one cell)
+template <int MODE>
+__host__ __device__ constexpr bool two_stages() { return MODE == MODE_RK2 || MODE == MODE_ADJ; }
 
 // values handed from the groups to the particle's lane: k1 and k2 (RK2), u
-// (AB, interpolation), u and its derivatives
+// (AB, interpolation), u and its derivatives; adjoint: J(X), J(X*), t*, the
+// cell of X* (in units of the cell width)
 template <int MODE, int NC>
-__host__ __device__ constexpr int result_count() { return MODE == MODE_RK2 ? 6 : (is_deriv<MODE>() ? 4 * NC : NC); }
+__host__ __device__ constexpr int result_count()
+{
+    return MODE == MODE_RK2 ? 6 : (MODE == MODE_ADJ ? 22 : (is_deriv<MODE>() ? 4 * NC : NC));
+}
 
 __host__ __device__ constexpr size_t align32(size_t x) { return (x + 31) & ~size_t(31); }
 
@@ -376,8 +386,9 @@ struct WarpPlan {
     static constexpr size_t k = align32(rec + 2 * 32 * 4 * sizeof(T));                     // [32][KS]
     static constexpr size_t w = align32(k + 32 * KS * sizeof(T));                          // [2][4 groups][WB]
     static constexpr int WB = is_deriv<MODE>() ? 40 : 24;                                  // groups 8 banks apart
-    static constexpr size_t x = align32(w + 2 * 4 * WB * sizeof(T));                       // [3][32] positions (steps)
-    static constexpr size_t rhs = align32(x + (is_step<MODE>() ? 3 * 32 * sizeof(double) : 0));   // [9][32] AB history
+    static constexpr bool HAS_X = is_step<MODE>() || MODE == MODE_ADJ;
+    static constexpr size_t x = align32(w + 2 * 4 * WB * sizeof(T));                       // [3][32] positions (steps), lambda
+    static constexpr size_t rhs = align32(x + (HAS_X ? 3 * 32 * sizeof(double) : 0));      // [9][32] AB history
     static constexpr size_t total = align32(rhs + (is_ab<MODE>() ? 3 * AB_MAX_HIST * 32 * sizeof(float) : 0));
 };
 
@@ -406,7 +417,7 @@ __device__ __forceinline__ void put_results(T* kb, const T (&v)[n])
 // ---------------------------------------------------------------------------
 template <typename T, int I, int MODE, int NC, int RW>
 struct HaloGeom {
-    static constexpr int MARGIN = MODE == MODE_RK2 ? 1 : 0;
+    static constexpr int MARGIN = two_stages<MODE>() ? 1 : 0;
     static constexpr HaloBox B = halo_box(I, MARGIN, sizeof(T) == 8);
     static constexpr int H = B.H, G = B.G, P = B.P, XOFF = B.XOFF;
     static constexpr int PL = P * H, SC = PL * H;
@@ -420,7 +431,7 @@ struct HaloGeom {
 // once: 64-byte rows, and H is odd).
 template <int I, int MODE>
 struct SlabGeom {
-    static constexpr HaloBox B = halo_box(I, MODE == MODE_RK2 ? 1 : 0, false);
+    static constexpr HaloBox B = halo_box(I, two_stages<MODE>() ? 1 : 0, false);
     static constexpr int H = B.H, G = B.G;
     static constexpr int SW = slab_width(I), SPT = BLK / SW;       // slabs a block is wide
     static constexpr int X0 = -((G + SW - 1) / SW) * SW;          // first slab's x1 relative to the block
@@ -434,9 +445,7 @@ enum { SRC_GLOBAL = 0, SRC_HALO = 1, SRC_SLABS = 2 };
 struct Place {
     const unsigned char* halo;   // SRC_HALO: the staged halo; SRC_SLABS: slot 0 of the slab ring
     int slab;                    // SRC_SLABS: sequence number of the block's first slab
-    int r1, r2, r3;              // the particle's cell relative to the halo
-    int o1, o2, o3;              // the halo's first node (unpadded coordinates)
-    int node;                    // SRC_GLOBAL: padded index of the stencil's first node
+    int c[3];                    // the particle's cell
 };
 
 // ---------------------------------------------------------------------------
@@ -460,7 +469,7 @@ template <typename T, int MODE, int NC>
 __device__ __forceinline__ void fetch_state(const BlockArgs& a, int64_t src, bool valid, unsigned char* ws, int lane)
 {
     using WPl = WarpPlan<T, MODE, NC>;
-    if constexpr (is_step<MODE>()) {
+    if constexpr (WPl::HAS_X) {   // (the adjoint's pos_in is lambda, src the caller index)
         if (!valid) return;
 #pragma unroll
         for (int ax = 0; ax < 3; ++ax)
@@ -487,6 +496,25 @@ __host__ __device__ constexpr int held_rows()
     return sizeof(T) == 8 || I == 8 ? 0 : (I == 4 ? 4 : (SRC == SRC_GLOBAL ? 6 : 0));
 }
 
+// One stage: contract the stencil of ld at the offsets s (less 1/2) from the
+// cell's centre; the rows held in f are loaded if `fresh`.
+template <typename T, int I, int DEG, int NC, bool D, int HR, class LD>
+__device__ __forceinline__ void interpolate_stage(const LD& ld, T s1, T s2, T s3, T* wb, bool fresh, const LaneMap<I>& m,
+                                                  const Basis<T, I, DEG, D>& B,
+                                                  T (&f)[HR > 0 ? HR : 1][LaneMap<I>::NZ][NC], T (&k)[D ? 4 * NC : NC])
+{
+    Weights<T, I, D> w;
+    if constexpr (HR > 0) {
+        if (fresh) load_rows<T, I, NC, HR>(ld, f);
+        __syncwarp();
+        B.eval(s1, s2, s3, m, wb, w);
+        contract<T, I, NC, D>(HeldLd<T, I, NC, HR, LD>{f, ld}, w, k);
+    } else {
+        B.eval(s1, s2, s3, m, wb, w);
+        contract<T, I, NC, D>(ld, w, k);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Q: a group interpolates its particle (offsets t, stencil at `at`), component
 // chunk ch; res: the particle's results, in every lane of the group.  live:
@@ -499,91 +527,81 @@ __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Plac
                                                   T (&res)[result_count<MODE, NC>()])
 {
     constexpr bool D = is_deriv<MODE>(), HALO = SRC != SRC_GLOBAL;
-    constexpr int LO = I / 2 - 1, ZS = LaneMap<I>::ZS;
-    auto halo_ld = [&](int r1, int r2, int r3) {
+    constexpr int LO = I / 2 - 1, ZS = LaneMap<I>::ZS, G = LO + (two_stages<MODE>() ? 1 : 0);
+    // the stencil of the cell displaced by d from the particle's, in the staged halo
+    auto halo_ld = [&](int d1, int d2, int d3) {
+        const int r1 = (at.c[0] & 7) + d1 + G - LO, r2 = (at.c[1] & 7) + d2 + G - LO, r3 = (at.c[2] & 7) + d3 + G - LO + m.z0;
         if constexpr (SRC == SRC_SLABS) {   // the lane's slab and column
             using SG = SlabGeom<I, MODE>;
-            const int x = r1 - LO + m.x - SG::G - SG::X0;
-            const int row = (r3 - LO + m.z0) * SG::H + (r2 - LO);
+            const int x = r1 + m.x - SG::G - SG::X0;
+            const int row = r3 * SG::H + r2;
             return HaloLd<T, STORE, RW, NC, SG::SW, ZS * SG::H * SG::SW, 0>{
                 at.halo + (unsigned)(at.slab + x / SG::SW) % NS * SG::slot + (row * SG::SW + x % SG::SW) * 16};
         } else {
             using HG = HaloGeom<T, I, MODE, NC, RW>;
-            const int e = (r3 - LO + m.z0) * HG::PL + (r2 - LO) * HG::P + (r1 - LO + m.x) + HG::XOFF;
+            const int e = r3 * HG::PL + r2 * HG::P + (r1 + m.x) + HG::XOFF;
             return HaloLd<T, STORE, RW, NC, HG::P, ZS * HG::PL, HG::SC>{at.halo + e * (STORE == ST_F64 ? 8 : 4 * RW)};
         }
     };
+    auto node_of = [&](int c1, int c2, int c3) { return (int)padded_index(a.f.NP, c1 - LO, c2 - LO, c3 - LO); };
     auto glob_ld = [&](int node) { return global_ld<T, I, STORE, RW, NC>(a.f, node, ch, m); };
-    Weights<T, I, D> w;
-    if constexpr (MODE != MODE_RK2) {
+    if constexpr (!two_stages<MODE>()) {
+        Weights<T, I, D> w;
         B.eval(t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, m, odd ? wb1 : wb0, w);
-        if constexpr (HALO) contract<T, I, NC, D>(halo_ld(at.r1, at.r2, at.r3), w, res);
-        else contract<T, I, NC, D>(glob_ld(at.node), w, res);
+        if constexpr (HALO) contract<T, I, NC, D>(halo_ld(0, 0, 0), w, res);
+        else contract<T, I, NC, D>(glob_ld(node_of(at.c[0], at.c[1], at.c[2])), w, res);
     } else {
         const T dtid = (T)(a.dt * a.g.inv_delta);
-        constexpr int HR = held_rows<T, I, SRC>();
+        constexpr int HR = MODE == MODE_RK2 ? held_rows<T, I, SRC>() : 0;
+        constexpr int NOUT = D ? 4 * NC : NC;
         T f[HR > 0 ? HR : 1][LaneMap<I>::NZ][NC];
-        T k1[NC], k2[NC];
-        // contract the stencil of ld; its held rows are loaded if `fresh`
-        auto stage = [&](const auto& ld, T s1, T s2, T s3, T* wb, bool fresh, T (&k)[NC]) {
-            if constexpr (HR > 0) {
-                if (fresh) load_rows<T, I, NC, HR>(ld, f);
-                __syncwarp();
-                B.eval(s1, s2, s3, m, wb, w);
-                contract<T, I, NC, false>(HeldLd<T, I, NC, HR, std::decay_t<decltype(ld)>>{f, ld}, w, k);
-            } else {
-                B.eval(s1, s2, s3, m, wb, w);
-                contract<T, I, NC, false>(ld, w, k);
-            }
-        };
-        if constexpr (HALO) stage(halo_ld(at.r1, at.r2, at.r3), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, k1);
-        else stage(glob_ld(at.node), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, k1);
+        T k1[NOUT], k2[NOUT];
+        if constexpr (HALO)
+            interpolate_stage<T, I, DEG, NC, D, HR>(halo_ld(0, 0, 0), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, m, B, f, k1);
+        else
+            interpolate_stage<T, I, DEG, NC, D, HR>(glob_ld(node_of(at.c[0], at.c[1], at.c[2])), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, m, B, f, k1);
         // stage-2 point, cell-relative: t* = t + dt k1 / delta
         T ts[3];
-        int dc[3];
+        int d[3];
 #pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
             ts[ax] = fma(dtid, k1[ax], t[ax]);
             const T fl = floor(ts[ax]);
-            dc[ax] = (int)fl;
+            d[ax] = (int)fl;
             ts[ax] -= fl;
         }
-        // where X* lies: in the halo, else by its padded node index (one cell
-        // away stays inside the ghost layers; farther it is wrapped)
-        const bool moved = (dc[0] | dc[1] | dc[2]) != 0;
-        const int s1 = at.r1 + dc[0], s2 = at.r2 + dc[1], s3 = at.r3 + dc[2];
-        // (unsigned: a saturated conversion is far as well)
-        const bool far = (unsigned)dc[0] + 1u > 2u || (unsigned)dc[1] + 1u > 2u || (unsigned)dc[2] + 1u > 2u;
-        int node2 = at.node + dc[0] + dc[1] * a.f.NP + dc[2] * a.f.NP * a.f.NP;
-        if (far) {
-            if ((lane & 7) == 0 && live) atomicOr(a.flags + FLAG_CFL, 1);
-            int c1, c2, c3;
-            if constexpr (HALO) {
-                c1 = at.o1 + at.r1, c2 = at.o2 + at.r2, c3 = at.o3 + at.r3;
-            } else {
-                c1 = at.node % a.f.NP - PAD + LO;
-                c2 = at.node / a.f.NP % a.f.NP - PAD + LO;
-                c3 = at.node / a.f.NP / a.f.NP - PAD + LO;
-            }
-            auto wrap = [&](int c, int d) { return (int)(((unsigned)c + (unsigned)d) & (unsigned)a.g.mask); };
-            node2 = (int)padded_index(a.f.NP, wrap(c1, dc[0]) - LO, wrap(c2, dc[1]) - LO, wrap(c3, dc[2]) - LO);
-        }
-        if constexpr (HALO) {   // the halo has a margin of one cell
+        // X* at most one cell away lies in the halo, or inside the ghost layers; farther
+        // its cell is wrapped (unsigned: a saturated conversion is far as well)
+        const bool moved = (d[0] | d[1] | d[2]) != 0;
+        const bool far = (unsigned)d[0] + 1u > 2u || (unsigned)d[1] + 1u > 2u || (unsigned)d[2] + 1u > 2u;
+        auto wrap = [&](int ax) { return (int)(((unsigned)at.c[ax] + (unsigned)d[ax]) & (unsigned)a.g.mask); };
+        if (far && (lane & 7) == 0 && live) atomicOr(a.flags + FLAG_CFL, 1);
+        if constexpr (HALO) {
             if (!__any_sync(0xffffffffu, far)) {
-                stage(halo_ld(s1, s2, s3), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, k2);
+                interpolate_stage<T, I, DEG, NC, D, HR>(halo_ld(d[0], d[1], d[2]), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, m, B, f, k2);
             } else {   // rare: every group of the warp gathers from global memory (the same values)
-                const int n2 = far ? node2
-                                   : (int)padded_index(a.f.NP, ((at.o1 + s1) & a.g.mask) - LO,
-                                                       ((at.o2 + s2) & a.g.mask) - LO, ((at.o3 + s3) & a.g.mask) - LO);
-                stage(glob_ld(n2), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, k2);
+                interpolate_stage<T, I, DEG, NC, D, HR>(glob_ld(node_of(wrap(0), wrap(1), wrap(2))), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, true, m, B, f, k2);
             }
         } else {
-            stage(glob_ld(node2), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, k2);
+            const int n2 = far ? node_of(wrap(0), wrap(1), wrap(2))
+                               : node_of(at.c[0] + d[0], at.c[1] + d[1], at.c[2] + d[2]);
+            interpolate_stage<T, I, DEG, NC, D, HR>(glob_ld(n2), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, m, B, f, k2);
         }
+        if constexpr (MODE == MODE_RK2) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            res[k] = k1[k];
-            res[3 + k] = k2[k];
+            for (int k = 0; k < 3; ++k) {
+                res[k] = k1[k];
+                res[3 + k] = k2[k];
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                res[k] = k1[3 + k];
+                res[9 + k] = k2[3 + k];
+            }
+#pragma unroll
+            for (int ax = 0; ax < 3; ++ax) res[18 + ax] = ts[ax];
+            res[21] = cell_as<T>(wrap(0) | wrap(1) << 10 | wrap(2) << 20);
         }
     }
 }
@@ -669,6 +687,47 @@ __device__ __forceinline__ void update_particle(const BlockArgs& a, int64_t j, i
     }
 }
 
+// Adjoint of one RK2 step, lane-dense (float64): with J in units of u per
+// cell (times inv_delta: per length),
+//   lambda* = dt/2 J(X*)^T lambda,  mu = dt/2 lambda + dt lambda*,
+//   lambda <- lambda + lambda* + J(X)^T mu;
+// lambda (caller order) is read and written, and what the field gradient's
+// scatter needs is left in grouped order: X* (offsets and cell), mu, dt/2 lambda.
+template <typename T, int MODE, int NC>
+__device__ __forceinline__ void adjoint_particle(const BlockArgs& a, int64_t j, int32_t id, bool valid,
+                                                 const unsigned char* ws, int lane)
+{
+    using WPl = WarpPlan<T, MODE, NC>;
+    if (!valid) return;
+    const T* kb = reinterpret_cast<const T*>(ws + WPl::k) + lane * WPl::KS;
+    const double* ls = reinterpret_cast<const double*>(ws + WPl::x) + lane;
+    const double dt = a.dt, hdi = 0.5 * dt * a.g.inv_delta;
+    const double lam[3] = {ls[0], ls[32], ls[64]};
+    double lstar[3], mu[3];
+#pragma unroll
+    for (int jj = 0; jj < 3; ++jj) {
+        double s = 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s = fma(widen(kb[9 + 3 * k + jj]), lam[k], s);
+        lstar[jj] = hdi * s;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) mu[k] = fma(dt, lstar[k], 0.5 * dt * lam[k]);
+#pragma unroll
+    for (int jj = 0; jj < 3; ++jj) {
+        double s = 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s = fma(widen(kb[3 * k + jj]), mu[k], s);
+        a.pos_out[jj * a.np + id] = lam[jj] + lstar[jj] + a.g.inv_delta * s;
+    }
+    if (a.adj) {
+        float4* o = a.adj + j;
+        o[0] = make_float4((float)kb[18], (float)kb[19], (float)kb[20], (float)kb[21]);
+        o[a.np] = make_float4((float)mu[0], (float)mu[1], (float)mu[2], 0.0f);
+        o[2 * a.np] = make_float4((float)(0.5 * dt * lam[0]), (float)(0.5 * dt * lam[1]), (float)(0.5 * dt * lam[2]), 0.0f);
+    }
+}
+
 // per-warp pointers into its shared memory
 template <typename T, int MODE, int NC>
 struct WarpMem {
@@ -691,7 +750,6 @@ template <typename T, int I, int DEG, int MODE, int NC, int STORE, int RW>
 __device__ __forceinline__ void run_direct(const BlockArgs& a, int64_t j0, int64_t j1, unsigned char* ws, int warp,
                                            int nw, int lane)
 {
-    constexpr int LO = I / 2 - 1;
     const int g = lane >> 3;
     const LaneMap<I> m(lane);
     Basis<T, I, DEG, is_deriv<MODE>()> B;
@@ -705,15 +763,13 @@ __device__ __forceinline__ void run_direct(const BlockArgs& a, int64_t j0, int64
         const int64_t src = !valid ? 0 : (a.perm ? a.perm[j] : j);
         const int32_t id = !valid ? 0 : (a.id_in ? a.id_in[src] : (int32_t)src);
         wm.recs[lane] = particle_record<T>(a, j, src, valid);
-        fetch_state<T, MODE, NC>(a, src, valid, ws, lane);
+        fetch_state<T, MODE, NC>(a, MODE == MODE_ADJ ? id : src, valid, ws, lane);
         __syncwarp();
-        for (int ch = 0; ch < (is_step<MODE>() ? 1 : (a.f.C + NC - 1) / NC); ++ch) {
+        for (int ch = 0; ch < (WarpPlan<T, MODE, NC>::HAS_X ? 1 : (a.f.C + NC - 1) / NC); ++ch) {
             for (int it = 0; it < 8 && it * 4 * nw < left; ++it) {
                 const PRec<T> rec = wm.recs[4 * it + g];
-                int c[3];
-                unpack_cell(cell_of(rec), c);
                 Place at{};
-                at.node = (int)padded_index(a.f.NP, c[0] - LO, c[1] - LO, c[2] - LO);
+                unpack_cell(cell_of(rec), at.c);
                 T res[result_count<MODE, NC>()];
                 interpolate_group<T, I, DEG, MODE, NC, STORE, RW, SRC_GLOBAL>(
                     a, at, ch, rec.t, it * 4 * nw + g < left, lane, B, m, wm.wb0, wm.wb1, it & 1, res);
@@ -723,6 +779,9 @@ __device__ __forceinline__ void run_direct(const BlockArgs& a, int64_t j0, int64
             if constexpr (is_step<MODE>()) {
                 cp_async_wait_all();
                 update_particle<T, MODE, NC>(a, j, id, valid, ws, lane);
+            } else if constexpr (MODE == MODE_ADJ) {
+                cp_async_wait_all();
+                adjoint_particle<T, MODE, NC>(a, j, id, valid, ws, lane);
             } else if (valid) write_outputs<T, MODE, NC>(a, id, ch, ws, lane);
             __syncwarp();
         }

@@ -1365,6 +1365,29 @@ static cudaError_t launch_adjoint(tracker* t, const AdjArgs& a)
     }
 }
 
+static cudaError_t launch_adj_particles(tracker* t, const BlockArgs& a, bool direct)
+{
+    ProfScope ps(t, PROF_STEP);
+    t->launches += 1;
+    const void* m = !direct && t->tmap_ok[1] ? &t->tmap[1] : nullptr;
+    switch (t->I) {
+        case 4: return launch_adj_particles_i4(a, m, t->deg_hi, t->stream);
+        case 6: return launch_adj_particles_i6(a, m, t->deg_hi, t->stream);
+        default: return launch_adj_particles_i8(a, m, t->deg_hi, t->stream);
+    }
+}
+
+static cudaError_t launch_adj_scatter(tracker* t, const AdjScatterArgs& a, int64_t nblocks)
+{
+    ProfScope ps(t, PROF_STEP);
+    t->launches += 1;
+    switch (t->I) {
+        case 4: return launch_adj_scatter_i4(a, nblocks, t->deg_hi, t->stream);
+        case 6: return launch_adj_scatter_i6(a, nblocks, t->deg_hi, t->stream);
+        default: return launch_adj_scatter_i8(a, nblocks, t->deg_hi, t->stream);
+    }
+}
+
 static int ensure_set(tracker* t, SetState& ss, int64_t np)
 {
     if (np <= ss.cap && ss.nb == t->nblocks) return TRK_OK;
@@ -1582,8 +1605,17 @@ int tracker_adjoint(tracker* t, int64_t np, const double* pos0, const double* la
     if ((rc = ensure_state(t, np))) return rc;
     const int K = std::min(ckpt_every, steps);
     const int nseg = (steps + K - 1) / K;
-    // layout: nseg checkpoints | K segment states | 2 lambdas
-    const size_t need = (size_t)(nseg + K + 2) * vec * 8;
+    const bool f64 = t->storage == TRK_F64;
+    // layout: nseg checkpoints, then
+    //   float64 fields: K segment states | 2 lambdas (caller order)
+    //   others, per step of a segment the grouped state the step's adjoint reads: K x [np] records |
+    //     X*, mu, dt/2 lambda of one step | K x [nblocks + 1] offsets | K x [np] ids
+    // (16-byte records, and offsets that the scan writes in 16-byte vectors: regions start on 256 bytes)
+    auto align256 = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t ckpt_bytes = align256((size_t)nseg * vec * 8), recs = (size_t)np * 16;
+    const size_t off_stride = align256((size_t)(t->nblocks + 1) * 4);
+    const size_t need = ckpt_bytes + (f64 ? (size_t)(K + 2) * vec * 8
+                                          : align256((size_t)(K + 3) * recs) + (size_t)K * off_stride + (size_t)K * np * 4);
     if (need > t->adj_bytes) {
         dev_free(t->adj_buf);
         t->adj_buf = nullptr;
@@ -1614,7 +1646,7 @@ int tracker_adjoint(tracker* t, int64_t np, const double* pos0, const double* la
             gscratch = t->adj_scratch;
             // every gather leaves the slabs it read zero; clearing them here as well
             // keeps a call that failed half-way from leaking into the next one
-            if (gscratch) CUDA_TRY(cudaMemsetAsync(gscratch, 0, sb, t->stream));
+            if (gscratch && f64) CUDA_TRY(cudaMemsetAsync(gscratch, 0, sb, t->stream));
         }
     }
     double* ckpt = t->adj_buf;
@@ -1626,6 +1658,89 @@ int tracker_adjoint(tracker* t, int64_t np, const double* pos0, const double* la
         double* dst = ckpt + (size_t)sg * vec;
         CUDA_TRY(cudaMemcpyAsync(dst, ckpt + (size_t)(sg - 1) * vec, vec * 8, cudaMemcpyDeviceToDevice, t->stream));
         if ((rc = tracker_advance(t, np, dst, nullptr, dt, K, TRK_RK2, 0))) return rc;
+    }
+    if (!f64) {
+        // backward sweep: recompute each segment from its checkpoint in grouped form, keeping each
+        // step's records, ids and offsets; then step back through it, lambda in place in grad_pos0
+        char* base = reinterpret_cast<char*>(t->adj_buf) + ckpt_bytes;
+        auto seg_rec = [&](int i) { return base + (size_t)i * recs; };
+        float4* adj = reinterpret_cast<float4*>(base + (size_t)K * recs);
+        char* offs = base + align256((size_t)(K + 3) * recs);
+        auto seg_off = [&](int i) { return reinterpret_cast<int32_t*>(offs + (size_t)i * off_stride); };
+        int32_t* ids = reinterpret_cast<int32_t*>(offs + (size_t)K * off_stride);
+        if (grad_pos0 != lambdaT) CUDA_TRY(cudaMemcpyAsync(grad_pos0, lambdaT, vec * 8, cudaMemcpyDeviceToDevice, t->stream));
+        if ((rc = ensure_bin(t, t->nblocks))) return rc;
+        for (int sg = nseg - 1; sg >= 0; --sg) {
+            const int n = std::min(steps, (sg + 1) * K) - sg * K;
+            const double* pos = ckpt + (size_t)sg * vec;
+            {
+                ProfScope ps(t, PROF_BIN);
+                CUDA_TRY(cudaMemsetAsync(t->d_counts, 0, (size_t)t->nblocks * sizeof(uint32_t), t->stream));
+                CUDA_TRY(launch_keys_count(t->g, np, pos, t->keys, t->d_counts, t->d_flags, t->stream));
+                t->launches += 1;
+            }
+            for (int i = 0; i < n; ++i) {
+                int32_t* off = seg_off(i);
+                int32_t* id = ids + (size_t)i * np;
+                const int nxt = i & 1;
+                {
+                    ProfScope ps(t, PROF_BIN);
+                    CUDA_TRY(launch_count_scan(t->d_counts, t->nblocks, off, t->d_cursor, t->d_scan_tmp, t->stream,
+                                               &t->launches));
+                    CUDA_TRY(launch_scatter_state(t->g, np, t->keys, t->d_cursor, i ? t->pos_s[nxt ^ 1] : pos,
+                                                  i ? id - np : nullptr, nullptr, 0, t->pos_s[nxt], id, nullptr, seg_rec(i),
+                                                  0, t->d_flags, t->stream));
+                    t->launches += 1;
+                }
+                if (i == n - 1) break;   // the next state is the following checkpoint (or X_T)
+                BlockArgs a = base_args(t);
+                a.np = np;
+                a.dt = dt;
+                a.offsets = off;
+                a.rec_in = seg_rec(i);
+                a.pos_in = a.pos_out = t->pos_s[nxt];
+                a.id_in = a.id_out = id;
+                a.key_out = t->keys;
+                a.counts = t->d_counts;
+                a.ppc = 0;
+                CUDA_TRY(adj_direct ? launch_direct(t, MODE_RK2, a) : launch_block(t, MODE_RK2, a, true));
+            }
+            for (int i = n - 1; i >= 0; --i) {
+                BlockArgs a = base_args(t);
+                a.np = np;
+                a.dt = dt;
+                a.offsets = seg_off(i);
+                a.rec_in = seg_rec(i);
+                a.id_in = ids + (size_t)i * np;
+                a.pos_in = a.pos_out = grad_pos0;   // lambda
+                a.adj = grad_field ? adj : nullptr;
+                a.ppc = 0;
+                CUDA_TRY(launch_adj_particles(t, a, adj_direct));
+                if (!grad_field) continue;
+                AdjScatterArgs sa{};
+                sa.g = t->g;
+                sa.cf = a.cf;
+                sa.np = np;
+                sa.offsets = a.offsets;
+                sa.rec = reinterpret_cast<const float4*>(a.rec_in);
+                sa.adj = adj;
+                sa.gfield = grad_field;
+                sa.gscratch = reinterpret_cast<float*>(gscratch);
+                CUDA_TRY(launch_adj_scatter(t, sa, adj_direct ? 0 : t->nblocks));
+                if (gscratch) {
+                    AdjArgs ga{};
+                    ga.g = t->g;
+                    ga.f = a.f;
+                    ga.offsets = a.offsets;
+                    ga.gfield = grad_field;
+                    ga.gscratch = gscratch;
+                    ProfScope ps(t, PROF_OTHER);   // the node gather of the field gradient
+                    t->launches += 1;
+                    CUDA_TRY(launch_adjoint_gather(t->I, ga, t->stream));
+                }
+            }
+        }
+        return TRK_OK;
     }
     // backward sweep: recompute each segment from its checkpoint, then step back through it
     CUDA_TRY(cudaMemcpyAsync(lam[0], lambdaT, vec * 8, cudaMemcpyDeviceToDevice, t->stream));
