@@ -129,10 +129,7 @@ struct GlobalLd {
     {
         const int64_t n = base + (a3 * f.NP + a2) * f.NP + a1;
         if constexpr (STORE == ST_F64) return (T)__ldg(f.f64 + k * f.plane + n);
-        else {
-            const uint32_t w = __ldg(f.rec + 4 * n + k);
-            return STORE == ST_BF16X2 ? (T)bf16x2_value(w) : (T)__uint_as_float(w);
-        }
+        else return (T)__ldg(f.rec + 4 * n + k);
     }
 };
 
@@ -155,7 +152,7 @@ __device__ __forceinline__ void stage_halo(T* halo, const FieldView& f, int o1, 
         if constexpr (STORE == ST_F64) {
             for (int k = 0; k < 3; ++k) v[k] = f.f64[k * f.plane + n];
         } else {
-            unpack<STORE, 4, 3>(reinterpret_cast<const uint4*>(f.rec)[n], v);
+            for (int k = 0; k < 3; ++k) v[k] = f.rec[4 * n + k];
         }
         for (int k = 0; k < 3; ++k) halo[k * SC + z * S3 + y * S2 + x] = v[k];
     }

@@ -315,11 +315,8 @@ __global__ void __launch_bounds__(NT, 4) k_adj_scatter_direct(const __grid_const
 template <int I, int DEG>
 cudaError_t launch_adj_particles(const BlockArgs& a, const CUtensorMap* tmap, cudaStream_t st)
 {
-    if (a.f.storage == ST_F32)
-        return tmap ? launch_slabs<I, DEG, MODE_ADJ, 3, ST_F32>(a, *tmap, st)
-                    : launch_direct_t<float, I, DEG, MODE_ADJ, 3, ST_F32, 4>(a, st);
-    return tmap ? launch_slabs<I, DEG, MODE_ADJ, 3, ST_BF16X2>(a, *tmap, st)
-                : launch_direct_t<float, I, DEG, MODE_ADJ, 3, ST_BF16X2, 4>(a, st);
+    return tmap ? launch_slabs<I, DEG, MODE_ADJ, 3>(a, *tmap, st)
+                : launch_direct_t<float, I, DEG, MODE_ADJ, 3, ST_F32, 4>(a, st);
 }
 
 template <int I, int DEG, bool SLAB>

@@ -18,14 +18,13 @@ __host__ __device__ constexpr size_t batched_warp_bytes()
     return WarpPlan<float, MODE_AB2_D, 3>::total;   // the larger of the two modes
 }
 
-template <int I, int DEG, int STORE>
+template <int I, int DEG>
 __device__ __forceinline__ void run_item(const BatchSet& S, int64_t j0, int64_t j1, unsigned char* ws, int warp, int lane)
 {
-    if (S.deriv) run_direct<float, I, DEG, MODE_AB2_D, 3, STORE, 4>(S.a, j0, j1, ws, warp, NW, lane);
-    else run_direct<float, I, DEG, MODE_AB2, 3, STORE, 4>(S.a, j0, j1, ws, warp, NW, lane);
+    if (S.deriv) run_direct<float, I, DEG, MODE_AB2_D, 3, ST_F32, 4>(S.a, j0, j1, ws, warp, NW, lane);
+    else run_direct<float, I, DEG, MODE_AB2, 3, ST_F32, 4>(S.a, j0, j1, ws, warp, NW, lane);
 }
 
-template <int STORE>
 __global__ void __launch_bounds__(NT, 4) k_batched(const BatchSet* __restrict__ sets, int nsets, int* ctr)
 {
     __shared__ __align__(128) unsigned char smem[NW * batched_warp_bytes()];
@@ -42,41 +41,33 @@ __global__ void __launch_bounds__(NT, 4) k_batched(const BatchSet* __restrict__ 
             if (it >= S.n_items) break;
             const int64_t j0 = (int64_t)it * PB, j1 = j0 + PB < S.a.np ? j0 + PB : S.a.np;
             switch (S.I * 2 + S.deg_hi) {
-                case 8: run_item<4, 3, STORE>(S, j0, j1, ws, warp, lane); break;
-                case 9: run_item<4, 5, STORE>(S, j0, j1, ws, warp, lane); break;
-                case 12: run_item<6, 5, STORE>(S, j0, j1, ws, warp, lane); break;
-                case 13: run_item<6, 7, STORE>(S, j0, j1, ws, warp, lane); break;
-                case 16: run_item<8, 7, STORE>(S, j0, j1, ws, warp, lane); break;
-                default: run_item<8, 9, STORE>(S, j0, j1, ws, warp, lane); break;
+                case 8: run_item<4, 3>(S, j0, j1, ws, warp, lane); break;
+                case 9: run_item<4, 5>(S, j0, j1, ws, warp, lane); break;
+                case 12: run_item<6, 5>(S, j0, j1, ws, warp, lane); break;
+                case 13: run_item<6, 7>(S, j0, j1, ws, warp, lane); break;
+                case 16: run_item<8, 7>(S, j0, j1, ws, warp, lane); break;
+                default: run_item<8, 9>(S, j0, j1, ws, warp, lane); break;
             }
         }
     }
 }
 
-template <int STORE>
-cudaError_t launch_batched_t(const BatchSet* sets, int nsets, int* ctr, int nsm, cudaStream_t st)
+}  // namespace
+
+cudaError_t launch_batched(const BatchSet* sets, int nsets, int* ctr, int nsm, cudaStream_t st)
 {
     static int ctas = 0;
     if (!ctas) {
-        cudaError_t e = cudaFuncSetAttribute(k_batched<STORE>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        cudaError_t e = cudaFuncSetAttribute(k_batched, cudaFuncAttributePreferredSharedMemoryCarveout,
                                              carveout_percent(NW * batched_warp_bytes(), 4));
         if (e != cudaSuccess) return e;
         int occ = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batched<STORE>, NT, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_batched, NT, 0);
         if (e != cudaSuccess) return e;
         ctas = std::max(occ, 1);
     }
-    k_batched<STORE><<<nsm * ctas, NT, 0, st>>>(sets, nsets, ctr);
+    k_batched<<<nsm * ctas, NT, 0, st>>>(sets, nsets, ctr);
     return cudaGetLastError();
-}
-
-}  // namespace
-
-cudaError_t launch_batched(int storage, const BatchSet* sets, int nsets, int* ctr, int nsm, cudaStream_t st)
-{
-    if (storage == ST_F32) return launch_batched_t<ST_F32>(sets, nsets, ctr, nsm, st);
-    if (storage == ST_BF16X2) return launch_batched_t<ST_BF16X2>(sets, nsets, ctr, nsm, st);
-    return cudaErrorInvalidValue;
 }
 
 }  // namespace trk

@@ -483,13 +483,12 @@ __global__ void k_unpermute_rhs(int64_t np, const float* __restrict__ src, const
 // blockIdx.z is the padded x3 plane, blockIdx.y counts groups of blockDim.y
 // padded rows, threads run along x1: reads are coalesced per component, a
 // record is one 16-byte (C = 1: 4-byte) store, and nothing divides.
-__device__ __forceinline__ uint32_t stored_word(int storage, float x)
+__device__ __forceinline__ float stored_value(int storage, float x)
 {
-    if (storage == ST_F32) return __float_as_uint(x);
+    if (storage == ST_F32) return x;
     // split of the float32-rounded value: hi = RN_bf16(x), lo = RN_bf16(x - hi)
-    const __nv_bfloat16 hi = __float2bfloat16_rn(x);
-    const __nv_bfloat16 lo = __float2bfloat16_rn(x - __bfloat162float(hi));
-    return (uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(lo) << 16);
+    const float hi = __bfloat162float(__float2bfloat16_rn(x));
+    return hi + __bfloat162float(__float2bfloat16_rn(x - hi));
 }
 
 template <typename S>
@@ -506,13 +505,13 @@ __global__ void k_convert_padded(int storage, const S* __restrict__ src, int C, 
         if (storage == ST_F64) {
             for (int k = 0; k < C; ++k) reinterpret_cast<double*>(dst)[k * plane + row + x] = (double)sx[k * n3];
         } else if (C == 1) {
-            reinterpret_cast<uint32_t*>(dst)[row + x] = stored_word(storage, (float)sx[0]);
+            reinterpret_cast<float*>(dst)[row + x] = stored_value(storage, (float)sx[0]);
         } else {
             for (int k0 = 0; k0 < C; k0 += 4) {
-                uint32_t w[4];
+                float w[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) w[k] = k0 + k < C ? stored_word(storage, (float)sx[(k0 + k) * n3]) : 0u;
-                reinterpret_cast<uint4*>(dst)[(k0 / 4) * plane + row + x] = make_uint4(w[0], w[1], w[2], w[3]);
+                for (int k = 0; k < 4; ++k) w[k] = k0 + k < C ? stored_value(storage, (float)sx[(k0 + k) * n3]) : 0.0f;
+                reinterpret_cast<float4*>(dst)[(k0 / 4) * plane + row + x] = make_float4(w[0], w[1], w[2], w[3]);
             }
         }
     }

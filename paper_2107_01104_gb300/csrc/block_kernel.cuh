@@ -176,10 +176,9 @@ __global__ void __launch_bounds__(NT, 4)
             for (int it = 0; it < 8 && it * 4 * NW < left; ++it) {
                 const PRec<T> rec = wm.recs[4 * it + g];
                 unpack_cell(cell_of(rec), at.c);   // (a particle lies in its own block)
-                T res[result_count<MODE, NC>()];
                 interpolate_group<T, I, DEG, MODE, NC, STORE, RW, SRC_HALO>(
-                    a, at, ch, rec.t, it * 4 * NW + g < left, lane, B, m, wm.wb0, wm.wb1, it & 1, res);
-                if ((lane & 7) == 0) put_results(wm.kbuf + (4 * it + g) * WarpMem<T, MODE, NC>::WPl::KS, res);
+                    a, at, ch, rec.t, it * 4 * NW + g < left, lane, B, m, wm.wb0, wm.wb1, it & 1,
+                    wm.kbuf + (4 * it + g) * WarpMem<T, MODE, NC>::WPl::KS);
             }
             __syncwarp();
             if constexpr (!STEP) {
@@ -332,7 +331,7 @@ struct Slabs {
     }
 };
 
-template <int I, int DEG, int MODE, int NC, int STORE>
+template <int I, int DEG, int MODE, int NC>
 __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
     k_slabs(const __grid_constant__ BlockArgs a, const __grid_constant__ CUtensorMap tmap)
 {
@@ -385,7 +384,8 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
         const int left = (int)min(j1 - b0 - 4 * warp, (int64_t)4 * nw * rounds);
         if (left <= 0) break;
         const bool valid = j < j1 && (lane >> 2) < rounds;
-        const int32_t id = !valid ? 0 : (a.id_in ? a.id_in[j] : (int32_t)j);
+        int32_t id = 0;   // (loaded where it is needed: a register less meanwhile)
+        if (MODE == MODE_ADJ && valid) id = a.id_in[j];
         fetch_state<T, MODE, NC>(a, MODE == MODE_ADJ ? id : j, valid, ws, lane);
         fetch_records(bn, 8, buf ^ 1);
         cp_async_commit();
@@ -410,14 +410,14 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
                 slabs.release_to(lo, lane, nw);
                 slabs.need((int)__reduce_max_sync(0xffffffffu, (unsigned)at.slab) + SG::NSL - 1);
                 at.halo = smem_raw;
-                T res[result_count<MODE, NC>()];
-                interpolate_group<T, I, DEG, MODE, NC, STORE, 4, SRC_SLABS, SP::NS>(a, at, slabs.ch, rec.t, now, lane, B, m,
-                                                                                    wm.wb0, wm.wb1, odd & 1, res);
+                interpolate_group<T, I, DEG, MODE, NC, ST_F32, 4, SRC_SLABS, SP::NS>(
+                    a, at, slabs.ch, rec.t, now, lane, B, m, wm.wb0, wm.wb1, odd & 1,
+                    wm.kbuf + (4 * it + g) * WarpMem<T, MODE, NC>::WPl::KS);
                 ++odd;
-                if (now && (lane & 7) == 0) put_results(wm.kbuf + (4 * it + g) * WarpMem<T, MODE, NC>::WPl::KS, res);
                 todo = todo && !now;
             } while (__any_sync(0xffffffffu, todo));
         }
+        if (MODE != MODE_ADJ && valid) id = a.id_in ? a.id_in[j] : (int32_t)j;
         __syncwarp();
         if constexpr (is_step<MODE>()) {
             cp_async_wait_all();
@@ -452,11 +452,11 @@ cudaError_t launch_block_hc(const BlockArgs& a, const CUtensorMap& tmap, int64_t
     return cudaGetLastError();
 }
 
-template <int I, int DEG, int MODE, int NC, int STORE>
+template <int I, int DEG, int MODE, int NC>
 cudaError_t launch_slabs(BlockArgs a, const CUtensorMap& tmap, cudaStream_t st)
 {
     using SP = SlabPlan<I, MODE, NC>;
-    auto kern = k_slabs<I, DEG, MODE, NC, STORE>;
+    auto kern = k_slabs<I, DEG, MODE, NC>;
     static int nsm = 0;
     if (!nsm) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SP::total);
@@ -481,7 +481,7 @@ cudaError_t launch_block_t(const BlockArgs& a, const CUtensorMap* tmap, int64_t 
     if constexpr (STORE == ST_F64) {
         if (tmap) return launch_block_hc<T, I, DEG, MODE, NC, STORE, RW, HC_TMA>(a, *tmap, nblocks, st);
     } else if constexpr (RW == 4) {
-        if (tmap) return launch_slabs<I, DEG, MODE, NC, STORE>(a, *tmap, st);
+        if (tmap) return launch_slabs<I, DEG, MODE, NC>(a, *tmap, st);
     }
     const CUtensorMap none{};
     return launch_block_hc<T, I, DEG, MODE, NC, STORE, RW, HC_ASYNC>(a, none, nblocks, st);

@@ -83,8 +83,7 @@ cudaError_t dispatch_mode(int mode, const FieldView& f, F&& go)
     const int s = f.storage;
 #define TRK_STORE(M, NC, RW)                                             \
     if (s == ST_F64) return go.template run<double, M, NC, ST_F64, 4>(); \
-    if (s == ST_F32) return go.template run<float, M, NC, ST_F32, RW>(); \
-    return go.template run<float, M, NC, ST_BF16X2, RW>();
+    return go.template run<float, M, NC, ST_F32, RW>();
 #define TRK_INTERP(M)                                      \
     if (f.C == 1) { TRK_STORE(M, 1, 1) }                   \
     if (f.C <= 3) { TRK_STORE(M, 3, 4) }                   \

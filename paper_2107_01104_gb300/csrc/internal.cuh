@@ -42,16 +42,18 @@ constexpr int PAD = 8;
 // fields are stored as node records, the layout every kernel gathers: four
 // components per 16-byte record (C = 1: one per 4-byte record), chunk ch
 // holding components 4 ch .. 4 ch + 3 of every node, absent components zero,
-// [chunks][NP^3] records.  A word is a float32 value, or a split-bf16 pair
-// (hi in the low half, lo in the high half).  One stencil row of I nodes is
-// then one contiguous run whatever the component.
+// [chunks][NP^3] records.  One stencil row of I nodes is then one contiguous
+// run whatever the component.  A split-bf16 value is kept as the float32 sum
+// of its two halves, which is what every use of the pair begins with (four
+// bytes either way; unpacking pairs in the gathers took 12 of the 17
+// instructions per node of a four-component chunk).
 struct FieldView {
     int storage;              // ST_*
     int C;                    // components
     int NP;                   // padded extent N + 2 PAD
     int64_t plane;            // NP^3 nodes
     const double* f64;        // [C][NP^3]                        (ST_F64)
-    const uint32_t* rec;      // [chunks][NP^3][4] (C = 1: [NP^3]) (ST_F32, ST_BF16X2)
+    const float* rec;         // [chunks][NP^3][4] (C = 1: [NP^3]) (ST_F32, ST_BF16X2)
 };
 
 __host__ __device__ constexpr int record_width(int C) { return C == 1 ? 1 : 4; }
@@ -368,7 +370,7 @@ size_t scan_scratch_bytes_u32(int64_t len);
 cudaError_t scan_exclusive_u32(uint32_t* data, int64_t len, uint32_t* scratch, cudaStream_t st, int64_t* launches);
 
 // One persistent launch over all sets (float32 or split-bf16 storage).
-cudaError_t launch_batched(int storage, const BatchSet* sets, int nsets, int* ctr, int nsm, cudaStream_t st);
+cudaError_t launch_batched(const BatchSet* sets, int nsets, int* ctr, int nsm, cudaStream_t st);
 
 // Sets the thread-local message returned by tracker_last_error().
 void set_error_message(const char* msg);

@@ -171,36 +171,24 @@ struct Basis {
 // Stencil loaders: ld(r, z, v) = components of the lane's node in row r and its
 // z-th plane
 // ---------------------------------------------------------------------------
-// value of a split-bf16 word (hi in the low half, lo in the high half)
-__device__ __forceinline__ float bf16x2_value(uint32_t w)
-{
-    return __uint_as_float(w << 16) + __uint_as_float(w & 0xffff0000u);
-}
-
-template <int STORE, int RW, int NC, typename T>
-__device__ __forceinline__ void unpack(const uint4& q, T (&v)[NC])
-{
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int k = 0; k < NC; ++k) v[k] = STORE == ST_BF16X2 ? bf16x2_value(w[k]) : __uint_as_float(w[k]);
-}
-
-// Records in global memory (float32 and split-bf16 fields).  A cell c in
+// Records in global memory.  A cell c in
 // [0, N) plus one is at least PAD - 1 > I / 2 nodes inside the ghost-padded
 // array, so a stencil is a box of fixed offsets from its first node.
-template <int STORE, int RW, int NC>
+template <int RW, int NC>
 struct RecordLd {
-    const uint32_t* p;     // the lane's first node
+    const float* p;        // the lane's first node
     int NP, NP2;           // record strides from row to row and from plane to plane of the lane
     __device__ __forceinline__ void operator()(int r, int z, float (&v)[NC]) const
     {
         const int off = z * NP2 + r * NP;
         if constexpr (RW == 4) {
-            unpack<STORE, RW, NC>(__ldg(reinterpret_cast<const uint4*>(p) + off), v);
+            const float4 q = __ldg(reinterpret_cast<const float4*>(p) + off);
+            const float w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int k = 0; k < NC; ++k) v[k] = w[k];
         } else {
             static_assert(NC == 1, "one component per 4-byte record");
-            const uint32_t w = __ldg(p + off);
-            v[0] = STORE == ST_BF16X2 ? bf16x2_value(w) : __uint_as_float(w);
+            v[0] = __ldg(p + off);
         }
     }
 };
@@ -229,7 +217,7 @@ __device__ __forceinline__ auto global_ld(const FieldView& f, int base, int ch, 
     if constexpr (STORE == ST_F64)
         return PlaneLd<NC>{f.f64 + (int64_t)ch * NC * f.plane + n, f.plane, f.NP, ZS * f.NP * f.NP, f.C - ch * NC};
     else
-        return RecordLd<STORE, RW, NC>{f.rec + ((int64_t)ch * f.plane + n) * RW, f.NP, ZS * f.NP * f.NP};
+        return RecordLd<RW, NC>{f.rec + ((int64_t)ch * f.plane + n) * RW, f.NP, ZS * f.NP * f.NP};
 }
 
 // A staged halo in shared memory: pitches P from row to row and PL from plane
@@ -243,10 +231,12 @@ struct HaloLd {
 #pragma unroll
             for (int k = 0; k < NC; ++k) v[k] = reinterpret_cast<const double*>(p)[k * SC + z * PL + r * P];
         } else if constexpr (RW == 4) {
-            unpack<STORE, RW, NC>(reinterpret_cast<const uint4*>(p)[z * PL + r * P], v);
+            const float4 q = reinterpret_cast<const float4*>(p)[z * PL + r * P];
+            const float w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int k = 0; k < NC; ++k) v[k] = w[k];
         } else {
-            const uint32_t w = reinterpret_cast<const uint32_t*>(p)[z * PL + r * P];
-            v[0] = STORE == ST_BF16X2 ? bf16x2_value(w) : __uint_as_float(w);
+            v[0] = reinterpret_cast<const float*>(p)[z * PL + r * P];
         }
     }
 };
@@ -282,21 +272,64 @@ __device__ __forceinline__ void load_rows(const LD& ld, T (&f)[HR][LaneMap<I>::N
 //   D = false: out[k] = u_k
 //   D = true:  out[k] = u_k, out[NC + 3k + j] = du_k / dt_j
 // ---------------------------------------------------------------------------
-// Sums v[0..n) over the group's eight lanes; every lane gets all of them.
+// Sums v[0..n) over the group's eight lanes, in three exchanges that halve the
+// values a lane carries (n = 12: 11 shuffles instead of 36; the shuffles share
+// the data path the stencils come through).  The lane is left with the sums
+// base .. base + count - 1 in v[0], v[1], ...
 template <typename T, int n>
-__device__ __forceinline__ void group_sum(T (&v)[n])
-{
+struct GroupSums {
+    static constexpr int m1 = (n + 1) / 2, m2 = (m1 + 1) / 2, m3 = (m2 + 1) / 2;
+    T v[m3];
+    int base, count;
+
+    template <int M, int O, int IN>
+    __device__ __forceinline__ static void exchange(T (&x)[IN], int lane, int& base, int& count)
+    {
+        constexpr int h = (M + 1) / 2;
+        const bool hi = lane & O;
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1)
+        for (int i = 0; i < h; ++i) {
+            const T a = x[i], b = i + h < M ? x[i + h < IN ? i + h : 0] : (T)0;
+            x[i] = (hi ? b : a) + __shfl_xor_sync(0xffffffffu, hi ? a : b, O);
+        }
+        base += hi ? h : 0;
+        count = hi ? max(count - h, 0) : min(count, h);
+    }
+    __device__ __forceinline__ GroupSums(T (&x)[n], int lane)
+    {
+        base = 0;
+        count = n;
+        exchange<n, 4>(x, lane, base, count);
+        exchange<m1, 2>(x, lane, base, count);
+        exchange<m2, 1>(x, lane, base, count);
 #pragma unroll
-        for (int i = 0; i < n; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-}
+        for (int i = 0; i < m3; ++i) v[i] = x[i];
+    }
+    // sum i in every lane of the group
+    template <int i>
+    __device__ __forceinline__ T all(int lane) const
+    {
+        constexpr bool h1 = i >= m1;
+        constexpr int i1 = i - (h1 ? m1 : 0);
+        constexpr bool h2 = i1 >= m2;
+        constexpr int i2 = i1 - (h2 ? m2 : 0);
+        constexpr bool h3 = i2 >= m3;
+        return __shfl_sync(0xffffffffu, v[i2 - (h3 ? m3 : 0)], (lane & 24) | (h1 ? 4 : 0) | (h2 ? 2 : 0) | (h3 ? 1 : 0));
+    }
+    // the sums from `first` on to the particle's slots
+    __device__ __forceinline__ void put(T* kb, int first, bool live) const
+    {
+#pragma unroll
+        for (int i = 0; i < m3; ++i)
+            if (live && i < count && base + i >= first) kb[base + i - first] = v[i];
+    }
+};
 
 // i-th term of a sum over n nodes taken from the ends inwards (0, n-1, 1, ...):
 // the small outer terms first, so that they are rounded while the partial sum is small
 __host__ __device__ constexpr int inward(int i, int n) { return i % 2 == 0 ? i / 2 : n - 1 - i / 2; }
 
-// the lane's column: out as above, to be summed over the group
+// the lane's column: out as above, to be summed over the group (GroupSums)
 template <typename T, int I, int NC, bool D, class LD>
 __device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D>& w, T (&out)[D ? 4 * NC : NC])
 {
@@ -335,7 +368,6 @@ __device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D>& w
             out[NC + 3 * k + 2] = w.w1 * c[k];
         }
     }
-    group_sum(out);
 }
 
 // ---------------------------------------------------------------------------
@@ -391,23 +423,6 @@ struct WarpPlan {
     static constexpr size_t rhs = align32(x + (HAS_X ? 3 * 32 * sizeof(double) : 0));      // [9][32] AB history
     static constexpr size_t total = align32(rhs + (is_ab<MODE>() ? 3 * AB_MAX_HIST * 32 * sizeof(float) : 0));
 };
-
-// one group's results (the same in all its lanes) into the particle's slots
-template <typename T, int n>
-__device__ __forceinline__ void put_results(T* kb, const T (&v)[n])
-{
-    if constexpr (sizeof(T) == 4) {
-#pragma unroll
-        for (int i = 0; i + 4 <= n; i += 4)
-            *reinterpret_cast<float4*>(kb + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-        if constexpr (n % 4 >= 2) *reinterpret_cast<float2*>(kb + n / 4 * 4) = make_float2(v[n / 4 * 4], v[n / 4 * 4 + 1]);
-        if constexpr (n % 2 == 1) kb[n - 1] = v[n - 1];
-    } else {
-#pragma unroll
-        for (int i = 0; i + 2 <= n; i += 2) *reinterpret_cast<double2*>(kb + i) = make_double2(v[i], v[i + 1]);
-        if constexpr (n % 2 == 1) kb[n - 1] = v[n - 1];
-    }
-}
 
 // ---------------------------------------------------------------------------
 // Halo of a cell block (block kernels): H^3 nodes from G nodes below the
@@ -517,14 +532,14 @@ __device__ __forceinline__ void interpolate_stage(const LD& ld, T s1, T s2, T s3
 
 // ---------------------------------------------------------------------------
 // Q: a group interpolates its particle (offsets t, stencil at `at`), component
-// chunk ch; res: the particle's results, in every lane of the group.  live:
-// false for an empty slot (whose results nobody reads).
+// chunk ch; the results go to the particle's slots kb.  live: false for an
+// empty slot.
 // ---------------------------------------------------------------------------
 template <typename T, int I, int DEG, int MODE, int NC, int STORE, int RW, int SRC, int NS = 1>
 __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Place& at, int ch, const T (&t)[3], bool live,
                                                   int lane, const Basis<T, I, DEG, is_deriv<MODE>()>& B,
                                                   const LaneMap<I>& m, T* wb0, T* wb1, bool odd,
-                                                  T (&res)[result_count<MODE, NC>()])
+                                                  T* kb)
 {
     constexpr bool D = is_deriv<MODE>(), HALO = SRC != SRC_GLOBAL;
     constexpr int LO = I / 2 - 1, ZS = LaneMap<I>::ZS, G = LO + (two_stages<MODE>() ? 1 : 0);
@@ -548,8 +563,17 @@ __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Plac
     if constexpr (!two_stages<MODE>()) {
         Weights<T, I, D> w;
         B.eval(t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, m, odd ? wb1 : wb0, w);
-        if constexpr (HALO) contract<T, I, NC, D>(halo_ld(0, 0, 0), w, res);
-        else contract<T, I, NC, D>(glob_ld(node_of(at.c[0], at.c[1], at.c[2])), w, res);
+        T out[D ? 4 * NC : NC];
+        if constexpr (HALO) contract<T, I, NC, D>(halo_ld(0, 0, 0), w, out);
+        else contract<T, I, NC, D>(glob_ld(node_of(at.c[0], at.c[1], at.c[2])), w, out);
+        if constexpr (MODE == MODE_INTERP_DERIV) {   // the derivatives only
+            T der[3 * NC];
+#pragma unroll
+            for (int i = 0; i < 3 * NC; ++i) der[i] = out[NC + i];
+            GroupSums<T, 3 * NC>(der, lane).put(kb + NC, 0, live);
+        } else {
+            GroupSums<T, D ? 4 * NC : NC>(out, lane).put(kb, 0, live);
+        }
     } else {
         const T dtid = (T)(a.dt * a.g.inv_delta);
         constexpr int HR = MODE == MODE_RK2 ? held_rows<T, I, SRC>() : 0;
@@ -560,12 +584,15 @@ __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Plac
             interpolate_stage<T, I, DEG, NC, D, HR>(halo_ld(0, 0, 0), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, m, B, f, k1);
         else
             interpolate_stage<T, I, DEG, NC, D, HR>(glob_ld(node_of(at.c[0], at.c[1], at.c[2])), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, m, B, f, k1);
+        const GroupSums<T, NOUT> s1(k1, lane);
+        const T u1[3] = {s1.template all<0>(lane), s1.template all<1>(lane), s1.template all<2>(lane)};
+        s1.put(kb, MODE == MODE_RK2 ? 0 : 3, live);
         // stage-2 point, cell-relative: t* = t + dt k1 / delta
         T ts[3];
         int d[3];
 #pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
-            ts[ax] = fma(dtid, k1[ax], t[ax]);
+            ts[ax] = fma(dtid, u1[ax], t[ax]);
             const T fl = floor(ts[ax]);
             d[ax] = (int)fl;
             ts[ax] -= fl;
@@ -587,21 +614,16 @@ __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Plac
                                : node_of(at.c[0] + d[0], at.c[1] + d[1], at.c[2] + d[2]);
             interpolate_stage<T, I, DEG, NC, D, HR>(glob_ld(n2), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, m, B, f, k2);
         }
+        const GroupSums<T, NOUT> s2(k2, lane);
         if constexpr (MODE == MODE_RK2) {
+            s2.put(kb + 3, 0, live);
+        } else {   // the Jacobians, t* and the cell of X*
+            s2.put(kb + 9, 3, live);
+            if (live && (lane & 7) == 0) {
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                res[k] = k1[k];
-                res[3 + k] = k2[k];
+                for (int ax = 0; ax < 3; ++ax) kb[18 + ax] = ts[ax];
+                kb[21] = cell_as<T>(wrap(0) | wrap(1) << 10 | wrap(2) << 20);
             }
-        } else {
-#pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                res[k] = k1[3 + k];
-                res[9 + k] = k2[3 + k];
-            }
-#pragma unroll
-            for (int ax = 0; ax < 3; ++ax) res[18 + ax] = ts[ax];
-            res[21] = cell_as<T>(wrap(0) | wrap(1) << 10 | wrap(2) << 20);
         }
     }
 }
@@ -770,10 +792,9 @@ __device__ __forceinline__ void run_direct(const BlockArgs& a, int64_t j0, int64
                 const PRec<T> rec = wm.recs[4 * it + g];
                 Place at{};
                 unpack_cell(cell_of(rec), at.c);
-                T res[result_count<MODE, NC>()];
                 interpolate_group<T, I, DEG, MODE, NC, STORE, RW, SRC_GLOBAL>(
-                    a, at, ch, rec.t, it * 4 * nw + g < left, lane, B, m, wm.wb0, wm.wb1, it & 1, res);
-                if ((lane & 7) == 0) put_results(wm.kbuf + (4 * it + g) * WarpMem<T, MODE, NC>::WPl::KS, res);
+                    a, at, ch, rec.t, it * 4 * nw + g < left, lane, B, m, wm.wb0, wm.wb1, it & 1,
+                    wm.kbuf + (4 * it + g) * WarpMem<T, MODE, NC>::WPl::KS);
             }
             __syncwarp();
             if constexpr (is_step<MODE>()) {

@@ -346,7 +346,7 @@ FieldView field_view(const tracker* t)
     f.NP = t->N + 2 * PAD;
     f.plane = (int64_t)f.NP * f.NP * f.NP;
     if (t->storage == ST_F64) f.f64 = reinterpret_cast<const double*>(t->field);
-    else f.rec = reinterpret_cast<const uint32_t*>(t->field);
+    else f.rec = reinterpret_cast<const float*>(t->field);
     return f;
 }
 
@@ -618,7 +618,7 @@ constexpr double kDirectDensity = 0.05;
 double direct_threshold(const tracker* t)
 {
     if (!column_available(t)) return 0.25;
-    return t->I == 4 ? 0.2 : kDirectDensity;
+    return t->I == 4 ? 0.25 : kDirectDensity;
 }
 
 // Below this many particles per grid cell the adjoint runs without halos
@@ -642,15 +642,16 @@ int step_path(const tracker* t, int64_t np)
 
 // AUTO interpolation: direct gathers below a density (and where the field has no
 // slabs to stage: C = 1, float64), the slab pipeline above.  Measured on GB300,
-// 256^3 float32, direct against slabs, us per call: u, I = 4 125 / 215 at 1/16
-// particle per cell, 488 / 386 at 1/4; I = 6 103 / 120 at 1/64, 300 / 221 at
-// 1/16; I = 8 160 / 183 at 1/64, 496 / 309 at 1/16; gradients, I = 6 378 / 380 at
-// 1/16, I = 8 238 / 224 at 1/64.
+// 256^3 float32, direct against slabs, us per call: u, I = 4 197 / 270 at 1/8
+// particle per cell, 374 / 381 at 1/4; I = 6 97 / 116 at 1/64, 158 / 149 at 1/32;
+// I = 8 150 / 178 at 1/64, 264 / 219 at 1/32; gradients, I = 4 1051 / 1047 at 1/4,
+// I = 6 140 / 165 at 1/64, 228 / 190 at 1/32, I = 8 186 / 229 at 1/128, 287 / 256
+// at 1/64.
 bool interp_direct(const tracker* t, int64_t np, int deriv)
 {
     if (t->storage == ST_F64 || !default_shape(t) || !t->tmap_ok[0] || t->halo_copy == TRK_HALO_ASYNC) return true;
     const double dens = (double)np / ((double)t->N * t->N * t->N);
-    return dens < (t->I == 4 ? 0.2 : (t->I == 6 && deriv ? 0.06 : 0.025));
+    return dens < (t->I == 4 ? 0.25 : (t->I == 6 ? 0.025 : (deriv ? 0.012 : 0.02)));
 }
 
 // One RK2/ABk step of tracker_advance: re-bin, then the fused step kernel.
@@ -1445,7 +1446,7 @@ static int batched_launch(tracker* t, const BatchSet* d_desc, int nsets)
 {
     ProfScope ps(t, PROF_STEP);
     CUDA_TRY(cudaMemsetAsync(t->d_ctr, 0, (size_t)nsets * sizeof(int), t->stream));
-    CUDA_TRY(launch_batched(t->storage, d_desc, nsets, t->d_ctr, t->nsm, t->stream));
+    CUDA_TRY(launch_batched(d_desc, nsets, t->d_ctr, t->nsm, t->stream));
     t->launches += 1;
     return TRK_OK;
 }
