@@ -311,57 +311,86 @@ __global__ void k_radix_hist(const uint32_t* __restrict__ keys, int64_t n, int s
 }
 
 // Stable scatter of one tile.  Warp w owns keys [base + 512 w, base + 512 (w+1))
-// in order; ranks among equal digits come from __match_any_sync.
-__global__ void k_radix_scatter(const uint32_t* __restrict__ keys_in, const int32_t* __restrict__ vals_in, int64_t n,
+// in order; ranks among equal digits come from __match_any_sync (once per key).
+// The tile is put in digit order in shared memory first, so that its keys
+// leave in runs (16 keys per digit on average) instead of one by one: 2^22 keys,
+// 82 us per pass with keys written from where they were read and ranked twice.
+__global__ void __launch_bounds__(RS_THREADS) k_radix_scatter(const uint32_t* __restrict__ keys_in, const int32_t* __restrict__ vals_in, int64_t n,
                                 int shift, int64_t ntiles, const uint32_t* __restrict__ tile_off,
                                 uint32_t* __restrict__ keys_out, int32_t* __restrict__ vals_out)
 {
     __shared__ uint32_t cnt[RS_WARPS][256];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    __shared__ uint32_t s_key[RS_TILE];
+    __shared__ int32_t s_val[RS_TILE];
+    __shared__ uint32_t start[256];   // of each digit in the tile; then its place in the output less that
+    __shared__ uint32_t wsum[RS_WARPS];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int64_t base = (int64_t)blockIdx.x * RS_TILE + (int64_t)w * RS_SUB;
     uint32_t k[RS_ITEMS];
     int32_t v[RS_ITEMS];
-    uint32_t d[RS_ITEMS];
+    uint32_t r[RS_ITEMS];             // rank among the warp's equal digits
 #pragma unroll
     for (int i = 0; i < RS_ITEMS; ++i) {
         const int64_t idx = base + i * 32 + lane;
         const bool valid = idx < n;
         k[i] = valid ? keys_in[idx] : 0u;
         v[i] = valid ? (vals_in ? vals_in[idx] : (int32_t)idx) : 0;
-        d[i] = valid ? ((k[i] >> shift) & 255u) : 256u;
     }
-    for (int e = threadIdx.x; e < RS_WARPS * 256; e += RS_THREADS) (&cnt[0][0])[e] = 0;
+    for (int e = tid; e < RS_WARPS * 256; e += RS_THREADS) (&cnt[0][0])[e] = 0;
     __syncthreads();
     const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
     for (int i = 0; i < RS_ITEMS; ++i) {
-        const unsigned peers = __match_any_sync(0xffffffffu, d[i]);
-        if (d[i] < 256u && lane == __ffs(peers) - 1) cnt[w][d[i]] += __popc(peers);
+        const bool valid = base + i * 32 + lane < n;
+        const uint32_t d = valid ? ((k[i] >> shift) & 255u) : 256u;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        uint32_t before = 0;
+        if (valid) before = cnt[w][d];
+        r[i] = before + __popc(peers & lt);
+        __syncwarp();
+        if (valid && lane == __ffs(peers) - 1) cnt[w][d] = before + __popc(peers);
         __syncwarp();
     }
     __syncthreads();
-    {
-        const int dg = threadIdx.x;   // one digit per thread
-        uint32_t run = tile_off[(int64_t)dg * ntiles + blockIdx.x];
+    {   // one digit per thread: its count in each warp -> the warps' first places in the tile
+        uint32_t tot = 0;
+#pragma unroll
+        for (int ww = 0; ww < RS_WARPS; ++ww) tot += cnt[ww][tid];
+        uint32_t inc = tot;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) wsum[w] = inc;
+        __syncthreads();
+        uint32_t run = inc - tot;
+        for (int ww = 0; ww < w; ++ww) run += wsum[ww];
+        start[tid] = tile_off[(int64_t)tid * ntiles + blockIdx.x] - run;
 #pragma unroll
         for (int ww = 0; ww < RS_WARPS; ++ww) {
-            const uint32_t x = cnt[ww][dg];
-            cnt[ww][dg] = run;
+            const uint32_t x = cnt[ww][tid];
+            cnt[ww][tid] = run;
             run += x;
         }
     }
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < RS_ITEMS; ++i) {
-        const unsigned peers = __match_any_sync(0xffffffffu, d[i]);
-        if (d[i] < 256u) {
-            const uint32_t pos = cnt[w][d[i]] + __popc(peers & lt);
-            keys_out[pos] = k[i];
-            vals_out[pos] = v[i];
+        if (base + i * 32 + lane < n) {
+            const uint32_t p = cnt[w][(k[i] >> shift) & 255u] + r[i];
+            s_key[p] = k[i];
+            s_val[p] = v[i];
         }
-        __syncwarp();
-        if (d[i] < 256u && lane == __ffs(peers) - 1) cnt[w][d[i]] += __popc(peers);
-        __syncwarp();
+    }
+    __syncthreads();
+    const int64_t left = n - (int64_t)blockIdx.x * RS_TILE;
+    const int m = left < RS_TILE ? (int)left : RS_TILE;
+    for (int p = tid; p < m; p += RS_THREADS) {
+        const uint32_t key = s_key[p];
+        const uint32_t pos = start[(key >> shift) & 255u] + (uint32_t)p;
+        keys_out[pos] = key;
+        vals_out[pos] = s_val[p];
     }
 }
 
