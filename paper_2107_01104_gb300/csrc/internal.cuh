@@ -123,7 +123,7 @@ struct BlockArgs {
     double* pos_out;          // [3][np], written at j
     int32_t* id_out;          // [np], written at j
     float* rhs_out;           // [ab_order-1][3][np], written at j
-    uint32_t* key_out;        // [np], written at j
+    uint32_t* key_out;        // [np], written at j, or null (a set that is not grouped: no id_out, counts)
     uint32_t* counts;         // [nblocks] block counts of the new keys (added into) or null
     void* out;                // interpolation outputs [nout][np], written at id
     int out_f64;

@@ -631,11 +631,23 @@ constexpr double kAdjDirectDensity = 0.125;
 constexpr size_t kCacheMax = 256;   // remembered tuning decisions (the oldest is dropped)
 constexpr double kProbeMin = 0.01;  // particles per cell from which the column order is a candidate
 
+// Sets this small are interpolated and stepped in the caller's order, without
+// binning: a pass is then one launch per step whose time is latency (a few
+// thousand particles do not share stencils in L1 whatever their order), where
+// the binning takes five launches more.  Only the direct kernel does that.
+constexpr int64_t kUngroupedNp = 32768;
+bool ungrouped(int64_t np, int path) { return path == TRK_STEP_DIRECT && np < kUngroupedNp; }
+
+// Below this many particles a step is latency, whatever the density: direct
+// gathers in one launch (float64 without a column kernel: up to the ungrouped limit).
+constexpr int64_t kSmallNp = 8192;
+
 // The kernel tracker_advance (and, between BLOCK and DIRECT, tracker_interpolate)
 // uses for np particles before any timing.
 int step_path(const tracker* t, int64_t np)
 {
     if (t->step_kernel != TRK_STEP_AUTO) return t->step_kernel;
+    if (np < (column_available(t) ? kSmallNp : kUngroupedNp)) return TRK_STEP_DIRECT;
     if ((double)np < direct_threshold(t) * (double)t->N * t->N * t->N) return TRK_STEP_DIRECT;
     return column_available(t) ? TRK_STEP_COLUMN : TRK_STEP_BLOCK;
 }
@@ -1178,12 +1190,17 @@ int tracker_interpolate(tracker* t, int64_t np, const double* pos, void* out, in
     const bool direct = t->step_kernel == TRK_STEP_DIRECT || (t->step_kernel == TRK_STEP_AUTO && interp_direct(t, np, deriv));
     if (!direct && (rc = check_block_kernel_shape(t))) return rc;
     if (np == 0) return TRK_OK;
-    if ((rc = ensure_sort(t, np))) return rc;
-    if ((rc = ensure_rec(t, np)) || (rc = bin_counting(t, np, pos, t->rec))) return rc;
+    const bool plain = ungrouped(np, direct ? TRK_STEP_DIRECT : TRK_STEP_BLOCK);
+    if (!plain && ((rc = ensure_sort(t, np)) || (rc = ensure_rec(t, np)) || (rc = bin_counting(t, np, pos, t->rec))))
+        return rc;
     BlockArgs a = base_args(t);
     a.np = np;
-    a.id_in = t->perm;   // grouped position -> caller index; the kernels read the records
-    a.rec_in = t->rec;
+    if (plain) {
+        a.pos_in = pos;
+    } else {
+        a.id_in = t->perm;   // grouped position -> caller index; the kernels read the records
+        a.rec_in = t->rec;
+    }
     a.ppc = 0;
     a.out = out;
     a.out_f64 = out_dtype == TRK_DTYPE_F64;
@@ -1240,6 +1257,23 @@ int tracker_advance(tracker* t, int64_t np, double* pos, float* rhs, double dt, 
     }
     if (path != TRK_STEP_DIRECT && (rc = check_block_kernel_shape(t))) return rc;
     if (np == 0 || steps == 0) return TRK_OK;
+    if (ungrouped(np, path)) {   // every step in place on the caller's arrays
+        int hist = k ? history_valid : 0;
+        for (int s = 0; s < steps; ++s) {
+            BlockArgs a = base_args(t);
+            a.np = np;
+            a.dt = dt;
+            a.pos_in = a.pos_out = pos;
+            a.rhs_in = a.rhs_out = rhs;
+            a.history_valid = hist;
+            a.ab_order = ab_order;
+            CUDA_TRY(launch_direct(t, mode, a));
+            if (k) hist = std::min(hist + 1, k - 1);
+        }
+        t->last_kernel = path;
+        t->last_tuning = {path, t->dir_blk, t->col_seg, halo_tmap(t, mode) ? 1 : 0, t->dir_ppc ? t->dir_ppc : 64};
+        return TRK_OK;
+    }
     if ((rc = ensure_sort(t, np))) return rc;
     if ((rc = ensure_state(t, np)) || (rc = ensure_rec(t, np))) return rc;
     for (const Cand& c : cands) {
