@@ -37,7 +37,11 @@ __global__ void __launch_bounds__(32 * direct_max_warps<T, I, MODE>(),
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int64_t j0 = (int64_t)blockIdx.x * a.ppc;
     const int64_t j1 = j0 + a.ppc < a.np ? j0 + a.ppc : a.np;
-    run_direct<T, I, DEG, MODE, NC, STORE, RW>(a, j0, j1, smem_raw + warp * WarpPlan<T, MODE, NC>::total, warp, nw, lane);
+    unsigned char* ws = smem_raw + warp * WarpPlan<T, MODE, NC>::total;
+    if constexpr (sizeof(T) == 4 && I == 8 && RW == 4 && !is_deriv<MODE>())
+        run_direct_warp<DEG, MODE, NC>(a, j0, j1, ws, warp, nw, lane);
+    else
+        run_direct<T, I, DEG, MODE, NC, STORE, RW>(a, j0, j1, ws, warp, nw, lane);
 }
 
 template <typename T, int I, int DEG, int MODE, int NC, int STORE, int RW>
@@ -59,16 +63,26 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
         if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     }
-    // a.ppc: a launch shape (every shape gives the same results); 0: 16 to 256
-    // particles per CTA, so that small sets still reach every SM; PPC_WIDE: CTAs
-    // that fill an SM, whose warps share one neighbourhood of the field in L1
+    // a.ppc: a launch shape (every shape gives the same results); PPC_WIDE: CTAs that
+    // fill an SM, whose warps share one neighbourhood of the field in L1; 0, by size:
+    // 16 to 256 particles per CTA, so that small sets still reach every SM and larger
+    // ones have eight CTAs per resident one.  On a field of many times the L2, at most
+    // 64: concurrent CTAs close together share what they pull into L2 (512^3, I = 8, 9e5
+    // tracers, AB2: 565 us per step against 675 with 128 and 743 with 256; not where two
+    // CTAs hold an SM, I = 6 RK2: 1.5e6 tracers 901 with 64, 850 with 256).  I = 8 on
+    // denser sets: wide (256^3, 1/16 per cell, RK2: 594 us against 638 with 256 by four
+    // warps; 512^3, 1/33: 2479 against 2658 with 64).
     int nw = NW;
+    if (a.ppc == 0) {
+        const int64_t even = (a.np + (int64_t)nsm * ctas_sm - 1) / ((int64_t)nsm * ctas_sm);
+        const int64_t n = a.f.NP - 2 * PAD, want = even <= 32 ? even : std::max<int64_t>(32, even / 8);
+        const int64_t cap = ctas_sm > 2 && n * n * n * 4 * (int64_t)sizeof(T) > ((int64_t)1 << 30) ? 64 : 256;
+        a.ppc = (int)std::min<int64_t>(cap, std::max<int64_t>(16, (want + 15) / 16 * 16));
+        if (sizeof(T) == 4 && I == 8 && a.np >= 64 * 16 * (int64_t)nsm && 34 * a.np >= n * n * n) a.ppc = PPC_WIDE;
+    }
     if (a.ppc == PPC_WIDE) {
         nw = maxw;
         a.ppc = 64 * nw;
-    } else if (a.ppc == 0) {
-        const int64_t even = (a.np + (int64_t)nsm * ctas_sm - 1) / ((int64_t)nsm * ctas_sm);
-        a.ppc = (int)std::min<int64_t>(256, std::max<int64_t>(16, (even + 15) / 16 * 16));
     }
     kern<<<(unsigned)((a.np + a.ppc - 1) / a.ppc), 32 * nw, nw * per_warp, st>>>(a);
     return cudaGetLastError();

@@ -329,33 +329,63 @@ struct GroupSums {
 // the small outer terms first, so that they are rounded while the partial sum is small
 __host__ __device__ constexpr int inward(int i, int n) { return i % 2 == 0 ? i / 2 : n - 1 - i / 2; }
 
-// the lane's column: out as above, to be summed over the group (GroupSums)
+// z sums of one row: pv (and pd with the derivative weights)
+template <typename T, int I, int NC, bool D, class LD>
+__device__ __forceinline__ void row_sums(const LD& ld, int r, const Weights<T, I, D>& w, T (&pv)[NC], T (&pd)[NC])
+{
+    constexpr int NZ = LaneMap<I>::NZ;
+#pragma unroll
+    for (int zz = 0; zz < NZ; ++zz) {
+        const int z = inward(zz, NZ);
+        T v[NC];
+        ld(r, z, v);
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            pv[k] = zz == 0 ? w.w3[z] * v[k] : fma(w.w3[z], v[k], pv[k]);
+            if constexpr (D) pd[k] = zz == 0 ? w.dw3[z] * v[k] : fma(w.dw3[z], v[k], pd[k]);
+        }
+    }
+}
+
+// the lane's column: out as above, to be summed over the group (GroupSums).
+// The rows are summed from the ends inwards; float32 values of I = 8 in the
+// order a whole warp on one particle sums them in (run_direct_warp): parts
+// {0, 4}, {1, 5}, {6, 2}, {7, 3}, then (p0 + p2) + (p1 + p3).
 template <typename T, int I, int NC, bool D, class LD>
 __device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D>& w, T (&out)[D ? 4 * NC : NC])
 {
-    constexpr int NY = LaneMap<I>::NY, NZ = LaneMap<I>::NZ;
-    T a[NC], b[NC], c[NC];
+    constexpr int NY = LaneMap<I>::NY;
+    T a[NC], b[NC], c[NC], pv[NC], pd[NC];
+    if constexpr (sizeof(T) == 4 && I == 8 && !D) {
+        T part[NC], pair[NC];
 #pragma unroll
-    for (int rr = 0; rr < NY; ++rr) {
-        const int r = inward(rr, NY);
-        T pv[NC], pd[NC];
+        for (int q = 0; q < 2; ++q)
 #pragma unroll
-        for (int zz = 0; zz < NZ; ++zz) {
-            const int z = inward(zz, NZ);
-            T v[NC];
-            ld(r, z, v);
+            for (int h = 0; h < 2; ++h) {
+                const int p = q + 2 * h, r0 = h ? p + 4 : p, r1 = h ? p : p + 4;
+                row_sums<T, I, NC, D>(ld, r0, w, pv, pd);
+#pragma unroll
+                for (int k = 0; k < NC; ++k) part[k] = w.w2[r0] * pv[k];
+                row_sums<T, I, NC, D>(ld, r1, w, pv, pd);
+#pragma unroll
+                for (int k = 0; k < NC; ++k) {
+                    part[k] = fma(w.w2[r1], pv[k], part[k]);
+                    pair[k] = h ? pair[k] + part[k] : part[k];
+                    if (h) a[k] = q ? a[k] + pair[k] : pair[k];
+                }
+            }
+    } else {
+#pragma unroll
+        for (int rr = 0; rr < NY; ++rr) {
+            const int r = inward(rr, NY);
+            row_sums<T, I, NC, D>(ld, r, w, pv, pd);
 #pragma unroll
             for (int k = 0; k < NC; ++k) {
-                pv[k] = zz == 0 ? w.w3[z] * v[k] : fma(w.w3[z], v[k], pv[k]);
-                if constexpr (D) pd[k] = zz == 0 ? w.dw3[z] * v[k] : fma(w.dw3[z], v[k], pd[k]);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            a[k] = rr == 0 ? w.w2[r] * pv[k] : fma(w.w2[r], pv[k], a[k]);
-            if constexpr (D) {
-                b[k] = rr == 0 ? w.dw2[r] * pv[k] : fma(w.dw2[r], pv[k], b[k]);
-                c[k] = rr == 0 ? w.w2[r] * pd[k] : fma(w.w2[r], pd[k], c[k]);
+                a[k] = rr == 0 ? w.w2[r] * pv[k] : fma(w.w2[r], pv[k], a[k]);
+                if constexpr (D) {
+                    b[k] = rr == 0 ? w.dw2[r] * pv[k] : fma(w.dw2[r], pv[k], b[k]);
+                    c[k] = rr == 0 ? w.w2[r] * pd[k] : fma(w.w2[r], pd[k], c[k]);
+                }
             }
         }
     }
@@ -700,6 +730,7 @@ __device__ __forceinline__ void update_particle(const BlockArgs& a, int64_t j, i
         }
     }
     if (!ok) atomicOr(a.flags + FLAG_NONFINITE, 1);
+    if (!a.key_out) return;   // a set that is not grouped
     a.id_out[j] = id;
     const uint32_t key = block_key(a.g, cn[0], cn[1], cn[2]);
     a.key_out[j] = key;
@@ -804,6 +835,153 @@ __device__ __forceinline__ void run_direct(const BlockArgs& a, int64_t j0, int64
                 cp_async_wait_all();
                 adjoint_particle<T, MODE, NC>(a, j, id, valid, ws, lane);
             } else if (valid) write_outputs<T, MODE, NC>(a, id, ch, ws, lane);
+            __syncwarp();
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// I = 8, float32, values: a whole warp per particle where stencils come from
+// beyond L1.  Lane (x, j) owns the rows y = j and j + 4 of column x: 16 nodes,
+// which it holds for RK2's second stage (eight lanes per particle would hold
+// 64, 256 registers, and gathering twice doubles the traffic beyond L1).  The
+// sums are those of the eight-lane form, bit for bit.  256^3, 1/16 per cell,
+// RK2, us per step: 690 with eight lanes at best; 512^3, 1.4e-2 per cell: 1717.
+// ---------------------------------------------------------------------------
+template <int DEG>
+struct WarpBasis {
+    Row<float, DEG> r;
+    int ax, i;
+    bool act;
+    __device__ __forceinline__ void init(const CoefTable<float>& tb, int lane)
+    {
+        act = lane < 24;
+        ax = act ? lane >> 3 : 0;
+        i = lane & 7;
+        r = load_row<float, DEG>(tb.c, i);
+    }
+    __device__ __forceinline__ void eval(float s1, float s2, float s3, float* wb) const
+    {
+        const float w = horner(r, ax == 0 ? s1 : (ax == 1 ? s2 : s3));
+        if (act) wb[ax * 8 + i] = w;
+        __syncwarp();
+    }
+};
+
+// the warp's sum of component comp = 2 bit4 + bit3 of the lane, in the eight lanes that share it
+template <int NC>
+__device__ __forceinline__ float warp_contract(const float (&f)[2][8][NC], const float* wb, int lane)
+{
+    const int x = lane & 7, j = lane >> 3;
+    float w3[8];
+    bcast_load(wb + 16, w3);
+    const float w1 = wb[x], w2[2] = {wb[8 + j], wb[12 + j]};
+    float p[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        float pv[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int zz = 0; zz < 8; ++zz) {
+                const int z = inward(zz, 8);
+                pv[h] = zz == 0 ? w3[z] * f[h][z][k] : fmaf(w3[z], f[h][z][k], pv[h]);
+            }
+        // rows in contract's order: j, j + 4 for j < 2, else j + 4, j
+        const bool up = j < 2;
+        p[k] = fmaf(up ? w2[1] : w2[0], up ? pv[1] : pv[0], (up ? w2[0] : w2[1]) * (up ? pv[0] : pv[1]));
+    }
+    const bool b4 = lane & 16, b3 = lane & 8;
+    float q0 = (b4 ? p[2] : p[0]) + __shfl_xor_sync(0xffffffffu, b4 ? p[0] : p[2], 16);
+    float q1 = (b4 ? p[3] : p[1]) + __shfl_xor_sync(0xffffffffu, b4 ? p[1] : p[3], 16);
+    float m = (b3 ? q1 : q0) + __shfl_xor_sync(0xffffffffu, b3 ? q0 : q1, 8);
+    m *= w1;
+    m += __shfl_xor_sync(0xffffffffu, m, 4);
+    m += __shfl_xor_sync(0xffffffffu, m, 2);
+    m += __shfl_xor_sync(0xffffffffu, m, 1);
+    return m;
+}
+
+template <int NC>
+__device__ __forceinline__ void warp_load(const FieldView& f, int node, int ch, int lane, float (&v)[2][8][NC])
+{
+    const RecordLd<4, NC> ld{f.rec + ((int64_t)ch * f.plane + node + (lane & 7) + (lane >> 3) * f.NP) * 4, f.NP, f.NP * f.NP};
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int z = 0; z < 8; ++z) ld(4 * h, z, v[h][z]);
+}
+
+template <int DEG, int MODE, int NC>
+__device__ __forceinline__ void run_direct_warp(const BlockArgs& a, int64_t j0, int64_t j1, unsigned char* ws, int warp,
+                                                int nw, int lane)
+{
+    using T = float;
+    using WPl = WarpPlan<T, MODE, NC>;
+    static_assert(!is_deriv<MODE>(), "values only");
+    constexpr int LO = 3;
+    WarpBasis<DEG> B;
+    B.init(a.cf, lane);
+    const WarpMem<T, MODE, NC> wm(ws, 0);
+    const int comp = (lane & 16 ? 2 : 0) + (lane & 8 ? 1 : 0);
+    const bool writer = (lane & 7) == 0 && comp < NC;
+    const float dtid = (float)(a.dt * a.g.inv_delta);
+    for (int64_t b0 = j0; b0 < j1; b0 += 32 * nw) {
+        const int64_t j = b0 + lane * nw + warp;
+        const int left = (int)min(j1 - b0 - warp, (int64_t)32 * nw);   // particles from this warp's first on
+        if (left <= 0) break;
+        const bool valid = j < j1;
+        const int64_t src = !valid ? 0 : (a.perm ? a.perm[j] : j);
+        const int32_t id = !valid ? 0 : (a.id_in ? a.id_in[src] : (int32_t)src);
+        wm.recs[lane] = particle_record<T>(a, j, src, valid);
+        fetch_state<T, MODE, NC>(a, src, valid, ws, lane);
+        __syncwarp();
+        for (int ch = 0; ch < (is_step<MODE>() ? 1 : (a.f.C + NC - 1) / NC); ++ch) {
+            for (int it = 0; it * nw < left; ++it) {
+                const PRec<T> rec = wm.recs[it];
+                int c[3];
+                unpack_cell(cell_of(rec), c);
+                float f[2][8][NC];
+                warp_load<NC>(a.f, (int)padded_index(a.f.NP, c[0] - LO, c[1] - LO, c[2] - LO), ch, lane, f);
+                float* kb = wm.kbuf + it * WPl::KS;
+                B.eval(rec.t[0] - 0.5f, rec.t[1] - 0.5f, rec.t[2] - 0.5f, MODE != MODE_RK2 && (it & 1) ? wm.wb1 : wm.wb0);
+                const float m = warp_contract<NC>(f, MODE != MODE_RK2 && (it & 1) ? wm.wb1 : wm.wb0, lane);
+                if (writer) kb[comp] = m;
+                if constexpr (MODE == MODE_RK2) {
+                    float ts[3];
+                    int d[3];
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) {
+                        const float u1 = __shfl_sync(0xffffffffu, m, ax == 0 ? 0 : (ax == 1 ? 8 : 16));
+                        ts[ax] = fmaf(dtid, u1, rec.t[ax]);
+                        const float fl = floorf(ts[ax]);
+                        d[ax] = (int)fl;
+                        ts[ax] -= fl;
+                    }
+                    if ((d[0] | d[1] | d[2]) != 0) {   // (the whole warp: one particle)
+                        const bool far = (unsigned)d[0] + 1u > 2u || (unsigned)d[1] + 1u > 2u || (unsigned)d[2] + 1u > 2u;
+                        if (far) {
+                            if (lane == 0) atomicOr(a.flags + FLAG_CFL, 1);
+#pragma unroll
+                            for (int ax = 0; ax < 3; ++ax) c[ax] = (int)(((unsigned)c[ax] + (unsigned)d[ax]) & (unsigned)a.g.mask);
+                        } else {
+#pragma unroll
+                            for (int ax = 0; ax < 3; ++ax) c[ax] += d[ax];
+                        }
+                        warp_load<NC>(a.f, (int)padded_index(a.f.NP, c[0] - LO, c[1] - LO, c[2] - LO), 0, lane, f);
+                    }
+                    B.eval(ts[0] - 0.5f, ts[1] - 0.5f, ts[2] - 0.5f, wm.wb1);
+                    const float m2 = warp_contract<NC>(f, wm.wb1, lane);
+                    if (writer) kb[3 + comp] = m2;
+                }
+            }
+            __syncwarp();
+            if constexpr (is_step<MODE>()) {
+                cp_async_wait_all();
+                update_particle<T, MODE, NC>(a, j, id, valid, ws, lane);
+            } else if (valid) {
+                write_outputs<T, MODE, NC>(a, id, ch, ws, lane);
+            }
             __syncwarp();
         }
     }
