@@ -226,7 +226,7 @@ template <int I, int MODE, int NC>
 struct SlabPlan {
     using SG = SlabGeom<I, MODE>;
     // (the adjoint hands 22 values per particle over: fewer warps leave room for the slabs)
-    static constexpr int warps = MODE == MODE_ADJ ? (I == 8 ? 8 : 12) : 4 * min_ctas<float, I, MODE, SRC_SLABS>();
+    static constexpr int warps = MODE == MODE_ADJ ? (I == 8 ? 8 : 12) : 4 * CTAS_SM;
     static constexpr size_t slab = SG::slot;
     static constexpr size_t per_warp = WarpPlan<float, MODE, NC>::total;
     static constexpr size_t room = 232448 - 256 - warps * per_warp;
@@ -340,7 +340,9 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
     using SG = typename SP::SG;
     constexpr int nw = SP::warps;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 3;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int GL = group_lanes<T, I, MODE, SRC_SLABS>(), P = 32 / GL;   // P particles at once
+    const int g = lane / GL;
     const int64_t j0 = (int64_t)blockIdx.x * a.ppc;
     const int64_t j1 = j0 + a.ppc < a.np ? j0 + a.ppc : a.np;
     const PRec<T>* recs_in = reinterpret_cast<const PRec<T>*>(a.rec_in);
@@ -363,37 +365,37 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
     __syncthreads();
     unsigned char* ws = smem_raw + SP::warp + warp * SP::per_warp;
     const WarpMem<T, MODE, NC> wm(ws, g);
-    const LaneMap<I> m(lane);
-    Basis<T, I, DEG, is_deriv<MODE>()> B;
+    const LaneMap<I, GL> m(lane);
+    Basis<T, I, DEG, is_deriv<MODE>(), GL> B;
     B.init(a.cf, m);
-    // A batch is 8 rounds of four particles per warp; the warps' first batches have 1
-    // to 8 rounds, so that their float64 phases do not all meet on that pipe at once.
+    // A batch is GL rounds of P particles per warp; the warps' first batches have 1/8
+    // to 8/8 of these rounds, so that their float64 phases do not all meet on that pipe at once.
     // The records of the next batch and the state of this one are copied to shared
     // memory (cp.async) while this one is interpolated.
-    int rounds = 1 + (warp & 7), odd = 0, buf = 0;
-    auto my_index = [&](int64_t b0) { return b0 + ((lane >> 2) * nw + warp) * 4 + (lane & 3); };
+    int rounds = (1 + (warp & 7)) * (GL / 8), odd = 0, buf = 0;
+    auto my_index = [&](int64_t b0) { return b0 + (lane / P * nw + warp) * P + lane % P; };
     auto fetch_records = [&](int64_t b0, int nrounds, int to) {
         const int64_t j = my_index(b0);
-        if (j < j1 && (lane >> 2) < nrounds) cp_async<16>(wm.recs + to * 32 + lane, recs_in + j);
+        if (j < j1 && lane / P < nrounds) cp_async<16>(wm.recs + to * 32 + lane, recs_in + j);
     };
     fetch_records(j0, rounds, 0);
     cp_async_commit();
     for (int64_t b0 = j0; b0 < j1; buf ^= 1) {
-        const int64_t bn = b0 + (int64_t)4 * nw * rounds;
+        const int64_t bn = b0 + (int64_t)P * nw * rounds;
         const int64_t j = my_index(b0);
-        const int left = (int)min(j1 - b0 - 4 * warp, (int64_t)4 * nw * rounds);
+        const int left = (int)min(j1 - b0 - P * warp, (int64_t)P * nw * rounds);
         if (left <= 0) break;
-        const bool valid = j < j1 && (lane >> 2) < rounds;
+        const bool valid = j < j1 && lane / P < rounds;
         int32_t id = 0;   // (loaded where it is needed: a register less meanwhile)
         if (MODE == MODE_ADJ && valid) id = a.id_in[j];
         fetch_state<T, MODE, NC>(a, MODE == MODE_ADJ ? id : j, valid, ws, lane);
-        fetch_records(bn, 8, buf ^ 1);
+        fetch_records(bn, GL, buf ^ 1);
         cp_async_commit();
         cp_async_wait_group<1>();
         __syncwarp();
-        for (int it = 0; it < 8 && it * 4 * nw < left; ++it) {
-            const bool live = it * 4 * nw + g < left;
-            const PRec<T> rec = wm.recs[buf * 32 + 4 * it + g];
+        for (int it = 0; it < rounds && it * P * nw < left; ++it) {
+            const bool live = it * P * nw + g < left;
+            const PRec<T> rec = wm.recs[buf * 32 + P * it + g];
             int c[3] = {0, 0, 0};
             if (live) unpack_cell(cell_of(rec), c);
             // (a particle lies in one of the CTA's blocks; the clamp only keeps corrupted
@@ -401,7 +403,7 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
             const int block = min(max((int)block_key(a.g, c[0], c[1], c[2]), slabs.b_first), slabs.b_last);
             const int q = slabs.first_slab(block);
             bool todo = live;
-            do {   // one round, unless the four particles lie in more than two adjacent blocks of a row
+            do {   // one round, unless the particles lie in more than two adjacent blocks of a row
                 const int lo = (int)__reduce_min_sync(0xffffffffu, todo ? (unsigned)q : 0x7fffffffu);
                 const bool now = todo && q - lo <= SG::SPT;
                 Place at{};
@@ -412,7 +414,7 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
                 at.halo = smem_raw;
                 interpolate_group<T, I, DEG, MODE, NC, ST_F32, 4, SRC_SLABS, SP::NS>(
                     a, at, slabs.ch, rec.t, now, lane, B, m, wm.wb0, wm.wb1, odd & 1,
-                    wm.kbuf + (4 * it + g) * WarpMem<T, MODE, NC>::WPl::KS);
+                    wm.kbuf + (P * it + g) * WarpMem<T, MODE, NC>::WPl::KS);
                 ++odd;
                 todo = todo && !now;
             } while (__any_sync(0xffffffffu, todo));
@@ -430,7 +432,7 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
         }
         __syncwarp();
         b0 = bn;
-        rounds = 8;
+        rounds = GL;
     }
     cp_async_wait_all();
     slabs.release_to(slabs.count, lane, nw);   // every copy has landed before the CTA ends

@@ -17,7 +17,7 @@ namespace trk {
 // Warps of a CTA that fills an SM at the kernel's register cap; float64
 // kernels, bound by the float64 pipe, four of 16.
 template <typename T, int I, int MODE>
-constexpr int direct_max_warps() { return sizeof(T) == 8 ? NW : 4 * min_ctas<T, I, MODE, SRC_GLOBAL>(); }
+constexpr int direct_max_warps() { return sizeof(T) == 8 ? NW : 4 * CTAS_SM; }
 
 // shared-memory carveout (percent of the SM's 228 KB) that holds `ctas` CTAs of
 // `smem` bytes each, with the 1 KB the system reserves per CTA
@@ -30,7 +30,7 @@ inline int carveout_percent(size_t smem, int ctas)
 
 template <typename T, int I, int DEG, int MODE, int NC, int STORE, int RW>
 __global__ void __launch_bounds__(32 * direct_max_warps<T, I, MODE>(),
-                                  4 * min_ctas<T, I, MODE, SRC_GLOBAL>() / direct_max_warps<T, I, MODE>())
+                                  4 * CTAS_SM / direct_max_warps<T, I, MODE>())
     k_direct(const __grid_constant__ BlockArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -49,7 +49,7 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
 {
     if (a.np <= 0) return cudaSuccess;
     constexpr size_t per_warp = WarpPlan<T, MODE, NC>::total;
-    constexpr int maxw = direct_max_warps<T, I, MODE>(), ctas_sm = min_ctas<T, I, MODE, SRC_GLOBAL>();
+    constexpr int maxw = direct_max_warps<T, I, MODE>(), ctas_sm = CTAS_SM;
     auto kern = k_direct<T, I, DEG, MODE, NC, STORE, RW>;
     static int nsm = 0;
     if (!nsm) {
@@ -63,22 +63,28 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
         if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     }
-    // a.ppc: a launch shape (every shape gives the same results); PPC_WIDE: CTAs that
-    // fill an SM, whose warps share one neighbourhood of the field in L1; 0, by size:
-    // 16 to 256 particles per CTA, so that small sets still reach every SM and larger
-    // ones have eight CTAs per resident one.  On a field of many times the L2, at most
-    // 64: concurrent CTAs close together share what they pull into L2 (512^3, I = 8, 9e5
-    // tracers, AB2: 565 us per step against 675 with 128 and 743 with 256; not where two
-    // CTAs hold an SM, I = 6 RK2: 1.5e6 tracers 901 with 64, 850 with 256).  I = 8 on
-    // denser sets: wide (256^3, 1/16 per cell, RK2: 594 us against 638 with 256 by four
-    // warps; 512^3, 1/33: 2479 against 2658 with 64).
+    // a.ppc: particles per CTA (every shape gives the same results); 0, by size (us per
+    // step, float32 unless noted):
+    //  - up to 64 each (I = 8, float64: 32), one wave: 128^3 float64 I = 6, 4e4 tracers,
+    //    RK2: 199 with 32, 222 with 64, 338 with 256; 64^3, I = 4, 3.5e4: 12 with 64, 16
+    //    with 32, 28 in CTAs of 1024.
+    //  - then an eighth of an even share per resident CTA, so that the last wave is short,
+    //    up to 256, which keeps a CTA's stencils close together (256^3, I = 4, AB2, 2^21: 235
+    //    with 256, 356 with 64).
+    //  - at most 64 on a field of many times the L2, whose concurrent CTAs then share what
+    //    they pull into it (512^3, I = 8, 9e5, AB2: 573 with 64, 702 with 256), and for RK2's
+    //    sixteen lanes on sets below 1/12 per cell (256^3, 8e5: 314 with 64, 330 with 1024).
+    //  - I = 8 on denser sets: CTAs that fill an SM, whose warps share one neighbourhood of
+    //    the field in L1 (PPC_WIDE; 256^3, 2^21, RK2: 1126, 1229 with 256, 1258 with 64).
     int nw = NW;
     if (a.ppc == 0) {
+        constexpr bool split = group_lanes<T, I, MODE, SRC_GLOBAL>() == 16, f32 = sizeof(T) == 4;
         const int64_t even = (a.np + (int64_t)nsm * ctas_sm - 1) / ((int64_t)nsm * ctas_sm);
-        const int64_t n = a.f.NP - 2 * PAD, want = even <= 32 ? even : std::max<int64_t>(32, even / 8);
-        const int64_t cap = ctas_sm > 2 && n * n * n * 4 * (int64_t)sizeof(T) > ((int64_t)1 << 30) ? 64 : 256;
-        a.ppc = (int)std::min<int64_t>(cap, std::max<int64_t>(16, (want + 15) / 16 * 16));
-        if (sizeof(T) == 4 && I == 8 && a.np >= 64 * 16 * (int64_t)nsm && 34 * a.np >= n * n * n) a.ppc = PPC_WIDE;
+        const int64_t n = a.f.NP - 2 * PAD, cells = n * n * n, one_wave = f32 && I < 8 ? 64 : 32;
+        const int64_t want = even <= one_wave ? even : std::max<int64_t>(one_wave, even / 8);
+        const bool small = cells * 4 * (int64_t)sizeof(T) > ((int64_t)1 << 30) || (split && 12 * a.np < cells);
+        a.ppc = (int)std::min<int64_t>(small ? 64 : 256, std::max<int64_t>(16, (want + 15) / 16 * 16));
+        if (f32 && I == 8 && a.np >= 64 * 16 * (int64_t)nsm && 34 * a.np >= cells) a.ppc = PPC_WIDE;
     }
     if (a.ppc == PPC_WIDE) {
         nw = maxw;

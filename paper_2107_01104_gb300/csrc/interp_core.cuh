@@ -106,27 +106,32 @@ __device__ __forceinline__ void bcast_load(const T* p, T (&w)[n])
 // ---------------------------------------------------------------------------
 // Lane map and weights of a group of eight lanes
 // ---------------------------------------------------------------------------
-template <int I>
+// Sixteen lanes (RK2, I = 6 float32): the eight of a half h own the x columns
+// of the rows y = h, h + 2, h + 4.
+template <int I, int GL = 8>
 struct LaneMap {
-    static constexpr int NY = I;                // rows along y per lane
+    static_assert(GL == 8 || (GL == 16 && I == 6), "sixteen lanes: I = 6");
+    static constexpr int YS = GL / 8;           // rows along y per lane: y0, y0 + YS, ...
+    static constexpr int NY = I / YS;
     static constexpr int NZ = I == 4 ? 2 : I;   // planes along z per lane: z0, z0 + ZS, ...
     static constexpr int ZS = I == 4 ? 2 : 1;
-    int x, z0;
+    int x, y0, z0;
     bool act;                                   // false: a repeated column (zero weight)
     __device__ __forceinline__ explicit LaneMap(int lane)
     {
         const int u = lane & 7;
         x = I == 8 ? u : (I == 6 ? (u < 6 ? u : u - 6) : (u & 3));
+        y0 = GL == 16 ? (lane >> 3 & 1) : 0;
         z0 = I == 4 ? u >> 2 : 0;
         act = I != 6 || u < 6;
     }
 };
 
-template <typename T, int I, bool D>
+template <typename T, int I, bool D, int GL = 8>
 struct Weights {
-    static constexpr int NY = LaneMap<I>::NY, NZ = LaneMap<I>::NZ;
+    static constexpr int NY = LaneMap<I, GL>::NY, NZ = LaneMap<I, GL>::NZ;
     T w1, dw1;
-    T w2[NY], w3[NZ];
+    T w2[GL == 16 ? 4 : NY], w3[NZ];
     T dw2[D ? NY : 1], dw3[D ? NZ : 1];
 };
 
@@ -135,16 +140,28 @@ struct Weights {
 // axis 3 at 8, their derivatives at 16 and 24; I = 4: axis 3 in the order 0, 2,
 // 1, 3, so that a lane's planes are adjacent).  Successive calls of a warp
 // alternate between two buffers, so one __syncwarp per call orders them.
-template <typename T, int I, int DEG, bool D>
+// Sixteen lanes: half 0 evaluates axis 2, half 1 axis 3; axis 2 is stored in the
+// order 0, 2, 4, -, 1, 3, 5, so that a half's rows are adjacent.
+template <typename T, int I, int DEG, bool D, int GL = 8>
 struct Basis {
     Row<T, DEG> r, dr;
-    __device__ __forceinline__ void init(const CoefTable<T>& tb, const LaneMap<I>& m)
+    __device__ __forceinline__ void init(const CoefTable<T>& tb, const LaneMap<I, GL>& m)
     {
         r = load_row<T, DEG>(tb.c, m.x);
         if (D) dr = load_row<T, DEG>(tb.d, m.x);
     }
-    __device__ __forceinline__ void eval(T s1, T s2, T s3, const LaneMap<I>& m, T* wb, Weights<T, I, D>& w) const
+    __device__ __forceinline__ void eval(T s1, T s2, T s3, const LaneMap<I, GL>& m, T* wb, Weights<T, I, D, GL>& w) const
     {
+        if constexpr (GL == 16) {
+            static_assert(!D, "values only");
+            const T a1 = horner(r, s1);
+            wb[m.y0 ? 8 + m.x : (m.x & 1) * 4 + (m.x >> 1)] = horner(r, m.y0 ? s3 : s2);
+            w.w1 = m.act ? a1 : (T)0;
+            __syncwarp();
+            bcast_load(wb + 4 * m.y0, w.w2);
+            bcast_load(wb + 8, w.w3);
+            return;
+        }
         const T a1 = horner(r, s1), a2 = horner(r, s2), a3 = horner(r, s3);
         // (repeated columns store the values their originals store)
         const int x3 = I == 4 ? (m.x & 1) * 2 + (m.x >> 1) : m.x;
@@ -209,15 +226,15 @@ struct PlaneLd {
 
 // Loader of the stencil whose first node has the padded index `base`, for the
 // component chunk ch (NC components of it)
-template <typename T, int I, int STORE, int RW, int NC>
-__device__ __forceinline__ auto global_ld(const FieldView& f, int base, int ch, const LaneMap<I>& m)
+template <typename T, int I, int STORE, int RW, int NC, int GL>
+__device__ __forceinline__ auto global_ld(const FieldView& f, int base, int ch, const LaneMap<I, GL>& m)
 {
-    constexpr int ZS = LaneMap<I>::ZS;
-    const int64_t n = (int64_t)base + m.x + m.z0 * f.NP * f.NP;
+    constexpr int ZS = LaneMap<I, GL>::ZS, YS = LaneMap<I, GL>::YS;
+    const int64_t n = (int64_t)base + m.x + m.y0 * f.NP + m.z0 * f.NP * f.NP;
     if constexpr (STORE == ST_F64)
-        return PlaneLd<NC>{f.f64 + (int64_t)ch * NC * f.plane + n, f.plane, f.NP, ZS * f.NP * f.NP, f.C - ch * NC};
+        return PlaneLd<NC>{f.f64 + (int64_t)ch * NC * f.plane + n, f.plane, YS * f.NP, ZS * f.NP * f.NP, f.C - ch * NC};
     else
-        return RecordLd<RW, NC>{f.rec + ((int64_t)ch * f.plane + n) * RW, f.NP, ZS * f.NP * f.NP};
+        return RecordLd<RW, NC>{f.rec + ((int64_t)ch * f.plane + n) * RW, YS * f.NP, ZS * f.NP * f.NP};
 }
 
 // A staged halo in shared memory: pitches P from row to row and PL from plane
@@ -245,7 +262,7 @@ struct HaloLd {
 // second stage), the others loaded as they are contracted.
 template <typename T, int I, int NC, int HR, class LD>
 struct HeldLd {
-    const T (&f)[HR][LaneMap<I>::NZ][NC];
+    const T (&f)[HR][LaneMap<I>::NZ][NC];   // (NZ: the same for either group size)
     const LD& rest;
     __device__ __forceinline__ void operator()(int r, int z, T (&v)[NC]) const
     {
@@ -325,13 +342,40 @@ struct GroupSums {
     }
 };
 
+// the same for three values over a group of sixteen (after join_halves): half 0 is
+// left with value 0 (lanes u < 4) or 1 (u >= 4), half 1 with value 2 (u < 4)
+template <typename T>
+struct HalfSums {
+    T v;
+    int which;   // -1: none
+    __device__ __forceinline__ HalfSums(const T (&x)[3], int lane)
+    {
+        const bool hi = lane & 4, second = lane & 8;
+        // half 1 adds value 2 in all its lanes
+        const T give = second ? x[0] : (hi ? x[0] : x[1]), keep = second ? x[0] : (hi ? x[1] : x[0]);
+        v = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        which = lane & 3 ? -1 : (second ? (hi ? -1 : 2) : (hi ? 1 : 0));
+    }
+    template <int i>
+    __device__ __forceinline__ T all(int lane) const
+    {
+        return __shfl_sync(0xffffffffu, v, (lane & 16) | (i == 0 ? 0 : (i == 1 ? 4 : 8)));
+    }
+    __device__ __forceinline__ void put(T* kb, int, bool live) const
+    {
+        if (live && which >= 0) kb[which] = v;
+    }
+};
+
 // i-th term of a sum over n nodes taken from the ends inwards (0, n-1, 1, ...):
 // the small outer terms first, so that they are rounded while the partial sum is small
 __host__ __device__ constexpr int inward(int i, int n) { return i % 2 == 0 ? i / 2 : n - 1 - i / 2; }
 
 // z sums of one row: pv (and pd with the derivative weights)
-template <typename T, int I, int NC, bool D, class LD>
-__device__ __forceinline__ void row_sums(const LD& ld, int r, const Weights<T, I, D>& w, T (&pv)[NC], T (&pd)[NC])
+template <typename T, int I, int NC, bool D, int GL, class LD>
+__device__ __forceinline__ void row_sums(const LD& ld, int r, const Weights<T, I, D, GL>& w, T (&pv)[NC], T (&pd)[NC])
 {
     constexpr int NZ = LaneMap<I>::NZ;
 #pragma unroll
@@ -350,23 +394,38 @@ __device__ __forceinline__ void row_sums(const LD& ld, int r, const Weights<T, I
 // the lane's column: out as above, to be summed over the group (GroupSums).
 // The rows are summed from the ends inwards; float32 values of I = 8 in the
 // order a whole warp on one particle sums them in (run_direct_warp): parts
-// {0, 4}, {1, 5}, {6, 2}, {7, 3}, then (p0 + p2) + (p1 + p3).
-template <typename T, int I, int NC, bool D, class LD>
-__device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D>& w, T (&out)[D ? 4 * NC : NC])
+// {0, 4}, {1, 5}, {6, 2}, {7, 3}, then (p0 + p2) + (p1 + p3); of I = 6 in the
+// order of sixteen lanes: rows 0, 4, 2 plus rows 1, 5, 3.
+template <typename T, int I, int NC, bool D, int GL, class LD>
+__device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D, GL>& w, T (&out)[D ? 4 * NC : NC])
 {
-    constexpr int NY = LaneMap<I>::NY;
+    constexpr int NY = LaneMap<I, GL>::NY;
     T a[NC], b[NC], c[NC], pv[NC], pd[NC];
-    if constexpr (sizeof(T) == 4 && I == 8 && !D) {
+    if constexpr (sizeof(T) == 4 && I == 6 && !D) {
+        T half[NC];
+#pragma unroll
+        for (int h = 0; h < (GL == 16 ? 1 : 2); ++h) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const int r = GL == 16 ? inward(q, 3) : h + 2 * inward(q, 3);
+                row_sums<T, I, NC, D, GL>(ld, r, w, pv, pd);
+#pragma unroll
+                for (int k = 0; k < NC; ++k) half[k] = q == 0 ? w.w2[r] * pv[k] : fma(w.w2[r], pv[k], half[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < NC; ++k) a[k] = h ? a[k] + half[k] : half[k];
+        }
+    } else if constexpr (sizeof(T) == 4 && I == 8 && !D) {
         T part[NC], pair[NC];
 #pragma unroll
         for (int q = 0; q < 2; ++q)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int p = q + 2 * h, r0 = h ? p + 4 : p, r1 = h ? p : p + 4;
-                row_sums<T, I, NC, D>(ld, r0, w, pv, pd);
+                row_sums<T, I, NC, D, GL>(ld, r0, w, pv, pd);
 #pragma unroll
                 for (int k = 0; k < NC; ++k) part[k] = w.w2[r0] * pv[k];
-                row_sums<T, I, NC, D>(ld, r1, w, pv, pd);
+                row_sums<T, I, NC, D, GL>(ld, r1, w, pv, pd);
 #pragma unroll
                 for (int k = 0; k < NC; ++k) {
                     part[k] = fma(w.w2[r1], pv[k], part[k]);
@@ -378,7 +437,7 @@ __device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D>& w
 #pragma unroll
         for (int rr = 0; rr < NY; ++rr) {
             const int r = inward(rr, NY);
-            row_sums<T, I, NC, D>(ld, r, w, pv, pd);
+            row_sums<T, I, NC, D, GL>(ld, r, w, pv, pd);
 #pragma unroll
             for (int k = 0; k < NC; ++k) {
                 a[k] = rr == 0 ? w.w2[r] * pv[k] : fma(w.w2[r], pv[k], a[k]);
@@ -391,7 +450,7 @@ __device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D>& w
     }
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
-        out[k] = w.w1 * a[k];
+        out[k] = GL == 16 ? a[k] : w.w1 * a[k];   // (sixteen lanes: join_halves multiplies)
         if constexpr (D) {
             out[NC + 3 * k] = w.dw1 * a[k];
             out[NC + 3 * k + 1] = w.w1 * b[k];
@@ -526,38 +585,59 @@ __device__ __forceinline__ void fetch_state(const BlockArgs& a, int64_t src, boo
     }
 }
 
-// Rows of the RK2 stencil a lane holds in registers between the stages: its
-// second stage then gathers these only where X* left the cell.  I = 4 (8
-// nodes): always.  I = 6 (36 nodes, 144 registers): in the direct kernel, whose
-// stencils come from beyond L1, eight warps per SM that hold them move less
-// than sixteen that gather twice (256^3 float32, RK2, us per step: 137 against
-// 158 at 1/64 particle per cell; 512^3 at 1.5e-3: 197 against 226; 168
-// registers with spills: 158, 220); from slabs in shared memory sixteen warps
-// without held rows are faster (1/4 per cell: 1238 against 1536).  I = 8 would
-// take 256 registers, float64 twice these: none.
-template <typename T, int I, int SRC>
+// Lanes per particle and rows of the RK2 stencil that a lane holds in registers
+// between the stages: its second stage then gathers these only where X* left
+// the cell.  I = 4 (8 nodes per lane): always.  I = 6 (36 nodes, 108 registers of
+// values): gathered from global memory, by sixteen lanes that hold 18 nodes each,
+// sixteen warps per SM (256^3 float32, RK2, us per step at 1/64 particle per cell:
+// 120, against 145 with eight lanes and eight warps that hold 36 nodes, 158 with
+// sixteen warps that gather twice; 512^3, 1.5e6: 671, 797); from slabs in shared
+// memory eight lanes without held rows, which issue fewer instructions (1/8 per
+// cell: 633 against 710 with sixteen lanes; 1/16: 377, 400, 12 warps with held
+// rows 407).  I = 8 would take 256 registers (run_direct_warp holds them),
+// float64 twice these: none.
+template <typename T, int I, int MODE, int SRC>
+__host__ __device__ constexpr int group_lanes()
+{
+    return sizeof(T) == 4 && I == 6 && MODE == MODE_RK2 && SRC == SRC_GLOBAL ? 16 : 8;
+}
+template <typename T, int I, int MODE, int SRC>
 __host__ __device__ constexpr int held_rows()
 {
-    return sizeof(T) == 8 || I == 8 ? 0 : (I == 4 ? 4 : (SRC == SRC_GLOBAL ? 6 : 0));
+    if (group_lanes<T, I, MODE, SRC>() == 16) return 3;
+    return sizeof(T) == 8 || I != 4 ? 0 : 4;
+}
+
+// The halves of a group of sixteen: half 0 goes on with values 0 and 1, half 1
+// with value 2 (then 0), so that the sums over x take three shuffles, not four.
+template <typename T>
+__device__ __forceinline__ void join_halves(T (&k)[3], T w1, int lane)
+{
+    const bool hi = lane & 8;
+    const T r = __shfl_xor_sync(0xffffffffu, hi ? k[0] : k[2], 8), r1 = __shfl_xor_sync(0xffffffffu, k[1], 8);
+    k[0] = w1 * ((hi ? k[2] : k[0]) + r);
+    k[1] = w1 * (k[1] + r1);
 }
 
 // One stage: contract the stencil of ld at the offsets s (less 1/2) from the
 // cell's centre; the rows held in f are loaded if `fresh`.
-template <typename T, int I, int DEG, int NC, bool D, int HR, class LD>
-__device__ __forceinline__ void interpolate_stage(const LD& ld, T s1, T s2, T s3, T* wb, bool fresh, const LaneMap<I>& m,
-                                                  const Basis<T, I, DEG, D>& B,
-                                                  T (&f)[HR > 0 ? HR : 1][LaneMap<I>::NZ][NC], T (&k)[D ? 4 * NC : NC])
+template <typename T, int I, int DEG, int NC, bool D, int HR, int GL, class LD>
+__device__ __forceinline__ void interpolate_stage(const LD& ld, T s1, T s2, T s3, T* wb, bool fresh,
+                                                  const LaneMap<I, GL>& m, const Basis<T, I, DEG, D, GL>& B,
+                                                  T (&f)[HR > 0 ? HR : 1][LaneMap<I>::NZ][NC], T (&k)[D ? 4 * NC : NC],
+                                                  int lane)
 {
-    Weights<T, I, D> w;
+    Weights<T, I, D, GL> w;
     if constexpr (HR > 0) {
         if (fresh) load_rows<T, I, NC, HR>(ld, f);
         __syncwarp();
         B.eval(s1, s2, s3, m, wb, w);
-        contract<T, I, NC, D>(HeldLd<T, I, NC, HR, LD>{f, ld}, w, k);
+        contract<T, I, NC, D, GL>(HeldLd<T, I, NC, HR, LD>{f, ld}, w, k);
     } else {
         B.eval(s1, s2, s3, m, wb, w);
-        contract<T, I, NC, D>(ld, w, k);
+        contract<T, I, NC, D, GL>(ld, w, k);
     }
+    if constexpr (GL == 16) join_halves(k, w.w1, lane);
 }
 
 // ---------------------------------------------------------------------------
@@ -567,35 +647,37 @@ __device__ __forceinline__ void interpolate_stage(const LD& ld, T s1, T s2, T s3
 // ---------------------------------------------------------------------------
 template <typename T, int I, int DEG, int MODE, int NC, int STORE, int RW, int SRC, int NS = 1>
 __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Place& at, int ch, const T (&t)[3], bool live,
-                                                  int lane, const Basis<T, I, DEG, is_deriv<MODE>()>& B,
-                                                  const LaneMap<I>& m, T* wb0, T* wb1, bool odd,
-                                                  T* kb)
+                                                  int lane,
+                                                  const Basis<T, I, DEG, is_deriv<MODE>(), group_lanes<T, I, MODE, SRC>()>& B,
+                                                  const LaneMap<I, group_lanes<T, I, MODE, SRC>()>& m, T* wb0, T* wb1,
+                                                  bool odd, T* kb)
 {
+    constexpr int GL = group_lanes<T, I, MODE, SRC>(), YS = LaneMap<I, GL>::YS;
     constexpr bool D = is_deriv<MODE>(), HALO = SRC != SRC_GLOBAL;
     constexpr int LO = I / 2 - 1, ZS = LaneMap<I>::ZS, G = LO + (two_stages<MODE>() ? 1 : 0);
     // the stencil of the cell displaced by d from the particle's, in the staged halo
     auto halo_ld = [&](int d1, int d2, int d3) {
-        const int r1 = (at.c[0] & 7) + d1 + G - LO, r2 = (at.c[1] & 7) + d2 + G - LO, r3 = (at.c[2] & 7) + d3 + G - LO + m.z0;
+        const int r1 = (at.c[0] & 7) + d1 + G - LO, r2 = (at.c[1] & 7) + d2 + G - LO + m.y0, r3 = (at.c[2] & 7) + d3 + G - LO + m.z0;
         if constexpr (SRC == SRC_SLABS) {   // the lane's slab and column
             using SG = SlabGeom<I, MODE>;
             const int x = r1 + m.x - SG::G - SG::X0;
             const int row = r3 * SG::H + r2;
-            return HaloLd<T, STORE, RW, NC, SG::SW, ZS * SG::H * SG::SW, 0>{
+            return HaloLd<T, STORE, RW, NC, YS * SG::SW, ZS * SG::H * SG::SW, 0>{
                 at.halo + (unsigned)(at.slab + x / SG::SW) % NS * SG::slot + (row * SG::SW + x % SG::SW) * 16};
         } else {
             using HG = HaloGeom<T, I, MODE, NC, RW>;
             const int e = r3 * HG::PL + r2 * HG::P + (r1 + m.x) + HG::XOFF;
-            return HaloLd<T, STORE, RW, NC, HG::P, ZS * HG::PL, HG::SC>{at.halo + e * (STORE == ST_F64 ? 8 : 4 * RW)};
+            return HaloLd<T, STORE, RW, NC, YS * HG::P, ZS * HG::PL, HG::SC>{at.halo + e * (STORE == ST_F64 ? 8 : 4 * RW)};
         }
     };
     auto node_of = [&](int c1, int c2, int c3) { return (int)padded_index(a.f.NP, c1 - LO, c2 - LO, c3 - LO); };
-    auto glob_ld = [&](int node) { return global_ld<T, I, STORE, RW, NC>(a.f, node, ch, m); };
+    auto glob_ld = [&](int node) { return global_ld<T, I, STORE, RW, NC, GL>(a.f, node, ch, m); };
     if constexpr (!two_stages<MODE>()) {
-        Weights<T, I, D> w;
+        Weights<T, I, D, GL> w;
         B.eval(t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, m, odd ? wb1 : wb0, w);
         T out[D ? 4 * NC : NC];
-        if constexpr (HALO) contract<T, I, NC, D>(halo_ld(0, 0, 0), w, out);
-        else contract<T, I, NC, D>(glob_ld(node_of(at.c[0], at.c[1], at.c[2])), w, out);
+        if constexpr (HALO) contract<T, I, NC, D, GL>(halo_ld(0, 0, 0), w, out);
+        else contract<T, I, NC, D, GL>(glob_ld(node_of(at.c[0], at.c[1], at.c[2])), w, out);
         if constexpr (MODE == MODE_INTERP_DERIV) {   // the derivatives only
             T der[3 * NC];
 #pragma unroll
@@ -606,15 +688,16 @@ __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Plac
         }
     } else {
         const T dtid = (T)(a.dt * a.g.inv_delta);
-        constexpr int HR = MODE == MODE_RK2 ? held_rows<T, I, SRC>() : 0;
+        constexpr int HR = MODE == MODE_RK2 ? held_rows<T, I, MODE, SRC>() : 0;
         constexpr int NOUT = D ? 4 * NC : NC;
         T f[HR > 0 ? HR : 1][LaneMap<I>::NZ][NC];
         T k1[NOUT], k2[NOUT];
         if constexpr (HALO)
-            interpolate_stage<T, I, DEG, NC, D, HR>(halo_ld(0, 0, 0), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, m, B, f, k1);
+            interpolate_stage<T, I, DEG, NC, D, HR, GL>(halo_ld(0, 0, 0), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, m, B, f, k1, lane);
         else
-            interpolate_stage<T, I, DEG, NC, D, HR>(glob_ld(node_of(at.c[0], at.c[1], at.c[2])), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, m, B, f, k1);
-        const GroupSums<T, NOUT> s1(k1, lane);
+            interpolate_stage<T, I, DEG, NC, D, HR, GL>(glob_ld(node_of(at.c[0], at.c[1], at.c[2])), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, m, B, f, k1, lane);
+        using Sums = std::conditional_t<GL == 16, HalfSums<T>, GroupSums<T, NOUT>>;
+        const Sums s1(k1, lane);
         const T u1[3] = {s1.template all<0>(lane), s1.template all<1>(lane), s1.template all<2>(lane)};
         s1.put(kb, MODE == MODE_RK2 ? 0 : 3, live);
         // stage-2 point, cell-relative: t* = t + dt k1 / delta
@@ -632,19 +715,19 @@ __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Plac
         const bool moved = (d[0] | d[1] | d[2]) != 0;
         const bool far = (unsigned)d[0] + 1u > 2u || (unsigned)d[1] + 1u > 2u || (unsigned)d[2] + 1u > 2u;
         auto wrap = [&](int ax) { return (int)(((unsigned)at.c[ax] + (unsigned)d[ax]) & (unsigned)a.g.mask); };
-        if (far && (lane & 7) == 0 && live) atomicOr(a.flags + FLAG_CFL, 1);
+        if (far && (lane & (GL - 1)) == 0 && live) atomicOr(a.flags + FLAG_CFL, 1);
         if constexpr (HALO) {
             if (!__any_sync(0xffffffffu, far)) {
-                interpolate_stage<T, I, DEG, NC, D, HR>(halo_ld(d[0], d[1], d[2]), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, m, B, f, k2);
+                interpolate_stage<T, I, DEG, NC, D, HR, GL>(halo_ld(d[0], d[1], d[2]), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, m, B, f, k2, lane);
             } else {   // rare: every group of the warp gathers from global memory (the same values)
-                interpolate_stage<T, I, DEG, NC, D, HR>(glob_ld(node_of(wrap(0), wrap(1), wrap(2))), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, true, m, B, f, k2);
+                interpolate_stage<T, I, DEG, NC, D, HR, GL>(glob_ld(node_of(wrap(0), wrap(1), wrap(2))), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, true, m, B, f, k2, lane);
             }
         } else {
             const int n2 = far ? node_of(wrap(0), wrap(1), wrap(2))
                                : node_of(at.c[0] + d[0], at.c[1] + d[1], at.c[2] + d[2]);
-            interpolate_stage<T, I, DEG, NC, D, HR>(glob_ld(n2), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, m, B, f, k2);
+            interpolate_stage<T, I, DEG, NC, D, HR, GL>(glob_ld(n2), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, m, B, f, k2, lane);
         }
-        const GroupSums<T, NOUT> s2(k2, lane);
+        const Sums s2(k2, lane);
         if constexpr (MODE == MODE_RK2) {
             s2.put(kb + 3, 0, live);
         } else {   // the Jacobians, t* and the cell of X*
@@ -803,14 +886,15 @@ template <typename T, int I, int DEG, int MODE, int NC, int STORE, int RW>
 __device__ __forceinline__ void run_direct(const BlockArgs& a, int64_t j0, int64_t j1, unsigned char* ws, int warp,
                                            int nw, int lane)
 {
-    const int g = lane >> 3;
-    const LaneMap<I> m(lane);
-    Basis<T, I, DEG, is_deriv<MODE>()> B;
+    constexpr int GL = group_lanes<T, I, MODE, SRC_GLOBAL>(), P = 32 / GL;   // P particles at once
+    const int g = lane / GL;
+    const LaneMap<I, GL> m(lane);
+    Basis<T, I, DEG, is_deriv<MODE>(), GL> B;
     B.init(table<T>(a), m);
     const WarpMem<T, MODE, NC> wm(ws, g);
     for (int64_t b0 = j0; b0 < j1; b0 += 32 * nw) {
-        const int64_t j = b0 + ((lane >> 2) * nw + warp) * 4 + (lane & 3);
-        const int left = (int)min(j1 - b0 - 4 * warp, (int64_t)32 * nw);   // particles from this warp's first on
+        const int64_t j = b0 + (lane / P * nw + warp) * P + lane % P;
+        const int left = (int)min(j1 - b0 - P * warp, (int64_t)32 * nw);   // particles from this warp's first on
         if (left <= 0) break;
         const bool valid = j < j1;
         const int64_t src = !valid ? 0 : (a.perm ? a.perm[j] : j);
@@ -819,13 +903,13 @@ __device__ __forceinline__ void run_direct(const BlockArgs& a, int64_t j0, int64
         fetch_state<T, MODE, NC>(a, MODE == MODE_ADJ ? id : src, valid, ws, lane);
         __syncwarp();
         for (int ch = 0; ch < (WarpPlan<T, MODE, NC>::HAS_X ? 1 : (a.f.C + NC - 1) / NC); ++ch) {
-            for (int it = 0; it < 8 && it * 4 * nw < left; ++it) {
-                const PRec<T> rec = wm.recs[4 * it + g];
+            for (int it = 0; it < GL && it * P * nw < left; ++it) {
+                const PRec<T> rec = wm.recs[P * it + g];
                 Place at{};
                 unpack_cell(cell_of(rec), at.c);
                 interpolate_group<T, I, DEG, MODE, NC, STORE, RW, SRC_GLOBAL>(
-                    a, at, ch, rec.t, it * 4 * nw + g < left, lane, B, m, wm.wb0, wm.wb1, it & 1,
-                    wm.kbuf + (4 * it + g) * WarpMem<T, MODE, NC>::WPl::KS);
+                    a, at, ch, rec.t, it * P * nw + g < left, lane, B, m, wm.wb0, wm.wb1, it & 1,
+                    wm.kbuf + (P * it + g) * WarpMem<T, MODE, NC>::WPl::KS);
             }
             __syncwarp();
             if constexpr (is_step<MODE>()) {
@@ -987,12 +1071,8 @@ __device__ __forceinline__ void run_direct_warp(const BlockArgs& a, int64_t j0, 
     }
 }
 
-// resident CTAs (of four warps) per SM the kernels are register-capped for: two
-// (255 registers) where 36 nodes are held, else four (128)
-template <typename T, int I, int MODE, int SRC>
-__host__ __device__ constexpr int min_ctas()
-{
-    return MODE == MODE_RK2 && held_rows<T, I, SRC>() > 4 ? 2 : 4;
-}
+// resident CTAs (of four warps) per SM the kernels are register-capped for
+// (128 registers)
+constexpr int CTAS_SM = 4;
 
 }  // namespace trk

@@ -161,7 +161,7 @@ struct tracker {
     int last_kernel = TRK_STEP_AUTO;  // kernel of the latest tracker_advance or tracker_interpolate
     int col_seg = 8;                  // column order: x3 slabs per segment (power of two)
     int dir_blk = BLK;                // direct path: edge of its cubic binning blocks (default shape only)
-    int dir_ppc = 256;                // direct path: particles per CTA
+    int dir_ppc = 256;                // direct path: launch shape (direct_shape)
     int64_t bin_cap = 0;              // entries of offsets / counts / cursor (largest geometry in use)
     int tune_source = TRK_TUNE_DEFAULT;   // how the latest call's parameters were chosen
     std::array<int, 5> last_tuning = {TRK_STEP_AUTO, BLK, 8, 0, 256};   // path, dir_blk, col_seg, tma, ppc of the latest call
@@ -495,8 +495,9 @@ int check_block_kernel_shape(const tracker* t)
     return TRK_OK;
 }
 
-// launch shape of the direct kernel for direct_particles = 64, 128, 256 (0: untimed)
-int direct_shape(int p) { return p == 256 ? PPC_WIDE : (p == 128 ? 256 : (p == 64 ? 64 : 0)); }
+// launch shape of the direct kernel for direct_particles = 64, 128, 256 (0: the
+// kernel's rule by size)
+int direct_shape(int p) { return p == 128 ? 256 : (p == 64 ? 64 : 0); }
 
 BlockArgs base_args(tracker* t)
 {
