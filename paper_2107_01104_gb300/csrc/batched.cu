@@ -1,6 +1,6 @@
 // Batched AB2 advection: many particle sets of uneven size and different
-// kernels (I = 4, 6, 8; value or value + gradient outputs) advanced by ONE
-// persistent launch per step.  CTAs take work items from a per-set atomic
+// kernels (I = 4, 6, 8; value or value + gradient outputs) advanced by one
+// persistent launch per step (dense sets: the slab pipeline).  CTAs take work items from a per-set atomic
 // counter, set after set: an item is a run of 128 grouped particles whose
 // stencils are gathered from the field through L1 (run_direct).  Large sets
 // come last in no particular order; the items are small, so the tail is
@@ -15,13 +15,14 @@ namespace {
 
 __host__ __device__ constexpr size_t batched_warp_bytes()
 {
-    return WarpPlan<float, MODE_AB2_D, 3>::total;   // the larger of the two modes
+    return std::max(WarpPlan<float, MODE_AB2_D, 3>::total, WarpPlan<float, MODE_AB2, 3>::total);
 }
 
 template <int I, int DEG>
 __device__ __forceinline__ void run_item(const BatchSet& S, int64_t j0, int64_t j1, unsigned char* ws, int warp, int lane)
 {
     if (S.deriv) run_direct<float, I, DEG, MODE_AB2_D, 3, ST_F32, 4>(S.a, j0, j1, ws, warp, NW, lane);
+    else if constexpr (I == 8) run_direct_warp<DEG, MODE_AB2, 3>(S.a, j0, j1, ws, warp, NW, lane);
     else run_direct<float, I, DEG, MODE_AB2, 3, ST_F32, 4>(S.a, j0, j1, ws, warp, NW, lane);
 }
 

@@ -7,6 +7,7 @@ namespace trk {
 cudaError_t launch_block_i8h(int mode, const BlockArgs& a, const void* tmap, int64_t nblocks, cudaStream_t st)
 {
     const CUtensorMap* m = static_cast<const CUtensorMap*>(tmap);
+    if (mode == MODE_AB2_D) return launch_slabs<8, 9, MODE_AB2_D, 3>(a, *m, st);   // (batched sets)
     return dispatch_mode<8, 9>(mode, a.f, GoBlock<8, 9>{a, m, nblocks, st});
 }
 

@@ -509,8 +509,9 @@ struct WarpPlan {
     static constexpr int WB = is_deriv<MODE>() ? 40 : 24;                                  // groups 8 banks apart
     static constexpr bool HAS_X = is_step<MODE>() || MODE == MODE_ADJ;
     static constexpr size_t x = align32(w + 2 * 4 * WB * sizeof(T));                       // [3][32] positions (steps), lambda
-    static constexpr size_t rhs = align32(x + (HAS_X ? 3 * 32 * sizeof(double) : 0));      // [9][32] AB history
-    static constexpr size_t total = align32(rhs + (is_ab<MODE>() ? 3 * AB_MAX_HIST * 32 * sizeof(float) : 0));
+    static constexpr size_t rhs = align32(x + (HAS_X ? 3 * 32 * sizeof(double) : 0));      // [3 HIST][32] AB history
+    static constexpr int HIST = MODE == MODE_AB2 ? AB_MAX_HIST : (MODE == MODE_AB2_D ? 1 : 0);   // entries (AB2_D: order 2)
+    static constexpr size_t total = align32(rhs + 3 * HIST * 32 * sizeof(float));
 };
 
 // ---------------------------------------------------------------------------

@@ -170,6 +170,8 @@ struct tracker {
     // one per stage-2 margin (interpolation and AB: 0, RK2: 1)
     CUtensorMap tmap[2];
     bool tmap_ok[2] = {false, false};
+    CUtensorMap set_tmap[3];          // slabs of I = 4, 6, 8 (batched sets)
+    bool set_tmap_ok[3] = {false, false, false};
     int halo_copy = TRK_HALO_AUTO;    // trk_halo_copy: how the block kernel stages its halo
     bool auto_tma = true;             // TRK_HALO_AUTO's current choice (tensor copies, where there is a map)
     uint32_t* d_counts = nullptr;     // [nblocks] block counts (counting-sort binning of the column path)
@@ -404,18 +406,18 @@ EncodeTiledFn encode_tiled()
 // reads zeros beyond C, which no output uses); node records
 // [chunks][NP][NP][4 NP] words, a slab of the halo per copy.  False where there is none (C = 1, float64 with C = 2: cp.async
 // staging).
-bool encode_field_map(const tracker* t, int margin, CUtensorMap* out)
+bool encode_field_map(const tracker* t, int I, int margin, CUtensorMap* out)
 {
     const EncodeTiledFn enc = encode_tiled();
     if (!enc || t->C < (t->storage == TRK_F64 ? 3 : 2) || !t->field) return false;
     const bool f64 = t->storage == TRK_F64;
-    const HaloBox b = halo_box(t->I, margin, f64);
+    const HaloBox b = halo_box(I, margin, f64);
     const cuuint64_t NP = (cuuint64_t)(t->N + 2 * PAD), unit = f64 ? 8 : 16;   // bytes per node and row element
     const cuuint64_t dims[4] = {f64 ? NP : 4 * NP, NP, NP, (cuuint64_t)(f64 ? t->C : record_chunks(t->C))};
     const cuuint64_t strides[3] = {NP * unit, NP * NP * unit, NP * NP * NP * unit};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     const cuuint32_t nc = f64 ? (cuuint32_t)(margin ? 3 : chunk_components(t->C)) : 1;
-    const cuuint32_t box[4] = {(cuuint32_t)(f64 ? b.P : 4 * slab_width(t->I)), (cuuint32_t)b.H, (cuuint32_t)b.H, nc};
+    const cuuint32_t box[4] = {(cuuint32_t)(f64 ? b.P : 4 * slab_width(I)), (cuuint32_t)b.H, (cuuint32_t)b.H, nc};
     return enc(out, f64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, t->field, dims,
                strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -423,7 +425,9 @@ bool encode_field_map(const tracker* t, int margin, CUtensorMap* out)
 
 void build_tmaps(tracker* t)
 {
-    for (int margin = 0; margin < 2; ++margin) t->tmap_ok[margin] = encode_field_map(t, margin, &t->tmap[margin]);
+    for (int margin = 0; margin < 2; ++margin) t->tmap_ok[margin] = encode_field_map(t, t->I, margin, &t->tmap[margin]);
+    for (int i = 0; i < 3; ++i)
+        t->set_tmap_ok[i] = t->storage != TRK_F64 && encode_field_map(t, 4 + 2 * i, 0, &t->set_tmap[i]);
 }
 
 cudaError_t launch_direct(tracker* t, int mode, const BlockArgs& a)
@@ -660,11 +664,21 @@ int step_path(const tracker* t, int64_t np)
 // I = 8 150 / 178 at 1/64, 264 / 219 at 1/32; gradients, I = 4 1051 / 1047 at 1/4,
 // I = 6 140 / 165 at 1/64, 228 / 190 at 1/32, I = 8 186 / 229 at 1/128, 287 / 256
 // at 1/64.
+bool sparse_for(const tracker* t, int64_t np, int I, int deriv)
+{
+    const double dens = (double)np / ((double)t->N * t->N * t->N);
+    return dens < (I == 4 ? 0.25 : (I == 6 ? 0.025 : (deriv ? 0.012 : 0.02)));
+}
 bool interp_direct(const tracker* t, int64_t np, int deriv)
 {
     if (t->storage == ST_F64 || !default_shape(t) || !t->tmap_ok[0] || t->halo_copy == TRK_HALO_ASYNC) return true;
-    const double dens = (double)np / ((double)t->N * t->N * t->N);
-    return dens < (t->I == 4 ? 0.25 : (t->I == 6 ? 0.025 : (deriv ? 0.012 : 0.02)));
+    return sparse_for(t, np, t->I, deriv);
+}
+
+bool overlap(const void* a, size_t na, const void* b, size_t nb)
+{
+    const uintptr_t x = (uintptr_t)a, y = (uintptr_t)b;
+    return x < y + nb && y < x + na;
 }
 
 // One RK2/ABk step of tracker_advance: re-bin, then the fused step kernel.
@@ -1191,7 +1205,9 @@ int tracker_interpolate(tracker* t, int64_t np, const double* pos, void* out, in
     const bool direct = t->step_kernel == TRK_STEP_DIRECT || (t->step_kernel == TRK_STEP_AUTO && interp_direct(t, np, deriv));
     if (!direct && (rc = check_block_kernel_shape(t))) return rc;
     if (np == 0) return TRK_OK;
-    const bool plain = ungrouped(np, direct ? TRK_STEP_DIRECT : TRK_STEP_BLOCK);
+    const int64_t out_values = (int64_t)t->C * (deriv ? 3 : 1) * np;
+    const bool plain = ungrouped(np, direct ? TRK_STEP_DIRECT : TRK_STEP_BLOCK) &&
+                       !overlap(pos, (size_t)np * 24, out, (size_t)out_values * 8);
     if (!plain && ((rc = ensure_sort(t, np)) || (rc = ensure_rec(t, np)) || (rc = bin_counting(t, np, pos, t->rec))))
         return rc;
     BlockArgs a = base_args(t);
@@ -1477,6 +1493,34 @@ static int bin_set(tracker* t, SetState& ss, const trk_set& S, bool first, bool 
     return TRK_OK;
 }
 
+// How a set of tracker_advance_batched steps: in the caller's order and arrays
+// (small sets, as in tracker_advance), or grouped, through the one persistent
+// launch of all such sets or, from the density on at which interpolation takes
+// it, through the slab pipeline in a launch of its own (256^3 float32, 2^21
+// particles, I = 6 with gradients: 438 us per step against 653).
+enum { SET_PLAIN, SET_GROUPED, SET_SLABS };
+static int set_route(const tracker* t, const trk_set& S, bool aliased)
+{
+    if (S.np < kUngroupedNp && !aliased) return SET_PLAIN;
+    if (!default_shape(t) || !t->set_tmap_ok[S.I / 2 - 2] || t->halo_copy == TRK_HALO_ASYNC ||
+        sparse_for(t, S.np, S.I, S.deriv))
+        return SET_GROUPED;
+    return SET_SLABS;
+}
+
+static cudaError_t launch_set_slabs(tracker* t, const BatchSet& B)
+{
+    ProfScope ps(t, PROF_STEP);
+    t->launches += 1;
+    const int mode = B.deriv ? MODE_AB2_D : MODE_AB2;
+    const void* m = &t->set_tmap[B.I / 2 - 2];
+    switch (B.I) {
+        case 4: return (B.deg_hi ? launch_block_i4h : launch_block_i4)(mode, B.a, m, t->nblocks, t->stream);
+        case 6: return (B.deg_hi ? launch_block_i6h : launch_block_i6)(mode, B.a, m, t->nblocks, t->stream);
+        default: return (B.deg_hi ? launch_block_i8h : launch_block_i8)(mode, B.a, m, t->nblocks, t->stream);
+    }
+}
+
 static int batched_launch(tracker* t, const BatchSet* d_desc, int nsets)
 {
     ProfScope ps(t, PROF_STEP);
@@ -1531,6 +1575,19 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
         }
         t->desc_cap = nsets;
     }
+    // small sets step in place on the caller's arrays, unless two sets share some of them
+    bool aliased = false;
+    for (int s = 0; s < nsets; ++s)
+        for (int r = 0; r < nsets; ++r)
+            aliased |= (r != s && overlap(sets[s].pos, (size_t)sets[s].np * 24, sets[r].pos, (size_t)sets[r].np * 24)) ||
+                       (r != s && overlap(sets[s].rhs, (size_t)sets[s].np * 12, sets[r].rhs, (size_t)sets[r].np * 12)) ||
+                       overlap(sets[s].pos, (size_t)sets[s].np * 24, sets[r].rhs, (size_t)sets[r].np * 12);
+    std::vector<int> route(nsets);
+    bool any_direct = false;
+    for (int s = 0; s < nsets; ++s) {
+        route[s] = set_route(t, sets[s], aliased);
+        any_direct |= sets[s].np > 0 && route[s] != SET_SLABS;
+    }
     // host-side descriptors: [0] first step (into buffer 1), [1] into buffer 0, [2] into buffer 1
     std::vector<BatchSet> h(3 * (size_t)nsets);
     const BlockArgs base = base_args(t);
@@ -1560,7 +1617,16 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
             B.a.id_in = B.a.id_out = ss.id_s[nxt];
             B.a.rhs_in = B.a.rhs_out = ss.rhs_s[nxt];
             B.a.history_valid = v == 0 ? history_valid : 1;
-            B.n_items = (int)((S.np + PB_HOST - 1) / PB_HOST);
+            if (route[s] == SET_PLAIN) {
+                B.a.rec_in = nullptr;
+                B.a.pos_in = B.a.pos_out = S.pos;
+                B.a.id_in = nullptr;
+                B.a.id_out = nullptr;
+                B.a.rhs_in = B.a.rhs_out = S.rhs;
+                B.a.key_out = nullptr;
+                B.a.counts = nullptr;
+            }
+            B.n_items = route[s] == SET_SLABS ? 0 : (int)((S.np + PB_HOST - 1) / PB_HOST);
             B.I = S.I;
             B.deg_hi = kTables[tabs[s]].deg > S.I - 1;
             B.deriv = S.deriv;
@@ -1570,7 +1636,7 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
     CUDA_TRY(cudaStreamSynchronize(t->stream));   // h may be released after this
     auto step = [&](int v) -> int {
         for (int s = 0; s < nsets; ++s) {
-            if (sets[s].np == 0) continue;
+            if (sets[s].np == 0 || route[s] == SET_PLAIN) continue;
             if (v == 0) {
                 int r = keys_set(t, t->sets[s], sets[s].np, sets[s].pos);
                 if (r) return r;
@@ -1578,7 +1644,13 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
             int r = bin_set(t, t->sets[s], sets[s], v == 0, v != 0 || history_valid, v == 1 ? 0 : 1);
             if (r) return r;
         }
-        return batched_launch(t, t->d_desc + (size_t)v * nsets, nsets);
+        if (any_direct) {
+            int r = batched_launch(t, t->d_desc + (size_t)v * nsets, nsets);
+            if (r) return r;
+        }
+        for (int s = 0; s < nsets; ++s)
+            if (sets[s].np > 0 && route[s] == SET_SLABS) CUDA_TRY(launch_set_slabs(t, h[(size_t)v * nsets + s]));
+        return TRK_OK;
     };
     if ((rc = step(0))) return rc;
     int cur = 1;
@@ -1587,7 +1659,7 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
         uint64_t key = mix(mix(mix(0, t->gen), (uint64_t)nsets), dbits(dt));
         for (int s = 0; s < nsets; ++s)
             key = mix(mix(mix(mix(mix(key, (uint64_t)sets[s].np), (uint64_t)sets[s].I), (uint64_t)tabs[s]),
-                          (uint64_t)sets[s].deriv),
+                          (uint64_t)(sets[s].deriv * 4 + route[s])),
                       (uint64_t)(uintptr_t)sets[s].out);
         // the state is in buffer 1 after the first step: into 0, then into 1
         rc = replay_graph(t, t->batch_graph, key, rest / 2, [&]() {
@@ -1603,7 +1675,7 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
     }
     ProfScope ps(t, PROF_OTHER);
     for (int s = 0; s < nsets; ++s) {
-        if (sets[s].np == 0) continue;
+        if (sets[s].np == 0 || route[s] == SET_PLAIN) continue;
         SetState& ss = t->sets[s];
         CUDA_TRY(launch_unpermute_pos(sets[s].np, ss.pos_s[cur], ss.id_s[cur], sets[s].pos, t->stream));
         CUDA_TRY(launch_unpermute_rhs(sets[s].np, ss.rhs_s[cur], ss.id_s[cur], sets[s].rhs, 3, t->stream));
