@@ -65,9 +65,10 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
     }
     // a.ppc: particles per CTA (every shape gives the same results); 0, by size (us per
     // step, float32 unless noted):
-    //  - up to 64 each (I = 8, float64: 32), one wave: 128^3 float64 I = 6, 4e4 tracers,
-    //    RK2: 199 with 32, 222 with 64, 338 with 256; 64^3, I = 4, 3.5e4: 12 with 64, 16
-    //    with 32, 28 in CTAs of 1024.
+    //  - float64, bound by its pipe: an even share per resident CTA, so that every SM has
+    //    its warps to the end (128^3, I = 6, 2e5 tracers, RK2: 712, 795 with 60 each).
+    //  - up to 64 each (I = 8: 32), the same (64^3, I = 4, 3.5e4: 12 with 64, 16 with 32,
+    //    28 in CTAs of 1024).
     //  - then an eighth of an even share per resident CTA, so that the last wave is short,
     //    up to 256, which keeps a CTA's stencils close together (256^3, I = 4, AB2, 2^21: 235
     //    with 256, 356 with 64).
@@ -80,10 +81,11 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
     if (a.ppc == 0) {
         constexpr bool split = group_lanes<T, I, MODE, SRC_GLOBAL>() == 16, f32 = sizeof(T) == 4;
         const int64_t even = (a.np + (int64_t)nsm * ctas_sm - 1) / ((int64_t)nsm * ctas_sm);
-        const int64_t n = a.f.NP - 2 * PAD, cells = n * n * n, one_wave = f32 && I < 8 ? 64 : 32;
-        const int64_t want = even <= one_wave ? even : std::max<int64_t>(one_wave, even / 8);
+        const int64_t n = a.f.NP - 2 * PAD, cells = n * n * n, one_wave = I < 8 ? 64 : 32;
+        const int64_t want = !f32 || even <= one_wave ? even : std::max<int64_t>(one_wave, even / 8);
         const bool small = cells * 4 * (int64_t)sizeof(T) > ((int64_t)1 << 30) || (split && 12 * a.np < cells);
-        a.ppc = (int)std::min<int64_t>(small ? 64 : 256, std::max<int64_t>(16, (want + 15) / 16 * 16));
+        const int64_t unit = std::max(16, NW * 32 / group_lanes<T, I, MODE, SRC_GLOBAL>());   // a round of the CTA
+        a.ppc = (int)std::min<int64_t>(!f32 ? 1 << 20 : (small ? 64 : 256) / unit * unit, (want + unit - 1) / unit * unit);
         if (f32 && I == 8 && a.np >= 64 * 16 * (int64_t)nsm && 34 * a.np >= cells) a.ppc = PPC_WIDE;
     }
     if (a.ppc == PPC_WIDE) {

@@ -107,11 +107,12 @@ __device__ __forceinline__ void bcast_load(const T* p, T (&w)[n])
 // Lane map and weights of a group of eight lanes
 // ---------------------------------------------------------------------------
 // Sixteen lanes (RK2, I = 6 float32): the eight of a half h own the x columns
-// of the rows y = h, h + 2, h + 4.
+// of the rows y = h, h + 2, h + 4.  Six lanes (steps, I = 6 float64): five groups
+// and two lanes that repeat lanes 24 and 25.
 template <int I, int GL = 8>
 struct LaneMap {
-    static_assert(GL == 8 || (GL == 16 && I == 6), "sixteen lanes: I = 6");
-    static constexpr int YS = GL / 8;           // rows along y per lane: y0, y0 + YS, ...
+    static_assert(GL == 8 || I == 6, "six or sixteen lanes: I = 6");
+    static constexpr int YS = GL == 16 ? 2 : 1; // rows along y per lane: y0, y0 + YS, ...
     static constexpr int NY = I / YS;
     static constexpr int NZ = I == 4 ? 2 : I;   // planes along z per lane: z0, z0 + ZS, ...
     static constexpr int ZS = I == 4 ? 2 : 1;
@@ -119,11 +120,11 @@ struct LaneMap {
     bool act;                                   // false: a repeated column (zero weight)
     __device__ __forceinline__ explicit LaneMap(int lane)
     {
-        const int u = lane & 7;
+        const int u = GL == 6 ? lane % 6 : lane & 7;
         x = I == 8 ? u : (I == 6 ? (u < 6 ? u : u - 6) : (u & 3));
         y0 = GL == 16 ? (lane >> 3 & 1) : 0;
         z0 = I == 4 ? u >> 2 : 0;
-        act = I != 6 || u < 6;
+        act = GL == 6 || I != 6 || u < 6;
     }
 };
 
@@ -369,6 +370,39 @@ struct HalfSums {
     }
 };
 
+// the same for three values over a group of six, in the order GroupSums has for
+// I = 6, ((x0 + x4) + x2) + ((x1 + x5) + x3): lanes 2q and 2q + 1 add the even and
+// the odd columns of value q
+template <typename T>
+struct TrioSums {
+    T v;
+    int u, base;
+    __device__ __forceinline__ TrioSums(const T (&x)[3], int lane)
+    {
+        u = lane % 6;
+        base = lane - u;
+        const int q = u >> 1, b = u & 1;
+        auto value = [&](int i) { return i == 0 ? x[0] : (i == 1 ? x[1] : x[2]); };
+        const int n1 = q == 2 ? 0 : q + 1, n2 = q == 0 ? 2 : q - 1;   // q + 1, q + 2 mod 3
+        // column n1 of value q comes from the lane n1, to whom q is n2
+        const T own = value(q);
+        const T c1 = __shfl_sync(0xffffffffu, value(n2), base + 2 * n1 + b);
+        const T c2 = __shfl_sync(0xffffffffu, value(n1), base + 2 * n2 + b);
+        v = (q == 1 ? c1 : own) + (q == 2 ? c1 : c2);
+        v += q == 0 ? c1 : (q == 1 ? own : c2);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+    }
+    template <int i>
+    __device__ __forceinline__ T all(int) const
+    {
+        return __shfl_sync(0xffffffffu, v, base + 2 * i);
+    }
+    __device__ __forceinline__ void put(T* kb, int, bool live) const
+    {
+        if (live && (u & 1) == 0) kb[u >> 1] = v;
+    }
+};
+
 // i-th term of a sum over n nodes taken from the ends inwards (0, n-1, 1, ...):
 // the small outer terms first, so that they are rounded while the partial sum is small
 __host__ __device__ constexpr int inward(int i, int n) { return i % 2 == 0 ? i / 2 : n - 1 - i / 2; }
@@ -505,10 +539,11 @@ struct WarpPlan {
     static constexpr int KS = (result_count<MODE, NC>() + 3) / 4 * 4;                      // values per particle
     static constexpr size_t rec = 0;                                                       // [2][32] records
     static constexpr size_t k = align32(rec + 2 * 32 * 4 * sizeof(T));                     // [32][KS]
-    static constexpr size_t w = align32(k + 32 * KS * sizeof(T));                          // [2][4 groups][WB]
+    static constexpr size_t w = align32(k + 32 * KS * sizeof(T));                          // [2][NG groups][WB]
     static constexpr int WB = is_deriv<MODE>() ? 40 : 24;                                  // groups 8 banks apart
     static constexpr bool HAS_X = is_step<MODE>() || MODE == MODE_ADJ;
-    static constexpr size_t x = align32(w + 2 * 4 * WB * sizeof(T));                       // [3][32] positions (steps), lambda
+    static constexpr int NG = sizeof(T) == 8 ? 5 : 4;
+    static constexpr size_t x = align32(w + 2 * NG * WB * sizeof(T));                       // [3][32] positions (steps), lambda
     static constexpr size_t rhs = align32(x + (HAS_X ? 3 * 32 * sizeof(double) : 0));      // [3 HIST][32] AB history
     static constexpr int HIST = MODE == MODE_AB2 ? AB_MAX_HIST : (MODE == MODE_AB2_D ? 1 : 0);   // entries (AB2_D: order 2)
     static constexpr size_t total = align32(rhs + 3 * HIST * 32 * sizeof(float));
@@ -596,11 +631,15 @@ __device__ __forceinline__ void fetch_state(const BlockArgs& a, int64_t src, boo
 // memory eight lanes without held rows, which issue fewer instructions (1/8 per
 // cell: 633 against 710 with sixteen lanes; 1/16: 377, 400, 12 warps with held
 // rows 407).  I = 8 would take 256 registers (run_direct_warp holds them),
-// float64 twice these: none.
+// float64 twice these: none.  float64 I = 6 steps are bound by the float64 pipe,
+// which idle lanes hold as long as busy ones: six lanes per particle, five
+// particles per warp (128^3, 4e5 tracers, RK2: 1410 us per step; eight lanes, two
+// of them idle: 1770).
 template <typename T, int I, int MODE, int SRC>
 __host__ __device__ constexpr int group_lanes()
 {
-    return sizeof(T) == 4 && I == 6 && MODE == MODE_RK2 && SRC == SRC_GLOBAL ? 16 : 8;
+    if (I != 6 || SRC != SRC_GLOBAL) return 8;
+    return sizeof(T) == 8 ? (MODE == MODE_RK2 || MODE == MODE_AB2 ? 6 : 8) : (MODE == MODE_RK2 ? 16 : 8);
 }
 template <typename T, int I, int MODE, int SRC>
 __host__ __device__ constexpr int held_rows()
@@ -654,6 +693,8 @@ __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Plac
                                                   bool odd, T* kb)
 {
     constexpr int GL = group_lanes<T, I, MODE, SRC>(), YS = LaneMap<I, GL>::YS;
+    using Sums = std::conditional_t<GL == 16, HalfSums<T>,
+                                    std::conditional_t<GL == 6, TrioSums<T>, GroupSums<T, is_deriv<MODE>() ? 4 * NC : NC>>>;
     constexpr bool D = is_deriv<MODE>(), HALO = SRC != SRC_GLOBAL;
     constexpr int LO = I / 2 - 1, ZS = LaneMap<I>::ZS, G = LO + (two_stages<MODE>() ? 1 : 0);
     // the stencil of the cell displaced by d from the particle's, in the staged halo
@@ -685,7 +726,7 @@ __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Plac
             for (int i = 0; i < 3 * NC; ++i) der[i] = out[NC + i];
             GroupSums<T, 3 * NC>(der, lane).put(kb + NC, 0, live);
         } else {
-            GroupSums<T, D ? 4 * NC : NC>(out, lane).put(kb, 0, live);
+            Sums(out, lane).put(kb, 0, live);
         }
     } else {
         const T dtid = (T)(a.dt * a.g.inv_delta);
@@ -697,7 +738,6 @@ __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Plac
             interpolate_stage<T, I, DEG, NC, D, HR, GL>(halo_ld(0, 0, 0), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, m, B, f, k1, lane);
         else
             interpolate_stage<T, I, DEG, NC, D, HR, GL>(glob_ld(node_of(at.c[0], at.c[1], at.c[2])), t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, wb0, true, m, B, f, k1, lane);
-        using Sums = std::conditional_t<GL == 16, HalfSums<T>, GroupSums<T, NOUT>>;
         const Sums s1(k1, lane);
         const T u1[3] = {s1.template all<0>(lane), s1.template all<1>(lane), s1.template all<2>(lane)};
         s1.put(kb, MODE == MODE_RK2 ? 0 : 3, live);
@@ -716,7 +756,7 @@ __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Plac
         const bool moved = (d[0] | d[1] | d[2]) != 0;
         const bool far = (unsigned)d[0] + 1u > 2u || (unsigned)d[1] + 1u > 2u || (unsigned)d[2] + 1u > 2u;
         auto wrap = [&](int ax) { return (int)(((unsigned)at.c[ax] + (unsigned)d[ax]) & (unsigned)a.g.mask); };
-        if (far && (lane & (GL - 1)) == 0 && live) atomicOr(a.flags + FLAG_CFL, 1);
+        if (far && m.x == 0 && live) atomicOr(a.flags + FLAG_CFL, 1);
         if constexpr (HALO) {
             if (!__any_sync(0xffffffffu, far)) {
                 interpolate_stage<T, I, DEG, NC, D, HR, GL>(halo_ld(d[0], d[1], d[2]), ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wb1, moved, m, B, f, k2, lane);
@@ -873,7 +913,7 @@ struct WarpMem {
     T *kbuf, *wb0, *wb1;
     __device__ __forceinline__ WarpMem(unsigned char* ws, int g)
         : recs(reinterpret_cast<PRec<T>*>(ws + WPl::rec)), kbuf(reinterpret_cast<T*>(ws + WPl::k)),
-          wb0(reinterpret_cast<T*>(ws + WPl::w) + g * WPl::WB), wb1(wb0 + 4 * WPl::WB)
+          wb0(reinterpret_cast<T*>(ws + WPl::w) + g * WPl::WB), wb1(wb0 + WPl::NG * WPl::WB)
     {
     }
 };
@@ -887,29 +927,30 @@ template <typename T, int I, int DEG, int MODE, int NC, int STORE, int RW>
 __device__ __forceinline__ void run_direct(const BlockArgs& a, int64_t j0, int64_t j1, unsigned char* ws, int warp,
                                            int nw, int lane)
 {
-    constexpr int GL = group_lanes<T, I, MODE, SRC_GLOBAL>(), P = 32 / GL;   // P particles at once
-    const int g = lane / GL;
+    constexpr int GL = group_lanes<T, I, MODE, SRC_GLOBAL>(), P = 32 / GL;   // P particles at once,
+    constexpr int R = 32 / P, PB_W = P * R;                                // R rounds of them per batch
+    const int g = GL == 6 ? min(lane / 6, 4) : lane / GL;
     const LaneMap<I, GL> m(lane);
     Basis<T, I, DEG, is_deriv<MODE>(), GL> B;
     B.init(table<T>(a), m);
     const WarpMem<T, MODE, NC> wm(ws, g);
-    for (int64_t b0 = j0; b0 < j1; b0 += 32 * nw) {
+    for (int64_t b0 = j0; b0 < j1; b0 += PB_W * nw) {
         const int64_t j = b0 + (lane / P * nw + warp) * P + lane % P;
-        const int left = (int)min(j1 - b0 - P * warp, (int64_t)32 * nw);   // particles from this warp's first on
+        const int left = (int)min(j1 - b0 - P * warp, (int64_t)PB_W * nw);   // particles from this warp's first on
         if (left <= 0) break;
-        const bool valid = j < j1;
+        const bool valid = j < j1 && lane < PB_W;
         const int64_t src = !valid ? 0 : (a.perm ? a.perm[j] : j);
         const int32_t id = !valid ? 0 : (a.id_in ? a.id_in[src] : (int32_t)src);
         wm.recs[lane] = particle_record<T>(a, j, src, valid);
         fetch_state<T, MODE, NC>(a, MODE == MODE_ADJ ? id : src, valid, ws, lane);
         __syncwarp();
         for (int ch = 0; ch < (WarpPlan<T, MODE, NC>::HAS_X ? 1 : (a.f.C + NC - 1) / NC); ++ch) {
-            for (int it = 0; it < GL && it * P * nw < left; ++it) {
+            for (int it = 0; it < R && it * P * nw < left; ++it) {
                 const PRec<T> rec = wm.recs[P * it + g];
                 Place at{};
                 unpack_cell(cell_of(rec), at.c);
                 interpolate_group<T, I, DEG, MODE, NC, STORE, RW, SRC_GLOBAL>(
-                    a, at, ch, rec.t, it * P * nw + g < left, lane, B, m, wm.wb0, wm.wb1, it & 1,
+                    a, at, ch, rec.t, it * P * nw + g < left && lane < GL * P, lane, B, m, wm.wb0, wm.wb1, it & 1,
                     wm.kbuf + (P * it + g) * WarpMem<T, MODE, NC>::WPl::KS);
             }
             __syncwarp();
