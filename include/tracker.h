@@ -63,7 +63,7 @@ typedef enum { TRK_LAGRANGE = 0, TRK_SPLINE = 1 } trk_family;
 
 /* Field storage inside the tracker.  Weights and accumulation are float32
  * for F32 and BF16X2, float64 for F64.  BF16X2 keeps hi = RN_bf16(x) and
- * lo = RN_bf16(x - hi) as two planes (4 bytes per value, about 16
+ * lo = RN_bf16(x - hi) (as node records of their sum, about 16
  * significant bits). */
 typedef enum { TRK_F64 = 0, TRK_F32 = 1, TRK_BF16X2 = 2 } trk_storage;
 
@@ -181,9 +181,10 @@ int tracker_interpolate(tracker* t, int64_t np, const double* pos, void* out, in
  *                   filled are zero) and min(history_valid + steps, k-1)
  *                   of them are valid.  rhs may be NULL for RK2.
  * pos[3][np] is read and overwritten in the caller's order.  Particles are
- * re-binned after every step (the update/re-sort of Sec. 3.3.1); the steps
- * are replayed from a captured CUDA graph (Adams-Bashforth runs step by step
- * until its history is full).  A particle that moves more
+ * re-binned after every step (the update/re-sort of Sec. 3.3.1), and the steps
+ * replayed from a captured CUDA graph (Adams-Bashforth runs step by step
+ * until its history is full); sets below 32768 particles on the direct kernel
+ * step in the caller's order and arrays, one launch per step.  A particle that moves more
  * than one cell in one stage is still computed exactly (through a slower
  * path) and raises TRK_ECFL at the next tracker_sync.
  * Errors: TRK_EINVAL, TRK_ENOFIELD, TRK_ENOMEM. */
@@ -191,46 +192,41 @@ int tracker_advance(tracker* t, int64_t np, double* pos, float* rhs, double dt, 
                     int history_valid);
 
 /* Step kernel used by tracker_advance and tracker_interpolate (trk_step_kernel):
- *   TRK_STEP_COLUMN: a persistent kernel that walks column segments of cell
- *     blocks along x3 (the x3 slabs of Sec. 3.3.1): the field halo stays in a
- *     ring of x3 planes, so a slab brings in only the planes it does not
- *     share with the previous one, and the next slab's planes and particles
- *     are copied in while the current slab is interpolated.  Its re-binning
- *     is a counting sort: the update phase counts the new block keys, a scan
- *     gives the offsets, and a scatter moves the particle state into its
- *     blocks (the order inside a block is not reproducible; no result
- *     depends on it).  Available for TRK_F32 storage with I = 4 or 6 in the
- *     8 x 8 x 8 block shape.
- *   TRK_STEP_BLOCK: one thread block per cell block, reading the state
- *     through the sort permutation (all storages and kernels).
+ *   TRK_STEP_COLUMN: the slab pipeline (a persistent thread block per SM takes
+ *     a contiguous run of grouped particles and keeps the field around them in
+ *     shared memory as a ring of slabs along x1, brought in by tensor copies
+ *     while earlier slabs are interpolated; the slabs of Sec. 3.3.1), with the
+ *     rows of cell blocks stacked along x3 in segments of column_segment
+ *     blocks.  Re-binning is a counting sort: the update phase counts the new
+ *     block keys, a scan gives the offsets, and a scatter moves the particle
+ *     state into its blocks (the order inside a block is not reproducible; no
+ *     result depends on it).  Available for TRK_F32 storage with I = 4 or 6 in
+ *     the 8 x 8 x 8 block shape.
+ *   TRK_STEP_BLOCK: the slab pipeline with the blocks in x1, x2, x3 order
+ *     where tensor copies stage the field (tracker_set_halo_copy; float32 and
+ *     split-bf16 fields of at least two components); else one thread block per
+ *     cell block with the block's halo in shared memory (all storages and
+ *     kernels).
  *   TRK_STEP_DIRECT: for sparse particle sets (the paper's production runs
- *     carry ~1e-3 tracers per grid cell, Sec. 4): particles sorted by block
- *     as for BLOCK, 64 to 256 of them per thread block, each stencil gathered
- *     from the field in global memory, so no field sweep and no halo per
- *     cell block (all storages and kernels, any block shape; float32 fields
- *     and split-bf16 fields whose component count is a multiple of three are
- *     read from a node-major copy the tracker keeps, made on first use: 16
- *     bytes per node for three float32 components, one 16-byte record per
- *     node and chunk of three split-bf16 components (a split-bf16 field
- *     whose copy cannot be allocated is read from the field itself); where
- *     a three-component copy is at most four times the L2 size (or the byte
- *     count in the environment variable TRK_NM_TEXTURE_BYTES, 0 for never)
- *     it is read through a texture object: the same bits, on the texture
- *     data path instead of the load/store one, which the gathers of a copy
- *     that mostly hits in L2 otherwise saturate).  The stage-2
- *     point of RK2 is gathered wherever it lies; TRK_ECFL is raised when it
- *     is more than one cell away.
+ *     carry ~1e-3 tracers per grid cell, Sec. 4): particles grouped as for
+ *     BLOCK, each stencil gathered from the field in global memory through L1,
+ *     so no field sweep (all storages and kernels, any block shape).  The
+ *     stage-2 point of RK2 is gathered wherever it lies; TRK_ECFL is raised
+ *     when it is more than one cell away.
+ * float32 and split-bf16 fields are kept as node records, 16 bytes per node and
+ * chunk of up to four components (C = 1: 4 bytes), split-bf16 values as the
+ * float32 sum hi + lo; float64 fields component by component.
  *   TRK_STEP_AUTO (default): the tuner's choice (see tracker_set_tuning):
  *     on the first call of a workload with enough steps, every candidate
  *     kernel and launch shape is timed on real steps of the call and the
  *     fastest kept; otherwise DIRECT below 0.05 particles per grid cell
  *     (np < 0.05 N^3), else COLUMN where available; without a column kernel
  *     DIRECT below 0.25 per cell, else BLOCK (measured crossovers).
- *     tracker_interpolate uses DIRECT or BLOCK; between 0.01 and 0.25 per
- *     cell its first call per (np, C, deriv, out_dtype) runs the block kernel
- *     with each halo copy and the direct kernel (they write the same values)
- *     and keeps the fastest: which one wins depends on C (the direct kernel
- *     gathers every component of a node at once for C = 3).
+ *     Below 8192 particles (32768 without a column kernel): DIRECT.
+ *     tracker_interpolate uses DIRECT below a density (float32 and split-bf16:
+ *     0.25 per cell for I = 4, 0.025 for I = 6, 0.02 for I = 8, 0.012 for its
+ *     gradients; float64, C = 1 and other block shapes: at every density),
+ *     else BLOCK.
  * All kernels perform the same floating-point operations in the same
  * order, so their results are bit-identical.  TRK_STEP_COLUMN on a tracker
  * without a column kernel is TRK_EINVAL.  Errors: TRK_EINVAL. */
@@ -247,21 +243,15 @@ int tracker_step_kernel_for(const tracker* t, int64_t np);
 int tracker_last_step_kernel(const tracker* t);
 
 /* How the block kernel (TRK_STEP_BLOCK, and the block side of interpolation)
- * stages each cell block's field halo in shared memory (the slab ghost
- * layers of Sec. 3.3.1, per cell block):
- *   TRK_HALO_ASYNC: cp.async copies of single elements (float32, float64) or
- *     16-byte vector loads through registers (split bf16);
- *   TRK_HALO_TMA: one tensor copy (cp.async.bulk.tensor) per chunk of three
- *     components, issued by one thread and awaited on an mbarrier, into a
- *     box padded so that the stencil loads meet few shared-memory bank
- *     conflicts (float32 and float64 storage with at least three
- *     components; elsewhere the cp.async staging is used);
- *   TRK_HALO_AUTO (default): TRK_HALO_TMA where the field has a tensor map
- *     (faster where few particles share a halo: 0.338 vs 0.526 ms per RK2
- *     step at 256^3, I = 6, 1/64 particle per cell), unless the tuner (the
- *     first timed tracker_advance or tracker_interpolate call of a workload)
- *     measured the cp.async halo faster (e.g. 2.93 vs 3.20 ms at 1/2 per
- *     cell, where the smem reads dominate); else TRK_HALO_ASYNC.
+ * brings the field into shared memory (the slab ghost layers of Sec. 3.3.1):
+ *   TRK_HALO_ASYNC: one thread block per cell block, the block's halo by
+ *     cp.async copies of nodes;
+ *   TRK_HALO_TMA: tensor copies (cp.async.bulk.tensor) awaited on mbarriers:
+ *     float32 fields of at least three components in the slab pipeline,
+ *     float64 ones one halo per cell block; elsewhere cp.async;
+ *   TRK_HALO_AUTO (default): tensor copies where the field has a tensor map
+ *     (float64 with at least three components, records of at least two, split
+ *     bf16 included), else TRK_HALO_ASYNC.
  * Both give bit-identical results.  A tensor copy that does not complete
  * within its wait limit skips its block and makes tracker_sync return
  * TRK_ECUDA.  Errors: TRK_EINVAL. */
@@ -269,14 +259,13 @@ int tracker_set_halo_copy(tracker* t, int kind);
 
 /* Launch shape of the time-step path.  step_kernel: TRK_STEP_COLUMN, _BLOCK
  * or _DIRECT; direct_block: edge of the cubic cell blocks the direct kernel's
- * particles are binned by (a power of two <= N; with the default 8^3 block
+ * particles are grouped by (a power of two <= N; with the default 8^3 block
  * shape; it sets how compact each thread block's particles are);
- * column_segment: x3 slabs per work item of the column kernel (a power of
+ * column_segment: cell blocks along x3 that TRK_STEP_COLUMN stacks (a power of
  * two <= 64, at most N/8); halo_copy: the block kernel's TRK_HALO_ASYNC or
- * TRK_HALO_TMA; direct_particles: particles per thread block of the direct
- * kernel (64, 128 or 256; 0 in tracker_set_tuning means 256; untimed calls
- * use the largest that gives three thread blocks per SM).  source
- * (tracker_get_tuning only): how they were chosen. */
+ * TRK_HALO_TMA; direct_particles: launch shape of the direct kernel: 256 (and
+ * 0): by the size of the set, 128: thread blocks of 256 particles, 64: of 64.
+ * source (tracker_get_tuning only): how they were chosen. */
 typedef enum { TRK_TUNE_DEFAULT = 0, TRK_TUNE_TIMED = 1, TRK_TUNE_CACHED = 2, TRK_TUNE_FIXED = 3 } trk_tune_source;
 typedef struct {
     int step_kernel;
@@ -295,13 +284,11 @@ typedef struct {
  * events; the host waits once; skipped while the stream is being captured)
  * and keeps the fastest for the rest of the call and for later calls
  * (TRK_TUNE_TIMED, then TRK_TUNE_CACHED).  Candidates: from 0.01 particles
- * per cell on, the column kernel with segments 8 and 16; the block kernel
- * with tensor-copy and with cp.async halos from 0.1 per cell on (from 0.01
- * without a column kernel); the direct kernel with block edges 8 and 16 and
- * 256 or 128 particles per thread block, up to one particle per cell.
+ * per cell on, TRK_STEP_COLUMN with segments of 1 and 8 (without a column
+ * kernel TRK_STEP_BLOCK with tensor copies); up to one particle per cell, the
+ * direct kernel with block edges 8 and 16 and launch shapes 256 and 128.
  * Other calls use the density rule of tracker_set_step_kernel with the
- * default shape, the direct kernel with the largest of 256, 128, 64
- * particles per thread block that gives three per SM (TRK_TUNE_DEFAULT).  Every
+ * default shape (TRK_TUNE_DEFAULT).  Every
  * candidate gives bit-identical steps.  When the environment variable
  * TRK_TUNE_CACHE names a file, decisions are appended to it (one line per
  * workload) and trackers created later read it.
@@ -317,14 +304,15 @@ int tracker_get_tuning(const tracker* t, trk_tuning* out);
  * for interpolation and AB steps (mode 0) or RK2 steps (mode 1). */
 int tracker_halo_copy(const tracker* t, int mode);
 
-/* 1 if the direct kernel reads the node-major copy of the current field
- * through a texture object, 0 if by plain loads or if no copy has been made
- * yet (the copy is made by the first direct launch after tracker_set_field);
- * negative status on error. */
+/* 1 if the three-component float32 or split-bf16 field's records are at most
+ * four times the L2 size (or the byte count in the environment variable
+ * TRK_NM_TEXTURE_BYTES, 0 for never), the range in which gathers mostly hit in
+ * L2; else 0.  Every load is a plain one: texture fetches of a row of records
+ * take 2.1 cycles against 1.2.  Negative status on error. */
 int tracker_field_texture(const tracker* t);
 
 /* ---------------------------------------------------------------------- */
-/* Batched advection: many particle sets, one persistent launch per step  */
+/* Batched advection: many particle sets advanced together                */
 /* ---------------------------------------------------------------------- */
 
 typedef struct {
@@ -342,8 +330,12 @@ typedef struct {
  * any other value = the one AB2 entry is valid; applied to all sets) in the
  * tracker's 3-component
  * field.  Each step is one persistent kernel over a shared work list of
- * (set, block) items, so sets of very different sizes and kernels share
- * one launch; the step sequence is captured in a CUDA graph and replayed.
+ * (set, run of 128 particles) items, so sets of very different sizes and
+ * kernels share one launch; sets as dense as those tracker_interpolate takes
+ * through the block kernel have a launch of the slab pipeline each.  Sets of
+ * 32768 particles and more are re-binned every step, smaller ones step in the
+ * caller's arrays (unless arrays of two sets overlap).  The step sequence is
+ * captured in a CUDA graph and replayed.
  * Errors: TRK_EINVAL, TRK_ENOFIELD, TRK_ENOMEM. */
 int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double dt, int steps,
                             int history_valid);
@@ -407,20 +399,21 @@ int tracker_state_read(const char* path, int64_t np, double* pos, float* rhs, tr
  *   lambda <- lambda + lambda* + J(X)^T mu.
  * Two modes (same values up to rounding order of the field gradient):
  *   halo mode (TRK_STEP_AUTO at 1/8 tracer per grid cell or more, or
- *     TRK_STEP_BLOCK / TRK_STEP_COLUMN): one thread block per cell block
- *     with the field halo in shared memory; the field gradient is
- *     accumulated per cell block (atomic adds into the block's slab of
- *     scratch) and then summed per grid node over the blocks whose halo
- *     holds it, in a fixed block order.  The scratch holds
+ *     TRK_STEP_BLOCK / TRK_STEP_COLUMN): the Jacobians through the slab
+ *     pipeline (float64: one thread block per cell block with its halo); the
+ *     field gradient is accumulated per cell block, into the block's slab of
+ *     scratch (float32 fields: sums of a block's particles held in registers;
+ *     float64: atomic adds), and then summed per grid node over the blocks
+ *     whose halo holds it, in a fixed block order.  The scratch holds
  *     nblocks * 3 * (I + 9)^3 values (float32, float64 for TRK_F64 storage;
  *     1.3 GB at N = 256, I = 6); when this exceeds the byte count in the
  *     environment variable TRK_ADJ_SCRATCH_BYTES (default 8 GiB) or cannot
- *     be allocated, each block accumulates in shared memory and adds its
- *     partial sums with float64 atomics instead.
+ *     be allocated, the partial sums are added to grad_field with float64
+ *     atomics instead.
  *   direct mode (TRK_STEP_AUTO below 1/8 tracer per cell, or
- *     TRK_STEP_DIRECT): no halos; 128 sorted particles per thread block,
- *     stencils gathered from the field in global memory, and each stencil
- *     node's contribution added to grad_field with a float64 atomic add.
+ *     TRK_STEP_DIRECT): stencils gathered from the field in global memory, and
+ *     each stencil node's contribution added to grad_field with a float64
+ *     atomic add.
  *     The position gradient is bit-identical to the halo mode's.
  * Errors: TRK_EINVAL, TRK_ENOFIELD, TRK_ENOMEM. */
 int tracker_adjoint(tracker* t, int64_t np, const double* pos0, const double* lambdaT, double dt, int steps,
