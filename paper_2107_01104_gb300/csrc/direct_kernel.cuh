@@ -73,9 +73,10 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
     //    up to 256, which keeps a CTA's stencils close together (256^3, I = 4, AB2, 2^21: 235
     //    with 256, 356 with 64).
     //  - at most 64 on a field of many times the L2, whose concurrent CTAs then share what
-    //    they pull into it (512^3, I = 8, 9e5, AB2: 573 with 64, 702 with 256), and for RK2's
-    //    sixteen lanes on sets below 1/12 per cell (256^3, 8e5: 314 with 64, 330 with 1024).
-    //  - I = 8 on denser sets: CTAs that fill an SM, whose warps share one neighbourhood of
+    //    they pull into it (512^3, I = 8, 9e5, AB2: 573 with 64, 702 with 256), for I = 8
+    //    (256^3, 5e5, RK2: 322, 352 with 256) and for RK2's sixteen lanes on sets below
+    //    1/12 per cell (256^3, 8e5: 314 with 64, 330 with 1024).
+    //  - I = 8 from 1/20 per cell on: CTAs that fill an SM, whose warps share one neighbourhood of
     //    the field in L1 (PPC_WIDE; 256^3, 2^21, RK2: 1126, 1229 with 256, 1258 with 64).
     int nw = NW;
     if (a.ppc == 0) {
@@ -83,10 +84,10 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
         const int64_t even = (a.np + (int64_t)nsm * ctas_sm - 1) / ((int64_t)nsm * ctas_sm);
         const int64_t n = a.f.NP - 2 * PAD, cells = n * n * n, one_wave = I < 8 ? 64 : 32;
         const int64_t want = !f32 || even <= one_wave ? even : std::max<int64_t>(one_wave, even / 8);
-        const bool small = cells * 4 * (int64_t)sizeof(T) > ((int64_t)1 << 30) || (split && 12 * a.np < cells);
+        const bool small = cells * 4 * (int64_t)sizeof(T) > ((int64_t)1 << 30) || I == 8 || (split && 12 * a.np < cells);
         const int64_t unit = std::max(16, NW * 32 / group_lanes<T, I, MODE, SRC_GLOBAL>());   // a round of the CTA
         a.ppc = (int)std::min<int64_t>(!f32 ? 1 << 20 : (small ? 64 : 256) / unit * unit, (want + unit - 1) / unit * unit);
-        if (f32 && I == 8 && a.np >= 64 * 16 * (int64_t)nsm && 34 * a.np >= cells) a.ppc = PPC_WIDE;
+        if (f32 && I == 8 && a.np >= 64 * 16 * (int64_t)nsm && 20 * a.np >= cells) a.ppc = PPC_WIDE;
     }
     if (a.ppc == PPC_WIDE) {
         nw = maxw;

@@ -407,8 +407,43 @@ struct TrioSums {
 // the small outer terms first, so that they are rounded while the partial sum is small
 __host__ __device__ constexpr int inward(int i, int n) { return i % 2 == 0 ? i / 2 : n - 1 - i / 2; }
 
+// a = w v (first) or a + w v, component-wise.  PACK: two float32 components per
+// instruction, rounded as single ones are; for gradients of I = 4, 6 from slabs
+// and for a warp per particle, whose registers hold the pairs (256^3, 2^21
+// particles, gradients: I = 6 431 -> 419 us; I = 8 RK2, 2^20: 592 -> 582; values
+// from slabs spill: I = 6 RK2 379 -> 462).
+template <bool PACK, int NC>
+__device__ __forceinline__ void axpy(bool first, float w, const float (&v)[NC], float (&a)[NC])
+{
+    if constexpr (PACK) {
+#pragma unroll
+        for (int k = 0; k + 1 < NC; k += 2) {
+            if (first)
+                asm("{.reg .b64 p, q, r;\n mov.b64 p, {%2, %2};\n mov.b64 q, {%3, %4};\n mul.rn.f32x2 r, p, q;\n"
+                    "mov.b64 {%0, %1}, r;}"
+                    : "=f"(a[k]), "=f"(a[k + 1])
+                    : "f"(w), "f"(v[k]), "f"(v[k + 1]));
+            else
+                asm("{.reg .b64 p, q, r;\n mov.b64 p, {%2, %2};\n mov.b64 q, {%3, %4};\n mov.b64 r, {%0, %1};\n"
+                    "fma.rn.f32x2 r, p, q, r;\n mov.b64 {%0, %1}, r;}"
+                    : "+f"(a[k]), "+f"(a[k + 1])
+                    : "f"(w), "f"(v[k]), "f"(v[k + 1]));
+        }
+        if constexpr (NC % 2) a[NC - 1] = first ? w * v[NC - 1] : fmaf(w, v[NC - 1], a[NC - 1]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) a[k] = first ? w * v[k] : fmaf(w, v[k], a[k]);
+    }
+}
+template <bool, int NC>
+__device__ __forceinline__ void axpy(bool first, double w, const double (&v)[NC], double (&a)[NC])
+{
+#pragma unroll
+    for (int k = 0; k < NC; ++k) a[k] = first ? w * v[k] : fma(w, v[k], a[k]);
+}
+
 // z sums of one row: pv (and pd with the derivative weights)
-template <typename T, int I, int NC, bool D, int GL, class LD>
+template <typename T, int I, int NC, bool D, int GL, bool PACK, class LD>
 __device__ __forceinline__ void row_sums(const LD& ld, int r, const Weights<T, I, D, GL>& w, T (&pv)[NC], T (&pd)[NC])
 {
     constexpr int NZ = LaneMap<I>::NZ;
@@ -417,11 +452,8 @@ __device__ __forceinline__ void row_sums(const LD& ld, int r, const Weights<T, I
         const int z = inward(zz, NZ);
         T v[NC];
         ld(r, z, v);
-#pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            pv[k] = zz == 0 ? w.w3[z] * v[k] : fma(w.w3[z], v[k], pv[k]);
-            if constexpr (D) pd[k] = zz == 0 ? w.dw3[z] * v[k] : fma(w.dw3[z], v[k], pd[k]);
-        }
+        axpy<PACK, NC>(zz == 0, w.w3[z], v, pv);
+        if constexpr (D) axpy<PACK, NC>(zz == 0, w.dw3[z], v, pd);
     }
 }
 
@@ -430,7 +462,7 @@ __device__ __forceinline__ void row_sums(const LD& ld, int r, const Weights<T, I
 // order a whole warp on one particle sums them in (run_direct_warp): parts
 // {0, 4}, {1, 5}, {6, 2}, {7, 3}, then (p0 + p2) + (p1 + p3); of I = 6 in the
 // order of sixteen lanes: rows 0, 4, 2 plus rows 1, 5, 3.
-template <typename T, int I, int NC, bool D, int GL, class LD>
+template <typename T, int I, int NC, bool D, int GL, bool PACK, class LD>
 __device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D, GL>& w, T (&out)[D ? 4 * NC : NC])
 {
     constexpr int NY = LaneMap<I, GL>::NY;
@@ -442,9 +474,8 @@ __device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D, GL
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
                 const int r = GL == 16 ? inward(q, 3) : h + 2 * inward(q, 3);
-                row_sums<T, I, NC, D, GL>(ld, r, w, pv, pd);
-#pragma unroll
-                for (int k = 0; k < NC; ++k) half[k] = q == 0 ? w.w2[r] * pv[k] : fma(w.w2[r], pv[k], half[k]);
+                row_sums<T, I, NC, D, GL, PACK>(ld, r, w, pv, pd);
+                axpy<PACK, NC>(q == 0, w.w2[r], pv, half);
             }
 #pragma unroll
             for (int k = 0; k < NC; ++k) a[k] = h ? a[k] + half[k] : half[k];
@@ -456,10 +487,10 @@ __device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D, GL
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int p = q + 2 * h, r0 = h ? p + 4 : p, r1 = h ? p : p + 4;
-                row_sums<T, I, NC, D, GL>(ld, r0, w, pv, pd);
+                row_sums<T, I, NC, D, GL, PACK>(ld, r0, w, pv, pd);
 #pragma unroll
                 for (int k = 0; k < NC; ++k) part[k] = w.w2[r0] * pv[k];
-                row_sums<T, I, NC, D, GL>(ld, r1, w, pv, pd);
+                row_sums<T, I, NC, D, GL, PACK>(ld, r1, w, pv, pd);
 #pragma unroll
                 for (int k = 0; k < NC; ++k) {
                     part[k] = fma(w.w2[r1], pv[k], part[k]);
@@ -471,14 +502,11 @@ __device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D, GL
 #pragma unroll
         for (int rr = 0; rr < NY; ++rr) {
             const int r = inward(rr, NY);
-            row_sums<T, I, NC, D, GL>(ld, r, w, pv, pd);
-#pragma unroll
-            for (int k = 0; k < NC; ++k) {
-                a[k] = rr == 0 ? w.w2[r] * pv[k] : fma(w.w2[r], pv[k], a[k]);
-                if constexpr (D) {
-                    b[k] = rr == 0 ? w.dw2[r] * pv[k] : fma(w.dw2[r], pv[k], b[k]);
-                    c[k] = rr == 0 ? w.w2[r] * pd[k] : fma(w.w2[r], pd[k], c[k]);
-                }
+            row_sums<T, I, NC, D, GL, PACK>(ld, r, w, pv, pd);
+            axpy<PACK, NC>(rr == 0, w.w2[r], pv, a);
+            if constexpr (D) {
+                axpy<PACK, NC>(rr == 0, w.dw2[r], pv, b);
+                axpy<PACK, NC>(rr == 0, w.w2[r], pd, c);
             }
         }
     }
@@ -672,10 +700,10 @@ __device__ __forceinline__ void interpolate_stage(const LD& ld, T s1, T s2, T s3
         if (fresh) load_rows<T, I, NC, HR>(ld, f);
         __syncwarp();
         B.eval(s1, s2, s3, m, wb, w);
-        contract<T, I, NC, D, GL>(HeldLd<T, I, NC, HR, LD>{f, ld}, w, k);
+        contract<T, I, NC, D, GL, false>(HeldLd<T, I, NC, HR, LD>{f, ld}, w, k);
     } else {
         B.eval(s1, s2, s3, m, wb, w);
-        contract<T, I, NC, D, GL>(ld, w, k);
+        contract<T, I, NC, D, GL, false>(ld, w, k);
     }
     if constexpr (GL == 16) join_halves(k, w.w1, lane);
 }
@@ -717,9 +745,10 @@ __device__ __forceinline__ void interpolate_group(const BlockArgs& a, const Plac
     if constexpr (!two_stages<MODE>()) {
         Weights<T, I, D, GL> w;
         B.eval(t[0] - (T)0.5, t[1] - (T)0.5, t[2] - (T)0.5, m, odd ? wb1 : wb0, w);
+        constexpr bool PACK = D && I <= 6 && SRC == SRC_SLABS;
         T out[D ? 4 * NC : NC];
-        if constexpr (HALO) contract<T, I, NC, D, GL>(halo_ld(0, 0, 0), w, out);
-        else contract<T, I, NC, D, GL>(glob_ld(node_of(at.c[0], at.c[1], at.c[2])), w, out);
+        if constexpr (HALO) contract<T, I, NC, D, GL, PACK>(halo_ld(0, 0, 0), w, out);
+        else contract<T, I, NC, D, GL, PACK>(glob_ld(node_of(at.c[0], at.c[1], at.c[2])), w, out);
         if constexpr (MODE == MODE_INTERP_DERIV) {   // the derivatives only
             T der[3 * NC];
 #pragma unroll
@@ -1002,20 +1031,16 @@ __device__ __forceinline__ float warp_contract(const float (&f)[2][8][NC], const
     float w3[8];
     bcast_load(wb + 16, w3);
     const float w1 = wb[x], w2[2] = {wb[8 + j], wb[12 + j]};
-    float p[4] = {0.f, 0.f, 0.f, 0.f};
+    float p[4] = {0.f, 0.f, 0.f, 0.f}, pv[2][NC];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int zz = 0; zz < 8; ++zz) axpy<true, NC>(zz == 0, w3[inward(zz, 8)], f[h][inward(zz, 8)], pv[h]);
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
-        float pv[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int zz = 0; zz < 8; ++zz) {
-                const int z = inward(zz, 8);
-                pv[h] = zz == 0 ? w3[z] * f[h][z][k] : fmaf(w3[z], f[h][z][k], pv[h]);
-            }
         // rows in contract's order: j, j + 4 for j < 2, else j + 4, j
         const bool up = j < 2;
-        p[k] = fmaf(up ? w2[1] : w2[0], up ? pv[1] : pv[0], (up ? w2[0] : w2[1]) * (up ? pv[0] : pv[1]));
+        p[k] = fmaf(up ? w2[1] : w2[0], up ? pv[1][k] : pv[0][k], (up ? w2[0] : w2[1]) * (up ? pv[0][k] : pv[1][k]));
     }
     const bool b4 = lane & 16, b3 = lane & 8;
     float q0 = (b4 ? p[2] : p[0]) + __shfl_xor_sync(0xffffffffu, b4 ? p[0] : p[2], 16);
