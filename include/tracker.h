@@ -398,7 +398,8 @@ int tracker_state_read(const char* path, int64_t np, double* pos, float* rhs, tr
  *   grad_field += W(X)^T mu + W(X*)^T (dt/2 lambda),
  *   lambda <- lambda + lambda* + J(X)^T mu.
  * Two modes (same values up to rounding order of the field gradient):
- *   halo mode (TRK_STEP_AUTO at 1/8 tracer per grid cell or more, or
+ *   halo mode (TRK_STEP_AUTO at 1/8 tracer per grid cell or more,
+ *     float32 and split-bf16 fields with I = 6 at 0.045; or
  *     TRK_STEP_BLOCK / TRK_STEP_COLUMN): the Jacobians through the slab
  *     pipeline (float64: one thread block per cell block with its halo); the
  *     field gradient is accumulated per cell block, into the block's slab of
@@ -410,7 +411,7 @@ int tracker_state_read(const char* path, int64_t np, double* pos, float* rhs, tr
  *     environment variable TRK_ADJ_SCRATCH_BYTES (default 8 GiB) or cannot
  *     be allocated, the partial sums are added to grad_field with float64
  *     atomics instead.
- *   direct mode (TRK_STEP_AUTO below 1/8 tracer per cell, or
+ *   direct mode (TRK_STEP_AUTO below that, or
  *     TRK_STEP_DIRECT): stencils gathered from the field in global memory, and
  *     each stencil node's contribution added to grad_field with a float64
  *     atomic add.

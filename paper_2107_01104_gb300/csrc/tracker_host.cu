@@ -608,18 +608,15 @@ bool same_geom(const GridGeom& a, const GridGeom& b)
 }
 
 // Below this many particles per grid cell the automatic choice gathers every
-// stencil straight from global memory (direct path) instead of sweeping the
-// field, without timing: on GB300 (float32, spline I = 6) the direct step wins
-// there for RK2 and AB on every grid measured (256^3: RK2 0.381 vs 0.534 ms at
-// 1/24 per cell, AB2 0.287 vs 0.328 ms).  Above it the kernels are timed.
+// stencil from global memory (direct path) instead of sweeping the field,
+// without timing.  Direct against the slab pipeline, us per RK2 step, 256^3
+// float32, I = 6: 216 / 313 at 1/32 per cell, 314 / 351 at 0.048, 404 / 377 at
+// 1/16; I = 4 (direct_threshold) stays ahead up to 1/4.
 constexpr double kDirectDensity = 0.05;
 
-// Without a column kernel (float64 or split-bf16 storage, I = 8, other block
-// shapes) the choice is between the block and the direct kernel, whose
-// binnings differ, so it is a density threshold, measured on GB300 (256^3,
-// RK2, block vs direct ms per step): float32 I = 8 1.24 vs 0.73 at 1/16 per
-// cell, 2.61 vs 2.65 at 1/4; float64 7.12 vs 6.02 and 24.7 vs 23.9;
-// split-bf16 (node-major copy) 1.19 vs 0.59 and 2.45 vs 2.20.
+// Without the column order (float64 or split-bf16 storage, I = 8, other block
+// shapes): block against direct, us per RK2 step: float32 I = 8, 256^3, 1/8 per
+// cell: 1204 / 1103, 1/4 1959 / 2073; float64 I = 6, 128^3, 0.1 per cell 950 / 712, 1/2 4460 / 3450.
 double direct_threshold(const tracker* t)
 {
     if (!column_available(t)) return 0.25;
@@ -627,11 +624,15 @@ double direct_threshold(const tracker* t)
 }
 
 // Below this many particles per grid cell the adjoint runs without halos
-// (direct mode); above it one CTA per cell block stages the block's halo.
-// Measured on GB300 (256^3 float32, spline I = 6, 20 RK2 steps, direct vs
-// halo ms per call): 23 vs 72 at 1/64 per cell, 74 vs 100 at 1/16, 282 vs
-// 221 at 1/4.
-constexpr double kAdjDirectDensity = 0.125;
+// (direct mode).  Direct against halo mode, us per call of four RK2 steps, 256^3
+// float32: I = 4 3982 / 7246 at 1/16 per cell, 7379 / 10006 at 1/8; I = 6 6560 /
+// 8413 at 1/32 (128^3: 1038 / 1179), 12375 / 9947 at 1/16 (1878 / 1421); I = 8
+// 20063 / 31984 at 1/16, 38857 / 40754 at 1/8.  float64 (both modes bound by its
+// pipe): 1/8.
+double adj_direct_density(const tracker* t)
+{
+    return t->storage == TRK_F64 || t->I != 6 ? 0.125 : 0.045;
+}
 
 constexpr size_t kCacheMax = 256;   // remembered tuning decisions (the oldest is dropped)
 constexpr double kProbeMin = 0.01;  // particles per cell from which the column order is a candidate
@@ -644,7 +645,7 @@ constexpr int64_t kUngroupedNp = 32768;
 bool ungrouped(int64_t np, int path) { return path == TRK_STEP_DIRECT && np < kUngroupedNp; }
 
 // Below this many particles a step is latency, whatever the density: direct
-// gathers in one launch (float64 without a column kernel: up to the ungrouped limit).
+// gathers in one launch (without the column order: up to the ungrouped limit).
 constexpr int64_t kSmallNp = 8192;
 
 // The kernel tracker_advance (and, between BLOCK and DIRECT, tracker_interpolate)
@@ -685,9 +686,8 @@ bool overlap(const void* a, size_t na, const void* b, size_t nb)
 // Every path re-bins with the counting sort: block counts (from the previous
 // step's update phase, or from the initial keys), one scan giving the offsets
 // and cursors, one scatter of the particle state into its blocks.  Then the
-// column kernel, the block kernel (one CTA per cell block), or the direct
-// kernel (PB grouped particles per CTA, stencils gathered from global
-// memory) updates the grouped state in place and counts the new keys.
+// slab pipeline or the block kernel, or the direct kernel (stencils gathered
+// from global memory) updates the grouped state in place and counts the new keys.
 // first: read the caller's arrays (identity ids).  AB steps: order
 // k = ab_order, `hist` valid history entries for this step.
 int advance_step(tracker* t, int64_t np, int path, int mode, int ab_order, int hist, double dt, int cur, bool first,
@@ -726,8 +726,8 @@ int advance_step(tracker* t, int64_t np, int path, int mode, int ab_order, int h
 
 // ---------------------------------------------------------------------------
 // Tuner of the time-step path.  A candidate fixes the step kernel and its
-// launch shape: the column kernel's segment length (x3 slabs per work item),
-// the direct kernel's binning block edge, the block kernel's halo copy
+// launch shape: the column order's segment length (blocks stacked along x3),
+// the direct kernel's binning block edge and CTAs, the block kernel's halo copy
 // (cp.async or tensor copies).  On the first tracker_advance call of a
 // workload (grid, kernel, storage, SM count, density bucket, scheme) with
 // enough steps, every candidate runs kTuneStepsPerCand real steps of the call,
@@ -815,15 +815,11 @@ void load_tune_file(tracker* t)
     fclose(f);
 }
 
-// The candidates for np particles (measured on GB300, 256^3 float32, spline
-// I = 6, RK2 and AB2 from 1.5e-3 to 1/2 particle per cell: the winners were
-// always among these): the column kernel with segments of 8 and 16 slabs
-// from kProbeMin particles per cell on; the block kernel with both halo
-// copies (the tensor-copy box wins where few particles share a halo, the
-// bank-conflict-free cp.async layout where many do) from kBlockMin on, or from
-// kProbeMin on without a column kernel; the direct kernel with binning edges
-// 8 and 16 up to one particle per cell.  Other block shapes than the default
-// run only the direct kernel.
+// The candidates for np particles: the slab pipeline from kProbeMin particles
+// per cell on (column order with segments of 1 and 8 blocks where available),
+// the direct kernel with binning edges 8 and 16 and two launch shapes up to one
+// particle per cell.  Other block shapes than the default run only the direct
+// kernel.
 std::vector<Cand> tune_candidates(const tracker* t, int64_t np)
 {
     std::vector<Cand> c;
@@ -1701,7 +1697,7 @@ int tracker_adjoint(tracker* t, int64_t np, const double* pos0, const double* la
     // float64 atomic adds straight into grad_field)
     const bool adj_direct = t->step_kernel == TRK_STEP_DIRECT ||
                             (t->step_kernel == TRK_STEP_AUTO &&
-                             (double)np < kAdjDirectDensity * (double)t->N * t->N * t->N);
+                             (double)np < adj_direct_density(t) * (double)t->N * t->N * t->N);
     if (!adj_direct && (rc = check_block_kernel_shape(t))) return rc;
     if (np == 0) return TRK_OK;
     const size_t vec = (size_t)3 * np;                 // doubles per position / lambda array
