@@ -482,7 +482,7 @@ class Tracker:
         return r
 
     def field_texture(self):
-        """True if the direct kernel reads the node-major field copy through a texture object."""
+        """True if a three-component field's records are at most four times the L2 size."""
         r = int(load_library().tracker_field_texture(self.h))
         _check(min(r, 0))
         return bool(r)
