@@ -1571,13 +1571,17 @@ int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double d
         }
         t->desc_cap = nsets;
     }
-    // small sets step in place on the caller's arrays, unless two sets share some of them
+    // small sets step in place on the caller's arrays, unless some of these share memory
     bool aliased = false;
     for (int s = 0; s < nsets; ++s)
         for (int r = 0; r < nsets; ++r)
             aliased |= (r != s && overlap(sets[s].pos, (size_t)sets[s].np * 24, sets[r].pos, (size_t)sets[r].np * 24)) ||
                        (r != s && overlap(sets[s].rhs, (size_t)sets[s].np * 12, sets[r].rhs, (size_t)sets[r].np * 12)) ||
-                       overlap(sets[s].pos, (size_t)sets[s].np * 24, sets[r].rhs, (size_t)sets[r].np * 12);
+                       overlap(sets[s].pos, (size_t)sets[s].np * 24, sets[r].rhs, (size_t)sets[r].np * 12) ||
+                       (sets[s].out && (overlap(sets[s].out, (size_t)sets[s].np * (sets[s].deriv ? 36 : 12), sets[r].pos,
+                                                (size_t)sets[r].np * 24) ||
+                                        overlap(sets[s].out, (size_t)sets[s].np * (sets[s].deriv ? 36 : 12), sets[r].rhs,
+                                                (size_t)sets[r].np * 12)));
     std::vector<int> route(nsets);
     bool any_direct = false;
     for (int s = 0; s < nsets; ++s) {
