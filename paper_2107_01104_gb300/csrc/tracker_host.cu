@@ -1040,6 +1040,7 @@ int tracker_set_field(tracker* t, const void* src, int C, int src_dtype, int src
         dev_free(t->field);
         t->field = nullptr;
         t->C = 0;
+        t->gen += 1;                  // captured step graphs hold the field's address and its tensor maps
         if (dev_alloc(&t->field, stored) != cudaSuccess) {
             cudaGetLastError();
             return fail(TRK_ENOMEM, "cannot allocate field storage (%zu bytes)", stored);
