@@ -33,6 +33,7 @@
 #include <cuda.h>   // CUtensorMap (type only; the library does not link the driver API)
 
 #include "internal.cuh"
+#include "six_lanes.h"
 
 namespace trk {
 
@@ -108,7 +109,7 @@ __device__ __forceinline__ void bcast_load(const T* p, T (&w)[n])
 // ---------------------------------------------------------------------------
 // Sixteen lanes (RK2, I = 6 float32): the eight of a half h own the x columns
 // of the rows y = h, h + 2, h + 4.  Six lanes (steps, I = 6 float64): five groups
-// and two lanes that repeat lanes 24 and 25.
+// and two lanes that repeat lanes 24 and 25 (six_lanes.h).
 template <int I, int GL = 8>
 struct LaneMap {
     static_assert(GL == 8 || I == 6, "six or sixteen lanes: I = 6");
@@ -120,7 +121,7 @@ struct LaneMap {
     bool act;                                   // false: a repeated column (zero weight)
     __device__ __forceinline__ explicit LaneMap(int lane)
     {
-        const int u = GL == 6 ? lane % 6 : lane & 7;
+        const int u = GL == 6 ? SixLanes(lane).u : lane & 7;
         x = I == 8 ? u : (I == 6 ? (u < 6 ? u : u - 6) : (u & 3));
         y0 = GL == 16 ? (lane >> 3 & 1) : 0;
         z0 = I == 4 ? u >> 2 : 0;
@@ -375,19 +376,15 @@ struct HalfSums {
 // the odd columns of value q
 template <typename T>
 struct TrioSums {
+    SixLanes at;
     T v;
-    int u, base;
-    __device__ __forceinline__ TrioSums(const T (&x)[3], int lane)
+    __device__ __forceinline__ TrioSums(const T (&x)[3], int lane) : at(lane)
     {
-        u = lane % 6;
-        base = lane - u;
-        const int q = u >> 1, b = u & 1;
+        const int q = at.value();
         auto value = [&](int i) { return i == 0 ? x[0] : (i == 1 ? x[1] : x[2]); };
-        const int n1 = q == 2 ? 0 : q + 1, n2 = q == 0 ? 2 : q - 1;   // q + 1, q + 2 mod 3
-        // column n1 of value q comes from the lane n1, to whom q is n2
         const T own = value(q);
-        const T c1 = __shfl_sync(0xffffffffu, value(n2), base + 2 * n1 + b);
-        const T c2 = __shfl_sync(0xffffffffu, value(n1), base + 2 * n2 + b);
+        const T c1 = __shfl_sync(0xffffffffu, value(at.next(2)), at.partner(1));
+        const T c2 = __shfl_sync(0xffffffffu, value(at.next(1)), at.partner(2));
         v = (q == 1 ? c1 : own) + (q == 2 ? c1 : c2);
         v += q == 0 ? c1 : (q == 1 ? own : c2);
         v += __shfl_xor_sync(0xffffffffu, v, 1);
@@ -395,11 +392,11 @@ struct TrioSums {
     template <int i>
     __device__ __forceinline__ T all(int) const
     {
-        return __shfl_sync(0xffffffffu, v, base + 2 * i);
+        return __shfl_sync(0xffffffffu, v, at.holder(i));
     }
     __device__ __forceinline__ void put(T* kb, int, bool live) const
     {
-        if (live && (u & 1) == 0) kb[u >> 1] = v;
+        if (live && (at.u & 1) == 0) kb[at.value()] = v;
     }
 };
 
@@ -958,7 +955,7 @@ __device__ __forceinline__ void run_direct(const BlockArgs& a, int64_t j0, int64
 {
     constexpr int GL = group_lanes<T, I, MODE, SRC_GLOBAL>(), P = 32 / GL;   // P particles at once,
     constexpr int R = 32 / P, PB_W = P * R;                                // R rounds of them per batch
-    const int g = GL == 6 ? min(lane / 6, 4) : lane / GL;
+    const int g = GL == 6 ? SixLanes(lane).group : lane / GL;
     const LaneMap<I, GL> m(lane);
     Basis<T, I, DEG, is_deriv<MODE>(), GL> B;
     B.init(table<T>(a), m);
