@@ -102,7 +102,11 @@ int tracker_set_stream(tracker* t, void* stream);
 
 /* Wait for the tracker's stream, then read and clear the device flags:
  * returns TRK_ENONFINITE or TRK_ECFL if a kernel raised one since the
- * last sync, else TRK_OK (or TRK_ECUDA). */
+ * last sync, else TRK_OK (or TRK_ECUDA).  TRK_ECUDA with "a tensor copy of
+ * the field did not complete" means that a wait inside a kernel ran out (after
+ * 2^22 polls, or the environment variable TRK_WAIT_LIMIT at creation, if that
+ * is less): the particles that needed the copy stayed as they were in that
+ * step (position, history, lambda; no outputs were written), the others did not. */
 int tracker_sync(tracker* t);
 
 /* ---------------------------------------------------------------------- */
@@ -253,8 +257,8 @@ int tracker_last_step_kernel(const tracker* t);
  *     (float64 with at least three components, records of at least two, split
  *     bf16 included), else TRK_HALO_ASYNC.
  * Both give bit-identical results.  A tensor copy that does not complete
- * within its wait limit skips its block and makes tracker_sync return
- * TRK_ECUDA.  Errors: TRK_EINVAL. */
+ * within its wait limit skips the particles that needed it and makes
+ * tracker_sync return TRK_ECUDA.  Errors: TRK_EINVAL. */
 int tracker_set_halo_copy(tracker* t, int kind);
 
 /* Launch shape of the time-step path.  step_kernel: TRK_STEP_COLUMN, _BLOCK

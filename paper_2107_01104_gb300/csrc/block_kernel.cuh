@@ -50,14 +50,12 @@ __device__ __forceinline__ void tma_issue(void* dst, const CUtensorMap* map, int
         : "memory");
 }
 
-// Waits for the barrier's phase `parity` to complete; false after the
-// iteration limit (each try_wait itself suspends for a bounded time), so a
-// copy that never lands cannot hang the kernel.
-constexpr int kTmaWaitLimit = 1 << 22;
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
+// Waits for the barrier's phase `parity` to complete; false after `limit` polls
+// (each try_wait itself suspends for a bounded time).
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int limit)
 {
     const uint32_t a = smem_addr(bar);
-    for (int it = 0; it < kTmaWaitLimit; ++it) {
+    for (int it = 0; it < limit; ++it) {
         uint32_t done = 0;
         asm volatile(
             "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
@@ -127,6 +125,7 @@ __global__ void __launch_bounds__(NT, 4)
     const int nchunks = STEP ? 1 : (a.f.C + NC - 1) / NC;
 
     uint32_t phase = 0;
+    bool hold = false;
     if constexpr (HC == HC_TMA) {
         static_assert(STORE == ST_F64, "node records are staged by k_slabs");
         if (tid == 0) mbar_init(mbar);
@@ -160,14 +159,16 @@ __global__ void __launch_bounds__(NT, 4)
             }
             if (issued) {
                 if constexpr (HC == HC_TMA) {
-                    // if the copy did not land within the limit the block is skipped (all
-                    // threads agree) and the host is told
-                    const bool ok = mbar_wait(mbar, phase);
-                    phase ^= 1u;
+                    // if the copy did not land within the limit (all threads agree) the block's
+                    // particles are held and the host is told; the shared memory is not
+                    // given up while the copy may still write to it
+                    const bool ok = mbar_wait(mbar, phase, a.wait_limit);
                     if (__syncthreads_or(!ok)) {
+                        hold = true;
                         if (tid == 0) atomicOr(a.flags + FLAG_HALO_TIMEOUT, 1);
-                        return;
+                        mbar_wait(mbar, phase, kWaitLimit);
                     }
+                    phase ^= 1u;
                 } else {
                     cp_async_wait_all();
                     __syncthreads();
@@ -182,13 +183,13 @@ __global__ void __launch_bounds__(NT, 4)
             }
             __syncwarp();
             if constexpr (!STEP) {
-                if (valid) write_outputs<T, MODE, NC>(a, id, ch, ws, lane);
+                if (valid && !hold) write_outputs<T, MODE, NC>(a, id, ch, ws, lane);
                 __syncwarp();
             }
         }
         if constexpr (STEP) {
             cp_async_wait_all();
-            update_particle<T, MODE, NC>(a, j, id, valid, ws, lane);
+            update_particle<T, MODE, NC>(a, j, id, valid, ws, lane, hold);
             __syncwarp();
         }
     }
@@ -233,9 +234,10 @@ struct SlabPlan {
     static constexpr int NS = room / slab < 12 ? (int)(room / slab) : 12;
     static constexpr size_t full = NS * slab;                // [NS] mbarriers
     static constexpr size_t done = full + 128;               // [NS] counters
-    static constexpr size_t warp = done + 64;
+    static constexpr size_t issued = done + 64;              // [NS] the last slab copied into the slot
+    static constexpr size_t warp = issued + 64;
     static constexpr size_t total = warp + warps * per_warp;
-    static_assert(NS >= SG::NSL + SG::SPT, "slabs of two adjacent blocks");
+    static_assert(NS >= SG::NSL + SG::SPT && NS <= 16, "slabs of two adjacent blocks; counters");
     static_assert(total <= 232448, "slab shared-memory plan exceeds the per-block limit");
 };
 
@@ -252,7 +254,7 @@ struct Slabs {
     int b_first, b_last;         // the CTA's cell blocks
     int l1, per_row, q0, count;  // log2 nb1; slabs per row of blocks; number of b_first's first slab; slabs of the CTA
     int held = 0, ready = -1;    // this warp: first slab not counted off; last slab waited for
-    bool dead = false;           // a wait ran out: no further waits (the host is told)
+    bool dead = false;           // (this lane's) a wait ran out: no further waits, nothing counted off (give_up)
 
     __device__ __forceinline__ void init()
     {
@@ -271,6 +273,7 @@ struct Slabs {
     {
         return reinterpret_cast<uint64_t*>(smem + SP::full) + q % NS;
     }
+    __device__ __forceinline__ int* issued(int q) const { return reinterpret_cast<int*>(smem + SP::issued) + q % NS; }
     // rows of blocks: x3 inside a segment of 2^lseg blocks, then x2, the segments along x3
     __device__ __forceinline__ void row_origin(int row, int& o2, int& o3) const
     {
@@ -285,6 +288,7 @@ struct Slabs {
     __device__ __forceinline__ void issue(int q) const
     {
         if (q >= count) return;
+        *issued(q) = q;
         const int row = (q + q0) / per_row, pos = (q + q0) - row * per_row;
         const int lo = max(max(pos - SG::NSL + SG::SPT, 0) / SG::SPT + (row << l1), b_first);
         const int hi = min(min(pos / SG::SPT, a.g.nb1 - 1) + (row << l1), b_last);
@@ -301,10 +305,23 @@ struct Slabs {
     {
         while (ready < q) {
             ++ready;
-            if (!dead && !mbar_wait(full(ready), (uint32_t)(ready / NS) & 1u)) {
+            if (!dead && !mbar_wait(full(ready), (uint32_t)(ready / NS) & 1u, a.wait_limit)) {
                 dead = true;
                 atomicOr(a.flags + FLAG_HALO_TIMEOUT, 1);
             }
+        }
+    }
+    // A lane whose wait runs out waits no more, and lane 0, if it is the one, counts no
+    // more slabs off: none is copied over before every warp has seen it land (the other
+    // warps' waits for what then never comes run out too).  The warp's particles stay as
+    // they are from that batch on (its lanes go on over whatever the slots hold), and
+    // before it leaves it waits, up to the full limit, for the copies on their way, those
+    // that it issued itself among them: the shared memory is not given up under them.
+    __device__ __forceinline__ void give_up()
+    {
+        for (int s = 0; s < NS; ++s) {
+            const int q = *static_cast<volatile int*>(issued(s));
+            if (q >= 0) mbar_wait(full(q), (uint32_t)(q / NS) & 1u, kWaitLimit);
         }
     }
     // count this warp off the slabs before q (their reads are consumed)
@@ -313,7 +330,7 @@ struct Slabs {
         while (held < q) {
             need(held);
             __syncwarp();
-            if (lane == 0) {
+            if (lane == 0 && !dead) {
                 int* d = reinterpret_cast<int*>(smem + SP::done) + held % NS;
                 int old;
                 asm volatile("atom.acq_rel.cta.shared::cta.add.s32 %0, [%1], 1;\n"
@@ -359,6 +376,7 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
         for (int s = 0; s < SP::NS; ++s) {
             mbar_init(slabs.full(s));
             reinterpret_cast<int*>(smem_raw + SP::done)[s] = 0;
+            *slabs.issued(s) = -1;
         }
         for (int s = 0; s < SP::NS; ++s) slabs.issue(s);
     }
@@ -383,7 +401,11 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
     for (int64_t b0 = j0; b0 < j1; buf ^= 1) {
         const int64_t bn = b0 + (int64_t)P * nw * rounds;
         const int64_t j = my_index(b0);
-        const int left = (int)min(j1 - b0 - P * warp, (int64_t)P * nw * rounds);
+        // (the same number; how it is formed, and the two calls of update_particle below, tip the
+        // register allocation: gradients 482 and 528 us per step of 2^21 particles at 256^3, RK2
+        // 402 and 385 per 2^20)
+        using Left = std::conditional_t<MODE == MODE_RK2, int64_t, int>;
+        const int left = (int)min((Left)(j1 - b0) - P * warp, (Left)(P * nw * rounds));
         if (left <= 0) break;
         const bool valid = j < j1 && lane / P < rounds;
         int32_t id = 0;   // (loaded where it is needed: a register less meanwhile)
@@ -421,13 +443,16 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
         }
         if (MODE != MODE_ADJ && valid) id = a.id_in ? a.id_in[j] : (int32_t)j;
         __syncwarp();
+        const bool dead = __any_sync(0xffffffffu, slabs.dead);
         if constexpr (is_step<MODE>()) {
             cp_async_wait_all();
-            update_particle<T, MODE, NC>(a, j, id, valid, ws, lane);
+            if (MODE == MODE_RK2 && !dead) update_particle<T, MODE, NC>(a, j, id, valid, ws, lane);
+            else update_particle<T, MODE, NC>(a, j, id, valid, ws, lane, dead);
         } else if constexpr (MODE == MODE_ADJ) {
             cp_async_wait_all();
-            adjoint_particle<T, MODE, NC>(a, j, id, valid, ws, lane);
-        } else if (valid) {
+            if (!dead) adjoint_particle<T, MODE, NC>(a, j, id, valid, ws, lane);
+            else if (valid) hold_adjoint(a, j, wm.recs[buf * 32 + lane]);
+        } else if (valid && !dead) {
             write_outputs<T, MODE, NC>(a, id, slabs.ch, ws, lane);
         }
         __syncwarp();
@@ -436,6 +461,7 @@ __global__ void __launch_bounds__(32 * SlabPlan<I, MODE, NC>::warps, 1)
     }
     cp_async_wait_all();
     slabs.release_to(slabs.count, lane, nw);   // every copy has landed before the CTA ends
+    if (__any_sync(0xffffffffu, slabs.dead)) slabs.give_up();
 }
 
 template <typename T, int I, int DEG, int MODE, int NC, int STORE, int RW, int HC>

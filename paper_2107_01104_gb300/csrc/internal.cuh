@@ -16,8 +16,9 @@ namespace trk {
 // ---------------------------------------------------------------------------
 // FLAG_BINNING: a counting-sort scatter found a block fuller than its count
 // (cannot happen when every step counts what it writes; guarded anyway).
-// FLAG_HALO_TIMEOUT: a tensor copy of a block's halo did not complete within
-// the wait limit (the block was skipped; reported as an internal error).
+// FLAG_HALO_TIMEOUT: a tensor copy of a block's halo or of a slab did not
+// complete within the wait limit (the particles that needed it stay as they
+// were; reported as an internal error).
 enum { FLAG_NONFINITE = 0, FLAG_CFL = 1, FLAG_BINNING = 2, FLAG_HALO_TIMEOUT = 3, NUM_FLAGS = 4 };
 
 // Storage codes (same values as trk_storage in tracker.h).
@@ -132,10 +133,14 @@ struct BlockArgs {
     int ppc;                  // direct kernel: particles per CTA (a multiple of 16), 0 (by size) or PPC_WIDE
     double dt;
     int* flags;
+    int wait_limit;           // polls of a tensor copy's barrier before a wait gives up
     float4* adj;              // MODE_ADJ: [3][np] X* (offsets, cell), mu, dt/2 lambda (grouped) or null
 };
 
 constexpr int PPC_WIDE = -1;
+// polls after which a wait for a tensor copy gives up (each suspends for a
+// bounded time), so that a copy that never lands cannot hang a kernel
+constexpr int kWaitLimit = 1 << 22;
 constexpr int AB_MAX_HIST = 3;   // history entries of the highest supported order (AB4)
 
 // dt-free Adams-Bashforth increment of order q (1..4): sum_j beta^q_j u_{n-j}

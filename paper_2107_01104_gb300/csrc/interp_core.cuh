@@ -833,9 +833,12 @@ __device__ __forceinline__ void write_outputs(const BlockArgs& a, int64_t id, in
     }
 }
 
+// hold: the field did not arrive (FLAG_HALO_TIMEOUT).  The particle stays as it was,
+// position and history, and writes no outputs; its key and block count are those of
+// its position, so that the next binning still finds every particle once.
 template <typename T, int MODE, int NC>
 __device__ __forceinline__ void update_particle(const BlockArgs& a, int64_t j, int32_t id, bool valid,
-                                                const unsigned char* ws, int lane)
+                                                const unsigned char* ws, int lane, bool hold = false)
 {
     using WPl = WarpPlan<T, MODE, NC>;
     const unsigned vm = __ballot_sync(0xffffffffu, valid);
@@ -863,17 +866,18 @@ __device__ __forceinline__ void update_particle(const BlockArgs& a, int64_t j, i
             const double inc = ab_increment(q, k1, [&](int e) { return widen(h[e]); });
             xn = x0 + a.dt * inc;
             // new history: u_n, then the older entries shifted by one
-            a.rhs_out[ax * a.np + j] = (float)k1;
+            a.rhs_out[ax * a.np + j] = hold ? h[0] : (float)k1;
 #pragma unroll
             for (int e = 1; e < AB_MAX_HIST; ++e)
-                if (e < a.ab_order - 1) a.rhs_out[(3 * e + ax) * a.np + j] = h[e - 1];
-            if (MODE == MODE_AB2 && a.out) reinterpret_cast<float*>(a.out)[ax * a.np + id] = (float)k1;
+                if (e < a.ab_order - 1) a.rhs_out[(3 * e + ax) * a.np + j] = hold ? h[e] : h[e - 1];
+            if (MODE == MODE_AB2 && a.out && !hold) reinterpret_cast<float*>(a.out)[ax * a.np + id] = (float)k1;
         }
+        if (hold) xn = x0;
         ok &= split_cell(xn, a.g.inv_delta, a.g.mask, cn[ax]);
         a.pos_out[ax * a.np + j] = xn;
     }
     if constexpr (MODE == MODE_AB2_D) {
-        if (a.out) {
+        if (a.out && !hold) {
 #pragma unroll
             for (int i = 0; i < 9; ++i)
                 reinterpret_cast<float*>(a.out)[i * a.np + id] = (float)((double)kb[3 + i] * a.g.inv_delta);
@@ -929,6 +933,14 @@ __device__ __forceinline__ void adjoint_particle(const BlockArgs& a, int64_t j, 
         o[a.np] = make_float4((float)mu[0], (float)mu[1], (float)mu[2], 0.0f);
         o[2 * a.np] = make_float4((float)(0.5 * dt * lam[0]), (float)(0.5 * dt * lam[1]), (float)(0.5 * dt * lam[2]), 0.0f);
     }
+}
+
+// the adjoint of a particle that is held (update_particle): lambda as it is, nothing for the field gradient
+__device__ __forceinline__ void hold_adjoint(const BlockArgs& a, int64_t j, const PRec<float>& rec)
+{
+    if (!a.adj) return;
+    a.adj[j] = make_float4(rec.t[0], rec.t[1], rec.t[2], rec.cell);
+    a.adj[a.np + j] = a.adj[2 * a.np + j] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // per-warp pointers into its shared memory

@@ -173,6 +173,7 @@ struct tracker {
     CUtensorMap set_tmap[3];          // slabs of I = 4, 6, 8 (batched sets)
     bool set_tmap_ok[3] = {false, false, false};
     int halo_copy = TRK_HALO_AUTO;    // trk_halo_copy: how the block kernel stages its halo
+    int wait_limit = kWaitLimit;      // polls of a tensor copy's barrier (TRK_WAIT_LIMIT)
     bool auto_tma = true;             // TRK_HALO_AUTO's current choice (tensor copies, where there is a map)
     uint32_t* d_counts = nullptr;     // [nblocks] block counts (counting-sort binning of the column path)
     int32_t* d_cursor = nullptr;      // [nblocks] scatter cursors
@@ -517,6 +518,7 @@ BlockArgs base_args(tracker* t)
         }
     a.offsets = t->offsets;
     a.flags = t->d_flags;
+    a.wait_limit = t->wait_limit;
     a.ab_order = 2;
     a.ppc = direct_shape(t->dir_ppc);
     return a;
@@ -918,6 +920,7 @@ int tracker_create(tracker** out, int N, double L, int family, int I, int m, int
         tracker_destroy(t);
         return rc;
     }
+    if (const char* env = getenv("TRK_WAIT_LIMIT")) t->wait_limit = std::max(0, std::min(atoi(env), kWaitLimit));
     load_tune_file(t);
     *out = t;
     return TRK_OK;
@@ -1020,7 +1023,7 @@ int tracker_sync(tracker* t)
     CUDA_TRY(cudaMemset(t->d_flags, 0, sizeof(h)));
     if (h[FLAG_NONFINITE]) return fail(TRK_ENONFINITE, "a position was non-finite or beyond 2^51 cells");
     if (h[FLAG_BINNING]) return fail(TRK_ECUDA, "internal error: block counts did not match the binned particles");
-    if (h[FLAG_HALO_TIMEOUT]) return fail(TRK_ECUDA, "internal error: a halo tensor copy did not complete (block skipped)");
+    if (h[FLAG_HALO_TIMEOUT]) return fail(TRK_ECUDA, "internal error: a tensor copy of the field did not complete (the particles that needed it were skipped)");
     if (h[FLAG_CFL]) return fail(TRK_ECFL, "a particle moved more than one cell in one stage (result computed exactly)");
     return TRK_OK;
 }

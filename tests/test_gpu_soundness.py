@@ -57,3 +57,85 @@ def test_batched_graph_after_the_field_moved(storage):
         assert torch.equal(x, y)
     for x in (t, taker, fresh):
         x.close()
+
+
+# A wait limit of no polls: every wait for a copy of the field gives up, so nothing
+# moves and nothing is written; of one poll: some do, and a particle has either made
+# the step or stayed.  Either way every particle is there once, and the tracker says so.
+def stopped(t):
+    with pytest.raises(trk.TrackerError) as e:
+        t.sync()
+    assert e.value.status == trk.TRK_ECUDA and "did not complete" in str(e.value)
+
+
+@pytest.mark.parametrize("storage,I,kind", [(F32, 4, trk.TRK_STEP_COLUMN), (F32, 6, trk.TRK_STEP_COLUMN),
+                                            (F32, 8, trk.TRK_STEP_BLOCK), (BF16, 6, trk.TRK_STEP_BLOCK),
+                                            (F64, 6, trk.TRK_STEP_BLOCK)])
+@pytest.mark.parametrize("scheme", [trk.TRK_RK2, trk.TRK_AB3])
+def test_waits_that_run_out(monkeypatch, storage, I, kind, scheme):
+    N, n, dt = 64, 70001, 4e-3
+    u, pos = velocity(N, 3), points(n)
+    rhs = 0.1 * torch.cos(pos.float()).repeat(2, 1, 1)
+
+    def tracker(limit):
+        monkeypatch.delenv("TRK_WAIT_LIMIT", raising=False)
+        if limit is not None:
+            monkeypatch.setenv("TRK_WAIT_LIMIT", str(limit))
+        t = trk.Tracker(N, I=I, m=I // 2 - 1, storage=storage)
+        t.set_field(u)
+        t.set_step_kernel(kind)
+        return t
+
+    def advance(t, steps):
+        p, r = pos.clone(), rhs.clone()
+        if scheme == trk.TRK_RK2:
+            t.advance(p, dt, steps)
+            return p, p
+        t.advance(p, dt, steps, scheme, rhs=r, history_valid=2)
+        return p, r
+
+    t = tracker(0)
+    p, r = advance(t, 6)
+    stopped(t)
+    assert torch.equal(p, pos) and (scheme == trk.TRK_RK2 or torch.equal(r, rhs))
+    out = torch.full((3, n), 7.0, dtype=torch.float64 if storage == F64 else torch.float32, device="cuda")
+    t.interpolate(pos, out_dtype=out.dtype, out=out)
+    stopped(t)
+    assert (out == 7).all()
+    t.close()
+
+    whole = tracker(None)
+    want, _ = advance(whole, 1)
+    whole.sync()
+    t = tracker(1)
+    for _ in range(3):
+        p, _ = advance(t, 1)
+        try:
+            t.sync()
+        except trk.TrackerError as e:
+            assert e.status == trk.TRK_ECUDA
+        assert ((p == want).all(0) | (p == pos).all(0)).all()
+    t.close()
+    whole.close()
+
+
+@pytest.mark.parametrize("I", [4, 6, 8])
+def test_adjoint_and_batched_waits_that_run_out(monkeypatch, I):
+    monkeypatch.setenv("TRK_WAIT_LIMIT", "0")
+    N, n = 64, 70001
+    t = trk.Tracker(N, I=I, m=I // 2 - 1, storage=F32)
+    t.set_field(velocity(N, 3))
+    t.set_step_kernel(trk.TRK_STEP_BLOCK)
+    pos = points(n)
+    lam = torch.sin(3 * pos)
+    gf = torch.zeros((3, N, N, N), dtype=torch.float64, device="cuda")
+    gpos, _ = t.adjoint(pos, lam, 4e-3, 3, 2, grad_field=gf)
+    stopped(t)
+    assert torch.equal(gpos, lam) and not gf.any()
+    for deriv in (0, 1):
+        s = dict(pos=pos.clone(), rhs=torch.cos(pos.float()), I=I, m=I // 2 - 1, family=trk.TRK_SPLINE, deriv=deriv,
+                 out=torch.full((9 if deriv else 3, n), 7.0, device="cuda"))
+        t.advance_batched([s], 4e-3, 5, history_valid=True)
+        stopped(t)
+        assert torch.equal(s["pos"], pos) and torch.equal(s["rhs"], torch.cos(pos.float())) and (s["out"] == 7).all()
+    t.close()
