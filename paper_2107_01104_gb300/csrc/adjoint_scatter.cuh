@@ -151,16 +151,22 @@ __global__ void __launch_bounds__(32 * ScatterPlan<I>::WARPS, ScatterPlan<I>::HA
         if (tid < 32) cnt[tid] = 0;
         __syncthreads();
         // one thread per stencil (a particle's two in adjacent lanes): where it goes
-        float4 at = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 at = make_float4(0.f, 0.f, 0.f, 0.f), mu = at;
         int key = -1, slot = 0, n1 = 0, n2 = 0, n3 = 0;
-        if (tid < n) at = (tid & 1) ? a.adj[b0 + (tid >> 1)] : a.rec[b0 + (tid >> 1)];
+        if (tid < n) {
+            at = (tid & 1) ? a.adj[b0 + (tid >> 1)] : a.rec[b0 + (tid >> 1)];
+            mu = a.adj[(1 + (tid & 1)) * a.np + b0 + (tid >> 1)];
+        }
         const int c = __float_as_int(at.w);
-        const bool same = __shfl_xor_sync(0xffffffffu, c, 1) == c;
+        // a stencil with a non-finite factor (or one near the end of the range) is added node by
+        // node: times the zeros that expand the weights it would put NaN into whole planes
+        const bool tame = fabsf(mu.x) + fabsf(mu.y) + fabsf(mu.z) + at.x + at.y + at.z < 1e37f;
+        const bool same = (__shfl_xor_sync(0xffffffffu, c, 1) == c) & tame & __shfl_xor_sync(0xffffffffu, (int)tame, 1);
         if (tid < n) {
             n1 = (((c & 1023) - o1) & mask) - LO;               // first node, relative to the halo
             n2 = (((c >> 10 & 1023) - o2) & mask) - LO;
             n3 = (((c >> 20 & 1023) - o3) & mask) - LO;
-            if ((unsigned)n1 <= (unsigned)(H - I) && (unsigned)n2 <= (unsigned)(H - I) && (unsigned)n3 <= (unsigned)(H - I)) {
+            if ((unsigned)n1 <= (unsigned)(H - I) && (unsigned)n2 <= (unsigned)(H - I) && (unsigned)n3 <= (unsigned)(H - I) && tame) {
                 key = 2 * n2 + (same ? 0 : 1);
                 if (!same) slot = atomicAdd(cnt + key, 1);
                 else if (!(tid & 1)) slot = atomicAdd(cnt + key, 2);
@@ -182,7 +188,6 @@ __global__ void __launch_bounds__(32 * ScatterPlan<I>::WARPS, ScatterPlan<I>::HA
         __syncthreads();
         // its weights, expanded over the halo
         if (tid < n) {
-            const float4 mu = a.adj[(1 + (tid & 1)) * a.np + b0 + (tid >> 1)];
             if (key >= 0) {
                 const int e = off[key] + slot;
                 float4* e1 = reinterpret_cast<float4*>(w1e + e * P::XE);
@@ -198,7 +203,7 @@ __global__ void __launch_bounds__(32 * ScatterPlan<I>::WARPS, ScatterPlan<I>::HA
                     const float w2 = axis_weight<I, DEG>(a.cf, at.y, i);
                     wme[e * I + i] = make_float4(w2 * mu.x, w2 * mu.y, w2 * mu.z, 0.f);
                 }
-            } else {   // X* left the halo (flagged by the gathers): straight into the gradient
+            } else {   // X* left the halo (flagged by the gathers), or not tame: straight into the gradient
 #pragma unroll 1
                 for (int q = 0; q < I * I * I; ++q) {
                     const int ix = q % I, iy = q / I % I, iz = q / (I * I);

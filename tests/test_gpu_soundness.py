@@ -139,3 +139,38 @@ def test_adjoint_and_batched_waits_that_run_out(monkeypatch, I):
         stopped(t)
         assert torch.equal(s["pos"], pos) and torch.equal(s["rhs"], torch.cos(pos.float())) and (s["out"] == 7).all()
     t.close()
+
+
+# A non-finite lambda, and a non-finite node of the field, reach the nodes of the
+# stencils they belong to and no others, whichever way the gradient is scattered.
+@pytest.mark.parametrize("I", [4, 6, 8])
+@pytest.mark.parametrize("what", ["lambda", "field"])
+def test_nonfinite_field_gradient_stays_in_its_stencils(monkeypatch, I, what):
+    N, n = 32, 4099
+    u, pos = velocity(N, 4).float(), points(n)
+    lam = torch.cos(pos)
+    if what == "lambda":
+        lam[1, 17], lam[0, 1234] = math.nan, math.inf
+    else:
+        u[2, 3, 4, 5], u[0, 20, 21, 22] = math.nan, math.inf
+    got = {}
+    for name, kind, scratch in (("gathers", trk.TRK_STEP_DIRECT, None), ("slabs", trk.TRK_STEP_BLOCK, None),
+                                ("atomics", trk.TRK_STEP_BLOCK, "0")):
+        monkeypatch.delenv("TRK_ADJ_SCRATCH_BYTES", raising=False)
+        if scratch is not None:
+            monkeypatch.setenv("TRK_ADJ_SCRATCH_BYTES", scratch)
+        t = trk.Tracker(N, I=I, m=I // 2 - 1, storage=F32)
+        t.set_field(u)
+        t.set_step_kernel(kind)
+        gf = torch.zeros((3, N, N, N), dtype=torch.float64, device="cuda")
+        t.adjoint(pos, lam, 5e-3, 1, 1, grad_field=gf)
+        torch.cuda.synchronize()
+        got[name] = gf
+        t.close()
+    ref = got.pop("gathers")
+    bad = ~torch.isfinite(ref)
+    assert 0 < bad.sum().item() < 0.2 * bad.numel()
+    top = ref[~bad].abs().max().item()
+    for gf in got.values():
+        assert torch.equal(~torch.isfinite(gf), bad)
+        assert (gf - ref)[~bad].abs().max().item() <= 1e-6 * top   # float32 sums within a block
