@@ -232,7 +232,8 @@ int tracker_advance(tracker* t, int64_t np, double* pos, float* rhs, double dt, 
  *     gradients; float64, C = 1 and other block shapes: at every density),
  *     else BLOCK.
  * All kernels perform the same floating-point operations in the same
- * order, so their results are bit-identical.  TRK_STEP_COLUMN on a tracker
+ * order, so their results are bit-identical (per kind of result: see
+ * tracker_advance_batched).  TRK_STEP_COLUMN on a tracker
  * without a column kernel is TRK_EINVAL.  Errors: TRK_EINVAL. */
 int tracker_set_step_kernel(tracker* t, int kind);
 
@@ -340,6 +341,9 @@ typedef struct {
  * 32768 particles and more are re-binned every step, smaller ones step in the
  * caller's arrays (unless arrays of two sets overlap).  The step sequence is
  * captured in a CUDA graph and replayed.
+ * For float32 I = 6 and 8, u is summed in another order beside its gradient
+ * (also in tracker_adjoint): a set with deriv = 1 follows the trajectory of the
+ * same set with deriv = 0 up to float32 rounding of u, not bit for bit.
  * Errors: TRK_EINVAL, TRK_ENOFIELD, TRK_ENOMEM. */
 int tracker_advance_batched(tracker* t, int nsets, const trk_set* sets, double dt, int steps,
                             int history_valid);

@@ -2,7 +2,8 @@
 //
 //   particles  MODE_ADJ of the interpolation kernels (k_slabs, or k_direct for
 //              sparse sets): J(X), J(X*) and the float64 lambda recurrence;
-//              leaves X*, mu and dt/2 lambda in grouped order;
+//              leaves X*, mu and dt/2 lambda in grouped order (X* from a u summed
+//              beside its derivatives: the forward step's up to rounding, contract);
 //   scatter    gfield += W(X)^T mu + W(X*)^T (dt/2 lambda), here.
 //
 // (Float64 fields: adjoint_kernel.cuh.)

@@ -24,8 +24,9 @@
 // 216-node stencil with loads, 56 / 68 / 75 with 1/4, 1/2, all rows as texture
 // fetches; shared memory 45), so every load is a plain one.
 //
-// Everything here gives the same bits whatever kernel runs it: the order of
-// the sums depends on the stencil only.
+// Everything here gives the same bits whatever kernel runs it, with one
+// exception: the order of the sums depends on the stencil and, for float32 I = 6
+// and 8, on whether derivatives are summed beside u (contract).
 #pragma once
 
 #include <type_traits>
@@ -458,7 +459,14 @@ __device__ __forceinline__ void row_sums(const LD& ld, int r, const Weights<T, I
 // The rows are summed from the ends inwards; float32 values of I = 8 in the
 // order a whole warp on one particle sums them in (run_direct_warp): parts
 // {0, 4}, {1, 5}, {6, 2}, {7, 3}, then (p0 + p2) + (p1 + p3); of I = 6 in the
-// order of sixteen lanes: rows 0, 4, 2 plus rows 1, 5, 3.
+// order of sixteen lanes: rows 0, 4, 2 plus rows 1, 5, 3.  With derivatives the
+// order stays from the ends inwards.  So u of a step that also writes gradients, and
+// the u that takes the adjoint to its stage-2 point, differ from the plain step's
+// in the last bits (each is as far from the exact sum); X*, which is u times dt, can
+// then lie on the other side of a face, where the interpolation has the other cell's
+// polynomial.  Summing u in the value's order there as well was measured (256^3):
+// batched sets 7.1 -> 7.7 ms and the gradients' error 5.1e-7 -> 5.4e-7, or, with the
+// rows from the ends inwards and u in parts, 11.7 ms, and the adjoint 36 -> 60 ms.
 template <typename T, int I, int NC, bool D, int GL, bool PACK, class LD>
 __device__ __forceinline__ void contract(const LD& ld, const Weights<T, I, D, GL>& w, T (&out)[D ? 4 * NC : NC])
 {

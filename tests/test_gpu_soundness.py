@@ -1,6 +1,6 @@
 """GPU: what a call keeps for later calls, and what stays apart inside a call:
 captured step graphs against fields set anew, waits that run out, non-finite
-particles, one order of the sums whatever a kernel outputs beside u."""
+particles."""
 import math
 
 import numpy as np
