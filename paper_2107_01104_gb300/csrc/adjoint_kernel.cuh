@@ -140,22 +140,24 @@ __device__ __forceinline__ GlobalLd<T, STORE, I> field_ld(const FieldView& f, in
     return GlobalLd<T, STORE, I>{f, (int)padded_index(f.NP, c1 - LO, c2 - LO, c3 - LO)};
 }
 
-// the halo of three components, through registers
-template <typename T, int STORE, int H, int S2, int S3, int SC>
-__device__ __forceinline__ void stage_halo(T* halo, const FieldView& f, int o1, int o2, int o3)
+// Starts the copies of the halo of three components (cp.async: they land while
+// the particles of the first batch are split; the caller waits).  Threads run
+// along x1 and walk the planes.
+template <int H, int S2, int S3, int SC>
+__device__ __forceinline__ void stage_halo(double* halo, const FieldView& f, int o1, int o2, int o3)
 {
+    constexpr int ROWS = NT / H;   // rows of a plane per pass
+    const int x = threadIdx.x % H, y0 = threadIdx.x / H;
     const int64_t NP = f.NP;
-    for (int e = threadIdx.x; e < H * H * H; e += NT) {
-        const int x = e % H, y = e / H % H, z = e / (H * H);
-        const int64_t n = ((int64_t)(o3 + PAD + z) * NP + (o2 + PAD + y)) * NP + (o1 + PAD + x);
-        T v[3];
-        if constexpr (STORE == ST_F64) {
-            for (int k = 0; k < 3; ++k) v[k] = f.f64[k * f.plane + n];
-        } else {
-            for (int k = 0; k < 3; ++k) v[k] = f.rec[4 * n + k];
+    const double* n0 = f.f64 + ((int64_t)(o3 + PAD) * NP + (o2 + PAD)) * NP + (o1 + PAD) + x;
+    for (int y = y0; y < H && y0 < ROWS; y += ROWS)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double* src = n0 + k * f.plane + y * NP;
+            double* dst = halo + k * SC + y * S2 + x;
+#pragma unroll 5
+            for (int z = 0; z < H; ++z, src += NP * NP, dst += S3) cp_async<8>(dst, src);
         }
-        for (int k = 0; k < 3; ++k) halo[k * SC + z * S3 + y * S2 + x] = v[k];
-    }
 }
 
 template <typename T, int I, int DEG, bool D>
@@ -573,6 +575,9 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
 
     for (int batch = j0; batch < j1; batch += PBA) {
         const int nbat = min(PBA, j1 - batch);
+        // the first batch's halo lands while P1 splits (later batches re-use the buffer
+        // as the previous batch's accumulator until it is flushed)
+        if (HALO && batch == j0) stage_halo<H, S2, S3, SC>(halo, a.f, o1, o2, o3);
         // ---------------- P1 ----------------
         double lam[3] = {0, 0, 0};
         int id = 0;
@@ -598,7 +603,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
             p_cell[tid] = pack_cell(c[0], c[1], c[2]);
         }
         if (batch != j0) __syncthreads();   // the accumulator of the previous batch is flushed
-        if constexpr (HALO) stage_halo<T, STORE, H, S2, S3, SC>(halo, a.f, o1, o2, o3);
+        if (HALO && batch != j0) stage_halo<H, S2, S3, SC>(halo, a.f, o1, o2, o3);
+        if (HALO) cp_async_wait_all();
         __syncthreads();
         // ---------------- Q1: u(X), J(X), J(X*) ----------------
         for (int q = warp; q < nbat; q += NW) {
