@@ -741,6 +741,10 @@ int advance_step(tracker* t, int64_t np, int path, int mode, int ab_order, int h
 constexpr int64_t kTuneMinNp = 32768;   // below this a step is launch-bound: no timing
 constexpr int kTuneStepsPerCand = 2;    // the first run of a kernel may load its module: keep the faster
 
+// What the numbers of a candidate mean, part of the key: lines of a file written when
+// direct_particles counted particles (no such field) are for other kernels.
+constexpr int kTuneShapes = 2;
+
 struct Cand {
     int path, dir_blk, col_seg, tma;
     int ppc = 256;                   // direct kernel: direct_particles
@@ -751,8 +755,8 @@ std::string tune_key(const tracker* t, int64_t np, int mode, int ab_order)
     const double dens = (double)np / ((double)t->N * t->N * t->N);
     const int bucket = (int)std::floor(2.0 * std::log2(dens));   // half-octave density buckets
     char buf[200];
-    snprintf(buf, sizeof(buf), "advance2 N=%d family=%d I=%d m=%d storage=%d sm=%d dens2=%d mode=%d order=%d", t->N,
-             t->family, t->I, t->m, t->storage, t->nsm, bucket, mode, ab_order);
+    snprintf(buf, sizeof(buf), "advance2 N=%d family=%d I=%d m=%d storage=%d sm=%d dens2=%d mode=%d order=%d shapes=%d",
+             t->N, t->family, t->I, t->m, t->storage, t->nsm, bucket, mode, ab_order, kTuneShapes);
     return buf;
 }
 

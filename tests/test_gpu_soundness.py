@@ -174,3 +174,25 @@ def test_nonfinite_field_gradient_stays_in_its_stencils(monkeypatch, I, what):
     for gf in got.values():
         assert torch.equal(~torch.isfinite(gf), bad)
         assert (gf - ref)[~bad].abs().max().item() <= 1e-6 * top   # float32 sums within a block
+
+
+# Tuning lines that an earlier library wrote, whose numbers meant other launch shapes,
+# are not taken over: the workload is timed again.
+def test_tunings_of_earlier_kernels_are_not_used(tmp_path, monkeypatch):
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("TRK_TUNE_CACHE", str(cache))
+    N, n = 64, 40000
+
+    def source():
+        t = trk.Tracker(N, storage=F32)
+        t.set_field(velocity(N, 8))
+        t.advance(points(n), 4e-3, 20)
+        s = t.tuning()["source"]
+        t.close()
+        return s
+
+    assert source() == trk.TRK_TUNE_TIMED and source() == trk.TRK_TUNE_CACHED
+    key = cache.read_text().split("|")[0]
+    old = key[:key.index(" order=") + len(" order=2")]   # the fields the earlier keys had
+    cache.write_text(old + f"|{trk.TRK_STEP_BLOCK} 8 8 0 256\n")
+    assert source() == trk.TRK_TUNE_TIMED
