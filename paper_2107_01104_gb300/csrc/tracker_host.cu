@@ -1130,7 +1130,7 @@ int tracker_set_tuning(tracker* t, const trk_tuning* p)
                  p->direct_particles == 0 ? 256 : p->direct_particles};
     if (!valid_cand(t, c))
         return fail(TRK_EINVAL, "invalid tuning (direct_block a power of two <= N, column_segment a power of two "
-                                "<= %d, direct_particles 128 or 256, a column kernel only for F32 storage with "
+                                "<= %d, direct_particles 64, 128 or 256, a column kernel only for F32 storage with "
                                 "I = 4, 6 and 8^3 blocks)", MAXSEG);
     t->step_kernel = c.path;
     t->halo_copy = p->halo_copy;
@@ -1292,7 +1292,7 @@ int tracker_advance(tracker* t, int64_t np, double* pos, float* rhs, double dt, 
             if (k) hist = std::min(hist + 1, k - 1);
         }
         t->last_kernel = path;
-        t->last_tuning = {path, t->dir_blk, t->col_seg, halo_tmap(t, mode) ? 1 : 0, t->dir_ppc ? t->dir_ppc : 64};
+        t->last_tuning = {path, t->dir_blk, t->col_seg, halo_tmap(t, mode) ? 1 : 0, t->dir_ppc ? t->dir_ppc : 256};
         return TRK_OK;
     }
     if ((rc = ensure_sort(t, np))) return rc;
@@ -1399,7 +1399,7 @@ int tracker_advance(tracker* t, int64_t np, double* pos, float* rhs, double dt, 
         cur ^= 1;
     }
     t->last_kernel = path;
-    t->last_tuning = {path, t->dir_blk, t->col_seg, halo_tmap(t, mode) ? 1 : 0, t->dir_ppc ? t->dir_ppc : 64};
+    t->last_tuning = {path, t->dir_blk, t->col_seg, halo_tmap(t, mode) ? 1 : 0, t->dir_ppc ? t->dir_ppc : 256};
     ProfScope ps(t, PROF_OTHER);
     CUDA_TRY(launch_unpermute_pos(np, t->pos_s[cur], t->id_s[cur], pos, t->stream));
     t->launches += 1;

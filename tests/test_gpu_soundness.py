@@ -196,3 +196,17 @@ def test_tunings_of_earlier_kernels_are_not_used(tmp_path, monkeypatch):
     old = key[:key.index(" order=") + len(" order=2")]   # the fields the earlier keys had
     cache.write_text(old + f"|{trk.TRK_STEP_BLOCK} 8 8 0 256\n")
     assert source() == trk.TRK_TUNE_TIMED
+
+
+# The launch shape an untimed call reports is one that can be fixed: the one by size.
+@pytest.mark.parametrize("n", [5000, 40000])
+def test_reported_launch_shape_is_the_one_by_size(n):
+    t = trk.Tracker(64, storage=F32)
+    t.set_field(velocity(64, 8))
+    t.advance(points(n), 4e-3, 2)
+    info = t.tuning()
+    assert info.pop("source") == trk.TRK_TUNE_DEFAULT and info["direct_particles"] == 256
+    t.set_tuning(**info)
+    t.advance(points(n), 4e-3, 2)
+    assert t.tuning() == dict(info, source=trk.TRK_TUNE_FIXED)
+    t.close()
