@@ -262,6 +262,7 @@ int set_geometry(tracker* t, int bx, int by, int bz)
     t->g.nb3 = N / bz;
     t->nblocks = (int64_t)t->g.nb1 * t->g.nb2 * t->g.nb3;
     t->key_bits = ilog2(t->nblocks);
+    t->gen += 1;                      // captured step graphs bin in the geometry they were captured with
     return ensure_bin(t, t->nblocks);
 }
 

@@ -210,3 +210,28 @@ def test_reported_launch_shape_is_the_one_by_size(n):
     t.advance(points(n), 4e-3, 2)
     assert t.tuning() == dict(info, source=trk.TRK_TUNE_FIXED)
     t.close()
+
+
+# Steps replayed from a graph bin in the block shape of now, not of the capture.
+def test_step_graph_after_the_block_shape_changed():
+    N, n, steps = 64, 40000, 8
+    u, pos = velocity(N, 9), points(n)
+
+    def run(t, edge):
+        trk.tracker_set_block(t.h, edge, edge, edge)
+        p = pos.clone()
+        t.advance(p, 4e-3, steps)
+        t.sync()
+        return p
+
+    t, want = trk.Tracker(N, storage=F32), None
+    t.set_field(u)
+    t.set_step_kernel(trk.TRK_STEP_DIRECT)
+    for edge in (4, 16, 4, 8, 2):
+        fresh = trk.Tracker(N, storage=F32)
+        fresh.set_field(u)
+        fresh.set_step_kernel(trk.TRK_STEP_DIRECT)
+        want = run(fresh, edge)
+        fresh.close()
+        assert torch.equal(run(t, edge), want), edge
+    t.close()
