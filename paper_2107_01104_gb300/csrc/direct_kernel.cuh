@@ -65,8 +65,10 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
     }
     // a.ppc: particles per CTA (every shape gives the same results); 0, by size (us per
     // step, float32 unless noted):
-    //  - float64, bound by its pipe: an even share per resident CTA, so that every SM has
-    //    its warps to the end (128^3, I = 6, 2e5 tracers, RK2: 712, 795 with 60 each).
+    //  - float64, bound by its pipe: an even share per resident CTA in whole rounds of a warp
+    //    (the warps of a CTA that have none cost nothing), so that every SM has its warps to
+    //    the end (128^3, I = 6, RK2, two steps with their binning: 4e4 tracers 348, in rounds of
+    //    a CTA 386; 1e5 762, 811; 2e5 1459, 1487).
     //  - up to 64 each (I = 8: 32), the same (64^3, I = 4, 3.5e4: 12 with 64, 16 with 32,
     //    28 in CTAs of 1024).
     //  - then an eighth of an even share per resident CTA, so that the last wave is short,
@@ -85,7 +87,9 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
         const int64_t n = a.f.NP - 2 * PAD, cells = n * n * n, one_wave = I < 8 ? 64 : 32;
         const int64_t want = !f32 || even <= one_wave ? even : std::max<int64_t>(one_wave, even / 8);
         const bool small = cells * 4 * (int64_t)sizeof(T) > ((int64_t)1 << 30) || I == 8 || (split && 12 * a.np < cells);
-        const int64_t unit = std::max(16, NW * 32 / group_lanes<T, I, MODE, SRC_GLOBAL>());   // a round of the CTA
+        // a round of the CTA; float64, of a warp
+        constexpr int round = 32 / group_lanes<T, I, MODE, SRC_GLOBAL>();
+        const int64_t unit = f32 ? std::max(16, NW * round) : round;
         a.ppc = (int)std::min<int64_t>(!f32 ? 1 << 20 : (small ? 64 : 256) / unit * unit, (want + unit - 1) / unit * unit);
         if (f32 && I == 8 && a.np >= 64 * 16 * (int64_t)nsm && 20 * a.np >= cells) a.ppc = PPC_WIDE;
     }
