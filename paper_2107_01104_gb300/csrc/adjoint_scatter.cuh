@@ -259,20 +259,22 @@ __global__ void __launch_bounds__(32 * ScatterPlan<I>::WARPS, ScatterPlan<I>::HA
     }
 }
 
-// Scatter of a sparse set: four particles at a time per warp (the lane map of
-// the interpolation), one float64 atomic per node and component, both stages in
-// one where X and X* share a cell.  Each pass over the nodes is 3 I^2
+// Scatter of a sparse set: four particles at a time per warp, I = 6 five (the lane
+// maps of the interpolation), one float64 atomic per node and component, both
+// stages in one where X and X* share a cell.  Each pass over the nodes is 3 I^2
 // conversions and atomics per warp (the bound) whether its lanes are busy or
-// not, so the warp first adds its 16 particles at X (with X* where they share a
-// cell), then the X* left over, four at a time again (256^3, I = 6, 1/32 per cell,
-// the whole adjoint of four steps: 9158 -> 6560 us against passes for "shared",
-// "X" and "X*" wherever one of the four differs).
-template <int I, bool TWO>
-__device__ __forceinline__ void add_direct(const AdjScatterArgs& a, const LaneMap<I>& m, int c, bool active,
-                                           const Weights<float, I, false>& wa, const float4& ma,
-                                           const Weights<float, I, false>& wb, const float4& mb)
+// not, so the CTA first adds its particles at X (with X* where they share a cell),
+// then the X* left over, as many per warp again (256^3, I = 6, 1/32 per cell, the
+// whole adjoint of four steps: 9158 -> 6560 us against passes for "shared", "X" and
+// "X*" wherever one of the four differs).  Five particles of six lanes instead of four
+// of eight, two of them idle, and few particles per CTA (its launch): 256^3, I = 6, us
+// per call of two steps, 1e5 particles 1195 -> 893, 6.4e5 3790 -> 3401.
+template <int I, int GL, bool TWO>
+__device__ __forceinline__ void add_direct(const AdjScatterArgs& a, const LaneMap<I, GL>& m, int c, bool active,
+                                           const Weights<float, I, false, GL>& wa, const float4& ma,
+                                           const Weights<float, I, false, GL>& wb, const float4& mb)
 {
-    using M = LaneMap<I>;
+    using M = LaneMap<I, GL>;
     constexpr int LO = I / 2 - 1;
     const int N = a.g.N, mask = a.g.mask;
     const int64_t NN3 = (int64_t)N * N * N;
@@ -293,22 +295,33 @@ __device__ __forceinline__ void add_direct(const AdjScatterArgs& a, const LaneMa
     }
 }
 
-constexpr int SD_ROUNDS = 4;   // of four particles, per warp
+template <int I>
+struct SparseScatter {
+    static constexpr int GL = I == 6 ? 6 : 8, P = 32 / GL;   // lanes per particle, particles at once
+    static constexpr int ROUND = NW * P;                     // particles of a CTA's round
+    static constexpr int ROUNDS = 2;                         // at most
+};
 
 template <int I, int DEG>
-__global__ void __launch_bounds__(NT, 4) k_adj_scatter_direct(const __grid_constant__ AdjScatterArgs a)
+__global__ void __launch_bounds__(NT, 4) k_adj_scatter_direct(const __grid_constant__ AdjScatterArgs a, int rounds)
 {
-    __shared__ __align__(16) float wbuf[NW][2][4][24];
-    __shared__ int rest[NW][4 * SD_ROUNDS];   // particles (from the warp's first) whose X* lies in another cell
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 3;
-    const LaneMap<I> m(lane);
-    Basis<float, I, DEG, false> B;
+    using S = SparseScatter<I>;
+    constexpr int GL = S::GL, P = S::P;
+    __shared__ __align__(16) float wbuf[NW][2][P][24];
+    __shared__ int rest[S::ROUNDS * S::ROUND], nrest;   // particles (from the CTA's first) whose X* lies in another cell
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = GL == 6 ? SixLanes(lane).group : lane / GL;
+    const LaneMap<I, GL> m(lane);
+    const bool act = m.act && lane < GL * P;
+    Basis<float, I, DEG, false, GL> B;
     B.init(a.cf, m);
-    const int64_t first = ((int64_t)blockIdx.x * NW + warp) * 4 * SD_ROUNDS;
-    int nrest = 0;
-    Weights<float, I, false> w0, w1;
-    for (int it = 0; it < SD_ROUNDS; ++it) {
-        const int64_t j = first + 4 * it + g;
+    const int64_t first = (int64_t)blockIdx.x * rounds * S::ROUND;
+    if (threadIdx.x == 0) nrest = 0;
+    __syncthreads();
+    Weights<float, I, false, GL> w0, w1;
+    for (int it = 0; it < rounds; ++it) {
+        const int q = it * S::ROUND + warp * P + g;
+        const int64_t j = first + q;
         const bool live = j < a.np;
         float4 at0{}, at1{}, m0{}, m1{};
         if (live) {
@@ -318,25 +331,25 @@ __global__ void __launch_bounds__(NT, 4) k_adj_scatter_direct(const __grid_const
             m1 = a.adj[2 * a.np + j];
         }
         const bool same = __float_as_int(at0.w) == __float_as_int(at1.w);
-        const unsigned left = __ballot_sync(0xffffffffu, live && !same && (lane & 7) == 0);
-        if (left >> lane & 1u) rest[warp][nrest + __popc(left & ((1u << lane) - 1u))] = 4 * it + g;
-        nrest += __popc(left);
+        if (live && !same && lane == GL * g) rest[atomicAdd(&nrest, 1)] = q;
         if (!same) m1.x = m1.y = m1.z = 0.0f;
         B.eval(at0.x - 0.5f, at0.y - 0.5f, at0.z - 0.5f, m, wbuf[warp][0][g], w0);
         B.eval(at1.x - 0.5f, at1.y - 0.5f, at1.z - 0.5f, m, wbuf[warp][1][g], w1);
-        add_direct<I, true>(a, m, __float_as_int(at0.w), live && m.act, w0, m0, w1, m1);
+        add_direct<I, GL, true>(a, m, __float_as_int(at0.w), live && act, w0, m0, w1, m1);
         __syncwarp();
     }
-    for (int k = 0; k < nrest; k += 4) {
-        const bool live = k + g < nrest;
+    __syncthreads();
+    const int n = nrest;
+    for (int k = warp * P, odd = 0; k < n; k += S::ROUND, odd ^= 1) {
+        const bool live = k + g < n;
         float4 at1{}, m1{};
         if (live) {
-            const int64_t j = first + rest[warp][k + g];
+            const int64_t j = first + rest[k + g];
             at1 = a.adj[j];
             m1 = a.adj[2 * a.np + j];
         }
-        B.eval(at1.x - 0.5f, at1.y - 0.5f, at1.z - 0.5f, m, wbuf[warp][k >> 2 & 1][g], w1);
-        add_direct<I, false>(a, m, __float_as_int(at1.w), live && m.act, w1, m1, w1, m1);
+        B.eval(at1.x - 0.5f, at1.y - 0.5f, at1.z - 0.5f, m, wbuf[warp][odd][g], w1);
+        add_direct<I, GL, false>(a, m, __float_as_int(at1.w), live && act, w1, m1, w1, m1);
         __syncwarp();
     }
 }
@@ -369,8 +382,21 @@ template <int I, int DEG>
 cudaError_t launch_adj_scatter(const AdjScatterArgs& a, int64_t nblocks, cudaStream_t st)
 {
     if (nblocks == 0) {
-        constexpr int per_cta = 4 * SD_ROUNDS * NW;
-        k_adj_scatter_direct<I, DEG><<<(unsigned)((a.np + per_cta - 1) / per_cta), NT, 0, st>>>(a);
+        using S = SparseScatter<I>;
+        static int nsm = 0;
+        if (!nsm) {
+            int dev = 0;
+            cudaError_t e = cudaGetDevice(&dev);
+            if (e != cudaSuccess || (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        }
+        // two rounds while the part of the gradient that the resident CTAs work on at once stays
+        // within half of the L2 (64 MB; the nodes' lines are otherwise fetched again by the next
+        // row of blocks): 256^3, I = 6, us per call of two steps, one round and two: 1e5 891 and
+        // 1005, 2.5e5 1589 and 1548, 6.4e5 3558 and 3401
+        const double share = std::min(1.0, 2.0 * S::ROUND * 4 * nsm / (double)a.np);
+        const int rounds = share * 24.0 * a.g.N * a.g.N * a.g.N <= (double)(1 << 26) ? 2 : 1;
+        const int64_t cta = (int64_t)rounds * S::ROUND;
+        k_adj_scatter_direct<I, DEG><<<(unsigned)((a.np + cta - 1) / cta), NT, 0, st>>>(a, rounds);
         return cudaGetLastError();
     }
     if (a.gscratch) return launch_adj_scatter_t<I, DEG, true>(a, nblocks, st);

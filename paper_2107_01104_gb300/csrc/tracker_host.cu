@@ -628,9 +628,9 @@ double direct_threshold(const tracker* t)
 
 // Below this many particles per grid cell the adjoint runs without halos
 // (direct mode).  Direct against halo mode, us per call of four RK2 steps, 256^3
-// float32: I = 4 3982 / 7246 at 1/16 per cell, 7379 / 10006 at 1/8; I = 6 6560 /
-// 8413 at 1/32 (128^3: 1038 / 1179), 12375 / 9947 at 1/16 (1878 / 1421); I = 8
-// 20063 / 31984 at 1/16, 38857 / 40754 at 1/8.  float64 (both modes bound by its
+// float32: I = 4 3944 / 7194 at 1/16 per cell, 7368 / 9986 at 1/8; I = 6 5770 /
+// 8252 at 1/32 (128^3: 918 / 1173), 10837 / 9804 at 1/16 (1654 / 1415); I = 8
+// 19444 / 31659 at 1/16, 37831 / 40357 at 1/8.  float64 (both modes bound by its
 // pipe): 1/8.
 double adj_direct_density(const tracker* t)
 {
