@@ -293,7 +293,9 @@ typedef struct {
  * kernel TRK_STEP_BLOCK with tensor copies); up to one particle per cell, the
  * direct kernel with block edges 8 and 16 and launch shapes 256 and 128.
  * Other calls use the density rule of tracker_set_step_kernel with the
- * default shape (TRK_TUNE_DEFAULT).  Every
+ * default shape (TRK_TUNE_DEFAULT; the direct kernel's block edge is 8, or 4
+ * for I = 6 and 8 at 0.02 to 0.06 particles per cell on float32 and split-bf16
+ * fields of one to eight times the L2).  Every
  * candidate gives bit-identical steps.  When the environment variable
  * TRK_TUNE_CACHE names a file, decisions are appended to it (one line per
  * workload) and trackers created later read it.

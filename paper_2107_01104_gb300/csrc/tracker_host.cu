@@ -845,6 +845,20 @@ std::vector<Cand> tune_candidates(const tracker* t, int64_t np)
     return c;
 }
 
+// Edge of the direct path's binning blocks where nothing was timed: 8, or 4 for
+// records of a few times the L2 with about one or two particles per 4^3 cells, whose
+// stencils are then fetched from beyond L1 in a better order than the smaller
+// blocks cost in the binning.  One step with its binning, us, edge 8 and 4, float32,
+// RK2: 256^3 I = 6, 5e5 tracers 246 and 240, 7e5 327 and 318; I = 8, 7e5 478 and 467;
+// but 2e5 127 and 130, I = 8 1.5e6 888 and 953, I = 4 7e5 192 and 195; 128^3 I = 6
+// 4e4 48 and 50; 512^3 I = 6 6e6 2664 and 2750.
+int untimed_edge(const tracker* t, int64_t np, int path)
+{
+    const double cells = (double)t->N * t->N * t->N, dens = (double)np / cells, l2s = 16.0 * cells / t->l2_bytes;
+    return path == TRK_STEP_DIRECT && t->storage != TRK_F64 && t->I >= 6 && l2s > 1 && l2s < 8 && dens >= 0.02 && dens < 0.06
+               ? 4 : BLK;
+}
+
 // keys and block counts of the grouped state pos_s[cur] in geometry bg (after
 // a change of binning geometry between two steps)
 int rekey(tracker* t, int64_t np, int cur, const BinGeom& bg)
@@ -1274,7 +1288,7 @@ int tracker_advance(tracker* t, int64_t np, double* pos, float* rhs, double dt, 
             const bool timed = np >= kTuneMinNp && cands.size() >= 2 &&
                                steps >= kTuneStepsPerCand * (int)cands.size() + 2 && cs == cudaStreamCaptureStatusNone;
             if (!timed) cands.clear();
-            apply_cand(t, Cand{path, BLK, 8, 1, 0});
+            apply_cand(t, Cand{path, untimed_edge(t, np, path), 8, 1, 0});
         }
     }
     if (path != TRK_STEP_DIRECT && (rc = check_block_kernel_shape(t))) return rc;

@@ -235,3 +235,22 @@ def test_sparse_field_gradient_rounds(I, m, N, n, dt):
         sync(t, cfl=dt > 0.1)
         t.close()
     assert (gf[0] - gf[1]).abs().max().item() <= 1e-6 * gf[1].abs().max().item()
+
+
+# untimed calls bin by 4^3 or 8^3 cells (256^3: 4^3 from 0.02 to 0.06 per cell for I = 6 and 8):
+# the same steps, and AB history, on either side of the rule and with the edge fixed
+@pytest.mark.parametrize("storage,I,m", [(F32, 6, 2), (BF16, 8, 3)])
+def test_untimed_binning_edge(storage, I, m):
+    N = 256
+    t = trk.Tracker(N, I=I, m=m, storage=storage)
+    t.set_field(synth.velocity_field_torch(N, 20, 5))
+    for n, edge in ((335544, 8), (335545, 4), (400001, 4)):
+        t.set_tuning()
+        pos = points(n)
+        got = steps_of(t, pos, trk.TRK_AB2, steps=5, hist=1)
+        assert t.tuning()["direct_block"] == edge and t.tuning()["source"] == trk.TRK_TUNE_DEFAULT
+        t.set_tuning(step_kernel=trk.TRK_STEP_DIRECT, direct_block=12 - edge)
+        for a, b in zip(got, steps_of(t, pos, trk.TRK_AB2, steps=5, hist=1)):
+            assert torch.equal(a, b)
+    sync(t, cfl=True)
+    t.close()
