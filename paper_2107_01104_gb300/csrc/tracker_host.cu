@@ -1293,7 +1293,8 @@ int tracker_advance(tracker* t, int64_t np, double* pos, float* rhs, double dt, 
     }
     if (path != TRK_STEP_DIRECT && (rc = check_block_kernel_shape(t))) return rc;
     if (np == 0 || steps == 0) return TRK_OK;
-    if (ungrouped(np, path)) {   // every step in place on the caller's arrays
+    // every step in place on the caller's arrays, unless they share memory
+    if (ungrouped(np, path) && !(k && overlap(pos, (size_t)np * 24, rhs, (size_t)np * 12 * (k - 1)))) {
         int hist = k ? history_valid : 0;
         for (int s = 0; s < steps; ++s) {
             BlockArgs a = base_args(t);

@@ -235,3 +235,23 @@ def test_step_graph_after_the_block_shape_changed():
         fresh.close()
         assert torch.equal(run(t, edge), want), edge
     t.close()
+
+
+# Positions and history in overlapping memory: a step starts from both as they were, and
+# the history is written last, in small sets (which step in place) as in large ones.
+def test_history_that_overlaps_the_positions():
+    n = 3000
+    rng = np.random.default_rng(3)
+    bits = (np.int64(0x3FF00000) + rng.integers(0, 1 << 20, 3 * n)) << 32 | 0x3DCCCCCD   # 1 <= x < 2, low word 0.1f
+    buf = torch.from_numpy(bits.view(np.float64)).cuda()
+    pos, rhs = buf.view(3, n), buf.view(torch.float32)[1001:1001 + 3 * n].view(3, n)
+    t = trk.Tracker(32, I=4, m=1, storage=F32)
+    t.set_field(velocity(32, 2))
+    p, r = pos.clone(), rhs.clone()
+    t.advance(p, 4e-3, 2, trk.TRK_AB2, rhs=r, history_valid=1)
+    t.advance(pos, 4e-3, 2, trk.TRK_AB2, rhs=rhs, history_valid=1)
+    t.sync()
+    want = p.clone().reshape(-1)
+    want.view(torch.float32)[1001:1001 + 3 * n] = r.reshape(-1)
+    assert torch.equal(buf.view(torch.int64), want.view(torch.int64))
+    t.close()
