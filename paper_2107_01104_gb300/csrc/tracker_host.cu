@@ -1800,7 +1800,12 @@ int tracker_adjoint(tracker* t, int64_t np, const double* pos0, const double* la
         char* offs = base + align256((size_t)(K + 3) * recs);
         auto seg_off = [&](int i) { return reinterpret_cast<int32_t*>(offs + (size_t)i * off_stride); };
         int32_t* ids = reinterpret_cast<int32_t*>(offs + (size_t)K * off_stride);
-        if (grad_pos0 != lambdaT) CUDA_TRY(cudaMemcpyAsync(grad_pos0, lambdaT, vec * 8, cudaMemcpyDeviceToDevice, t->stream));
+        const double* lam0 = lambdaT;
+        if (grad_pos0 != lambdaT && overlap(grad_pos0, vec * 8, lambdaT, vec * 8)) {   // through scratch
+            lam0 = reinterpret_cast<double*>(adj);
+            CUDA_TRY(cudaMemcpyAsync(adj, lambdaT, vec * 8, cudaMemcpyDeviceToDevice, t->stream));
+        }
+        if (grad_pos0 != lam0) CUDA_TRY(cudaMemcpyAsync(grad_pos0, lam0, vec * 8, cudaMemcpyDeviceToDevice, t->stream));
         if ((rc = ensure_bin(t, t->nblocks))) return rc;
         for (int sg = nseg - 1; sg >= 0; --sg) {
             const int n = std::min(steps, (sg + 1) * K) - sg * K;

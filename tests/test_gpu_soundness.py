@@ -255,3 +255,18 @@ def test_history_that_overlaps_the_positions():
     want.view(torch.float32)[1001:1001 + 3 * n] = r.reshape(-1)
     assert torch.equal(buf.view(torch.int64), want.view(torch.int64))
     t.close()
+
+
+@pytest.mark.parametrize("shift", [-64, 0, 1000])
+def test_adjoint_into_memory_that_overlaps_lambda(shift):
+    n = 5000
+    pos = points(n)
+    buf = torch.cos(torch.arange(3 * n + 2000, dtype=torch.float64, device="cuda"))
+    lam, grad = buf[1000:1000 + 3 * n].view(3, n), buf[1000 + shift:1000 + shift + 3 * n].view(3, n)
+    t = trk.Tracker(32, I=6, m=2, storage=F32)
+    t.set_field(velocity(32, 2))
+    want = trk.tracker_adjoint(t.h, pos, lam.clone(), 4e-3, 3, 2)[0].clone()
+    trk.tracker_adjoint(t.h, pos, lam, 4e-3, 3, 2, grad_pos0=grad)
+    t.sync()
+    assert torch.equal(grad, want)
+    t.close()
