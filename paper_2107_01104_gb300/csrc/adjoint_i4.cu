@@ -1,4 +1,4 @@
-// Adjoint block kernels for kernel width I = 4 (all storages).
+// Adjoint block kernels for kernel width I = 4 (float64 fields).
 #include "adjoint_kernel.cuh"
 
 namespace trk {

@@ -1,4 +1,4 @@
-// Adjoint block kernels for kernel width I = 6 (all storages).
+// Adjoint block kernels for kernel width I = 6 (float64 fields), and the node gather (all).
 #include "adjoint_kernel.cuh"
 
 namespace trk {

@@ -1,4 +1,5 @@
-// Discrete adjoint of one RK2 (Heun) step, per cell block.
+// Discrete adjoint of one RK2 (Heun) step, per cell block, for float64 fields
+// (float32 and split-bf16 ones: adjoint_scatter.cuh; their node gather is here).
 //
 // Forward map (Eq. tracers, RK2): X* = X + dt u(X), X' = X + dt/2 (u(X) + u(X*)).
 // Given lambda = dLoss/dX' per particle, with J = du/dX and W(X) the linear
@@ -120,24 +121,21 @@ struct SmemLd {
 
 
 // Stencils from the stored field: three components of node c + a - (I/2 - 1)
-template <typename T, int STORE, int I>
 struct GlobalLd {
     static constexpr bool kShared = false;
     FieldView f;
     int base;
-    __device__ __forceinline__ T operator()(int k, int a1, int a2, int a3) const
+    __device__ __forceinline__ double operator()(int k, int a1, int a2, int a3) const
     {
-        const int64_t n = base + (a3 * f.NP + a2) * f.NP + a1;
-        if constexpr (STORE == ST_F64) return (T)__ldg(f.f64 + k * f.plane + n);
-        else return (T)__ldg(f.rec + 4 * n + k);
+        return __ldg(f.f64 + k * f.plane + base + (a3 * f.NP + a2) * f.NP + a1);
     }
 };
 
-template <typename T, int STORE, int I>
-__device__ __forceinline__ GlobalLd<T, STORE, I> field_ld(const FieldView& f, int c1, int c2, int c3)
+template <int I>
+__device__ __forceinline__ GlobalLd field_ld(const FieldView& f, int c1, int c2, int c3)
 {
     constexpr int LO = I / 2 - 1;
-    return GlobalLd<T, STORE, I>{f, (int)padded_index(f.NP, c1 - LO, c2 - LO, c3 - LO)};
+    return GlobalLd{f, (int)padded_index(f.NP, c1 - LO, c2 - LO, c3 - LO)};
 }
 
 // Starts the copies of the halo of three components (cp.async: they land while
@@ -501,20 +499,6 @@ constexpr int PBA = 128;   // particles per adjoint batch (keeps the float64 I =
 
 enum { ADJ_SMEM = 0, ADJ_SLAB = 1, ADJ_DIRECT = 2 };   // where the W^T scatter goes (see above)
 
-// two-element vector of T for zeroing shared memory
-template <typename T>
-struct Vec2;
-template <>
-struct Vec2<float> {
-    using type = float2;
-    __device__ static float2 zero() { return make_float2(0.0f, 0.0f); }
-};
-template <>
-struct Vec2<double> {
-    using type = double2;
-    __device__ static double2 zero() { return make_double2(0.0, 0.0); }
-};
-
 template <typename T, int SC>
 struct AdjPlan {
     static constexpr size_t rec = align32((size_t)3 * SC * sizeof(T));
@@ -528,9 +512,10 @@ struct AdjPlan {
     static_assert(total <= 232448, "adjoint shared-memory plan exceeds the per-block limit");
 };
 
-template <typename T, int I, int DEG, int STORE, int AM>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __grid_constant__ AdjArgs a)
+template <int I, int DEG, int AM>
+__global__ void __launch_bounds__(NT, 1) k_adjoint(const __grid_constant__ AdjArgs a)
 {
+    using T = double;
     constexpr bool HALO = AM != ADJ_DIRECT;
     constexpr int H = BLK + I - 1 + 2;
     constexpr int G = I / 2;
@@ -597,8 +582,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
             const int r1 = (c[0] - o1) & mask, r2 = (c[1] - o2) & mask, r3 = (c[2] - o3) & mask;
             const bool in = HALO && r1 >= LO && r1 <= RMAX && r2 >= LO && r2 <= RMAX && r3 >= LO && r3 <= RMAX;
             const int rp = in ? pack_rel(r1, r2, r3) : -1;
-            if constexpr (sizeof(T) == 4) rec.cell = __int_as_float(rp);
-            else rec.cell = __longlong_as_double((long long)rp);
+            rec.cell = cell_as<T>(rp);
             p_rec[tid] = rec;
             p_cell[tid] = pack_cell(c[0], c[1], c[2]);
         }
@@ -609,14 +593,12 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
         // ---------------- Q1: u(X), J(X), J(X*) ----------------
         for (int q = warp; q < nbat; q += NW) {
             const PRec<T> rec = p_rec[q];
-            int rp;
-            if constexpr (sizeof(T) == 4) rp = __float_as_int(rec.cell);
-            else rp = (int)__double_as_longlong(rec.cell);
+            const int rp = cell_of(rec);
             const int r1 = rp & 255, r2 = (rp >> 8) & 255, r3 = (rp >> 16) & 255;
             const int pc = p_cell[q];
             const int c1 = pc & 1023, c2 = (pc >> 10) & 1023, c3 = (pc >> 20) & 1023;
             if (rp >= 0) L.load(SL{halo + (r3 - LO) * S3 + (r2 - LO) * S2 + (r1 - LO)});
-            else L.load(field_ld<T, STORE, I>(a.f, c1, c2, c3));
+            else L.load(field_ld<I>(a.f, c1, c2, c3));
             W.eval(rec.t[0] - (T)0.5, rec.t[1] - (T)0.5, rec.t[2] - (T)0.5, wv, wd);
             T acc[12];
             L.contract(wv, wd, acc);
@@ -645,7 +627,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
                     // left the staged halo, or (direct) moved more than one cell
                     const bool far = HALO || abs(dc[0]) > 1 || abs(dc[1]) > 1 || abs(dc[2]) > 1;
                     if (far && lane == 0) atomicOr(a.flags + FLAG_CFL, 1);
-                    L.load(field_ld<T, STORE, I>(a.f, cs1, cs2, cs3));
+                    L.load(field_ld<I>(a.f, cs1, cs2, cs3));
                 }
             }
             W.eval(ts[0] - (T)0.5, ts[1] - (T)0.5, ts[2] - (T)0.5, wv, wd);
@@ -658,8 +640,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
                 r2c.t[1] = ts[1];
                 r2c.t[2] = ts[2];
                 const int rp2 = in2 ? pack_rel(s1, s2, s3) : -1;
-                if constexpr (sizeof(T) == 4) r2c.cell = __int_as_float(rp2);
-                else r2c.cell = __longlong_as_double((long long)rp2);
+                r2c.cell = cell_as<T>(rp2);
                 p_rec2[q] = r2c;
                 p_cell2[q] = pack_cell(cs1, cs2, cs3);
             }
@@ -709,12 +690,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
             const int64_t NN3g = (int64_t)N * N * N;
             for (int q = warp; q < nbat; q += NW) {
                 const PRec<T> recs[2] = {p_rec[q], p_rec2[q]};
-                int rps[2];
-#pragma unroll
-                for (int stage = 0; stage < 2; ++stage) {
-                    if constexpr (sizeof(T) == 4) rps[stage] = __float_as_int(recs[stage].cell);
-                    else rps[stage] = (int)__double_as_longlong(recs[stage].cell);
-                }
+                const int rps[2] = {cell_of(recs[0]), cell_of(recs[1])};
                 const T mus[2][3] = {{p_mu[q * 6 + 0], p_mu[q * 6 + 1], p_mu[q * 6 + 2]},
                                      {p_mu[q * 6 + 3], p_mu[q * 6 + 4], p_mu[q * 6 + 5]}};
                 const bool same = HALO ? (rps[0] >= 0 && rps[0] == rps[1]) : p_cell[q] == p_cell2[q];
@@ -759,7 +735,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
             continue;
         }
         static_assert(SC % 2 == 0, "the accumulator is zeroed two values at a time");
-        for (int e = tid; e < 3 * SC / 2; e += NT) reinterpret_cast<typename Vec2<T>::type*>(halo)[e] = Vec2<T>::zero();
+        for (int e = tid; e < 3 * SC / 2; e += NT) reinterpret_cast<double2*>(halo)[e] = make_double2(0.0, 0.0);
         __syncthreads();
         const int64_t NN3 = (int64_t)N * N * N;
         auto add_smem = [&](T* base) {
@@ -770,12 +746,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_adjoint(const __
         };
         for (int q = warp; q < nbat; q += NW) {
             const PRec<T> recs[2] = {p_rec[q], p_rec2[q]};
-            int rps[2];
-#pragma unroll
-            for (int stage = 0; stage < 2; ++stage) {
-                if constexpr (sizeof(T) == 4) rps[stage] = __float_as_int(recs[stage].cell);
-                else rps[stage] = (int)__double_as_longlong(recs[stage].cell);
-            }
+            const int rps[2] = {cell_of(recs[0]), cell_of(recs[1])};
             const T mus[2][3] = {{p_mu[q * 6 + 0], p_mu[q * 6 + 1], p_mu[q * 6 + 2]},
                                  {p_mu[q * 6 + 3], p_mu[q * 6 + 4], p_mu[q * 6 + 5]}};
             if (rps[0] >= 0 && rps[0] == rps[1]) {
@@ -925,12 +896,12 @@ __global__ void k_adj_gather(const __grid_constant__ AdjArgs a)
     a.gfield[2 * NN3 + node] += s2;
 }
 
-template <typename T, int I, int DEG, int STORE, int AM>
+template <int I, int DEG, int AM>
 cudaError_t launch_adjoint_g(const AdjArgs& a, int64_t nblocks, cudaStream_t st)
 {
     constexpr int H = BLK + I - 1 + 2;
-    constexpr size_t smem = AdjPlan<T, Layout<I, H>::SC>::total;
-    auto kern = k_adjoint<T, I, DEG, STORE, AM>;
+    constexpr size_t smem = AdjPlan<double, Layout<I, H>::SC>::total;
+    auto kern = k_adjoint<I, DEG, AM>;
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -944,18 +915,12 @@ cudaError_t launch_adjoint_g(const AdjArgs& a, int64_t nblocks, cudaStream_t st)
 
 // no offsets: the direct mode over a.np sorted particles; with per-block
 // scratch the W^T adds go to the block's slab in global memory
-template <typename T, int I, int DEG, int STORE>
-cudaError_t launch_adjoint_t(const AdjArgs& a, int64_t nblocks, cudaStream_t st)
-{
-    if (!a.offsets) return launch_adjoint_g<T, I, DEG, STORE, ADJ_DIRECT>(a, (a.np + PBA - 1) / PBA, st);
-    if (a.gscratch) return launch_adjoint_g<T, I, DEG, STORE, ADJ_SLAB>(a, nblocks, st);
-    return launch_adjoint_g<T, I, DEG, STORE, ADJ_SMEM>(a, nblocks, st);
-}
-
 template <int I, int DEG>
 cudaError_t dispatch_adjoint(const AdjArgs& a, int64_t nblocks, cudaStream_t st)
 {
-    return launch_adjoint_t<double, I, DEG, ST_F64>(a, nblocks, st);
+    if (!a.offsets) return launch_adjoint_g<I, DEG, ADJ_DIRECT>(a, (a.np + PBA - 1) / PBA, st);
+    if (a.gscratch) return launch_adjoint_g<I, DEG, ADJ_SLAB>(a, nblocks, st);
+    return launch_adjoint_g<I, DEG, ADJ_SMEM>(a, nblocks, st);
 }
 
 }  // namespace adj

@@ -282,18 +282,6 @@ __global__ void k_scatter_perm(GridGeom g, int64_t np, const uint32_t* __restric
     write_record<RT>(g, np, pos, j, rec, d, flags);
 }
 
-// Block counts of np keys, one atomic add per group of equal keys in a warp
-// (keys written by a step kernel arrive grouped by the previous binning).
-__global__ void k_count_keys(int64_t np, const uint32_t* __restrict__ keys, uint32_t* __restrict__ counts)
-{
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const unsigned valid = __ballot_sync(0xffffffffu, j < np);
-    if (j >= np) return;
-    const uint32_t key = keys[j];
-    const unsigned peers = __match_any_sync(valid, key);
-    if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(counts + key, (uint32_t)__popc(peers));
-}
-
 __global__ void k_radix_hist(const uint32_t* __restrict__ keys, int64_t n, int shift, int64_t ntiles,
                              uint32_t* __restrict__ tile_hist)
 {
@@ -666,13 +654,6 @@ cudaError_t launch_scatter_perm(const GridGeom& g, int64_t np, const uint32_t* k
     if (np <= 0) return cudaSuccess;
     auto kern = !rec ? k_scatter_perm<void> : (rec_f64 ? k_scatter_perm<double> : k_scatter_perm<float>);
     kern<<<grid_for(np, 256), 256, 0, st>>>(g, np, keys, cursor, pos, perm, rec, flags);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_count_keys(int64_t np, const uint32_t* keys, uint32_t* counts, cudaStream_t st)
-{
-    if (np <= 0) return cudaSuccess;
-    k_count_keys<<<grid_for(np, 256), 256, 0, st>>>(np, keys, counts);
     return cudaGetLastError();
 }
 

@@ -399,8 +399,6 @@ cudaError_t launch_count_scan(uint32_t* counts, int64_t nblocks, int32_t* offset
 // records PRec<float or double> rec[d] of pos (null: none)
 cudaError_t launch_scatter_perm(const GridGeom& g, int64_t np, const uint32_t* keys, int32_t* cursor, const double* pos,
                                 int32_t* perm, void* rec, int rec_f64, int* flags, cudaStream_t st);
-// counts[key] += number of particles with that key
-cudaError_t launch_count_keys(int64_t np, const uint32_t* keys, uint32_t* counts, cudaStream_t st);
 // the same for the particle state, with its records
 cudaError_t launch_scatter_state(const GridGeom& g, int64_t np, const uint32_t* keys, int32_t* cursor,
                                  const double* pos_in, const int32_t* id_in, const float* rhs_in, int rhs_rows,

@@ -261,20 +261,14 @@ struct HaloLd {
     }
 };
 
-// A lane's stencil, its first HR rows held in registers (re-used by RK2's
-// second stage), the others loaded as they are contracted.
-template <typename T, int I, int NC, int HR, class LD>
+// A lane's stencil, its HR rows held in registers (re-used by RK2's second stage)
+template <typename T, int I, int NC, int HR>
 struct HeldLd {
     const T (&f)[HR][LaneMap<I>::NZ][NC];   // (NZ: the same for either group size)
-    const LD& rest;
     __device__ __forceinline__ void operator()(int r, int z, T (&v)[NC]) const
     {
-        if (r < HR) {
 #pragma unroll
-            for (int k = 0; k < NC; ++k) v[k] = f[r < HR ? r : 0][z][k];
-        } else {
-            rest(r, z, v);
-        }
+        for (int k = 0; k < NC; ++k) v[k] = f[r][z][k];
     }
 };
 
@@ -702,10 +696,11 @@ __device__ __forceinline__ void interpolate_stage(const LD& ld, T s1, T s2, T s3
 {
     Weights<T, I, D, GL> w;
     if constexpr (HR > 0) {
+        static_assert(HR == (LaneMap<I, GL>::NY), "all of the lane's rows");
         if (fresh) load_rows<T, I, NC, HR>(ld, f);
         __syncwarp();
         B.eval(s1, s2, s3, m, wb, w);
-        contract<T, I, NC, D, GL, false>(HeldLd<T, I, NC, HR, LD>{f, ld}, w, k);
+        contract<T, I, NC, D, GL, false>(HeldLd<T, I, NC, HR>{f}, w, k);
     } else {
         B.eval(s1, s2, s3, m, wb, w);
         contract<T, I, NC, D, GL, false>(ld, w, k);
