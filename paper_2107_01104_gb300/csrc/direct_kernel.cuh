@@ -65,10 +65,11 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
     }
     // a.ppc: particles per CTA (every shape gives the same results); 0, by size (us per
     // step, float32 unless noted):
-    //  - float64, bound by its pipe: an even share per resident CTA in whole rounds of a warp
-    //    (the warps of a CTA that have none cost nothing), so that every SM has its warps to
-    //    the end (128^3, I = 6, RK2, two steps with their binning: 4e4 tracers 348, in rounds of
-    //    a CTA 386; 1e5 762, 811; 2e5 1459, 1487).
+    //  - float64, bound by its pipe: an even share per resident CTA, so that every SM has its
+    //    warps to the end, in rounds of a warp where that is less for the fullest SM (warps of a
+    //    CTA that have none cost nothing; 128^3, I = 6, RK2, two steps with their binning: 4e4
+    //    tracers 348, in rounds of a CTA 386; 1e5 762, 811; 2e5 1459, 1487), else of a CTA, whose
+    //    warps then end together (32^3, I = 8, RK2, one step: 2e4 tracers 164, 169).
     //  - up to 64 each (I = 8: 32), the same (64^3, I = 4, 3.5e4: 12 with 64, 16 with 32,
     //    28 in CTAs of 1024).
     //  - then an eighth of an even share per resident CTA, so that the last wave is short,
@@ -87,10 +88,13 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
         const int64_t n = a.f.NP - 2 * PAD, cells = n * n * n, one_wave = I < 8 ? 64 : 32;
         const int64_t want = !f32 || even <= one_wave ? even : std::max<int64_t>(one_wave, even / 8);
         const bool small = cells * 4 * (int64_t)sizeof(T) > ((int64_t)1 << 30) || I == 8 || (split && 12 * a.np < cells);
-        // a round of the CTA; float64, of a warp
+        // whole rounds of the CTA, or (float64) of a warp where an SM then has fewer of these in all
         constexpr int round = 32 / group_lanes<T, I, MODE, SRC_GLOBAL>();
-        const int64_t unit = f32 ? std::max(16, NW * round) : round;
-        a.ppc = (int)std::min<int64_t>(!f32 ? 1 << 20 : (small ? 64 : 256) / unit * unit, (want + unit - 1) / unit * unit);
+        const auto ceil_to = [](int64_t x, int64_t u) { return (x + u - 1) / u * u; };
+        const auto per_sm = [&](int64_t p) { return ceil_to(ceil_to(a.np, p) / p, nsm) / nsm * ceil_to(p, round); };
+        int64_t unit = f32 ? std::max(16, NW * round) : NW * round;
+        if (!f32 && per_sm(ceil_to(want, round)) < per_sm(ceil_to(want, unit))) unit = round;
+        a.ppc = (int)std::min<int64_t>(!f32 ? 1 << 20 : (small ? 64 : 256) / unit * unit, ceil_to(want, unit));
         if (f32 && I == 8 && a.np >= 64 * 16 * (int64_t)nsm && 20 * a.np >= cells) a.ppc = PPC_WIDE;
     }
     if (a.ppc == PPC_WIDE) {
