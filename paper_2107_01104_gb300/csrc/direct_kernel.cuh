@@ -75,19 +75,24 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
     //  - then an eighth of an even share per resident CTA, so that the last wave is short,
     //    up to 256, which keeps a CTA's stencils close together (256^3, I = 4, AB2, 2^21: 235
     //    with 256, 356 with 64).
-    //  - at most 64 on a field of many times the L2, whose concurrent CTAs then share what
-    //    they pull into it (512^3, I = 8, 9e5, AB2: 573 with 64, 702 with 256), for I = 8
-    //    (256^3, 5e5, RK2: 322, 352 with 256) and for RK2's sixteen lanes on sets below
-    //    1/12 per cell (256^3, 8e5: 314 with 64, 330 with 1024).
-    //  - I = 8 from 1/20 per cell on: CTAs that fill an SM, whose warps share one neighbourhood of
-    //    the field in L1 (PPC_WIDE; 256^3, 2^21, RK2: 1126, 1229 with 256, 1258 with 64).
+    //  - at most 64 on sets below 1/80 per cell in a field of many times the L2 (records above
+    //    1 GB), whose concurrent CTAs then share what they pull into it (512^3, AB2, 64 and
+    //    256: 1e6 I = 4 266, 288, I = 6 430, 468, I = 8 584, 641; but 3e6 492, 457 and 966, 846
+    //    and 1406, 1353; 3e7 I = 4 4610, 2943; 1024^3, I = 6, 6e6 3191, 3541, 2e7 6437, 6189).
+    //    In smaller fields for I = 8 (256^3, 5e5, RK2: 322, 352 with 256) and for RK2's
+    //    sixteen lanes on sets below 1/12 per cell (256^3, 8e5: 314 with 64, 330 with 1024).
+    //  - I = 8 from 1/20 per cell on (big fields 1/32), sets of at least one such CTA per SM: CTAs
+    //    that fill an SM, whose warps share one neighbourhood of the field in L1 (PPC_WIDE;
+    //    256^3, 2^21, RK2: 1126, 1229 with 256, 1258 with 64; 4e5 264, 244 with 64; 512^3, 4.5e6
+    //    2504, 2585 with 256, 3e6 1800, 1763).
     int nw = NW;
     if (a.ppc == 0) {
         constexpr bool split = group_lanes<T, I, MODE, SRC_GLOBAL>() == 16, f32 = sizeof(T) == 4;
         const int64_t even = (a.np + (int64_t)nsm * ctas_sm - 1) / ((int64_t)nsm * ctas_sm);
         const int64_t n = a.f.NP - 2 * PAD, cells = n * n * n, one_wave = I < 8 ? 64 : 32;
         const int64_t want = !f32 || even <= one_wave ? even : std::max<int64_t>(one_wave, even / 8);
-        const bool small = cells * 4 * (int64_t)sizeof(T) > ((int64_t)1 << 30) || I == 8 || (split && 12 * a.np < cells);
+        const bool big = cells * 16 > (int64_t)1 << 30;
+        const bool small = big ? 80 * a.np < cells : I == 8 || (split && 12 * a.np < cells);
         // whole rounds of the CTA, or (float64) of a warp where an SM then has fewer of these in all
         constexpr int round = 32 / group_lanes<T, I, MODE, SRC_GLOBAL>();
         const auto ceil_to = [](int64_t x, int64_t u) { return (x + u - 1) / u * u; };
@@ -95,7 +100,7 @@ cudaError_t launch_direct_t(BlockArgs a, cudaStream_t st)
         int64_t unit = f32 ? std::max(16, NW * round) : NW * round;
         if (!f32 && per_sm(ceil_to(want, round)) < per_sm(ceil_to(want, unit))) unit = round;
         a.ppc = (int)std::min<int64_t>(!f32 ? 1 << 20 : (small ? 64 : 256) / unit * unit, ceil_to(want, unit));
-        if (f32 && I == 8 && a.np >= 64 * 16 * (int64_t)nsm && 20 * a.np >= cells) a.ppc = PPC_WIDE;
+        if (f32 && I == 8 && a.np >= 64 * 16 * (int64_t)nsm && (big ? 32 : 20) * a.np >= cells) a.ppc = PPC_WIDE;
     }
     if (a.ppc == PPC_WIDE) {
         nw = maxw;

@@ -619,7 +619,10 @@ constexpr double kDirectDensity = 0.05;
 
 // Without the column order (float64 or split-bf16 storage, I = 8, other block
 // shapes): block against direct, us per RK2 step: float32 I = 8, 256^3, 1/8 per
-// cell: 1204 / 1103, 1/4 1959 / 2073; float64 I = 6, 128^3, 0.1 per cell 950 / 712, 1/2 4460 / 3450.
+// cell: 1204 / 1103, 1/4 1959 / 2073.  float64, 128^3: I = 4 986 / 936 at 1/4 per
+// cell, 7616 / 7411 at 2; I = 6 2373 / 1804, 18520 / 14277; I = 8 4627 / 3579, at 1
+// 17468 / 14264: direct is ahead at every density, and a timed call chooses it; the
+// rule of untimed calls, which tracker_step_kernel_for reports, is the storages' common one.
 double direct_threshold(const tracker* t)
 {
     if (!column_available(t)) return 0.25;
@@ -649,6 +652,9 @@ bool ungrouped(int64_t np, int path) { return path == TRK_STEP_DIRECT && np < kU
 
 // Below this many particles a step is latency, whatever the density: direct
 // gathers in one launch (without the column order: up to the ungrouped limit).
+// Column order and direct, us per RK2 step of a call of eight: 16^3, I = 6, 8000
+// particles (two per cell) 17 / 10; 64^3, I = 4, 20 / 8; up to the ungrouped limit
+// direct stays ahead there (32^3, I = 6, 32000: 27 / 18).
 constexpr int64_t kSmallNp = 8192;
 
 // The kernel tracker_advance (and, between BLOCK and DIRECT, tracker_interpolate)
