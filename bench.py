@@ -941,6 +941,7 @@ def tuner_table(trk, dev, stream, dev_index, args, fma):
     Nt = 256
     field = torch.from_numpy(synth.velocity_field_np(Nt, 85, 1001).astype("float32")).to(dev)
     rows = []
+    # direct_particles: 256 the shape by size, 128 thread blocks of 256 particles, 64 of 64
     cands = [("column seg 4", dict(step_kernel=trk.TRK_STEP_COLUMN, column_segment=4)),
              ("column seg 8", dict(step_kernel=trk.TRK_STEP_COLUMN, column_segment=8)),
              ("column seg 16", dict(step_kernel=trk.TRK_STEP_COLUMN, column_segment=16)),
@@ -949,9 +950,9 @@ def tuner_table(trk, dev, stream, dev_index, args, fma):
              ("direct edge 8", dict(step_kernel=trk.TRK_STEP_DIRECT, direct_block=8)),
              ("direct edge 16", dict(step_kernel=trk.TRK_STEP_DIRECT, direct_block=16)),
              ("direct edge 32", dict(step_kernel=trk.TRK_STEP_DIRECT, direct_block=32)),
-             ("direct edge 8, 128 per CTA", dict(step_kernel=trk.TRK_STEP_DIRECT, direct_block=8, direct_particles=128)),
-             ("direct edge 16, 128 per CTA", dict(step_kernel=trk.TRK_STEP_DIRECT, direct_block=16,
-                                                   direct_particles=128)),
+             ("direct edge 8, 256 per CTA", dict(step_kernel=trk.TRK_STEP_DIRECT, direct_block=8, direct_particles=128)),
+             ("direct edge 16, 256 per CTA", dict(step_kernel=trk.TRK_STEP_DIRECT, direct_block=16,
+                                                  direct_particles=128)),
              ("direct edge 8, 64 per CTA", dict(step_kernel=trk.TRK_STEP_DIRECT, direct_block=8, direct_particles=64))]
     names = {trk.TRK_STEP_COLUMN: "column", trk.TRK_STEP_BLOCK: "block", trk.TRK_STEP_DIRECT: "direct"}
     for scheme, sname in ((trk.TRK_RK2, "RK2"), (trk.TRK_AB2, "AB2")):
