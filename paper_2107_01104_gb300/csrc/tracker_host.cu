@@ -857,7 +857,8 @@ std::vector<Cand> tune_candidates(const tracker* t, int64_t np)
 // blocks cost in the binning.  One step with its binning, us, edge 8 and 4, float32,
 // RK2: 256^3 I = 6, 5e5 tracers 246 and 240, 7e5 327 and 318; I = 8, 7e5 478 and 467;
 // but 2e5 127 and 130, I = 8 1.5e6 888 and 953, I = 4 7e5 192 and 195; 128^3 I = 6
-// 4e4 48 and 50; 512^3 I = 6 6e6 2664 and 2750.
+// 4e4 48 and 50; 512^3 I = 6 6e6 2664 and 2750.  (Not while the stream is being captured:
+// the smaller blocks may need larger binning arrays.)
 int untimed_edge(const tracker* t, int64_t np, int path)
 {
     const double cells = (double)t->N * t->N * t->N, dens = (double)np / cells, l2s = 16.0 * cells / t->l2_bytes;
@@ -1294,7 +1295,7 @@ int tracker_advance(tracker* t, int64_t np, double* pos, float* rhs, double dt, 
             const bool timed = np >= kTuneMinNp && cands.size() >= 2 &&
                                steps >= kTuneStepsPerCand * (int)cands.size() + 2 && cs == cudaStreamCaptureStatusNone;
             if (!timed) cands.clear();
-            apply_cand(t, Cand{path, untimed_edge(t, np, path), 8, 1, 0});
+            apply_cand(t, Cand{path, cs == cudaStreamCaptureStatusNone ? untimed_edge(t, np, path) : BLK, 8, 1, 0});
         }
     }
     if (path != TRK_STEP_DIRECT && (rc = check_block_kernel_shape(t))) return rc;

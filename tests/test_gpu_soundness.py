@@ -270,3 +270,26 @@ def test_adjoint_into_memory_that_overlaps_lambda(shift):
     t.sync()
     assert torch.equal(grad, want)
     t.close()
+
+
+# A step captured by the caller, on a tracker whose buffers a larger set has sized, allocates
+# nothing whatever the density.
+def test_captured_step_after_a_larger_set():
+    N = 256
+    t = trk.Tracker(N, I=8, m=3, storage=F32)
+    t.set_field(synth.velocity_field_torch(N, 20, 5))
+    big, pos = points(1100000), points(500000)       # bins of 8^3 and, outside a capture, 4^3 cells
+    t.advance(big, 1e-3, 1)
+    p = pos.clone()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        t.advance(p, 1e-3, 1)
+    p.copy_(pos)
+    g.replay()
+    torch.cuda.synchronize()
+    want = pos.clone()
+    t.advance(want, 1e-3, 1)
+    t.sync()
+    assert torch.equal(p, want)
+    t.close()
