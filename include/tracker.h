@@ -103,9 +103,9 @@ int tracker_set_stream(tracker* t, void* stream);
 /* Wait for the tracker's stream, then read and clear the device flags:
  * returns TRK_ENONFINITE or TRK_ECFL if a kernel raised one since the
  * last sync, else TRK_OK (or TRK_ECUDA).  TRK_ECUDA with "a tensor copy of
- * the field did not complete" means that a wait inside a kernel ran out (after
- * 2^22 polls, or the environment variable TRK_WAIT_LIMIT at creation, if that
- * is less): the particles that needed the copy stayed as they were in that
+ * the field did not complete" means that a wait inside a kernel ran out (2^20
+ * polls, 1.5 s; fewer with the environment variable TRK_WAIT_LIMIT, a number of
+ * polls, at creation): the particles that needed the copy stayed as they were in that
  * step (position, history, lambda; no outputs were written), the others did not. */
 int tracker_sync(tracker* t);
 

@@ -321,7 +321,8 @@ struct Slabs {
     {
         for (int s = 0; s < NS; ++s) {
             const int q = *static_cast<volatile int*>(issued(s));
-            if (q >= 0) mbar_wait(full(q), (uint32_t)(q / NS) & 1u, kWaitLimit);
+            // (one that does not land leaves the others no less time)
+            if (q >= 0 && !mbar_wait(full(q), (uint32_t)(q / NS) & 1u, kWaitLimit)) break;
         }
     }
     // count this warp off the slabs before q (their reads are consumed)

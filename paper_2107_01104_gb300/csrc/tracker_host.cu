@@ -946,7 +946,11 @@ int tracker_create(tracker** out, int N, double L, int family, int I, int m, int
         tracker_destroy(t);
         return rc;
     }
-    if (const char* env = getenv("TRK_WAIT_LIMIT")) t->wait_limit = std::max(0, std::min(atoi(env), kWaitLimit));
+    if (const char* env = getenv("TRK_WAIT_LIMIT")) {   // (anything but a number: the default)
+        char* end = nullptr;
+        const long v = strtol(env, &end, 10);
+        if (end != env && *end == 0) t->wait_limit = (int)std::max(0L, std::min(v, (long)kWaitLimit));
+    }
     load_tune_file(t);
     *out = t;
     return TRK_OK;

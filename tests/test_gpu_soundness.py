@@ -293,3 +293,14 @@ def test_captured_step_after_a_larger_set():
     t.sync()
     assert torch.equal(p, want)
     t.close()
+
+
+@pytest.mark.parametrize("value", ["", "none", "12x"])
+def test_wait_limit_that_is_no_number(monkeypatch, value):
+    monkeypatch.setenv("TRK_WAIT_LIMIT", value)
+    t = trk.Tracker(32, storage=F32)
+    t.set_field(velocity(32, 2))
+    p = points(40000)
+    t.advance(p, 4e-3, 2)
+    t.sync()
+    t.close()
